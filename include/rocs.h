@@ -82,11 +82,12 @@ rocs_status_t rocs_set_path(rocs_path_t path);
  *                      tile planning use it and the call does not synchronise; when NULL
  *                      the offsets are copied back from the device (the call synchronises
  *                      `stream`).
- * The plan owns device arrays of O(N + number of tiles) int32, allocated and freed in stream
- * order on `stream` (from a memory pool of the library's own, which keeps what a destroyed plan
- * frees for the next plan instead of returning it to the driver); use the plan on that stream, or order other streams
- * behind it yourself.  Tile lists for a given number of rows per candidate are created on
- * first use by the attention / interaction calls (one allocation + copy) and cached.
+ * The plan owns device arrays of O(N + number of tiles) int32 (from a memory pool of the library's
+ * own, which keeps what a destroyed plan frees for the next plan instead of returning it to the
+ * driver): the candidate-to-request map and the work lists of the attention / interaction calls.
+ * Each is made on the stream of the first call that needs it (one allocation + one launch), kept
+ * for that stream's later calls, and freed in stream order on `stream`; use the plan on that
+ * stream, or order other streams behind it (and it behind them before the plan is destroyed).
  * Errors: INVALID_ARG, SEGMENTS, CUDA.
  */
 rocs_status_t rocs_plan_create(rocs_plan_t** out, int32_t R, int64_t N,

@@ -36,7 +36,7 @@ __device__ uint32_t g_device_status;
 
 }  // namespace
 
-// Stream-ordered allocations of the plan (request ids, work lists) come from a pool of the library's
+// Stream-ordered allocations of the plan's lists (request ids, tiles, items) come from a pool of the library's
 // own that keeps freed memory instead of returning it to the driver at the next synchronisation: a
 // serving loop builds and drops one plan per batch, and with the default pool's zero release
 // threshold every batch would pay the driver's allocation path again.
@@ -74,135 +74,162 @@ uint32_t* device_status_word() {
   return p;
 }
 
-// Work lists are expanded on the device: the host only adds up the tile counts of the R requests
-// (tile_base, R + 1 integers), every list entry then finds its request by binary search in that
-// prefix array, so a batch with hundreds of thousands of entries costs one small copy and one launch.
-__global__ void expand_tiles_kernel(int32_t R, int32_t total, int32_t cands_per_tile,
-                                    const int32_t* __restrict__ off, const int32_t* __restrict__ tile_base,
-                                    Tile* __restrict__ out) {
-  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  int32_t lo = 0, hi = R;  // largest r with tile_base[r] <= i
-  while (hi - lo > 1) {
-    const int32_t mid = lo + (hi - lo) / 2;
-    if (tile_base[mid] <= i) lo = mid; else hi = mid;
+// Work lists are expanded on the device from the offsets alone: every block adds up the list entries
+// ceil(n_r / cands_per_tile) of the R requests into a prefix array in its shared memory, every entry then
+// finds its request by binary search in it.  One launch and no host copy per list: adding up on the host
+// also takes a staged copy to the device and an allocation for it (plan + query projection + attention of
+// 3 requests x 574 candidates: 49.5 us that way, 42.3 us this way; plan + interaction of 128 x 1024
+// candidates: 159.6 and 156.4 us).  All blocks read the same R offsets, from L2; beyond kMaxScan requests
+// (the 48 KB of shared memory a block has without asking for more) the host adds up.
+constexpr int kListThreads = 256;
+constexpr int32_t kMaxScan = 12000;
+
+// Prefix sums of the entries per request in shared memory; all threads of the block take part.
+__device__ void scan_entries(int32_t R, int32_t cands_per_tile, const int32_t* __restrict__ off, int32_t* pre) {
+  __shared__ int32_t warp_sum[kListThreads / 32];
+  for (int32_t r = threadIdx.x; r < R; r += kListThreads) pre[r] = (off[r + 1] - off[r] + cands_per_tile - 1) / cands_per_tile;
+  __syncthreads();
+  const int32_t chunk = (R + kListThreads - 1) / kListThreads;
+  const int32_t r0 = min((int32_t)threadIdx.x * chunk, R), r1 = min(r0 + chunk, R);
+  int32_t sum = 0;
+  for (int32_t r = r0; r < r1; ++r) sum += pre[r];
+  int32_t incl = sum;
+  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += up;
   }
-  const int32_t c = off[lo] + (i - tile_base[lo]) * cands_per_tile;
-  out[i] = Tile{lo, c, min(cands_per_tile, off[lo + 1] - c), 0};
+  if (lane == 31) warp_sum[warp] = incl;
+  __syncthreads();
+  int32_t acc = incl - sum;
+  for (int w = 0; w < warp; ++w) acc += warp_sum[w];
+  for (int32_t r = r0; r < r1; ++r) {
+    const int32_t n = pre[r];
+    pre[r] = acc;
+    acc += n;
+  }
+  if (r1 == R && r0 < R) pre[R] = acc;
+  __syncthreads();
 }
 
-// Attention items in the order request, head, tile (or tile pair).
-__global__ void expand_dca_items_kernel(int32_t R, int32_t total, int32_t cands_per_tile, int32_t heads,
-                                        int32_t tiles_per_item, const int32_t* __restrict__ off,
-                                        const int32_t* __restrict__ item_base, DcaItem* __restrict__ out) {
-  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  int32_t lo = 0, hi = R;  // largest r with item_base[r] * heads <= i
+// Entry i of the list is entry `local` of request `req`, which has `per_head` of them for every head.
+__device__ __forceinline__ void find_entry(int32_t R, int32_t heads, const int32_t* __restrict__ base, int32_t i,
+                                           int32_t& req, int32_t& local, int32_t& per_head) {
+  int32_t lo = 0, hi = R;  // largest r with base[r] * heads <= i
   while (hi - lo > 1) {
     const int32_t mid = lo + (hi - lo) / 2;
-    if ((int64_t)item_base[mid] * heads <= i) lo = mid; else hi = mid;
+    if ((int64_t)base[mid] * heads <= i) lo = mid; else hi = mid;
   }
-  const int32_t per_head = item_base[lo + 1] - item_base[lo];
-  const int32_t local = i - item_base[lo] * heads;
+  req = lo;
+  local = i - base[lo] * heads;
+  per_head = base[lo + 1] - base[lo];
+}
+
+// heads == 0: interaction tiles, in the order request, tile.  heads > 0: attention items, in the order
+// request, head, tile.  base: prefix sums of the entries per request, or null to add them up here.
+__global__ void __launch_bounds__(kListThreads) expand_list_kernel(int32_t R, int32_t total, int32_t cands_per_tile,
+                                                                   int32_t heads, const int32_t* __restrict__ off,
+                                                                   const int32_t* __restrict__ base,
+                                                                   void* __restrict__ out) {
+  extern __shared__ int32_t pre[];
+  if (base == nullptr) {
+    scan_entries(R, cands_per_tile, off, pre);
+    base = pre;
+  }
+  const int32_t i = blockIdx.x * kListThreads + threadIdx.x;
+  if (i >= total) return;
+  int32_t req, local, per_head;
+  find_entry(R, max(heads, 1), base, i, req, local, per_head);
   const int32_t h = local / per_head, t = local % per_head;
-  const int32_t c = off[lo] + t * tiles_per_item * cands_per_tile, c_end = off[lo + 1];
-  const int32_t a = min(cands_per_tile, c_end - c);
-  const int32_t b = tiles_per_item == 2 ? min(cands_per_tile, c_end - c - a) : 0;
-  out[i] = DcaItem{lo, c, (int16_t)a, (int16_t)b, h};
+  const int32_t c = off[req] + t * cands_per_tile;
+  const int32_t count = min(cands_per_tile, off[req + 1] - c);
+  if (heads == 0)
+    static_cast<Tile*>(out)[i] = Tile{req, c, count, 0};
+  else
+    static_cast<DcaItem*>(out)[i] = DcaItem{req, c, count, h};
 }
 
-// Prefix sums of ceil(n_r / per_entry) over the requests, copied to the device.  Returns the total
-// through *total; *base_dev is a stream-ordered allocation the caller frees after its kernel.
-static rocs_status_t upload_entry_base(const rocs_plan* plan, int32_t per_entry, cudaStream_t stream,
-                                       int32_t** base_dev, int64_t* total) {
-  std::vector<int32_t> base((size_t)plan->R + 1);
-  int64_t acc = 0;
-  for (int32_t r = 0; r < plan->R; ++r) {
-    base[r] = (int32_t)acc;
-    const int64_t n = (int64_t)plan->offsets_host[r + 1] - plan->offsets_host[r];
-    acc += (n + per_entry - 1) / per_entry;
-    if (acc > 0x7fffffffLL) return ROCS_ERR_UNSUPPORTED;
+static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, cudaStream_t stream,
+                               DeviceList* out) {
+  static_assert(sizeof(Tile) == 16 && sizeof(DcaItem) == 16, "list entries");
+  unsigned long long id = 0;
+  ROCS_CUDA_TRY(cudaStreamGetId(stream, &id));
+  std::lock_guard<std::mutex> lock(plan->mu);
+  const auto key = std::make_tuple(id, cands_per_tile, heads);
+  auto it = plan->lists.find(key);
+  if (it != plan->lists.end()) {
+    *out = it->second;
+    return ROCS_OK;
   }
-  base[plan->R] = (int32_t)acc;
-  *total = acc;
-  ROCS_CUDA_TRY(pool_alloc((void**)base_dev, sizeof(int32_t) * base.size(), stream));
-  // Pageable source: the copy is staged before the call returns, so `base` may go away.
-  if (cudaMemcpyAsync(*base_dev, base.data(), sizeof(int32_t) * base.size(), cudaMemcpyHostToDevice, stream) !=
-      cudaSuccess) {
-    cudaFreeAsync(*base_dev, stream);
+  DeviceList list;
+  if (plan->N > 0 && cands_per_tile == 0) {
+    ROCS_CUDA_TRY(pool_alloc(&list.dev, sizeof(int32_t) * (size_t)plan->N, stream));
+    fill_row2req_kernel<<<(unsigned)((plan->N + 255) / 256), 256, 0, stream>>>(plan->R, plan->N, plan->cand_offsets,
+                                                                              static_cast<int32_t*>(list.dev));
+  } else if (plan->N > 0) {
+    const int32_t R = plan->R;
+    std::vector<int32_t> base(R > kMaxScan ? (size_t)R + 1 : 0);
+    int64_t entries = 0;
+    for (int32_t r = 0; r < R; ++r) {
+      if (R > kMaxScan) base[r] = (int32_t)entries;
+      const int64_t n = (int64_t)plan->offsets_host[r + 1] - plan->offsets_host[r];
+      entries += (n + cands_per_tile - 1) / cands_per_tile;
+    }
+    const int64_t total = entries * std::max(heads, 1);
+    if (total > 0x7fffffffLL) return ROCS_ERR_UNSUPPORTED;
+    list.num = (int32_t)total;
+    ROCS_CUDA_TRY(pool_alloc(&list.dev, sizeof(Tile) * (size_t)total, stream));
+    int32_t* base_dev = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (R > kMaxScan) {
+      base[R] = (int32_t)entries;
+      e = pool_alloc((void**)&base_dev, sizeof(int32_t) * base.size(), stream);
+      // Pageable source: the copy is staged before the call returns, so `base` may go away.
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(base_dev, base.data(), sizeof(int32_t) * base.size(), cudaMemcpyHostToDevice, stream);
+    }
+    if (e == cudaSuccess)
+      expand_list_kernel<<<(unsigned)((total + kListThreads - 1) / kListThreads), kListThreads,
+                           base_dev ? 0 : sizeof(int32_t) * ((size_t)R + 1), stream>>>(
+          R, list.num, cands_per_tile, heads, plan->cand_offsets, base_dev, list.dev);
+    if (base_dev) cudaFreeAsync(base_dev, stream);
+    if (e != cudaSuccess) {
+      cudaFreeAsync(list.dev, stream);
+      return ROCS_ERR_CUDA;
+    }
+  }
+  if (cudaGetLastError() != cudaSuccess) {
+    if (list.dev) cudaFreeAsync(list.dev, stream);
     return ROCS_ERR_CUDA;
   }
+  plan->lists[key] = list;
+  *out = list;
   return ROCS_OK;
 }
 
-rocs_status_t plan_tiles(const rocs_plan* plan, int32_t cands_per_tile, cudaStream_t stream,
-                         TileList* out) {
+rocs_status_t plan_row2req(const rocs_plan* plan, cudaStream_t stream, const int32_t** out) {
+  DeviceList list;
+  const rocs_status_t st = plan_list(plan, 0, 0, stream, &list);
+  *out = static_cast<const int32_t*>(list.dev);
+  return st;
+}
+
+rocs_status_t plan_tiles(const rocs_plan* plan, int32_t cands_per_tile, cudaStream_t stream, TileList* out) {
   if (cands_per_tile < 1) return ROCS_ERR_INVALID_ARG;
-  std::lock_guard<std::mutex> lock(plan->mu);
-  auto it = plan->tiles.find(cands_per_tile);
-  if (it != plan->tiles.end()) {
-    *out = it->second;
-    return ROCS_OK;
-  }
-  TileList tl;
-  if (plan->N > 0) {
-    int32_t* base_dev = nullptr;
-    int64_t total = 0;
-    rocs_status_t st = upload_entry_base(plan, cands_per_tile, stream, &base_dev, &total);
-    if (st != ROCS_OK) return st;
-    tl.num = (int32_t)total;
-    cudaError_t e = pool_alloc((void**)&tl.dev, sizeof(Tile) * (size_t)total, stream);
-    if (e == cudaSuccess) {
-      expand_tiles_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(plan->R, tl.num, cands_per_tile,
-                                                                              plan->cand_offsets, base_dev, tl.dev);
-      e = cudaGetLastError();
-      if (e != cudaSuccess) cudaFreeAsync(tl.dev, stream);
-    }
-    cudaFreeAsync(base_dev, stream);
-    if (e != cudaSuccess) return ROCS_ERR_CUDA;
-  }
-  plan->tiles[cands_per_tile] = tl;
-  *out = tl;
-  return ROCS_OK;
+  DeviceList list;
+  const rocs_status_t st = plan_list(plan, cands_per_tile, 0, stream, &list);
+  *out = TileList{static_cast<Tile*>(list.dev), list.num};
+  return st;
 }
 
-rocs_status_t plan_dca_items(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, int32_t tiles_per_item,
-                             cudaStream_t stream, DcaItemList* out) {
-  if (cands_per_tile < 1 || cands_per_tile > 32767 || heads < 1 || heads > 65535 || tiles_per_item < 1 ||
-      tiles_per_item > 2)
-    return ROCS_ERR_INVALID_ARG;
-  std::lock_guard<std::mutex> lock(plan->mu);
-  const int64_t key = ((int64_t)cands_per_tile * 65536 + heads) * 2 + (tiles_per_item - 1);
-  auto it = plan->dca_items.find(key);
-  if (it != plan->dca_items.end()) {
-    *out = it->second;
-    return ROCS_OK;
-  }
-  DcaItemList il;
-  if (plan->N > 0) {
-    int32_t* base_dev = nullptr;
-    int64_t per_head = 0;
-    rocs_status_t st = upload_entry_base(plan, cands_per_tile * tiles_per_item, stream, &base_dev, &per_head);
-    if (st != ROCS_OK) return st;
-    const int64_t total = per_head * heads;
-    if (total > 0x7fffffffLL) {
-      cudaFreeAsync(base_dev, stream);
-      return ROCS_ERR_UNSUPPORTED;
-    }
-    il.num = (int32_t)total;
-    cudaError_t e = pool_alloc((void**)&il.dev, sizeof(DcaItem) * (size_t)total, stream);
-    if (e == cudaSuccess) {
-      expand_dca_items_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(
-          plan->R, il.num, cands_per_tile, heads, tiles_per_item, plan->cand_offsets, base_dev, il.dev);
-      e = cudaGetLastError();
-      if (e != cudaSuccess) cudaFreeAsync(il.dev, stream);
-    }
-    cudaFreeAsync(base_dev, stream);
-    if (e != cudaSuccess) return ROCS_ERR_CUDA;
-  }
-  plan->dca_items[key] = il;
-  *out = il;
-  return ROCS_OK;
+rocs_status_t plan_dca_items(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, cudaStream_t stream,
+                             DcaItemList* out) {
+  if (cands_per_tile < 1 || heads < 1) return ROCS_ERR_INVALID_ARG;
+  DeviceList list;
+  const rocs_status_t st = plan_list(plan, cands_per_tile, heads, stream, &list);
+  *out = DcaItemList{static_cast<DcaItem*>(list.dev), list.num};
+  return st;
 }
 
 }  // namespace rocs
@@ -284,20 +311,6 @@ rocs_status_t rocs_plan_create(rocs_plan_t** out, int32_t R, int64_t N, const in
         }
       });
   }
-  if (N > 0) {
-    // Stream-ordered allocation: after the first batch the pool hands the block back without a
-    // device synchronisation, so building a plan per batch stays off the critical path.
-    if (pool_alloc((void**)&p->row2req, sizeof(int32_t) * (size_t)N, stream) != cudaSuccess) {
-      delete p;
-      return ROCS_ERR_CUDA;
-    }
-    fill_row2req_kernel<<<(unsigned)((N + 255) / 256), 256, 0, stream>>>(R, N, cand_offsets, p->row2req);
-    if (cudaGetLastError() != cudaSuccess) {
-      cudaFreeAsync(p->row2req, stream);
-      delete p;
-      return ROCS_ERR_CUDA;
-    }
-  }
   p->stream = stream;
   *out = p;
   return ROCS_OK;
@@ -307,10 +320,7 @@ rocs_status_t rocs_plan_destroy(rocs_plan_t* plan) {
   if (!plan) return ROCS_OK;
   rocs_status_t st = ROCS_OK;
   // Freed in stream order behind whatever the caller enqueued on the plan's stream.
-  if (plan->row2req && cudaFreeAsync(plan->row2req, plan->stream) != cudaSuccess) st = ROCS_ERR_CUDA;
-  for (auto& kv : plan->tiles)
-    if (kv.second.dev && cudaFreeAsync(kv.second.dev, plan->stream) != cudaSuccess) st = ROCS_ERR_CUDA;
-  for (auto& kv : plan->dca_items)
+  for (auto& kv : plan->lists)
     if (kv.second.dev && cudaFreeAsync(kv.second.dev, plan->stream) != cudaSuccess) st = ROCS_ERR_CUDA;
   delete plan;
   return st;
@@ -366,12 +376,16 @@ static rocs_status_t ikbo_linear_impl(const rocs_plan_t* plan, rocs_dtype_t dtyp
     if (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255u))
       return ROCS_ERR_WORKSPACE;
   }
+  const int32_t* row2req = nullptr;
   if (d_req > 0) {
     const size_t need = z_bytes;
     if (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255u))
       return ROCS_ERR_WORKSPACE;
+    // In front of the request half: the candidate kernel may start beside that one and reads the map at once.
+    rocs_status_t st = plan_row2req(plan, stream, &row2req);
+    if (st != ROCS_OK) return st;
     // Request half, once per request (Section 4.1): Z = X^R W_CR^T + bias, fp32.
-    rocs_status_t st = linear_dispatch(dtype, plan->R, d_req, d_out, XR, ld_xr, W_CR, ld_wcr, bias,
+    st = linear_dispatch(dtype, plan->R, d_req, d_out, XR, ld_xr, W_CR, ld_wcr, bias,
                                        nullptr, 0, nullptr, ROCS_ACT_NONE, workspace, d_out,
                                        /*out_f32=*/true, stream);
     if (st != ROCS_OK) return st;
@@ -391,7 +405,7 @@ static rocs_status_t ikbo_linear_impl(const rocs_plan_t* plan, rocs_dtype_t dtyp
       umma_linear_ws2_supported(plan->N, d_cand, d_out, false))
     partials = reinterpret_cast<float2*>(static_cast<uint8_t*>(workspace) + z_bytes);
   rocs_status_t st = linear_dispatch(dtype, plan->N, d_cand, d_out, XC, ld_xc, W_CC, ld_wcc, bias, Z, d_out,
-                                     Z ? plan->row2req : nullptr, act, Y, ld_y, /*out_f32=*/false, stream,
+                                     row2req, act, Y, ld_y, /*out_f32=*/false, stream,
                                      request_half_on_umma, partials, plan->R);
   if (st != ROCS_OK || row_stats == nullptr) return st;
   if (partials != nullptr)
@@ -522,8 +536,12 @@ rocs_status_t rocs_glm_interaction(const rocs_plan_t* plan, rocs_dtype_t dtype, 
     zr = (float*)workspace;
   }
   if (dtype == ROCS_BF16 && g_path.load() == ROCS_PATH_AUTO && umma_glm_supported(n_r, n_c, d, n_ro, n_co)) {
+    // The candidate kernel's tile list first: that kernel then starts beside the request kernel.
+    TileList tiles;
+    rocs_status_t st = (YC || OC) ? plan_tiles(plan, 128 / n_c, stream, &tiles) : ROCS_OK;
+    if (st != ROCS_OK) return st;
     // Request side once per request (tiny), candidate side on tensor cores.
-    rocs_status_t st = glm_request_mma_supported(n_r, d, n_ro, n_co)
+    st = glm_request_mma_supported(n_r, d, n_ro, n_co)
                            ? glm_request_mma(plan, n_r, n_c, d, XR, W, n_ro, n_co, YR, OR_, zr, stream)
                            : simt_glm(dtype, plan, n_r, n_c, d, XR, nullptr, W, n_ro, n_co, YR, nullptr, OR_,
                                       nullptr, zr, stream);

@@ -431,8 +431,8 @@ int sm_count_fm() {
 }
 
 template <int D>
-rocs_status_t launch_fm_mma(const rocs_plan* plan, int32_t n_r, int32_t k, const void* XC, const void* P,
-                            const float* TT, void* FC, cudaStream_t stream) {
+rocs_status_t launch_fm_mma(const rocs_plan* plan, const int32_t* row2req, int32_t n_r, int32_t k, const void* XC,
+                            const void* P, const float* TT, void* FC, cudaStream_t stream) {
   constexpr int kStages = D <= 64 ? 8 : D <= 128 ? 6 : 3;
   constexpr int kSmem = kStages * (D / 64) * kSlabBytes + 512;
   CUtensorMap map_xc;
@@ -447,7 +447,7 @@ rocs_status_t launch_fm_mma(const rocs_plan* plan, int32_t n_r, int32_t k, const
   p.k = k;
   p.num_tiles = (int32_t)((plan->N + kTileCands - 1) / kTileCands);
   p.P = (const __nv_bfloat16*)P;
-  p.row2req = plan->row2req;
+  p.row2req = row2req;
   p.TT = TT;
   p.FC = (__nv_bfloat16*)FC;
   p.status = status;
@@ -479,6 +479,12 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
   if (smem_r > kMaxSmem || smem_c > kMaxSmem) return ROCS_ERR_UNSUPPORTED;
   const size_t n_rp = (size_t)(n_r + 15) / 16 * 16, kp = (size_t)(k + 15) / 16 * 16;
   const size_t smem_mma = n_rp * ((size_t)(d + 8) * 2 + (kp + 8) * 2) + 2 * kp * (size_t)(d + 8) * 2;
+  // in front of the request kernel: the candidate kernel may start beside that one and reads the map at once
+  const int32_t* row2req = nullptr;
+  if (plan->N > 0 && FC) {
+    const rocs_status_t st = plan_row2req(plan, stream, &row2req);
+    if (st != ROCS_OK) return st;
+  }
   if (plan->R > 0 && tensor_core_request && sizeof(T) == 2 && d % 16 == 0 && k % 8 == 0 && smem_mma <= kMaxSmem) {
     ROCS_CUDA_TRY(cudaFuncSetAttribute(fm_request_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_mma));
     fm_request_mma_kernel<<<plan->R, 256, smem_mma, stream>>>(n_r, d, k, (const __nv_bfloat16*)XR,
@@ -492,16 +498,16 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
   if (plan->N == 0 || !FC) return ROCS_OK;
   if (fast_candidates) {
     switch (d) {
-      case 64: return launch_fm_mma<64>(plan, n_r, k, XC, P, TT, FC, stream);
-      case 128: return launch_fm_mma<128>(plan, n_r, k, XC, P, TT, FC, stream);
-      case 192: return launch_fm_mma<192>(plan, n_r, k, XC, P, TT, FC, stream);
-      case 256: return launch_fm_mma<256>(plan, n_r, k, XC, P, TT, FC, stream);
+      case 64: return launch_fm_mma<64>(plan, row2req, n_r, k, XC, P, TT, FC, stream);
+      case 128: return launch_fm_mma<128>(plan, row2req, n_r, k, XC, P, TT, FC, stream);
+      case 192: return launch_fm_mma<192>(plan, row2req, n_r, k, XC, P, TT, FC, stream);
+      case 256: return launch_fm_mma<256>(plan, row2req, n_r, k, XC, P, TT, FC, stream);
       default: break;
     }
   }
   ROCS_CUDA_TRY(cudaFuncSetAttribute(fm_candidate_simt_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
   fm_candidate_simt_kernel<T><<<(unsigned)plan->N, 128, smem_c, stream>>>(n_r, n_c, d, k, (const T*)XC, (const T*)P,
-                                                                         plan->row2req, TT, (T*)FC);
+                                                                         row2req, TT, (T*)FC);
   ROCS_CUDA_TRY(cudaGetLastError());
   return ROCS_OK;
 }

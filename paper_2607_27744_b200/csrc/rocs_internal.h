@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <map>
 #include <mutex>
+#include <tuple>
 #include <vector>
 
 #include "../../include/rocs.h"
@@ -26,13 +27,17 @@ struct TileList {
   int32_t num = 0;
 };
 
-// One unit of work of the tensor-core attention kernel: one head of up to two consecutive tiles
-// (A and B) of the same request, which then share every K/V block that is loaded.
+// A list of a plan in device memory, of whatever kind its key says.
+struct DeviceList {
+  void* dev = nullptr;
+  int32_t num = 0;
+};
+
+// One unit of work of the attention kernels: one head of `count` consecutive candidates of a request.
 struct DcaItem {
   int32_t req;
-  int32_t cand0;    // first candidate of tile A; tile B starts at cand0 + count_a
-  int16_t count_a;  // candidates in tile A (>= 1)
-  int16_t count_b;  // candidates in tile B (0 = no second tile)
+  int32_t cand0;
+  int32_t count;
   int32_t head;
 };
 
@@ -47,11 +52,12 @@ struct rocs_plan {
   int32_t R = 0;
   int64_t N = 0;
   const int32_t* cand_offsets = nullptr;  // device, borrowed
-  int32_t* row2req = nullptr;             // device [N], m_i of Section 4.1
   std::vector<int32_t> offsets_host;      // [R+1]
   mutable std::mutex mu;
-  mutable std::map<int32_t, rocs::TileList> tiles;  // key: candidates per tile
-  mutable std::map<int64_t, rocs::DcaItemList> dca_items;  // key: (candidates per tile * 65536 + heads) * 2 + tiles per item - 1
+  // Device lists, made on first use and kept per stream (its id, which is never reused): a list is only
+  // ever read on the stream whose order puts its making in front of the reader.
+  // Key: stream id, candidates per tile (0: the candidate -> request map), heads (0: no head dimension).
+  mutable std::map<std::tuple<unsigned long long, int32_t, int32_t>, rocs::DeviceList> lists;
   int device = 0;
   cudaStream_t stream = nullptr;  // stream the plan was created on; its memory is freed there
 };
@@ -68,14 +74,16 @@ inline size_t elem_size(rocs_dtype_t dt) { return dt == ROCS_BF16 ? 2 : 4; }
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// m_i of Section 4.1, int32 [N] on the device; made on first use.
+rocs_status_t plan_row2req(const rocs_plan* plan, cudaStream_t stream, const int32_t** out);
+
 // Returns the cached tile list for `cands_per_tile`, building it on first use.
 rocs_status_t plan_tiles(const rocs_plan* plan, int32_t cands_per_tile, cudaStream_t stream,
                          TileList* out);
 
-// Work items for the attention kernel, ordered request, head, tile (or tile pair when tiles_per_item is 2);
-// cached in the plan.
-rocs_status_t plan_dca_items(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, int32_t tiles_per_item,
-                             cudaStream_t stream, DcaItemList* out);
+// Work items for the attention kernels, ordered request, head, tile; cached in the plan.
+rocs_status_t plan_dca_items(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, cudaStream_t stream,
+                             DcaItemList* out);
 
 // ---- general (CUDA-core) kernels: simt_kernels.cu -------------------------------------
 // Y[i, :] = act(add[row2req ? row2req[i] : -, :] + X[i, :] W^T + bias).  out_f32 selects an

@@ -294,14 +294,17 @@ rocs_status_t simt_dca(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_q, int3
   if (items == 0) return ROCS_OK;
   const int64_t blocks = (items + DCA_WARPS - 1) / DCA_WARPS;
   if (blocks > 0x7fffffffLL) return ROCS_ERR_UNSUPPORTED;
+  const int32_t* row2req = nullptr;
+  const rocs_status_t st = plan_row2req(plan, stream, &row2req);
+  if (st != ROCS_OK) return st;
   if (dt == ROCS_F32)
     dca_simt_kernel<float><<<(unsigned)blocks, DCA_WARPS * 32, 0, stream>>>(
-        n_rows, n_q, H, dh, scale, (const float*)Q, (const float*)K, (const float*)V, plan->row2req,
+        n_rows, n_q, H, dh, scale, (const float*)Q, (const float*)K, (const float*)V, row2req,
         seq_offsets, (float*)O);
   else
     dca_simt_kernel<__nv_bfloat16><<<(unsigned)blocks, DCA_WARPS * 32, 0, stream>>>(
         n_rows, n_q, H, dh, scale, (const __nv_bfloat16*)Q, (const __nv_bfloat16*)K,
-        (const __nv_bfloat16*)V, plan->row2req, seq_offsets, (__nv_bfloat16*)O);
+        (const __nv_bfloat16*)V, row2req, seq_offsets, (__nv_bfloat16*)O);
   ROCS_CUDA_TRY(cudaGetLastError());
   return ROCS_OK;
 }
@@ -324,10 +327,13 @@ static rocs_status_t launch_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c,
     ROCS_CUDA_TRY(cudaGetLastError());
   }
   if (candidate_side && plan->N > 0 && (YC || OC)) {
+    const int32_t* row2req = nullptr;
+    const rocs_status_t st = plan_row2req(plan, stream, &row2req);
+    if (st != ROCS_OK) return st;
     ROCS_CUDA_TRY(cudaFuncSetAttribute(glm_candidate_simt_kernel<T>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
     glm_candidate_simt_kernel<T><<<(unsigned)plan->N, 128, smem_c, stream>>>(
-        n_r, n_c, d, (const T*)XR, (const T*)XC, (const T*)W, n_ro, n_co, plan->row2req, zr, (T*)YC,
+        n_r, n_c, d, (const T*)XR, (const T*)XC, (const T*)W, n_ro, n_co, row2req, zr, (T*)YC,
         (T*)OC);
     ROCS_CUDA_TRY(cudaGetLastError());
   }

@@ -464,7 +464,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     for (int32_t i = item0 + side; i < p.num_items; i += item_step) {
       const DcaItem item = p.items[i];
       const int32_t L = p.seq_offsets[item.req + 1] - p.seq_offsets[item.req];
-      const int32_t rows_valid = item.count_a * p.n_q;
+      const int32_t rows_valid = item.count * p.n_q;
       // this thread's half of the output columns of its row
       auto out_ptr = [&]() { return p.O + ((int64_t)item.cand0 * p.n_q + row) * row_width + item.head * DH + half * kOutCols; };
       bool aborted = false;
@@ -668,7 +668,7 @@ static rocs_status_t launch_dca(const rocs_plan* plan, int32_t n_q, int32_t H, f
                                 cudaStream_t stream) {
   using C = DcaCfg<DH, BKV>;
   DcaItemList items;
-  rocs_status_t st = plan_dca_items(plan, BQ / n_q, H, /*tiles_per_item=*/1, stream, &items);
+  rocs_status_t st = plan_dca_items(plan, BQ / n_q, H, stream, &items);
   if (st != ROCS_OK) return st;
   if (items.num == 0) return ROCS_OK;
   const uint64_t width = (uint64_t)H * DH;

@@ -405,6 +405,16 @@ def test_glm_bf16_other_split(path):
     assert _run_glm(cfg, co, path=path) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("R", [1, 255, 257, 12000, 12001])
+def test_work_lists_of_many_requests(R):
+    # the lists are scanned by 256 threads per block up to 12000 requests and on the host beyond: counts of
+    # 0..3 candidates put empty requests at both ends of every thread's share
+    co = wl.offsets_from_counts([(i * 5 + 3) % 4 for i in range(R)])
+    assert _run_glm(wl.CONFIGS[5].with_(R=R, n_r=8, d_emb=64, n_ro=0, n_co=0), co) <= tol_for("bf16")
+    so = wl.offsets_from_counts([(i * 3) % 5 for i in range(R)])
+    assert _run_dca(wl.CONFIGS[3].with_(R=R, H=2, dh=32), co, so) <= tol_for("bf16")
+
+
 def test_glm_config4_full_size_sampled():
     cfg = wl.CONFIGS[4]
     co = wl.cand_offsets(cfg)
