@@ -150,6 +150,13 @@ __global__ void __launch_bounds__(kListThreads) expand_list_kernel(int32_t R, in
     static_cast<DcaItem*>(out)[i] = DcaItem{req, c, count, h};
 }
 
+int64_t plan_entries(const rocs_plan* plan, int32_t cands_per_tile) {
+  int64_t entries = 0;
+  for (int32_t r = 0; r < plan->R; ++r)
+    entries += ((int64_t)plan->offsets_host[r + 1] - plan->offsets_host[r] + cands_per_tile - 1) / cands_per_tile;
+  return entries;
+}
+
 static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, cudaStream_t stream,
                                DeviceList* out) {
   static_assert(sizeof(Tile) == 16 && sizeof(DcaItem) == 16, "list entries");
@@ -169,21 +176,17 @@ static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, in
                                                                               static_cast<int32_t*>(list.dev));
   } else if (plan->N > 0) {
     const int32_t R = plan->R;
-    std::vector<int32_t> base(R > kMaxScan ? (size_t)R + 1 : 0);
-    int64_t entries = 0;
-    for (int32_t r = 0; r < R; ++r) {
-      if (R > kMaxScan) base[r] = (int32_t)entries;
-      const int64_t n = (int64_t)plan->offsets_host[r + 1] - plan->offsets_host[r];
-      entries += (n + cands_per_tile - 1) / cands_per_tile;
-    }
-    const int64_t total = entries * std::max(heads, 1);
+    const int64_t total = plan_entries(plan, cands_per_tile) * std::max(heads, 1);
     if (total > 0x7fffffffLL) return ROCS_ERR_UNSUPPORTED;
     list.num = (int32_t)total;
     ROCS_CUDA_TRY(pool_alloc(&list.dev, sizeof(Tile) * (size_t)total, stream));
     int32_t* base_dev = nullptr;
     cudaError_t e = cudaSuccess;
     if (R > kMaxScan) {
-      base[R] = (int32_t)entries;
+      std::vector<int32_t> base((size_t)R + 1, 0);
+      for (int32_t r = 0; r < R; ++r)
+        base[r + 1] = base[r] + (int32_t)(((int64_t)plan->offsets_host[r + 1] - plan->offsets_host[r] + cands_per_tile - 1) /
+                                          cands_per_tile);
       e = pool_alloc((void**)&base_dev, sizeof(int32_t) * base.size(), stream);
       // Pageable source: the copy is staged before the call returns, so `base` may go away.
       if (e == cudaSuccess)

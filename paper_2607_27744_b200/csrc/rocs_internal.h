@@ -74,6 +74,9 @@ inline size_t elem_size(rocs_dtype_t dt) { return dt == ROCS_BF16 ? 2 : 4; }
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// Tiles of at most `cands_per_tile` candidates that the batch's requests are cut into.
+int64_t plan_entries(const rocs_plan* plan, int32_t cands_per_tile);
+
 // m_i of Section 4.1, int32 [N] on the device; made on first use.
 rocs_status_t plan_row2req(const rocs_plan* plan, cudaStream_t stream, const int32_t** out);
 

@@ -89,78 +89,6 @@ rocs_status_t launch_linear(int64_t M, int32_t d_in, int32_t d_out, const void* 
 }
 
 // ---------------------------------------------------------------------------------------------
-// Cross attention (Eq. 13): one warp per (query row, head).  Keys are visited 32 at a time (one
-// per lane) with a running maximum and normaliser; values are accumulated with lanes spread
-// over the head dimension.  The request of the row comes from row2req, its keys from
-// seq_offsets: K/V are read in place, never copied per candidate.
-// ---------------------------------------------------------------------------------------------
-constexpr int DCA_WARPS = 4;
-constexpr int DCA_MAX_DH = 256;
-
-template <typename T>
-__global__ void __launch_bounds__(DCA_WARPS * 32) dca_simt_kernel(
-    int64_t n_rows, int32_t n_q, int32_t H, int32_t dh, float scale, const T* __restrict__ Q,
-    const T* __restrict__ K, const T* __restrict__ V, const int32_t* __restrict__ row2req,
-    const int32_t* __restrict__ seq_offsets, T* __restrict__ O) {
-  __shared__ float qs[DCA_WARPS][DCA_MAX_DH];
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int64_t item = (int64_t)blockIdx.x * DCA_WARPS + warp;
-  if (item >= n_rows * H) return;
-  const int64_t qrow = item / H;
-  const int32_t h = (int32_t)(item % H);
-  const int32_t r = row2req[qrow / n_q];
-  const int64_t s0 = seq_offsets[r];
-  const int32_t L = seq_offsets[r + 1] - seq_offsets[r];
-  const int64_t hd = (int64_t)H * dh;
-  const int64_t qbase = qrow * hd + (int64_t)h * dh;
-  for (int e = lane; e < dh; e += 32) qs[warp][e] = ld_f(Q, qbase + e);
-  __syncwarp();
-  float m = -INFINITY, l = 0.f;
-  float acc[DCA_MAX_DH / 32];
-#pragma unroll
-  for (int u = 0; u < DCA_MAX_DH / 32; ++u) acc[u] = 0.f;
-  for (int32_t j0 = 0; j0 < L; j0 += 32) {
-    const int32_t j = j0 + lane;
-    float s = -INFINITY;
-    if (j < L) {
-      const int64_t kb = (s0 + j) * hd + (int64_t)h * dh;
-      float dot = 0.f;
-      for (int e = 0; e < dh; ++e) dot = fmaf(qs[warp][e], ld_f(K, kb + e), dot);
-      s = dot * scale;
-    }
-    float cmax = s;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
-    const float m_new = fmaxf(m, cmax);
-    const float corr = (m == -INFINITY) ? 0.f : expf(m - m_new);
-    const float p = (j < L) ? expf(s - m_new) : 0.f;
-    float psum = p;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, o);
-    l = l * corr + psum;
-#pragma unroll
-    for (int u = 0; u < DCA_MAX_DH / 32; ++u) acc[u] *= corr;
-    const int32_t cnt = min(32, L - j0);
-    for (int jj = 0; jj < cnt; ++jj) {
-      const float pj = __shfl_sync(0xffffffffu, p, jj);
-      const int64_t vb = (s0 + j0 + jj) * hd + (int64_t)h * dh;
-#pragma unroll
-      for (int u = 0; u < DCA_MAX_DH / 32; ++u) {
-        const int e = lane + 32 * u;
-        if (e < dh) acc[u] = fmaf(pj, ld_f(V, vb + e), acc[u]);
-      }
-    }
-    m = m_new;
-  }
-  const float inv = (L > 0) ? 1.f / l : 0.f;
-#pragma unroll
-  for (int u = 0; u < DCA_MAX_DH / 32; ++u) {
-    const int e = lane + 32 * u;
-    if (e < dh) st_f(O, qbase + e, acc[u] * inv);
-  }
-}
-
-// ---------------------------------------------------------------------------------------------
 // GLM factorization machine (Eq. 9-10) and row-axis compression (Eq. 5-6).
 // Request kernel (one block per request): YR = [X^R X^R^T, 0], OR = W_RR YR, and the request
 // term ZR = W_CR YR that the candidate kernel adds to every candidate of the request.
@@ -283,30 +211,6 @@ rocs_status_t simt_linear(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_ou
                                                row2req, act, Y, ld_y, stream);
   return launch_linear<__nv_bfloat16, __nv_bfloat16>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add,
                                                      ld_add, row2req, act, Y, ld_y, stream);
-}
-
-rocs_status_t simt_dca(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh,
-                       float scale, const void* Q, const void* K, const void* V,
-                       const int32_t* seq_offsets, void* O, cudaStream_t stream) {
-  if (dh > DCA_MAX_DH) return ROCS_ERR_UNSUPPORTED;
-  const int64_t n_rows = plan->N * n_q;
-  const int64_t items = n_rows * H;
-  if (items == 0) return ROCS_OK;
-  const int64_t blocks = (items + DCA_WARPS - 1) / DCA_WARPS;
-  if (blocks > 0x7fffffffLL) return ROCS_ERR_UNSUPPORTED;
-  const int32_t* row2req = nullptr;
-  const rocs_status_t st = plan_row2req(plan, stream, &row2req);
-  if (st != ROCS_OK) return st;
-  if (dt == ROCS_F32)
-    dca_simt_kernel<float><<<(unsigned)blocks, DCA_WARPS * 32, 0, stream>>>(
-        n_rows, n_q, H, dh, scale, (const float*)Q, (const float*)K, (const float*)V, row2req,
-        seq_offsets, (float*)O);
-  else
-    dca_simt_kernel<__nv_bfloat16><<<(unsigned)blocks, DCA_WARPS * 32, 0, stream>>>(
-        n_rows, n_q, H, dh, scale, (const __nv_bfloat16*)Q, (const __nv_bfloat16*)K,
-        (const __nv_bfloat16*)V, row2req, seq_offsets, (__nv_bfloat16*)O);
-  ROCS_CUDA_TRY(cudaGetLastError());
-  return ROCS_OK;
 }
 
 template <typename T>

@@ -56,4 +56,107 @@ __device__ __forceinline__ void rows_to_shared(const T* __restrict__ src, float*
   }
 }
 
+// Entry i of the list of tiles of at most `per` consecutive candidates of one request, in the order
+// request, head, tile (heads = 1: request, tile), found by the block itself from the offsets of R <= THREADS
+// requests: one request per thread and one scan.  A list in memory is one more launch and allocation in
+// front of the kernel (4 us of a 68 us pass over 4 tiny requests); where there are more requests than
+// threads the caller brings the plan's list.  All threads of the block call this.
+struct FoundTile {
+  int32_t req, cand0, count, head;
+};
+template <int THREADS>
+__device__ __forceinline__ FoundTile find_tile_in_block(int32_t R, int32_t per, int32_t heads,
+                                                        const int32_t* __restrict__ off, int32_t i) {
+  __shared__ int32_t warp_sum[THREADS / 32];
+  __shared__ FoundTile found;
+  const int32_t t = threadIdx.x, lane = t % 32;
+  const int32_t c0 = t < R ? off[t] : 0, n = t < R ? off[t + 1] - c0 : 0;
+  const int32_t tiles = (n + per - 1) / per, entries = tiles * heads;
+  int32_t incl = entries;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += up;
+  }
+  if (lane == 31) warp_sum[t / 32] = incl;
+  __syncthreads();
+  int32_t first = incl - entries;
+  for (int w = 0; w < t / 32; ++w) first += warp_sum[w];
+  if (first <= i && i < first + entries) {
+    const int32_t local = i - first, h = local / tiles, c = (local - h * tiles) * per;
+    found = FoundTile{t, c0 + c, min(per, n - c), h};
+  }
+  __syncthreads();
+  return found;
+}
+
+__device__ __forceinline__ void cp_async_16(uint32_t smem_dst, const void* src, int bytes) {  // the rest of the 16 is zeros
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
+
+// Eight bf16 values of one 16-byte vector as fp32.
+__device__ __forceinline__ void bf16x8_to_f32(const uint4& raw, float4& lo, float4& hi) {
+  lo = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u), __uint_as_float(raw.y << 16),
+                   __uint_as_float(raw.y & 0xffff0000u));
+  hi = make_float4(__uint_as_float(raw.z << 16), __uint_as_float(raw.z & 0xffff0000u), __uint_as_float(raw.w << 16),
+                   __uint_as_float(raw.w & 0xffff0000u));
+}
+
+// A tile of `rows` rows of up to COLS columns into shared memory as fp32 (row stride `stride` floats, a
+// multiple of 4), zeros beyond `valid` rows and beyond d columns.  Rows are `ld` elements apart in
+// global memory and start on 16-byte boundaries; d is a multiple of a 16-byte vector.  fp32 goes by
+// cp.async (the caller commits and waits), bf16 through registers.
+template <typename T, int COLS>
+__device__ __forceinline__ void rows_to_shared_async(const T* __restrict__ src, int64_t ld, int valid, int rows, int d,
+                                                     float* __restrict__ dst, int stride, int tid, int threads) {
+  constexpr int kVec = 16 / (int)sizeof(T), kPerRow = COLS / kVec;
+#pragma unroll 4
+  for (int v = tid; v < rows * kPerRow; v += threads) {
+    const int r = v / kPerRow, c = (v % kPerRow) * kVec;
+    const bool in = r < valid && c < d;
+    const T* from = src + (in ? r * ld + c : 0);
+    float* to = dst + r * stride + c;
+    if constexpr (sizeof(T) == 4) {
+      cp_async_16((uint32_t)__cvta_generic_to_shared(to), from, in ? 16 : 0);
+    } else {
+      float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+      if (in) bf16x8_to_f32(__ldg(reinterpret_cast<const uint4*>(from)), lo, hi);
+      *reinterpret_cast<float4*>(to) = lo;
+      *reinterpret_cast<float4*>(to + 4) = hi;
+    }
+  }
+}
+
+// Packed fp32 pairs: one issue slot for two FMAs.
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+__device__ __forceinline__ void store_pair(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
+__device__ __forceinline__ void store_pair(__nv_bfloat16* p, float a, float b) {
+  *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(a, b);
+}
+
 }  // namespace rocs

@@ -290,6 +290,17 @@ def test_dca_bf16_scores_that_outgrow_the_first_key_block(dh):
     assert rocs.last_device_status() == 0
 
 
+@pytest.mark.parametrize("dtype,dh,n_q", [("f32", 4, 1), ("f32", 36, 3), ("f32", 64, 70), ("f32", 128, 1), ("f32", 200, 1),
+                                          ("bf16", 96, 1), ("bf16", 256, 2)])
+def test_dca_general_kernel_edges(dtype, dh, n_q):
+    # tiles of 32 query rows and 64 keys: one row / key, one less, exact, one more; empty request and sequence;
+    # head widths between the compiled ones; more query tokens than a tile has rows
+    co = wl.offsets_from_counts([1, 31, 32, 0, 65, 2] if n_q < 64 else [1, 0, 2, 1, 1, 3])
+    so = wl.offsets_from_counts([63, 64, 1, 40, 129, 0])
+    cfg = wl.CONFIGS[3].with_(R=6, H=3, dh=dh, n_q=n_q, dtype=dtype)
+    assert _run_dca(cfg, co, so) <= tol_for(dtype)
+
+
 def test_dca_bf16_64_query_tokens_per_candidate():
     # two candidates fill a 128-row tile (Section 4.3.2 names query tiles of 32 and 64 tokens)
     co = wl.offsets_from_counts([5, 1, 12, 2])
@@ -405,13 +416,14 @@ def test_glm_bf16_other_split(path):
     assert _run_glm(cfg, co, path=path) <= tol_for("bf16")
 
 
-@pytest.mark.parametrize("R", [1, 255, 257, 12000, 12001])
+@pytest.mark.parametrize("R", [1, 127, 128, 129, 255, 257, 12000, 12001])
 def test_work_lists_of_many_requests(R):
     # the lists are scanned by 256 threads per block up to 12000 requests and on the host beyond: counts of
     # 0..3 candidates put empty requests at both ends of every thread's share
     co = wl.offsets_from_counts([(i * 5 + 3) % 4 for i in range(R)])
     assert _run_glm(wl.CONFIGS[5].with_(R=R, n_r=8, d_emb=64, n_ro=0, n_co=0), co) <= tol_for("bf16")
     so = wl.offsets_from_counts([(i * 3) % 5 for i in range(R)])
+    assert _run_dca(wl.CONFIGS[3].with_(R=R, H=2, dh=8), co, so) <= tol_for("bf16")
     assert _run_dca(wl.CONFIGS[3].with_(R=R, H=2, dh=32), co, so) <= tol_for("bf16")
 
 
