@@ -1,0 +1,186 @@
+// Linear layer on the CUDA cores (Eq. 4 / Eq. 14):
+//     Y[i, n] = act( sum_k X[i, k] W[n, k] + bias[n] + add[row2req[i], n] )
+// in fp32 FMA on fp32 or bf16 storage: the fp32 path, and bf16 shapes the tensor-core kernels do not take.
+//
+// A block computes a BM x BN tile.  Its threads form KS groups of 64 (8 x 8 threads, TM x TN outputs each)
+// that take the 16-wide slices of K in turn, each through a three-stage cp.async ring of its own with a
+// barrier of its own, and add their partial tiles up in shared memory in a fixed order at the end.
+// Operands stay row-major in shared memory (20-float rows): a thread reads four k of a row at once, the
+// eight rows a quarter-warp reads hit eight different bank groups.
+//
+// Which tile (`simt_linear`): the largest that still gives every SM work, since the FMAs per shared-memory
+// read fall with it (8 x 8 outputs: 16 FMAs per 16-byte read, 4 x 4: 8, 2 x 2: 4) and what bounds the large
+// shapes is the FMA pipe and those reads, while a small batch (the request half at R rows) is bound by the
+// length of its K chain on a few SMs.  Measured, fp32: 24 requests x 768 -> 1024 with 2613 candidates x
+// 256 -> 1024 behind it, 61 us for both (one 64 x 64 tile of 16-wide synchronous slices for every shape:
+// 160 us, half of it the 16 blocks of the request half).
+// Every output is produced by a sequence that depends on the shape only, so results are deterministic and
+// independent of the other rows' values (Eq. 1).
+#include "rocs_internal.h"
+#include "simt_util.cuh"
+
+namespace rocs {
+namespace {
+
+constexpr int kBk = 16, kRow = kBk + 4;  // k per slice; floats per shared-memory row
+constexpr int kGroup = 64, kStages = 3;
+
+template <int BM, int BN, int KS>
+constexpr int smem_bytes() {
+  constexpr int ring = KS * kStages * (BM + BN) * kRow, tiles = KS * BM * BN;
+  return (ring > tiles ? ring : tiles) * (int)sizeof(float);
+}
+
+__device__ __forceinline__ float ld_f(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+__device__ __forceinline__ void st_f(float* p, float v) { *p = v; }
+__device__ __forceinline__ void st_f(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+
+// 16 columns from k0 of `rows` rows starting at row0 of a matrix, zeros outside it.
+__device__ __forceinline__ void load_slice(const float* __restrict__ src, int64_t ld, int64_t row0, int64_t n_rows,
+                                           int rows, int32_t k0, int32_t d, float* dst, int t) {
+  for (int v = t; v < rows * (kBk / 4); v += kGroup) {
+    const int r = v / (kBk / 4), k = k0 + (v % (kBk / 4)) * 4;
+    const int left = row0 + r < n_rows ? min(max(d - k, 0), 4) : 0;
+    cp_async_16((uint32_t)__cvta_generic_to_shared(dst + r * kRow + (v % (kBk / 4)) * 4),
+                src + (left > 0 ? (row0 + r) * ld + k : 0), left * 4);
+  }
+}
+__device__ __forceinline__ void load_slice(const __nv_bfloat16* __restrict__ src, int64_t ld, int64_t row0,
+                                           int64_t n_rows, int rows, int32_t k0, int32_t d, float* dst, int t) {
+  for (int v = t; v < rows * (kBk / 8); v += kGroup) {
+    const int r = v / (kBk / 8), k = k0 + (v % (kBk / 8)) * 8;
+    const int left = row0 + r < n_rows ? min(max(d - k, 0), 8) : 0;
+    const __nv_bfloat16* from = src + (row0 + r) * ld + k;
+    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+    if (left == 8) {
+      bf16x8_to_f32(__ldg(reinterpret_cast<const uint4*>(from)), lo, hi);
+    } else if (left > 0) {
+      float f[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) f[e] = e < left ? ld_f(from + e) : 0.f;
+      lo = make_float4(f[0], f[1], f[2], f[3]);
+      hi = make_float4(f[4], f[5], f[6], f[7]);
+    }
+    float* to = dst + r * kRow + (v % (kBk / 8)) * 8;
+    *reinterpret_cast<float4*>(to) = lo;
+    *reinterpret_cast<float4*>(to + 4) = hi;
+  }
+}
+
+template <typename TIn, typename TOut, int TM, int TN, int KS>
+__global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kernel(
+    int64_t M, int32_t d_in, int32_t d_out, const TIn* __restrict__ X, int64_t ld_x, const TIn* __restrict__ W,
+    int64_t ld_w, const float* __restrict__ bias, const float* __restrict__ add, int64_t ld_add,
+    const int32_t* __restrict__ row2req, int act, TOut* __restrict__ Y, int64_t ld_y) {
+  constexpr int BM = 8 * TM, BN = 8 * TN;
+  extern __shared__ __align__(16) float sm[];
+  const int group = threadIdx.x / kGroup, t = threadIdx.x % kGroup;
+  const int tx = t % 8, ty = t / 8;
+  const int64_t m0 = (int64_t)blockIdx.x * BM;
+  const int32_t n0 = blockIdx.y * BN;
+  const int32_t slices = (d_in + kBk - 1) / kBk;
+  const int32_t mine = (slices - group + KS - 1) / KS;  // slices group, group + KS, ...
+  float* ring = sm + group * kStages * (BM + BN) * kRow;
+  auto fetch = [&](int32_t it) {
+    if (it < mine) {
+      float* st = ring + (it % kStages) * (BM + BN) * kRow;
+      const int32_t k0 = (group + it * KS) * kBk;
+      load_slice(X, ld_x, m0, M, BM, k0, d_in, st, t);
+      load_slice(W, ld_w, n0, d_out, BN, k0, d_in, st + BM * kRow, t);
+    }
+    cp_async_commit();
+  };
+  auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kGroup) : "memory"); };
+
+  float acc[TM][TN];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+#pragma unroll
+  for (int s = 0; s < kStages - 1; ++s) fetch(s);
+  for (int32_t it = 0; it < mine; ++it) {
+    cp_async_wait<kStages - 2>();
+    group_sync();  // slice `it` has landed for the group, and everybody is done with slice it - 1
+    fetch(it + kStages - 1);
+    const float* a_s = ring + (it % kStages) * (BM + BN) * kRow + ty * kRow;
+    const float* b_s = ring + (it % kStages) * (BM + BN) * kRow + (BM + tx) * kRow;
+#pragma unroll
+    for (int k = 0; k < kBk; k += 4) {
+      float4 a[TM], b[TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(a_s + i * 8 * kRow + k);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) b[j] = *reinterpret_cast<const float4*>(b_s + j * 8 * kRow + k);
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+          acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+          acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+          acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+        }
+    }
+  }
+  cp_async_wait<0>();
+  __syncthreads();  // the rings become the groups' partial tiles
+  float* part = sm + group * BM * BN;
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) part[(ty + 8 * i) * BN + tx + 8 * j] = acc[i][j];
+  __syncthreads();
+  for (int e = threadIdx.x; e < BM * BN; e += kGroup * KS) {
+    const int64_t m = m0 + e / BN;
+    const int32_t n = n0 + e % BN;
+    if (m >= M || n >= d_out) continue;
+    float v = sm[e];
+#pragma unroll
+    for (int g = 1; g < KS; ++g) v += sm[g * BM * BN + e];
+    if (bias) v += bias[n];
+    if (add) v += add[(int64_t)(row2req ? row2req[m] : m) * ld_add + n];
+    if (act == ROCS_ACT_RELU) v = fmaxf(v, 0.f);
+    st_f(Y + m * ld_y + n, v);
+  }
+}
+
+template <typename TIn, typename TOut>
+rocs_status_t launch_linear(int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x, const void* W,
+                            int64_t ld_w, const float* bias, const float* add, int64_t ld_add,
+                            const int32_t* row2req, int act, void* Y, int64_t ld_y, cudaStream_t stream) {
+  if (M == 0 || d_out == 0) return ROCS_OK;
+  auto tiles = [&](int b) { return ((M + b - 1) / b) * ((d_out + b - 1) / b); };
+#define ROCS_LAUNCH(T_, KS_)                                                                                         \
+  do {                                                                                                               \
+    constexpr int smem = smem_bytes<8 * T_, 8 * T_, KS_>();                                                          \
+    auto kernel = linear_simt_kernel<TIn, TOut, T_, T_, KS_>;                                                        \
+    ROCS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));                  \
+    kernel<<<dim3((unsigned)((M + 8 * T_ - 1) / (8 * T_)), (unsigned)((d_out + 8 * T_ - 1) / (8 * T_))), kGroup * KS_, \
+             smem, stream>>>(M, d_in, d_out, (const TIn*)X, ld_x, (const TIn*)W, ld_w, bias, add, ld_add, row2req,   \
+                             act, (TOut*)Y, ld_y);                                                                   \
+  } while (0)
+  if (tiles(64) >= 296) ROCS_LAUNCH(8, 2);
+  else if (tiles(32) >= 148) ROCS_LAUNCH(4, 4);
+  else ROCS_LAUNCH(2, 8);
+#undef ROCS_LAUNCH
+  ROCS_CUDA_TRY(cudaGetLastError());
+  return ROCS_OK;
+}
+
+}  // namespace
+
+rocs_status_t simt_linear(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x,
+                          const void* W, int64_t ld_w, const float* bias, const float* add, int64_t ld_add,
+                          const int32_t* row2req, int act, void* Y, int64_t ld_y, bool out_f32, cudaStream_t stream) {
+  if (dt == ROCS_F32)
+    return launch_linear<float, float>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act, Y, ld_y,
+                                       stream);
+  if (out_f32)
+    return launch_linear<__nv_bfloat16, float>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act, Y,
+                                               ld_y, stream);
+  return launch_linear<__nv_bfloat16, __nv_bfloat16>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act,
+                                                     Y, ld_y, stream);
+}
+
+}  // namespace rocs

@@ -15,80 +15,6 @@ __device__ __forceinline__ void st_f(float* p, int64_t i, float v) { p[i] = v; }
 __device__ __forceinline__ void st_f(__nv_bfloat16* p, int64_t i, float v) { p[i] = __float2bfloat16_rn(v); }
 
 // ---------------------------------------------------------------------------------------------
-// Linear: Y[i, n] = act(sum_k X[i, k] W[n, k] + bias[n] + add[row2req[i], n])      (Eq. 4 / Eq. 14)
-// 64x64 output tile per block, 16-wide k slices through shared memory, 4x4 outputs per thread.
-// ---------------------------------------------------------------------------------------------
-constexpr int LBM = 64, LBN = 64, LBK = 16;
-
-template <typename TIn, typename TOut>
-__global__ void __launch_bounds__(256) linear_simt_kernel(
-    int64_t M, int32_t d_in, int32_t d_out, const TIn* __restrict__ X, int64_t ld_x,
-    const TIn* __restrict__ W, int64_t ld_w, const float* __restrict__ bias,
-    const float* __restrict__ add, int64_t ld_add, const int32_t* __restrict__ row2req, int act,
-    TOut* __restrict__ Y, int64_t ld_y) {
-  __shared__ float As[LBK][LBM + 4];
-  __shared__ float Bs[LBK][LBN + 4];
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
-  const int64_t m0 = (int64_t)blockIdx.x * LBM;
-  const int32_t n0 = blockIdx.y * LBN;
-  float acc[4][4] = {};
-  for (int32_t k0 = 0; k0 < d_in; k0 += LBK) {
-    for (int e = tid; e < LBM * LBK; e += 256) {
-      const int r = e / LBK, k = e % LBK;
-      const int64_t gm = m0 + r;
-      As[k][r] = (gm < M && k0 + k < d_in) ? ld_f(X, gm * ld_x + k0 + k) : 0.f;
-      const int32_t gn = n0 + r;
-      Bs[k][r] = (gn < d_out && k0 + k < d_in) ? ld_f(W, (int64_t)gn * ld_w + k0 + k) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < LBK; ++k) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[k][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[k][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t gm = m0 + ty * 4 + i;
-    if (gm >= M) continue;
-    const float* add_row = add ? add + (int64_t)(row2req ? row2req[gm] : gm) * ld_add : nullptr;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int32_t gn = n0 + tx * 4 + j;
-      if (gn >= d_out) continue;
-      float v = acc[i][j];
-      if (bias) v += bias[gn];
-      if (add_row) v += add_row[gn];
-      if (act == ROCS_ACT_RELU) v = fmaxf(v, 0.f);
-      st_f(Y, gm * ld_y + gn, v);
-    }
-  }
-}
-
-template <typename TIn, typename TOut>
-rocs_status_t launch_linear(int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x,
-                            const void* W, int64_t ld_w, const float* bias, const float* add,
-                            int64_t ld_add, const int32_t* row2req, int act, void* Y, int64_t ld_y,
-                            cudaStream_t stream) {
-  if (M == 0 || d_out == 0) return ROCS_OK;
-  dim3 grid((unsigned)((M + LBM - 1) / LBM), (unsigned)((d_out + LBN - 1) / LBN));
-  linear_simt_kernel<TIn, TOut><<<grid, 256, 0, stream>>>(
-      M, d_in, d_out, (const TIn*)X, ld_x, (const TIn*)W, ld_w, bias, add, ld_add, row2req, act,
-      (TOut*)Y, ld_y);
-  ROCS_CUDA_TRY(cudaGetLastError());
-  return ROCS_OK;
-}
-
-// ---------------------------------------------------------------------------------------------
 // GLM factorization machine (Eq. 9-10) and row-axis compression (Eq. 5-6).
 // Request kernel (one block per request): YR = [X^R X^R^T, 0], OR = W_RR YR, and the request
 // term ZR = W_CR YR that the candidate kernel adds to every candidate of the request.
@@ -198,20 +124,6 @@ __global__ void __launch_bounds__(128) glm_candidate_simt_kernel(
 }
 
 }  // namespace
-
-rocs_status_t simt_linear(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_out, const void* X,
-                          int64_t ld_x, const void* W, int64_t ld_w, const float* bias,
-                          const float* add, int64_t ld_add, const int32_t* row2req, int act,
-                          void* Y, int64_t ld_y, bool out_f32, cudaStream_t stream) {
-  if (dt == ROCS_F32)
-    return launch_linear<float, float>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req,
-                                       act, Y, ld_y, stream);
-  if (out_f32)
-    return launch_linear<__nv_bfloat16, float>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add,
-                                               row2req, act, Y, ld_y, stream);
-  return launch_linear<__nv_bfloat16, __nv_bfloat16>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add,
-                                                     ld_add, row2req, act, Y, ld_y, stream);
-}
 
 template <typename T>
 static rocs_status_t launch_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d,

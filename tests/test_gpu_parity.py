@@ -97,6 +97,30 @@ def test_plain_linear_bf16_wide_many_rows(relu, bias):
     assert rel_err(to_host_f64(y), want) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("M,d_in,d_out", [(1, 3, 1), (35, 19, 17), (33, 130, 1024), (600, 100, 397), (2600, 35, 517)])
+def test_linear_general_kernel_tiles(dtype, M, d_in, d_out):
+    # the three tile sizes (16, 32, 64), each with remainders in rows, columns and K; rows padded to 16 bytes
+    # with NaN behind the last column, which must not be read into the sum
+    rocs.set_path(rocs.PATH_GENERAL)
+    g = np.random.default_rng(M)
+    X, W = g.standard_normal((M, d_in), dtype=np.float32), g.standard_normal((d_out, d_in), dtype=np.float32)
+    b = g.standard_normal(d_out).astype(np.float32)
+    X, W = wl.store(X, dtype), wl.store(W * d_in ** -0.5, dtype)
+    ld = rocs.padded_ld(d_in, rocs.BF16 if dtype == "bf16" else rocs.F32)
+
+    def padded(a):
+        t = torch.full((a.shape[0], ld), float("nan"), dtype=torch.bfloat16 if dtype == "bf16" else torch.float32, device="cuda")
+        t[:, :d_in] = to_dev(a)
+        return t[:, :d_in]
+
+    ldo = rocs.padded_ld(d_out, rocs.BF16 if dtype == "bf16" else rocs.F32)
+    Y = torch.empty((M, ldo), dtype=torch.bfloat16 if dtype == "bf16" else torch.float32, device="cuda")[:, :d_out]
+    rocs.linear(padded(X), padded(W), bias=to_dev(b), relu=True, out=Y)
+    want = ref.ikbo_linear(wl.offsets_from_counts([M]), None, X, W, bias=b, relu=True)
+    assert rel_err(to_host_f64(Y), want) <= tol_for(dtype)
+
+
 def test_linear_empty_batch():
     co = np.zeros(3, np.int32)
     cfg = wl.CONFIGS[2].with_(R=2, d_req=64, d_cand=64, d_out=64)
