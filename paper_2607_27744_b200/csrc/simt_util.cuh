@@ -132,26 +132,26 @@ __device__ __forceinline__ void rows_to_shared_async(const T* __restrict__ src, 
   }
 }
 
-// Packed fp32 pairs: one issue slot for two FMAs.
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float2 unpack2(uint64_t v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
+// `rows` dense rows of d elements (d a multiple of a 16-byte vector) into shared memory as fp32 with row
+// stride `stride` floats; fp32 by cp.async, bf16 through registers.
+template <typename T>
+__device__ __forceinline__ void dense_rows_to_shared_async(const T* __restrict__ src, int rows, int d,
+                                                           float* __restrict__ dst, int stride, int tid, int threads) {
+  constexpr int kVec = 16 / (int)sizeof(T);
+  const int per_row = d / kVec;
+#pragma unroll 4
+  for (int v = tid; v < rows * per_row; v += threads) {
+    const int r = v / per_row;
+    float* to = dst + r * stride + (v - r * per_row) * kVec;
+    if constexpr (sizeof(T) == 4) {
+      cp_async_16((uint32_t)__cvta_generic_to_shared(to), src + (int64_t)v * kVec, 16);
+    } else {
+      float4 lo, hi;
+      bf16x8_to_f32(__ldg(reinterpret_cast<const uint4*>(src) + v), lo, hi);
+      *reinterpret_cast<float4*>(to) = lo;
+      *reinterpret_cast<float4*>(to + 4) = hi;
+    }
+  }
 }
 
 __device__ __forceinline__ void store_pair(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }

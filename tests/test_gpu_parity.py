@@ -440,6 +440,16 @@ def test_glm_bf16_other_split(path):
     assert _run_glm(cfg, co, path=path) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("dtype,n_r,n_c,d,n_co", [("f32", 4, 2, 16, 0), ("f32", 1, 1, 4, 1), ("f32", 30, 7, 20, 5), ("f32", 24, 8, 128, 4),
+                                                   ("f32", 5, 70, 12, 3), ("f32", 8, 220, 4, 64), ("bf16", 20, 12, 72, 6), ("bf16", 3, 5, 8, 9)])
+def test_glm_general_kernel_tiles(dtype, n_r, n_c, d, n_co):
+    # tiles of about 64 rows: several candidates, one candidate wider than a tile, embedding counts that leave
+    # remainders in every 4 x 4 group, a compression block too large for shared memory
+    co = wl.offsets_from_counts([1, 0, 9, 33, 2] if n_c < 100 else [1, 0, 3])
+    cfg = wl.CONFIGS[4].with_(R=len(co) - 1, dtype=dtype, n_r=n_r, n_c=n_c, d_emb=d, n_ro=min(2, n_co), n_co=n_co)
+    assert _run_glm(cfg, co) <= tol_for(dtype)
+
+
 @pytest.mark.parametrize("R", [1, 127, 128, 129, 255, 257, 12000, 12001])
 def test_work_lists_of_many_requests(R):
     # the lists are scanned by 256 threads per block up to 12000 requests and on the host beyond: counts of
