@@ -122,13 +122,16 @@ __global__ void __launch_bounds__(128) fm_candidate_simt_kernel(int32_t n_r, int
 }
 
 // ---------------------------------------------------------------------------------------------
-// Candidate side, bf16 streaming kernel: n_c = 16, k in {8, 16}, d a multiple of 64 up to 256.
+// Candidate side, bf16 streaming kernel: n_c up to 16, even k up to 32, d a multiple of 64 up to 256.
+// The fragments hold 16 candidate rows: of a candidate with fewer the rest are the next candidate's, which
+// step 1 masks to zero (0 x NaN of a neighbour must not arise) and step 2 computes and drops.  Bound by HBM.
+// 18 399 candidates of 12 embeddings x 128, k = 16: the general kernel (a block per candidate) took 284 us, a
+// whole pass through this one 34 us, most of it host work.
 // ---------------------------------------------------------------------------------------------
-constexpr int kNc = 16;            // rows per candidate
+constexpr int kFragRows = 16;      // rows of a candidate's fragments
 constexpr int kTileCands = 8;      // candidates per tile = compute warps per CTA
-constexpr int kTileRows = kNc * kTileCands;  // 128
 constexpr int kFmThreads = (kTileCands + 1) * 32;
-constexpr int kSlabBytes = kTileRows * 128;  // 64 columns of the tile, 128-byte swizzled rows
+constexpr int kMaxStages = 12;
 constexpr uint32_t kStatusFm = 0x600;
 
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
@@ -261,31 +264,36 @@ __global__ void __launch_bounds__(256) fm_request_mma_kernel(int32_t n_r, int32_
 
 struct FmParams {
   int64_t N;
-  int32_t n_r, k, num_tiles;
-  const __nv_bfloat16* P;        // [n_r + 16, k]
+  int32_t n_r, n_c, k, num_tiles, stages;
+  const __nv_bfloat16* P;        // [n_r + n_c, k]
   const int32_t* row2req;        // [N]
   const float* TT;               // [R, k, d]
-  __nv_bfloat16* FC;             // [N, 16, k]
+  __nv_bfloat16* FC;             // [N, n_c, k]
   uint32_t* status;
 };
 
-template <int D, int STAGES>
+// KT: blocks of 16 projection columns.  With one, the request's T stays in registers while consecutive
+// candidates share it; with two it would not fit beside H and comes from L1 for every candidate.
+template <int D, int KT, bool FULL>
 __global__ void __launch_bounds__(kFmThreads, 1)
 fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmParams p) {
   constexpr int kSlabs = D / 64;
-  constexpr int kStageBytes = kSlabs * kSlabBytes;
   constexpr int kPairs = D / 16;  // pairs of 8-column groups = k-steps of step 2
   extern __shared__ __align__(1024) uint8_t smem[];
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * kStageBytes);
-  uint64_t* empty = full + STAGES;
-  AbortFlag* abort_flag = reinterpret_cast<AbortFlag*>(empty + STAGES);
+  const int32_t n_c = FULL ? kFragRows : p.n_c;
+  const int32_t slab_bytes = kTileCands * n_c * 128;  // 64 columns of the tile, 128-byte swizzled rows
+  const int32_t stage_bytes = kSlabs * slab_bytes;
+  // behind the stages: rows that the last candidate's fragments read past the tile
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.stages * stage_bytes + (FULL ? 0 : kFragRows * 128));
+  uint64_t* empty = full + kMaxStages;
+  AbortFlag* abort_flag = reinterpret_cast<AbortFlag*>(empty + kMaxStages);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   if ((smem_u32(smem) & 1023u) != 0) {  // the swizzled tiles assume a 1024-byte aligned base
     if (threadIdx.x == 0) atomicCAS(p.status, 0u, kStatusFm | 15);
     return;
   }
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < p.stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], kTileCands);
     }
@@ -303,119 +311,145 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
     // ------------------------------ TMA producer ------------------------------------------
     if (lane == 0) {
       prefetch_tensormap(&map_xc);
-      uint32_t it = 0;
+      int s = 0;
+      uint32_t phase = 0, it = 0;
       for (int32_t t = tile_begin; t < tile_end; ++t, ++it) {
-        const int s = it % STAGES;
-        if (!mbar_wait(&empty[s], ((it / STAGES) & 1) ^ 1, abort_flag, p.status, kStatusFm | 1)) break;
-        mbar_expect_tx(&full[s], kStageBytes);
+        if (!mbar_wait(&empty[s], phase ^ 1, abort_flag, p.status, kStatusFm | 1)) break;
+        mbar_expect_tx(&full[s], stage_bytes);
 #pragma unroll
         for (int sl = 0; sl < kSlabs; ++sl)
-          tma_load_2d(smem + s * kStageBytes + sl * kSlabBytes, &map_xc, &full[s], sl * 64, t * kTileRows);
+          tma_load_2d(smem + s * stage_bytes + sl * slab_bytes, &map_xc, &full[s], sl * 64, t * kTileCands * n_c);
+        if (++s == p.stages) { s = 0; phase ^= 1; }
       }
       // loads in flight land in this CTA's shared memory: wait for them before the CTA may exit
-      for (int s = 0; s < STAGES; ++s) {
-        const uint32_t n_issued = it / STAGES + (((int)(it % STAGES) > s) ? 1 : 0);
+      for (int st = 0; st < p.stages; ++st) {
+        const uint32_t n_issued = it / p.stages + (((int)(it % p.stages) > st) ? 1 : 0);
         if (n_issued == 0) continue;
         const uint64_t t0 = globaltimer_ns();
-        while (!mbar_try_wait(&full[s], (n_issued - 1) & 1) && globaltimer_ns() - t0 < kWaitLimitNs) {}
+        while (!mbar_try_wait(&full[st], (n_issued - 1) & 1) && globaltimer_ns() - t0 < kWaitLimitNs) {}
       }
     }
   } else {
     // ------------------------------ one candidate per warp ---------------------------------
     const int g = lane / 4, tq = lane % 4;  // fragment row group and column pair
     // P_C^T as the M x K operand of step 1: A[m = projection column][kk = candidate row]
-    uint32_t pa[4];
+    uint32_t pa[KT][4];
     {
       const __nv_bfloat16* pc = p.P + (int64_t)p.n_r * p.k;
-      auto at = [&](int row, int col) -> float {  // P_C[row][col], zero beyond k columns
-        return col < p.k ? __bfloat162float(pc[row * p.k + col]) : 0.f;
+      auto at = [&](int row, int col) -> float {  // P_C[row][col], zero beyond n_c rows and k columns
+        return row < n_c && col < p.k ? __bfloat162float(pc[row * p.k + col]) : 0.f;
       };
-      pa[0] = pack_bf16(at(2 * tq, g), at(2 * tq + 1, g));
-      pa[1] = pack_bf16(at(2 * tq, g + 8), at(2 * tq + 1, g + 8));
-      pa[2] = pack_bf16(at(2 * tq + 8, g), at(2 * tq + 9, g));
-      pa[3] = pack_bf16(at(2 * tq + 8, g + 8), at(2 * tq + 9, g + 8));
+#pragma unroll
+      for (int kt = 0; kt < KT; ++kt) {
+        const int c = kt * 16 + g;
+        pa[kt][0] = pack_bf16(at(2 * tq, c), at(2 * tq + 1, c));
+        pa[kt][1] = pack_bf16(at(2 * tq, c + 8), at(2 * tq + 1, c + 8));
+        pa[kt][2] = pack_bf16(at(2 * tq + 8, c), at(2 * tq + 9, c));
+        pa[kt][3] = pack_bf16(at(2 * tq + 8, c + 8), at(2 * tq + 9, c + 8));
+      }
     }
+    // rows of the K x N operand of step 1 that are this candidate's: 2 tq, 2 tq + 1 and the two 8 further on
+    auto row_mask = [&](int row) { return (row < n_c ? 0xffffu : 0u) | (row + 1 < n_c ? 0xffff0000u : 0u); };
+    const uint32_t keep_lo = row_mask(2 * tq), keep_hi = row_mask(2 * tq + 8);
     // this lane's address pattern inside a candidate's 16 rows: row, and which of the two
     // 8-column groups of a pair
-    const int lrow = (lane % 8) + ((lane / 8) % 2) * 8;
+    const int trow = warp * n_c + (lane % 8) + ((lane / 8) % 2) * 8;
     const int lsel = lane / 16;
-    float tfrag[kPairs][2][4];  // T^T of the cached request in step-1 accumulator layout
+    float tfrag[KT == 1 ? kPairs : 1][2][4];  // T^T of the cached request in step-1 accumulator layout
+    auto load_t = [&](const float* tt, int kt, int cp, float (&f)[2][4]) {
+      const int c = kt * 16 + g;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int col = (2 * cp + h) * 8 + 2 * tq;
+        const float2 lo = c < p.k ? *reinterpret_cast<const float2*>(tt + c * D + col) : make_float2(0.f, 0.f);
+        const float2 hi = c + 8 < p.k ? *reinterpret_cast<const float2*>(tt + (c + 8) * D + col) : make_float2(0.f, 0.f);
+        f[h][0] = lo.x;
+        f[h][1] = lo.y;
+        f[h][2] = hi.x;
+        f[h][3] = hi.y;
+      }
+    };
     int32_t cached_req = -1;
-    uint32_t it = 0;
+    int s = 0;
+    uint32_t phase = 0;
     // the request of this warp's candidate, fetched one tile ahead of its use (the load would
     // otherwise sit on every candidate's critical path)
     int32_t r_next = 0;
     if (tile_begin < tile_end && (int64_t)tile_begin * kTileCands + warp < p.N)
       r_next = p.row2req[(int64_t)tile_begin * kTileCands + warp];
-    for (int32_t t = tile_begin; t < tile_end; ++t, ++it) {
-      const int s = it % STAGES;
+    for (int32_t t = tile_begin; t < tile_end; ++t) {
       const int32_t r = r_next;
       {
         const int64_t cand_next = (int64_t)(t + 1) * kTileCands + warp;
         if (t + 1 < tile_end && cand_next < p.N) r_next = p.row2req[cand_next];
       }
-      if (!mbar_wait(&full[s], (it / STAGES) & 1, abort_flag, p.status, kStatusFm | 2)) break;
+      if (!mbar_wait(&full[s], phase, abort_flag, p.status, kStatusFm | 2)) break;
       const int64_t cand = (int64_t)t * kTileCands + warp;
       if (cand < p.N) {
+        const float* tt = p.TT + (int64_t)r * p.k * D;
         if (r != cached_req) {
           if (cached_req < 0) griddep_wait();  // TT comes from the request kernel launched just before
           cached_req = r;
-          const float* tt = p.TT + (int64_t)r * p.k * D;
+          if constexpr (KT == 1) {
 #pragma unroll
-          for (int cp = 0; cp < kPairs; ++cp)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int col = (2 * cp + h) * 8 + 2 * tq;
-              const float2 lo = g < p.k ? *reinterpret_cast<const float2*>(tt + g * D + col) : make_float2(0.f, 0.f);
-              const float2 hi = g + 8 < p.k ? *reinterpret_cast<const float2*>(tt + (g + 8) * D + col) : make_float2(0.f, 0.f);
-              tfrag[cp][h][0] = lo.x;
-              tfrag[cp][h][1] = lo.y;
-              tfrag[cp][h][2] = hi.x;
-              tfrag[cp][h][3] = hi.y;
-            }
-        }
-        const uint32_t tile = smem_u32(smem + s * kStageBytes);
-        const int trow = warp * kNc + lrow;
-        // step 1: H^T (16 x D) = T^T + P_C^T X^C, rounded to bf16 as the K x N operand of step 2
-        uint32_t hb[kPairs][2][2];  // [k-step][projection columns 0-7 | 8-15][b0, b1]
-#pragma unroll
-        for (int cp = 0; cp < kPairs; ++cp) {
-          const int chunk = 2 * cp + lsel;  // 16-byte chunk along d
-          uint32_t xb[4];
-          ldmatrix_x4_trans(tile + (chunk / 8) * kSlabBytes + trow * 128 + (((chunk % 8) ^ (trow & 7)) << 4), xb);
-          float acc0[4], acc1[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            acc0[e] = tfrag[cp][0][e];
-            acc1[e] = tfrag[cp][1][e];
+            for (int cp = 0; cp < kPairs; ++cp) load_t(tt, 0, cp, tfrag[cp]);
           }
-          mma_bf16(acc0, pa, xb[0], xb[1]);
-          mma_bf16(acc1, pa, xb[2], xb[3]);
-          hb[cp][0][0] = pack_bf16(acc0[0], acc0[1]);
-          hb[cp][0][1] = pack_bf16(acc1[0], acc1[1]);
-          hb[cp][1][0] = pack_bf16(acc0[2], acc0[3]);
-          hb[cp][1][1] = pack_bf16(acc1[2], acc1[3]);
         }
-        // step 2: FC (16 x 16) = X^C H
-        float out0[4] = {0.f, 0.f, 0.f, 0.f}, out1[4] = {0.f, 0.f, 0.f, 0.f};
+        const uint32_t tile = smem_u32(smem + s * stage_bytes) + trow * 128;
+        __nv_bfloat16* fc = p.FC + cand * n_c * p.k;
 #pragma unroll
-        for (int cp = 0; cp < kPairs; ++cp) {
-          const int chunk = 2 * cp + lsel;
-          uint32_t xa[4];
-          ldmatrix_x4(tile + (chunk / 8) * kSlabBytes + trow * 128 + (((chunk % 8) ^ (trow & 7)) << 4), xa);
-          mma_bf16(out0, xa, hb[cp][0][0], hb[cp][0][1]);
-          mma_bf16(out1, xa, hb[cp][1][0], hb[cp][1][1]);
-        }
-        __nv_bfloat16* fc = p.FC + cand * kNc * p.k;
-        *reinterpret_cast<uint32_t*>(fc + g * p.k + 2 * tq) = pack_bf16(out0[0], out0[1]);
-        *reinterpret_cast<uint32_t*>(fc + (g + 8) * p.k + 2 * tq) = pack_bf16(out0[2], out0[3]);
-        if (p.k > 8) {
-          *reinterpret_cast<uint32_t*>(fc + g * p.k + 8 + 2 * tq) = pack_bf16(out1[0], out1[1]);
-          *reinterpret_cast<uint32_t*>(fc + (g + 8) * p.k + 8 + 2 * tq) = pack_bf16(out1[2], out1[3]);
+        for (int kt = 0; kt < KT; ++kt) {
+          // step 1: H^T (16 x D) = T^T + P_C^T X^C, rounded to bf16 as the K x N operand of step 2
+          uint32_t hb[kPairs][2][2];  // [k-step][projection columns 0-7 | 8-15][b0, b1]
+#pragma unroll
+          for (int cp = 0; cp < kPairs; ++cp) {
+            const int chunk = 2 * cp + lsel;  // 16-byte chunk along d
+            uint32_t xb[4];
+            ldmatrix_x4_trans(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xb);
+            if constexpr (!FULL) {
+              xb[0] &= keep_lo;
+              xb[1] &= keep_hi;
+              xb[2] &= keep_lo;
+              xb[3] &= keep_hi;
+            }
+            float f[2][4];
+            if constexpr (KT == 1) {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) f[e / 4][e % 4] = tfrag[cp][e / 4][e % 4];
+            } else {
+              load_t(tt, kt, cp, f);
+            }
+            mma_bf16(f[0], pa[kt], xb[0], xb[1]);
+            mma_bf16(f[1], pa[kt], xb[2], xb[3]);
+            hb[cp][0][0] = pack_bf16(f[0][0], f[0][1]);
+            hb[cp][0][1] = pack_bf16(f[1][0], f[1][1]);
+            hb[cp][1][0] = pack_bf16(f[0][2], f[0][3]);
+            hb[cp][1][1] = pack_bf16(f[1][2], f[1][3]);
+          }
+          // step 2: FC (16 x 16) = X^C H
+          float out[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+          for (int cp = 0; cp < kPairs; ++cp) {
+            const int chunk = 2 * cp + lsel;
+            uint32_t xa[4];
+            ldmatrix_x4(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xa);
+            mma_bf16(out[0], xa, hb[cp][0][0], hb[cp][0][1]);
+            mma_bf16(out[1], xa, hb[cp][1][0], hb[cp][1][1]);
+          }
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int col = kt * 16 + 8 * h + 2 * tq;
+            if (col < p.k) {
+              if (FULL || g < n_c) *reinterpret_cast<uint32_t*>(fc + g * p.k + col) = pack_bf16(out[h][0], out[h][1]);
+              if (FULL || g + 8 < n_c)
+                *reinterpret_cast<uint32_t*>(fc + (g + 8) * p.k + col) = pack_bf16(out[h][2], out[h][3]);
+            }
+          }
         }
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[s]);
+      if (++s == p.stages) { s = 0; phase ^= 1; }
     }
   }
 }
@@ -430,35 +464,38 @@ int sm_count_fm() {
   return n;
 }
 
-template <int D>
-rocs_status_t launch_fm_mma(const rocs_plan* plan, const int32_t* row2req, int32_t n_r, int32_t k, const void* XC,
-                            const void* P, const float* TT, void* FC, cudaStream_t stream) {
-  constexpr int kStages = D <= 64 ? 8 : D <= 128 ? 6 : 3;
-  constexpr int kSmem = kStages * (D / 64) * kSlabBytes + 512;
+template <int D, int KT, bool FULL>
+rocs_status_t launch_fm_mma_as(const rocs_plan* plan, const int32_t* row2req, int32_t n_r, int32_t n_c, int32_t k,
+                               const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
+  const int stage_bytes = D / 64 * kTileCands * n_c * 128;
+  constexpr int kFixed = kFragRows * 128 + 2 * kMaxStages * 8 + 16;
   CUtensorMap map_xc;
-  if (!make_tensor_map_2d(&map_xc, XC, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)plan->N * kNc, D, D, kTileRows, 64,
-                          true))
+  if (!make_tensor_map_2d(&map_xc, XC, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)plan->N * n_c, D, D,
+                          (uint32_t)(kTileCands * n_c), 64, true))
     return ROCS_ERR_CUDA;
   uint32_t* status = device_status_word();
   if (!status) return ROCS_ERR_CUDA;
   FmParams p{};
   p.N = plan->N;
   p.n_r = n_r;
+  p.n_c = n_c;
   p.k = k;
   p.num_tiles = (int32_t)((plan->N + kTileCands - 1) / kTileCands);
+  p.stages = std::min(kMaxStages, (227 * 1024 - kFixed) / stage_bytes);
   p.P = (const __nv_bfloat16*)P;
   p.row2req = row2req;
   p.TT = TT;
   p.FC = (__nv_bfloat16*)FC;
   p.status = status;
-  auto kern = fm_candidate_mma_kernel<D, kStages>;
-  ROCS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
+  const int smem = p.stages * stage_bytes + kFixed;
+  auto kern = fm_candidate_mma_kernel<D, KT, FULL>;
+  ROCS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   // Launched so that it may overlap the request kernel in front of it on the stream (that kernel
   // releases its dependents at once); nothing else this kernel reads is written by that launch.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)std::min(p.num_tiles, sm_count_fm()));
   cfg.blockDim = dim3(kFmThreads);
-  cfg.dynamicSmemBytes = kSmem;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -467,6 +504,14 @@ rocs_status_t launch_fm_mma(const rocs_plan* plan, const int32_t* row2req, int32
   cfg.numAttrs = 1;
   ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, map_xc, p));
   return ROCS_OK;
+}
+
+template <int D>
+rocs_status_t launch_fm_mma(const rocs_plan* plan, const int32_t* row2req, int32_t n_r, int32_t n_c, int32_t k,
+                            const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
+  if (k > 16) return launch_fm_mma_as<D, 2, false>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
+  if (n_c < kFragRows) return launch_fm_mma_as<D, 1, false>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
+  return launch_fm_mma_as<D, 1, true>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
 }
 
 template <typename T>
@@ -498,10 +543,10 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
   if (plan->N == 0 || !FC) return ROCS_OK;
   if (fast_candidates) {
     switch (d) {
-      case 64: return launch_fm_mma<64>(plan, row2req, n_r, k, XC, P, TT, FC, stream);
-      case 128: return launch_fm_mma<128>(plan, row2req, n_r, k, XC, P, TT, FC, stream);
-      case 192: return launch_fm_mma<192>(plan, row2req, n_r, k, XC, P, TT, FC, stream);
-      case 256: return launch_fm_mma<256>(plan, row2req, n_r, k, XC, P, TT, FC, stream);
+      case 64: return launch_fm_mma<64>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 128: return launch_fm_mma<128>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 192: return launch_fm_mma<192>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 256: return launch_fm_mma<256>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
       default: break;
     }
   }
@@ -515,7 +560,7 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
 }  // namespace
 
 bool fm_projection_fast_supported(int32_t n_c, int32_t d, int32_t k) {
-  return n_c == kNc && (k == 8 || k == 16) && d % 64 == 0 && d >= 64 && d <= 256;
+  return n_c <= kFragRows && k % 2 == 0 && k <= 32 && d % 64 == 0 && d >= 64 && d <= 256;
 }
 
 rocs_status_t fm_projection(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, int32_t k,

@@ -50,6 +50,23 @@ def test_bf16_ragged_segments_and_tail_tile(path, k, d_emb):
     assert _run(cfg, co, k, path=path) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("n_c,k,d_emb", [(12, 16, 128), (4, 24, 192), (1, 2, 64), (15, 32, 256), (16, 18, 128), (8, 10, 64)])
+def test_bf16_streaming_kernel_with_partial_fragments(n_c, k, d_emb):
+    # fewer than 16 rows per candidate (fragments reach into the next candidate's rows), one and two blocks of
+    # projection columns, the last of them partial; a candidate full of NaN must not show in its neighbours
+    co = wl.offsets_from_counts([1, 0, 9, 8, 33, 7, 0, 133])
+    cfg = wl.CONFIGS[4].with_(R=len(co) - 1, n_r=20, n_c=n_c, d_emb=d_emb)
+    assert _run(cfg, co, k) <= tol_for("bf16")
+    d = wl.glm_inputs(cfg, co)
+    P, XC = to_dev(wl.fm_projection_weight(cfg, k)), to_dev(d["XC"])
+    plan = rocs.plan_create(to_dev(co), co)
+    base = _bits(rocs.glm_fm_projection(plan, to_dev(d["XR"]), XC, P)["FC"])
+    XC[60] = float("nan")
+    pert = _bits(rocs.glm_fm_projection(plan, to_dev(d["XR"]), XC, P)["FC"])
+    others = np.arange(len(base)) != 60
+    assert np.array_equal(base[others], pert[others])
+
+
 @pytest.mark.parametrize("path", PATHS)
 def test_bf16_shapes_outside_the_streaming_kernel(path):
     co = wl.offsets_from_counts([20, 3, 41])
