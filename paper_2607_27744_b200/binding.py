@@ -1,8 +1,9 @@
-"""ctypes binding of ``librocs.so`` (declared in ``include/rocs.h``).
+"""Binding of ``librocs.so`` (declared in ``include/rocs.h``).
 
 Argument marshalling only: torch supplies device memory and streams, every step of the
 computation runs inside the library's CUDA kernels.  There is no CPU or eager fallback: if the
-library is missing or a call fails, an exception is raised.
+library is missing or a call fails, an exception is raised.  The calls of a scoring loop go through
+the extension ``_native`` (``csrc/binding.cpp``), the rest through ctypes.
 
 Functions mirror the C entry points (``rocs_`` prefix dropped): :func:`plan_create`,
 :func:`ikbo_linear`, :func:`linear`, :func:`dca_attention`, :func:`glm_interaction`.
@@ -19,6 +20,7 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "librocs.so")
 _lib = None
+_ext = None
 
 OK = 0
 BF16, F32 = 0, 1
@@ -118,49 +120,38 @@ def last_device_status() -> int:
     return detail.value
 
 
-def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.bfloat16:
-        return BF16
-    if t.dtype == torch.float32:
-        return F32
-    raise TypeError(f"unsupported dtype {t.dtype}")
-
-
-def _p(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
-
-
-def _stream() -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-
-
-def _rows_2d(t: torch.Tensor):
-    assert t.dim() == 2 and t.stride(1) == 1 and t.is_cuda, "expect a row-major 2-D CUDA tensor"
-    return t.stride(0) if t.shape[0] > 1 else max(t.stride(0), t.shape[1])
+def _native():
+    """Loads the extension on first use; raises if it (or the library it calls) has not been built."""
+    global _ext
+    lib()
+    try:
+        from . import _native as ext
+    except ImportError as e:
+        raise RuntimeError(f"the extension _native is missing or broken ({e}): build it with "
+                           "`python -m paper_2607_27744_b200.build` (there is no fallback path)") from e
+    ext.set_error_type(RocsError)
+    _ext = ext
+    return ext
 
 
 class Plan:
     """Owns a ``rocs_plan_t`` (Section 4.1: the request-candidate map in segment form)."""
 
     def __init__(self, cand_offsets: torch.Tensor, cand_offsets_host=None):
-        assert cand_offsets.is_cuda and cand_offsets.dtype == torch.int32 and cand_offsets.is_contiguous()
+        self.handle = None
         self.cand_offsets = cand_offsets
-        self.R = cand_offsets.numel() - 1
-        if cand_offsets_host is None:
+        host = cand_offsets_host
+        if host is None:
             host = cand_offsets.cpu()
-        else:
-            host = torch.as_tensor(cand_offsets_host, dtype=torch.int32).contiguous()
+        elif not (isinstance(host, torch.Tensor) and host.dtype is torch.int32 and host.is_contiguous()):
+            host = torch.as_tensor(host, dtype=torch.int32).contiguous()
         self._host = host
-        self.N = int(host[-1]) if host.numel() else 0
-        handle = ctypes.c_void_p()
-        _check(lib().rocs_plan_create(ctypes.byref(handle), self.R, self.N, _p(cand_offsets),
-                                      ctypes.c_void_p(host.data_ptr()), _stream()), "rocs_plan_create")
-        self.handle = handle
+        self.handle, self.R, self.N = (_ext or _native()).plan_create(cand_offsets, host)
 
     def close(self):
-        if getattr(self, "handle", None):
-            lib().rocs_plan_destroy(self.handle)
-            self.handle = None
+        handle, self.handle = self.handle, None
+        if handle:
+            _ext.plan_destroy(handle)
 
     def __del__(self):
         try:
@@ -182,24 +173,7 @@ def ikbo_linear(plan: Plan, XR: Optional[torch.Tensor], XC: torch.Tensor, W_CR: 
                 out: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Y_i = act(Z[m_i] + X^C_i W_CC^T), Z = X^R W_CR^T + bias (Eq. 14).  W_CR / W_CC may be column
     slices of one [d_out, d_req + d_cand] weight."""
-    d_req = 0 if XR is None else XR.shape[1]
-    d_cand, d_out = XC.shape[1], W_CC.shape[0]
-    assert XC.shape[0] == plan.N
-    if out is None:
-        out = torch.empty((plan.N, d_out), dtype=XC.dtype, device=XC.device)
-    need = ikbo_linear_workspace(plan, d_out) if d_req > 0 else 0
-    if need and workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=XC.device)
-    if bias is not None:
-        assert bias.dtype == torch.float32 and bias.is_contiguous()
-    code = lib().rocs_ikbo_linear(
-        plan.handle, _dtype_code(XC), d_req, d_cand, d_out,
-        _p(XR), _rows_2d(XR) if d_req else 0, _p(XC), _rows_2d(XC),
-        _p(W_CR) if d_req else None, _rows_2d(W_CR) if d_req else 0, _p(W_CC), _rows_2d(W_CC),
-        _p(bias), ACT_RELU if relu else ACT_NONE, _p(out), _rows_2d(out),
-        _p(workspace), workspace.numel() if workspace is not None else 0, _stream())
-    _check(code, "rocs_ikbo_linear")
-    return out
+    return (_ext or _native()).ikbo_linear(plan.handle, plan.R, plan.N, XR, XC, W_CR, W_CC, bias, relu, out, workspace)
 
 
 def ikbo_linear_stats(plan: Plan, XR: torch.Tensor, XC: torch.Tensor, W_CR: torch.Tensor, W_CC: torch.Tensor,
@@ -207,31 +181,13 @@ def ikbo_linear_stats(plan: Plan, XR: torch.Tensor, XC: torch.Tensor, W_CR: torc
                       row_stats: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None):
     """ikbo_linear that also leaves each output row's (sum, sum of squares) for a normalisation folded
     into the next layer (Eq. 7).  Returns (Y, row_stats [N, 2] fp32)."""
-    d_req, d_cand, d_out = XR.shape[1], XC.shape[1], W_CC.shape[0]
-    assert XC.shape[0] == plan.N
-    if out is None:
-        out = torch.empty((plan.N, d_out), dtype=XC.dtype, device=XC.device)
-    if row_stats is None:
-        row_stats = torch.empty((plan.N, 2), dtype=torch.float32, device=XC.device)
-    need = int(lib().rocs_ikbo_linear_stats_workspace(plan.handle, d_out))
-    if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=XC.device)
-    code = lib().rocs_ikbo_linear_stats(
-        plan.handle, _dtype_code(XC), d_req, d_cand, d_out, _p(XR), _rows_2d(XR), _p(XC), _rows_2d(XC),
-        _p(W_CR), _rows_2d(W_CR), _p(W_CC), _rows_2d(W_CC), _p(bias), ACT_RELU if relu else ACT_NONE, _p(out),
-        _rows_2d(out), _p(row_stats), _p(workspace), workspace.numel(), _stream())
-    _check(code, "rocs_ikbo_linear_stats")
-    return out, row_stats
+    return (_ext or _native()).ikbo_linear_stats(plan.handle, plan.R, plan.N, XR, XC, W_CR, W_CC, bias, relu, out, row_stats,
+                                                 workspace)
 
 
 def weight_row_sums(W: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """wbar[n] = sum_k W[n, k] in fp32: the W 1 term of a LayerNorm folded into the layer."""
-    d_out, d_in = W.shape
-    if out is None:
-        out = torch.empty(d_out, dtype=torch.float32, device=W.device)
-    _check(lib().rocs_weight_row_sums(_dtype_code(W), d_out, d_in, _p(W), _rows_2d(W), _p(out), _stream()),
-           "rocs_weight_row_sums")
-    return out
+    return (_ext or _native()).weight_row_sums(W, out)
 
 
 def linear_normed(X: torch.Tensor, row_stats: torch.Tensor, W: torch.Tensor, wbar: Optional[torch.Tensor] = None,
@@ -239,46 +195,20 @@ def linear_normed(X: torch.Tensor, row_stats: torch.Tensor, W: torch.Tensor, wba
                   out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Y = act(norm(X) W^T + bias) with the normalisation applied to the layer's accumulators (Eq. 7
     folded into the epilogue); gamma and beta are folded into W and bias by the caller."""
-    M, d_in = X.shape
-    d_out = W.shape[0]
-    assert row_stats.dtype == torch.float32 and row_stats.shape == (M, 2) and row_stats.is_contiguous()
-    if out is None:
-        out = torch.empty((M, d_out), dtype=X.dtype, device=X.device)
-    code = lib().rocs_linear_normed(_dtype_code(X), kind, M, d_in, d_out, _p(X), _rows_2d(X), _p(row_stats), float(eps),
-                                    _p(W), _rows_2d(W), _p(wbar), _p(bias), ACT_RELU if relu else ACT_NONE, _p(out),
-                                    _rows_2d(out), _stream())
-    _check(code, "rocs_linear_normed")
-    return out
+    return (_ext or _native()).linear_normed(X, row_stats, W, wbar, bias, eps, kind, relu, out)
 
 
 def linear(X: torch.Tensor, W: torch.Tensor, bias: Optional[torch.Tensor] = None, relu: bool = False,
            out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Y = act(X W^T + bias), the one-group case of Eq. 4."""
-    M, d_in = X.shape
-    d_out = W.shape[0]
-    if out is None:
-        out = torch.empty((M, d_out), dtype=X.dtype, device=X.device)
-    code = lib().rocs_linear(_dtype_code(X), M, d_in, d_out, _p(X), _rows_2d(X), _p(W), _rows_2d(W), _p(bias),
-                             ACT_RELU if relu else ACT_NONE, _p(out), _rows_2d(out), _stream())
-    _check(code, "rocs_linear")
-    return out
+    return (_ext or _native()).linear(X, W, bias, relu, out)
 
 
 def dca_attention(plan: Plan, Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, seq_offsets: torch.Tensor,
                   scale: float = 0.0, out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Candidate-side cross attention over the request's shared K/V (Eq. 13).
     Q [N, n_q, H, dh]; K, V [T, H, dh]; seq_offsets int32 [R+1] on the device."""
-    N, n_q, H, dh = Q.shape
-    assert N == plan.N and Q.is_contiguous() and K.is_contiguous() and V.is_contiguous()
-    assert seq_offsets.dtype == torch.int32 and seq_offsets.is_cuda and seq_offsets.numel() == plan.R + 1
-    if out is None:
-        out = torch.empty_like(Q)
-    need = int(lib().rocs_dca_attention_workspace(plan.handle, n_q, H, dh))
-    ws = torch.empty(need, dtype=torch.uint8, device=Q.device) if need else None
-    code = lib().rocs_dca_attention(plan.handle, _dtype_code(Q), n_q, H, dh, float(scale), _p(Q), _p(K), _p(V),
-                                    K.shape[0], _p(seq_offsets), _p(out), _p(ws), need, _stream())
-    _check(code, "rocs_dca_attention")
-    return out
+    return (_ext or _native()).dca_attention(plan.handle, plan.R, plan.N, Q, K, V, seq_offsets, scale, out)
 
 
 def glm_interaction_workspace(plan: Plan, n_r: int, n_c: int, n_co: int) -> int:
@@ -290,29 +220,25 @@ def glm_interaction(plan: Plan, XR: torch.Tensor, XC: torch.Tensor, W: Optional[
                     workspace: Optional[torch.Tensor] = None, outs: Optional[dict] = None) -> dict:
     """GLM factorization machine (Eq. 9-10) with optional row-axis compression (Eq. 5-6).
     Returns a dict with the tensors that were requested among YR, YC, OR, OC."""
-    R, n_r, d = XR.shape
+    R, n_r, _ = XR.shape
     N, n_c, _ = XC.shape
     n = n_r + n_c
-    assert R == plan.R and N == plan.N and XR.is_contiguous() and XC.is_contiguous()
-    dev, dt = XC.device, XC.dtype
-    outs = dict(outs or {})
+    outs = dict(outs) if outs else {}
+
+    def fill(key, *shape):
+        if key not in outs:
+            outs[key] = torch.empty(shape, dtype=XC.dtype, device=XC.device)
+
     if want_raw:
         if want_request_side:
-            outs.setdefault("YR", torch.empty((R, n_r, n), dtype=dt, device=dev))
-        outs.setdefault("YC", torch.empty((N, n_c, n), dtype=dt, device=dev))
+            fill("YR", R, n_r, n)
+        fill("YC", N, n_c, n)
     if W is not None:
-        assert W.shape == (n_ro + n_co, n) and W.is_contiguous()
         if want_request_side:
-            outs.setdefault("OR", torch.empty((R, n_ro, n), dtype=dt, device=dev))
-        outs.setdefault("OC", torch.empty((N, n_co, n), dtype=dt, device=dev))
-    need = glm_interaction_workspace(plan, n_r, n_c, n_co) if W is not None else 0
-    if need and workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=dev)
-    code = lib().rocs_glm_interaction(
-        plan.handle, _dtype_code(XC), n_r, n_c, d, _p(XR), _p(XC), _p(W), n_ro, n_co,
-        _p(outs.get("YR")), _p(outs.get("YC")), _p(outs.get("OR")), _p(outs.get("OC")),
-        _p(workspace), workspace.numel() if workspace is not None else 0, _stream())
-    _check(code, "rocs_glm_interaction")
+            fill("OR", R, n_ro, n)
+        fill("OC", N, n_co, n)
+    (_ext or _native()).glm_interaction(plan.handle, plan.R, plan.N, XR, XC, W, n_ro, n_co, outs.get("YR"), outs.get("YC"),
+                                        outs.get("OR"), outs.get("OC"), workspace)
     return outs
 
 
@@ -325,37 +251,20 @@ def glm_fm_projection(plan: Plan, XR: torch.Tensor, XC: torch.Tensor, P: torch.T
                       outs: Optional[dict] = None) -> dict:
     """GLM factorization machine (Eq. 9-10) projected to k columns, F = G P with P [n_r + n_c, k].
     Returns a dict with FC [N, n_c, k] and, if requested, FR [R, n_r, k]."""
-    R, n_r, d = XR.shape
-    N, n_c, _ = XC.shape
     k = P.shape[1]
-    assert R == plan.R and N == plan.N and XR.is_contiguous() and XC.is_contiguous()
-    assert P.shape[0] == n_r + n_c and P.is_contiguous() and P.dtype == XC.dtype
-    dev, dt = XC.device, XC.dtype
-    outs = dict(outs or {})
-    if want_request_side:
-        outs.setdefault("FR", torch.empty((R, n_r, k), dtype=dt, device=dev))
-    outs.setdefault("FC", torch.empty((N, n_c, k), dtype=dt, device=dev))
-    need = glm_fm_projection_workspace(plan, d, k)
-    if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=dev)
-    code = lib().rocs_glm_fm_projection(
-        plan.handle, _dtype_code(XC), n_r, n_c, d, k, _p(XR), _p(XC), _p(P), _p(outs.get("FR")), _p(outs.get("FC")),
-        _p(workspace), workspace.numel(), _stream())
-    _check(code, "rocs_glm_fm_projection")
+    outs = dict(outs) if outs else {}
+    if want_request_side and "FR" not in outs:
+        outs["FR"] = torch.empty((XR.shape[0], XR.shape[1], k), dtype=XC.dtype, device=XC.device)
+    if "FC" not in outs:
+        outs["FC"] = torch.empty((XC.shape[0], XC.shape[1], k), dtype=XC.dtype, device=XC.device)
+    (_ext or _native()).glm_fm_projection(plan.handle, plan.R, plan.N, XR, XC, P, outs.get("FR"), outs.get("FC"), workspace)
     return outs
 
 
 def group_norm(X: torch.Tensor, gamma: Optional[torch.Tensor] = None, beta: Optional[torch.Tensor] = None,
                eps: float = 1e-5, kind: int = NORM_LAYER, out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Group-local LayerNorm / RMSNorm (Eq. 7) of one group's tensor X [M, d], row by row."""
-    assert X.dim() == 2 and X.stride(1) == 1
-    M, d = X.shape
-    if out is None:
-        out = torch.empty((M, d), dtype=X.dtype, device=X.device)
-    code = lib().rocs_group_norm(_dtype_code(X), kind, M, d, _p(X), _rows_2d(X), _p(gamma), _p(beta), eps, _p(out),
-                                 _rows_2d(out), _stream())
-    _check(code, "rocs_group_norm")
-    return out
+    return (_ext or _native()).group_norm(X, gamma, beta, eps, kind, out)
 
 
 def ikbo_linear_static(cand_offsets: torch.Tensor, XR: torch.Tensor, XC: torch.Tensor, W_CR: torch.Tensor,
@@ -365,10 +274,4 @@ def ikbo_linear_static(cand_offsets: torch.Tensor, XR: torch.Tensor, XC: torch.T
     allocates nothing -- for hosts that cannot call cudaMalloc while scoring.  The caller passes the
     output tensor; scratch lives in a fixed array inside the library (limits: R * d_out <= 1 Mi,
     N <= 256 Ki; calls share the array, so do not let two of them overlap on the GPU)."""
-    R, N = cand_offsets.numel() - 1, XC.shape[0]
-    code = lib().rocs_ikbo_linear_static(
-        _dtype_code(XC), R, N, _p(cand_offsets), XR.shape[1], XC.shape[1], W_CC.shape[0], _p(XR), _rows_2d(XR),
-        _p(XC), _rows_2d(XC), _p(W_CR), _rows_2d(W_CR), _p(W_CC), _rows_2d(W_CC), _p(bias),
-        ACT_RELU if relu else ACT_NONE, _p(out), _rows_2d(out), _stream())
-    _check(code, "rocs_ikbo_linear_static")
-    return out
+    return (_ext or _native()).ikbo_linear_static(cand_offsets, XR, XC, W_CR, W_CC, out, bias, relu)

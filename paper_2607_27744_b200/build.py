@@ -1,15 +1,18 @@
-"""Builds ``librocs.so`` in-tree with nvcc for sm_100a (no other architecture)."""
+"""Builds ``librocs.so`` in-tree with nvcc for sm_100a (no other architecture), and the Python extension
+``_native`` (the native half of binding.py) that calls it."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "librocs.so")
+EXT = os.path.join(HERE, "_native.so")
 SOURCES = ["api.cu", "simt_kernels.cu", "linear_simt.cu", "tensor_map.cu", "umma_linear.cu", "umma_linear_ws2.cu", "umma_linear_pair.cu", "umma_dca.cu", "dca_simt.cu", "umma_glm.cu", "fm_projection.cu", "group_norm.cu", "no_alloc.cu", "selftest.cu", "row_stats.cu", "glm_request_mma.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -60,7 +63,24 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
         # through cudaGetDriverEntryPoint, so the library loads on a machine without a GPU.
         run([_nvcc(), "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a",
              "-Xcompiler", "-fPIC", "-cudart", "static"])
+    build_extension(run, force)
     return LIB
+
+
+def build_extension(run, force: bool):
+    """The extension sits beside librocs.so and finds it there; torch's own libraries are loaded by `import torch`."""
+    import torch
+    src = os.path.join(CSRC, "binding.cpp")
+    header = os.path.join(os.path.dirname(HERE), "include", "rocs.h")
+    if not force and os.path.exists(EXT) and os.path.getmtime(EXT) >= max(os.path.getmtime(src), os.path.getmtime(header)):
+        return
+    base = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+         "-I" + os.path.join(base, "include"), "-I" + os.path.join(base, "include", "torch", "csrc", "api", "include"),
+         "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(cuda, "include"), src, "-o", EXT,
+         "-L" + os.path.join(base, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10", "-L" + HERE,
+         "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"])
 
 
 if __name__ == "__main__":

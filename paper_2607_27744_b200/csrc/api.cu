@@ -69,8 +69,14 @@ static cudaError_t pool_alloc(void** ptr, size_t bytes, cudaStream_t stream) {
 }
 
 uint32_t* device_status_word() {
-  uint32_t* p = nullptr;
-  if (cudaGetSymbolAddress((void**)&p, g_device_status) != cudaSuccess) return nullptr;
+  static std::atomic<uint32_t*> found[64];  // the word's address on each device: fixed while the library is loaded
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  uint32_t* p = dev < 64 ? found[dev].load(std::memory_order_acquire) : nullptr;
+  if (p == nullptr) {
+    if (cudaGetSymbolAddress((void**)&p, g_device_status) != cudaSuccess) return nullptr;
+    if (dev < 64) found[dev].store(p, std::memory_order_release);
+  }
   return p;
 }
 

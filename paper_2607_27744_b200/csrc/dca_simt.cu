@@ -201,7 +201,7 @@ rocs_status_t launch(const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh, 
   }
   constexpr int smem = smem_floats<DHP>() * (int)sizeof(float);
   auto kernel = dca_simt_kernel<T, DHP>;
-  ROCS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  ROCS_ALLOW_SMEM(kernel, smem);
   const dim3 grid((unsigned)items.num, (unsigned)std::min<int64_t>(((int64_t)cands * n_q + kRows - 1) / kRows, 65535));
   kernel<<<grid, kThreads, smem, stream>>>(n_q, H, dh, scale, (const T*)Q, (const T*)K, (const T*)V, plan->R, cands,
                                            plan->cand_offsets, items.dev, seq_offsets, (T*)O);

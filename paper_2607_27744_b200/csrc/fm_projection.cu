@@ -489,7 +489,7 @@ rocs_status_t launch_fm_mma_as(const rocs_plan* plan, const int32_t* row2req, in
   p.status = status;
   const int smem = p.stages * stage_bytes + kFixed;
   auto kern = fm_candidate_mma_kernel<D, KT, FULL>;
-  ROCS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  ROCS_ALLOW_SMEM(kern, kMaxDynamicSmem);
   // Launched so that it may overlap the request kernel in front of it on the stream (that kernel
   // releases its dependents at once); nothing else this kernel reads is written by that launch.
   cudaLaunchConfig_t cfg = {};
@@ -531,12 +531,12 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
     if (st != ROCS_OK) return st;
   }
   if (plan->R > 0 && tensor_core_request && sizeof(T) == 2 && d % 16 == 0 && k % 8 == 0 && smem_mma <= kMaxSmem) {
-    ROCS_CUDA_TRY(cudaFuncSetAttribute(fm_request_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_mma));
+    ROCS_ALLOW_SMEM(fm_request_mma_kernel, kMaxSmem);
     fm_request_mma_kernel<<<plan->R, 256, smem_mma, stream>>>(n_r, d, k, (const __nv_bfloat16*)XR,
                                                               (const __nv_bfloat16*)P, TT, (__nv_bfloat16*)FR);
     ROCS_CUDA_TRY(cudaGetLastError());
   } else if (plan->R > 0) {
-    ROCS_CUDA_TRY(cudaFuncSetAttribute(fm_request_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
+    ROCS_ALLOW_SMEM(fm_request_kernel<T>, kMaxSmem);
     fm_request_kernel<T><<<plan->R, 256, smem_r, stream>>>(n_r, d, k, (const T*)XR, (const T*)P, TT, (T*)FR);
     ROCS_CUDA_TRY(cudaGetLastError());
   }
@@ -550,7 +550,7 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
       default: break;
     }
   }
-  ROCS_CUDA_TRY(cudaFuncSetAttribute(fm_candidate_simt_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
+  ROCS_ALLOW_SMEM(fm_candidate_simt_kernel<T>, kMaxSmem);
   fm_candidate_simt_kernel<T><<<(unsigned)plan->N, 128, smem_c, stream>>>(n_r, n_c, d, k, (const T*)XC, (const T*)P,
                                                                          row2req, TT, (T*)FC);
   ROCS_CUDA_TRY(cudaGetLastError());

@@ -145,7 +145,7 @@ rocs_status_t glm_request_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, i
                               cudaStream_t stream) {
   if (plan->R == 0) return ROCS_OK;
   const size_t smem = request_smem(n_r, d, n_ro, n_co);
-  ROCS_CUDA_TRY(cudaFuncSetAttribute(glm_request_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  ROCS_ALLOW_SMEM(glm_request_mma_kernel, kMaxDynamicSmem);
   glm_request_mma_kernel<<<plan->R, kThreads, smem, stream>>>(n_r, n_c, d, (const __nv_bfloat16*)XR,
                                                              (const __nv_bfloat16*)W, n_ro, n_co,
                                                              (__nv_bfloat16*)YR, (__nv_bfloat16*)OR_, zr);

@@ -155,7 +155,7 @@ rocs_status_t launch_linear(int64_t M, int32_t d_in, int32_t d_out, const void* 
   do {                                                                                                               \
     constexpr int smem = smem_bytes<8 * T_, 8 * T_, KS_>();                                                          \
     auto kernel = linear_simt_kernel<TIn, TOut, T_, T_, KS_>;                                                        \
-    ROCS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));                  \
+    ROCS_ALLOW_SMEM(kernel, smem);                                                                                   \
     kernel<<<dim3((unsigned)((M + 8 * T_ - 1) / (8 * T_)), (unsigned)((d_out + 8 * T_ - 1) / (8 * T_))), kGroup * KS_, \
              smem, stream>>>(M, d_in, d_out, (const TIn*)X, ld_x, (const TIn*)W, ld_w, bias, add, ld_add, row2req,   \
                              act, (TOut*)Y, ld_y);                                                                   \

@@ -3,6 +3,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 #include <map>
 #include <mutex>
@@ -69,6 +70,21 @@ namespace rocs {
     cudaError_t _e = (expr);                   \
     if (_e != cudaSuccess) return ROCS_ERR_CUDA; \
   } while (0)
+
+// Raises a kernel's limit of dynamic shared memory to `bytes` (a constant of the kernel), once per device: the
+// attribute stays with the function, and setting it again cost half a microsecond of every launch.
+#define ROCS_ALLOW_SMEM(kernel, bytes)                                                                     \
+  do {                                                                                                     \
+    static std::atomic<uint64_t> _done{0};                                                                 \
+    int _dev = 0;                                                                                          \
+    ROCS_CUDA_TRY(cudaGetDevice(&_dev));                                                                   \
+    const uint64_t _bit = _dev < 64 ? 1ull << _dev : 0;                                                    \
+    if ((_done.load(std::memory_order_acquire) & _bit) == 0) {                                             \
+      ROCS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(bytes))); \
+      _done.fetch_or(_bit, std::memory_order_release);                                                     \
+    }                                                                                                      \
+  } while (0)
+constexpr int kMaxDynamicSmem = 227 * 1024;  // per block on sm_100
 
 inline size_t elem_size(rocs_dtype_t dt) { return dt == ROCS_BF16 ? 2 : 4; }
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

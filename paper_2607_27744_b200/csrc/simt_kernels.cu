@@ -235,15 +235,14 @@ static rocs_status_t launch_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c,
     tiles.num = (int32_t)total;
   }
   if (plan->R > 0) {
-    ROCS_CUDA_TRY(cudaFuncSetAttribute(glm_request_simt_kernel<T>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
+    ROCS_ALLOW_SMEM(glm_request_simt_kernel<T>, kMaxSmem);
     glm_request_simt_kernel<T><<<plan->R, 256, smem_r, stream>>>(
         n_r, n_c, d, (const T*)XR, (const T*)W, n_ro, n_co, (T*)YR, (T*)OR_, zr);
     ROCS_CUDA_TRY(cudaGetLastError());
   }
   if (candidate_side) {
     auto kernel = glm_candidate_simt_kernel<T>;
-    ROCS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemC));
+    ROCS_ALLOW_SMEM(kernel, kMaxSmemC);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)tiles.num);
     cfg.blockDim = dim3(kGlmThreads);

@@ -705,7 +705,7 @@ static rocs_status_t launch_dca(const rocs_plan* plan, int32_t n_q, int32_t H, f
   p.trace = (long long*)rocs_dca_trace_buffer;
 #endif
   auto kernel = dca_umma_kernel<DH, BKV>;
-  ROCS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
+  ROCS_ALLOW_SMEM(kernel, C::kSmemBytes);
   const int grid = std::min((items.num + 1) / 2, sm_count_dca());  // one CTA per SM, two item streams per CTA
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);

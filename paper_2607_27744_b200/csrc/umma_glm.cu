@@ -403,8 +403,7 @@ rocs_status_t umma_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t 
   cfg.numAttrs = p.zr_from_previous_launch ? 1 : 0;
 #define ROCS_GLM_LAUNCH(NC_)                                                                                  \
   do {                                                                                                        \
-    ROCS_CUDA_TRY(cudaFuncSetAttribute(glm_umma_kernel<NC_>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
-                                       L.smem_bytes));                                                        \
+    ROCS_ALLOW_SMEM(glm_umma_kernel<NC_>, kMaxSmem);                                                          \
     ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, glm_umma_kernel<NC_>, map_xr, map_xc, p));                         \
   } while (0)
   if (n_c == 8) ROCS_GLM_LAUNCH(8);

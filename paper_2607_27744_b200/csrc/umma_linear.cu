@@ -295,7 +295,7 @@ rocs_status_t launch(int64_t M, int32_t d_in, int32_t d_out, const void* X, int6
   uint32_t* status = device_status_word();
   if (!status) return ROCS_ERR_CUDA;
   auto kernel = linear_umma_kernel<BN, OutT>;
-  ROCS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
+  ROCS_ALLOW_SMEM(kernel, Cfg::kSmemBytes);
   const int64_t tiles = ((M + BM - 1) / BM) * ((d_out + BN - 1) / BN);
   const int grid = (int)std::min<int64_t>(tiles, sm_count());
   LinearParams p{M, d_in, d_out, bias, add, ld_add, row2req, act, status};

@@ -300,7 +300,7 @@ rocs_status_t umma_linear_pair(int64_t M, int32_t d_in, int32_t d_out, const voi
   }
   const int64_t tiles = ((M + 2 * BM - 1) / (2 * BM)) * ((d_out + BN - 1) / BN);
   const int pairs = (int)std::min<int64_t>(tiles, sm_count_pair() / 2);
-  ROCS_CUDA_TRY(cudaFuncSetAttribute(linear_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+  ROCS_ALLOW_SMEM(linear_pair_kernel, kSmemBytes);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * pairs);
   cfg.blockDim = dim3(kThreads);

@@ -378,7 +378,7 @@ rocs_status_t umma_linear_ws2(int64_t M, int32_t d_in, int32_t d_out, const void
   p.wait_for_previous = (add_from_previous_launch && add != nullptr) ? 1 : 0;
   p.stat_partials = stat_partials;
   const int smem_bytes = fixed + p.a_stages * kAStageBytes;
-  ROCS_CUDA_TRY(cudaFuncSetAttribute(linear_ws2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes));
+  ROCS_ALLOW_SMEM(linear_ws2_kernel, kMaxDynamicSmem);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * p.n_slices * p.groups);
   cfg.blockDim = dim3(kThreads);
