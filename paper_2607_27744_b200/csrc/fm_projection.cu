@@ -309,7 +309,7 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
 
   if (warp == kTileCands) {
     // ------------------------------ TMA producer ------------------------------------------
-    if (lane == 0) {
+    if (elect_one()) {
       prefetch_tensormap(&map_xc);
       int s = 0;
       uint32_t phase = 0, it = 0;

@@ -105,6 +105,17 @@ __device__ __forceinline__ bool mbar_wait_paced(uint64_t* bar, uint32_t parity, 
   }
 }
 
+// True in one lane of a converged warp, the same one every time.  TMA and tcgen05 instructions take their
+// descriptors from uniform registers: under an elect.sync predicate the compiler knows that one thread
+// issues them and emits the instruction alone, under `lane == 0` it wraps each of them in a loop over the
+// active lanes (measured in the ring GEMM: four products and a commit 309 cycles that way, 72 this way; two
+// TMA loads with their expect 333 and 202).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok));
+  return ok != 0;
+}
+
 // ---- programmatic dependent launch ------------------------------------------------------------
 // A kernel launched with the programmatic-stream-serialization attribute may start while its
 // predecessor still runs; it must call griddep_wait() before touching anything the predecessor

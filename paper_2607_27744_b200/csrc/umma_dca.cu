@@ -284,7 +284,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
   if (warp == kControlWarp0 || warp == kControlWarp0 + 3) {
     // ------------------------------ TMA producers: one warp per side --------------------------
     const int side = warp == kControlWarp0 ? 0 : 1;
-    if (lane == 0) {
+    if (elect_one()) {
       prefetch_tensormap(&map_q);
       prefetch_tensormap(&map_k);
       prefetch_tensormap(&map_v);
@@ -393,7 +393,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
       if (!mbar_wait_paced(kv_full + 8 * (kv_it % kKvStages), (kv_it / kKvStages) & 1, abort_flag, p.status, kStatusDca | 4)) { ok = false; break; }
       if (nblk == 1 && tail_valid < BKV) zero_v_tail(kv_it % kKvStages, tail_valid);
       tc_fence_after_sync();
-      if (lane == 0) {
+      if (elect_one()) {
         issue_s(desc_k(kv_it % kKvStages));
         if (nblk == 1) umma_commit(q_empty);
       }
@@ -414,7 +414,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         TRACE_EV(2 + side, 2);
         if (j + 1 < nblk) {
           tc_fence_after_sync();
-          if (lane == 0) {
+          if (elect_one()) {
             issue_s(dk_next);
             if (j + 2 == nblk) umma_commit(q_empty);  // last S of the item: the Q tile is free
           }
@@ -426,7 +426,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         ++cnt_p;
         TRACE_EV(2 + side, 4);
         tc_fence_after_sync();
-        if (lane == 0) {
+        if (elect_one()) {
           issue_pv(dv, j == 0);
           umma_commit(kv_empty + 8 * stage);  // K_j and V_j are no longer needed
         }

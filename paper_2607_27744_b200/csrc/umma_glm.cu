@@ -96,7 +96,7 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------------------
-    if (lane == 0) {
+    if (elect_one()) {
       prefetch_tensormap(&map_xr);
       prefetch_tensormap(&map_xc);
       uint32_t it = 0;
@@ -123,16 +123,16 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ---------------------------------------------
-    const uint32_t idesc = umma_idesc_bf16(128, (uint32_t)(p.n_r_pad + 128), false, false);
-    uint32_t it = 0;
-    bool ok = true;
-    for (int32_t t = t_begin; t < t_end; ++t, ++it) {
-      const uint32_t acc = it & 1;
-      const int s = it % p.stages;
-      if (!mbar_wait(&tmem_empty[acc], ((it >> 1) & 1) ^ 1, abort_flag, p.status, kStatusGlm | 2)) { ok = false; break; }
-      if (!mbar_wait(&full[s], (it / p.stages) & 1, abort_flag, p.status, kStatusGlm | 3)) { ok = false; break; }
-      tc_fence_after_sync();
-      if (lane == 0) {
+    if (elect_one()) {
+      const uint32_t idesc = umma_idesc_bf16(128, (uint32_t)(p.n_r_pad + 128), false, false);
+      uint32_t it = 0;
+      bool ok = true;
+      for (int32_t t = t_begin; t < t_end; ++t, ++it) {
+        const uint32_t acc = it & 1;
+        const int s = it % p.stages;
+        if (!mbar_wait(&tmem_empty[acc], ((it >> 1) & 1) ^ 1, abort_flag, p.status, kStatusGlm | 2)) { ok = false; break; }
+        if (!mbar_wait(&full[s], (it / p.stages) & 1, abort_flag, p.status, kStatusGlm | 3)) { ok = false; break; }
+        tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + acc * kAccStride;
         const uint32_t st = smem_u32(smem + s * p.stage_bytes);
         for (int32_t ks = 0; ks < k_slices; ++ks) {
@@ -144,12 +144,11 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
         umma_commit(&empty[s]);
         umma_commit(&tmem_full[acc]);
       }
-      __syncwarp();
-    }
-    if (!ok && lane == 0) {
-      umma_commit(drain);
-      const uint64_t t0 = globaltimer_ns();
-      while (!mbar_try_wait(drain, 0) && globaltimer_ns() - t0 < kWaitLimitNs) {}
+      if (!ok) {
+        umma_commit(drain);
+        const uint64_t t0 = globaltimer_ns();
+        while (!mbar_try_wait(drain, 0) && globaltimer_ns() - t0 < kWaitLimitNs) {}
+      }
     }
   } else {
     // ------------------------------ epilogue groups ----------------------------------------

@@ -106,7 +106,7 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------------------
-    if (lane == 0) {
+    if (elect_one()) {
       prefetch_tensormap(&map_x);
       prefetch_tensormap(&map_w);
       uint32_t it = 0;
@@ -136,19 +136,19 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ---------------------------------------------
-    constexpr uint32_t idesc = umma_idesc_bf16(BM, BN, false, false);
-    uint32_t it = 0, lt = 0;
-    bool ok = true;
-    for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++lt) {
-      const uint32_t acc = lt & 1;
-      if (!mbar_wait(&tmem_empty[acc], ((lt >> 1) & 1) ^ 1, abort_flag, p.status, kStatusLinear | 2)) { ok = false; break; }
-      tc_fence_after_sync();
-      const uint32_t d_tmem = tmem_base + acc * BN;
-      for (int32_t kb = 0; kb < k_blocks; ++kb, ++it) {
-        const int s = it % kStages;
-        if (!mbar_wait(&full[s], (it / kStages) & 1, abort_flag, p.status, kStatusLinear | 3)) { ok = false; break; }
+    if (elect_one()) {
+      constexpr uint32_t idesc = umma_idesc_bf16(BM, BN, false, false);
+      uint32_t it = 0, lt = 0;
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++lt) {
+        const uint32_t acc = lt & 1;
+        if (!mbar_wait(&tmem_empty[acc], ((lt >> 1) & 1) ^ 1, abort_flag, p.status, kStatusLinear | 2)) { ok = false; break; }
         tc_fence_after_sync();
-        if (lane == 0) {
+        const uint32_t d_tmem = tmem_base + acc * BN;
+        for (int32_t kb = 0; kb < k_blocks; ++kb, ++it) {
+          const int s = it % kStages;
+          if (!mbar_wait(&full[s], (it / kStages) & 1, abort_flag, p.status, kStatusLinear | 3)) { ok = false; break; }
+          tc_fence_after_sync();
           const uint32_t a_addr = smem_u32(smem + s * Cfg::kStageBytes);
           const uint64_t a_desc = smem_desc_sw128(a_addr, 1024, 16);
           const uint64_t b_desc = smem_desc_sw128(a_addr + Cfg::kABytes, 1024, 16);
@@ -157,15 +157,13 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             umma_ss(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
           umma_commit(&empty[s]);  // frees the stage once these MMAs have read it
         }
-        __syncwarp();
+        if (ok) umma_commit(&tmem_full[acc]);
       }
-      if (ok && lane == 0) umma_commit(&tmem_full[acc]);
-      __syncwarp();
-    }
-    if (!ok && lane == 0) {
-      umma_commit(drain);
-      const uint64_t t0 = globaltimer_ns();
-      while (!mbar_try_wait(drain, 0) && globaltimer_ns() - t0 < kWaitLimitNs) {}
+      if (!ok) {
+        umma_commit(drain);
+        const uint64_t t0 = globaltimer_ns();
+        while (!mbar_try_wait(drain, 0) && globaltimer_ns() - t0 < kWaitLimitNs) {}
+      }
     }
   } else {
     // ------------------------------ epilogue -----------------------------------------------
@@ -225,7 +223,7 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         }
         // staging buffer (two per warp): make sure the TMA store that last read it has finished
         uint8_t* buf = my_stage + (stores & 1) * 4096;
-        if (lane == 0) tma_store_wait_read<1>();
+        if (elect_one()) tma_store_wait_read<1>();
         __syncwarp();
         uint8_t* row_ptr = buf + lane * 128;
 #pragma unroll
@@ -250,14 +248,14 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         }
         fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0) {
+        if (elect_one()) {
           tma_store_2d(&map_y, buf, col0, m0 + q * 32);
           tma_store_commit();
         }
         ++stores;
       }
     }
-    if (lane == 0) tma_store_wait_all<0>();
+    if (elect_one()) tma_store_wait_all<0>();
   }
 
   tc_fence_before_sync();

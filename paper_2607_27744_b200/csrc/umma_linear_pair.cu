@@ -97,7 +97,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 
   if (warp == 0) {
     // ------------------------------ TMA producer (both CTAs) -------------------------------
-    if (lane == 0) {
+    if (elect_one()) {
       prefetch_tensormap(&map_x);
       prefetch_tensormap(&map_w);
       uint32_t it = 0;
@@ -122,7 +122,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer (leader CTA only) ---------------------------
-    if (rank == 0 && lane == 0) {
+    if (rank == 0 && elect_one()) {
       constexpr uint32_t idesc = umma_idesc_bf16(2 * BM, BN, false, false);
       uint32_t it = 0, lt = 0;
       bool ok = true;
@@ -165,7 +165,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       const int32_t n0 = (int32_t)(t % n_tiles) * BN;
       if (!mbar_wait(&tmem_full[acc], (lt >> 1) & 1, abort_flag, p.status, kStatusPair | 4)) break;
       tc_fence_after_sync();
-      if (lane == 0) tma_store_wait_read<0>();  // the previous tile's stores have read this warp's boxes
+      if (elect_one()) tma_store_wait_read<0>();  // the previous tile's stores have read this warp's boxes
       __syncwarp();
       const uint32_t t_row = tmem_base + acc * BN + half * 128 + ((uint32_t)(q * 32) << 16);
       float sc = 1.f, sh = 0.f;
@@ -223,7 +223,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           for (int i = 0; i < 64; ++i) f[i] = fmaxf(f[i], 0.f);
         }
         if (c == 1) {  // the store of the first chunk has finished reading the box
-          if (lane == 0) tma_store_wait_read<0>();
+          if (elect_one()) tma_store_wait_read<0>();
           __syncwarp();
         }
         uint8_t* row_ptr = my_stage + lane * 128;
@@ -242,13 +242,13 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         }
         fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0) {
+        if (elect_one()) {
           if (col0 < p.d_out && (int64_t)m0 + q * 32 < p.M) tma_store_2d(&map_y, my_stage, col0, m0 + q * 32);
           tma_store_commit();
         }
       }
     }
-    if (lane == 0) tma_store_wait_all<0>();
+    if (elect_one()) tma_store_wait_all<0>();
   }
 
   tc_fence_before_sync();

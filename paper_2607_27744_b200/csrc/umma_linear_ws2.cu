@@ -123,7 +123,7 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
 
   if (warp == 0) {
     // ------------------------------ TMA producer (both CTAs) -------------------------------
-    if (lane == 0) {
+    if (elect_one()) {
       prefetch_tensormap(&map_x);
       prefetch_tensormap(&map_w);
       const uint32_t w_full_leader = map_to_cta(smem_u32(w_full), 0);
@@ -174,7 +174,7 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer (leader CTA only): a single thread -----------
-    if (rank == 0 && lane == 0) {
+    if (rank == 0 && elect_one()) {
       constexpr uint32_t idesc = umma_idesc_bf16(2 * BM, BN, false, false);
       uint32_t it = 0, lt = 0;
       bool ok = mbar_wait(w_full, 0, abort_flag, p.status, kStatusWs2 | 6);
@@ -229,7 +229,7 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       if (!mbar_wait(&tmem_full[acc], (lt >> 1) & 1, abort_flag, p.status, kStatusWs2 | 4)) break;
       tc_fence_after_sync();
       // the TMA stores of the previous tile have finished reading this warp's staging boxes
-      if (lane == 0) tma_store_wait_read<0>();
+      if (elect_one()) tma_store_wait_read<0>();
       __syncwarp();
       const uint32_t t_row = tmem_base + acc * BN + half * 128 + ((uint32_t)(q * 32) << 16);
       float st_sum = 0.f, st_sq = 0.f;  // this row's 128 output columns, for a normalisation that follows (Eq. 7)
@@ -286,7 +286,7 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
           }
         }
         if (c == 1) {  // the store of the first chunk has finished reading the box
-          if (lane == 0) tma_store_wait_read<0>();
+          if (elect_one()) tma_store_wait_read<0>();
           __syncwarp();
         }
         uint8_t* row_ptr = my_stage + lane * 128;
@@ -305,7 +305,7 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         }
         fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0) {
+        if (elect_one()) {
           if (n0 + half * 128 + c * 64 < p.d_out && (int64_t)m0 + q * 32 < p.M)
             tma_store_2d(&map_y, my_stage, n0 + half * 128 + c * 64, m0 + q * 32);
           tma_store_commit();
@@ -315,7 +315,7 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         p.stat_partials[row * (2 * p.n_slices) + slice * 2 + half] = make_float2(st_sum, st_sq);
       if (lane == 0 && has_add) mbar_arrive(&z_empty[lt % kZBufs]);
     }
-    if (lane == 0) tma_store_wait_all<0>();
+    if (elect_one()) tma_store_wait_all<0>();
   }
 
   tc_fence_before_sync();
