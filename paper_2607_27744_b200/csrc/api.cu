@@ -37,7 +37,7 @@ __device__ uint32_t g_device_status;
 }  // namespace
 
 // Stream-ordered allocations of the plan's lists (request ids, tiles, items) come from a pool of the library's
-// own that keeps freed memory instead of returning it to the driver at the next synchronisation: a
+// own that keeps up to 1 GiB of freed memory instead of returning it to the driver at the next synchronisation: a
 // serving loop builds and drops one plan per batch, and with the default pool's zero release
 // threshold every batch would pay the driver's allocation path again.
 static cudaError_t pool_alloc(void** ptr, size_t bytes, cudaStream_t stream) {
@@ -58,7 +58,7 @@ static cudaError_t pool_alloc(void** ptr, size_t bytes, cudaStream_t stream) {
       props.location.id = dev;
       e = cudaMemPoolCreate(&pool, &props);
       if (e != cudaSuccess) return e;
-      uint64_t keep = UINT64_MAX;
+      uint64_t keep = 1ull << 30;
       cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
       pools[dev] = pool;
     } else {
@@ -163,22 +163,15 @@ int64_t plan_entries(const rocs_plan* plan, int32_t cands_per_tile) {
   return entries;
 }
 
-static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, cudaStream_t stream,
-                               DeviceList* out) {
+// Allocates and fills one list of the plan (key as in rocs_plan::lists) in the order of `stream`, from the
+// offsets at `off`.
+static rocs_status_t make_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, const int32_t* off,
+                               cudaStream_t stream, DeviceList* out) {
   static_assert(sizeof(Tile) == 16 && sizeof(DcaItem) == 16, "list entries");
-  unsigned long long id = 0;
-  ROCS_CUDA_TRY(cudaStreamGetId(stream, &id));
-  std::lock_guard<std::mutex> lock(plan->mu);
-  const auto key = std::make_tuple(id, cands_per_tile, heads);
-  auto it = plan->lists.find(key);
-  if (it != plan->lists.end()) {
-    *out = it->second;
-    return ROCS_OK;
-  }
   DeviceList list;
   if (plan->N > 0 && cands_per_tile == 0) {
     ROCS_CUDA_TRY(pool_alloc(&list.dev, sizeof(int32_t) * (size_t)plan->N, stream));
-    fill_row2req_kernel<<<(unsigned)((plan->N + 255) / 256), 256, 0, stream>>>(plan->R, plan->N, plan->cand_offsets,
+    fill_row2req_kernel<<<(unsigned)((plan->N + 255) / 256), 256, 0, stream>>>(plan->R, plan->N, off,
                                                                               static_cast<int32_t*>(list.dev));
   } else if (plan->N > 0) {
     const int32_t R = plan->R;
@@ -201,7 +194,7 @@ static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, in
     if (e == cudaSuccess)
       expand_list_kernel<<<(unsigned)((total + kListThreads - 1) / kListThreads), kListThreads,
                            base_dev ? 0 : sizeof(int32_t) * ((size_t)R + 1), stream>>>(
-          R, list.num, cands_per_tile, heads, plan->cand_offsets, base_dev, list.dev);
+          R, list.num, cands_per_tile, heads, off, base_dev, list.dev);
     if (base_dev) cudaFreeAsync(base_dev, stream);
     if (e != cudaSuccess) {
       cudaFreeAsync(list.dev, stream);
@@ -212,9 +205,69 @@ static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, in
     if (list.dev) cudaFreeAsync(list.dev, stream);
     return ROCS_ERR_CUDA;
   }
-  plan->lists[key] = list;
   *out = list;
   return ROCS_OK;
+}
+
+// The same list outside any stream capture, complete on return: on a stream of its own, from the plan's host
+// copy of the offsets (work in front of the plan's stream may itself be captured and never run).
+static rocs_status_t make_list_now(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, DeviceList* out) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  ROCS_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
+  rocs_status_t st = ROCS_ERR_CUDA;
+  cudaStream_t own = nullptr;
+  int32_t* off = nullptr;
+  const size_t bytes = sizeof(int32_t) * plan->offsets_host.size();
+  if (cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking) == cudaSuccess) {
+    if (pool_alloc((void**)&off, bytes, own) == cudaSuccess) {
+      if (cudaMemcpyAsync(off, plan->offsets_host.data(), bytes, cudaMemcpyHostToDevice, own) == cudaSuccess)
+        st = make_list(plan, cands_per_tile, heads, off, own, out);
+      cudaFreeAsync(off, own);
+    }
+    if (cudaStreamSynchronize(own) != cudaSuccess) st = ROCS_ERR_CUDA;
+    cudaStreamDestroy(own);
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return st;
+}
+
+static unsigned long long capture_of(cudaStream_t stream) {  // 0: the stream is not being captured
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(stream, &status, &id) != cudaSuccess || status != cudaStreamCaptureStatusActive) {
+    cudaGetLastError();
+    return 0;
+  }
+  return id;
+}
+
+static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, cudaStream_t stream,
+                               DeviceList* out) {
+  const unsigned long long capture = capture_of(stream);
+  std::lock_guard<std::mutex> lock(plan->mu);
+  if (capture != 0 && capture != plan->capture) {
+    // A graph that outlives this call: it must hold a list that exists now, not one that its own replays would
+    // allocate.  Any list made outside a capture will do, since the graph is launched behind the plan.
+    for (const auto& kv : plan->lists)
+      if (std::get<1>(kv.first) == cands_per_tile && std::get<2>(kv.first) == heads) {
+        *out = kv.second;
+        return ROCS_OK;
+      }
+    const rocs_status_t st = make_list_now(plan, cands_per_tile, heads, out);
+    if (st == ROCS_OK) plan->lists[std::make_tuple(0ull, cands_per_tile, heads)] = *out;
+    return st;
+  }
+  unsigned long long id = 0;
+  if (plan->capture == 0) ROCS_CUDA_TRY(cudaStreamGetId(stream, &id));
+  const auto key = std::make_tuple(id, cands_per_tile, heads);
+  auto it = plan->lists.find(key);
+  if (it != plan->lists.end()) {
+    *out = it->second;
+    return ROCS_OK;
+  }
+  const rocs_status_t st = make_list(plan, cands_per_tile, heads, plan->cand_offsets, stream, out);
+  if (st == ROCS_OK) plan->lists[key] = *out;
+  return st;
 }
 
 rocs_status_t plan_row2req(const rocs_plan* plan, cudaStream_t stream, const int32_t** out) {
@@ -321,6 +374,7 @@ rocs_status_t rocs_plan_create(rocs_plan_t** out, int32_t R, int64_t N, const in
       });
   }
   p->stream = stream;
+  p->capture = capture_of(stream);
   *out = p;
   return ROCS_OK;
 }

@@ -56,11 +56,12 @@ struct rocs_plan {
   std::vector<int32_t> offsets_host;      // [R+1]
   mutable std::mutex mu;
   // Device lists, made on first use and kept per stream (its id, which is never reused): a list is only
-  // ever read on the stream whose order puts its making in front of the reader.
+  // ever read on the stream whose order puts its making in front of the reader, or by a graph captured later.
   // Key: stream id, candidates per tile (0: the candidate -> request map), heads (0: no head dimension).
   mutable std::map<std::tuple<unsigned long long, int32_t, int32_t>, rocs::DeviceList> lists;
   int device = 0;
   cudaStream_t stream = nullptr;  // stream the plan was created on; its memory is freed there
+  unsigned long long capture = 0; // the capture the plan was created in, and lives in; 0: none
 };
 
 namespace rocs {

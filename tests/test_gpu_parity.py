@@ -534,6 +534,43 @@ def test_candidate_isolation_is_bit_exact(path):
         assert np.all(np.any(a[seg] != b[seg], axis=1))
 
 
+# ------------------------------------------------------------------ streams and graphs -------
+@pytest.mark.parametrize("warm", [False, True])
+def test_calls_captured_in_a_graph_replay(warm):
+    # a plan made outside the capture, its lists made or not yet made when the capture begins; and a plan that
+    # lives inside the capture
+    cfg = wl.CONFIGS[5].with_(R=5, d_req=64, d_cand=64, d_out=128, n_ro=4, n_co=4)
+    co, so = wl.offsets_from_counts([30, 0, 700, 1, 9]), wl.offsets_from_counts([40, 10, 200, 5, 64])
+    lin, att, g = wl.linear_inputs(cfg, co), wl.dca_inputs(cfg, co, so), wl.glm_inputs(cfg, co)
+    W, XR, XC = to_dev(lin["W"]), to_dev(lin["XR"]), to_dev(lin["XC"])
+    Q, K, V, sod = to_dev(att["Q"]), to_dev(att["K"]), to_dev(att["V"]), to_dev(so)
+    GR, GC, GW = to_dev(g["XR"]), to_dev(g["XC"]), to_dev(g["W"])
+    cod, host = to_dev(co), torch.from_numpy(co)
+
+    def layers(plan):
+        y = rocs.ikbo_linear(plan, XR, XC, W[:, :cfg.d_req], W[:, cfg.d_req:], relu=True)
+        o = rocs.dca_attention(plan, Q, K, V, sod)
+        return [y, o, rocs.glm_interaction(plan, GR, GC, GW, cfg.n_ro, cfg.n_co)["OC"]]
+
+    other = rocs.plan_create(cod, host)
+    want = [_bits(t) for t in layers(other)]
+    plan = other if warm else rocs.plan_create(cod, host)
+    for inside in (False, True):
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            p = rocs.plan_create(cod, host) if inside else plan
+            outs = layers(p)
+            if inside:
+                p.close()
+        for _ in range(3):
+            for t in outs:
+                t.zero_()
+            graph.replay()
+            assert all(np.array_equal(_bits(t), w) for t, w in zip(outs, want))
+    again = layers(plan)   # and the plan still serves calls outside the graph
+    assert all(np.array_equal(_bits(t), w) for t, w in zip(again, want))
+
+
 # ------------------------------------------------------------------ ABI errors --------------
 def test_error_codes_on_bad_arguments():
     co = wl.offsets_from_counts([4, 4])
