@@ -11,9 +11,14 @@
 // swizzle); the description below gives the figures of the first.
 //
 // One persistent CTA per SM runs TWO independent item streams (sides A and B), 20 warps:
-//   warps 16,19 TMA producers of sides A, B: the Q tile of the item, then (K_j, V_j) blocks through a ring
+//   warps 16,19 TMA producers of sides A, B: the Q tile of the item, then its K and V blocks through a ring of
+//               slots that hold one block each, in the order of their use (K_0, K_1, V_0, K_2, V_1, ...): a K
+//               block gives its slot back when its S is done, half a block before its V does.  With a stage
+//               per (K_j, V_j) pair two stages were all that fits at dh = 128 and the issuer waited for them
+//               (821 candidates x 32 query tokens, 4 heads of 128, 500..1500 keys: 113 us, 90 us with slots)
 //   warps 17,18 tcgen05.mma issuers of sides A, B:  S = Q K_j^T (128x128x64, operands in shared memory)
-//               and O += P V_j (128x64x128, P read from tensor memory, V from shared memory)
+//               and O += P V_j (128x64x128, P read from tensor memory, V from shared memory); the last block's
+//               products end at the next multiple of 16 keys
 //   warps 0-15  softmax: 8 warps per side, TWO threads per query row, each owning 64 of the 128 key
 //               columns of a block: S from TMEM into registers (one read), exp2 on scaled scores,
 //               fp32 partial sums, P rounded to bf16 and stored to tensor memory.
@@ -21,11 +26,11 @@
 // P has its own columns, so S_{j+1} is issued as soon as S_j sits in registers, and the wait on
 // P V_{j-1} comes in the middle of block j, just before P_j starts to overwrite P_{j-1}.
 //
-// Reference of the softmax: the maximum of the row's FIRST block, rounded up to an integer, found
-// by both threads of the row (each scans all 128 columns, so they agree bit for bit without
+// Reference of the softmax: the maximum over the row's FIRST 32 keys, rounded up to an integer, found
+// by both threads of the row (each scans those columns, so they agree bit for bit without
 // talking) and never moved: later blocks need no maximum, no rescaling of O and no exchange.
-// fp32 holds 2^x up to x = 128, so a row overflows only if a later score exceeds its first block's
-// maximum by about 88 nats; such a row shows Inf/NaN in its sums at the end of the item and is then
+// fp32 holds 2^x up to x = 128, so a row overflows only if a later score exceeds that maximum by about
+// 88 nats; such a row shows Inf/NaN in its sums at the end of the item and is then
 // computed again by its two threads alone in plain fp32 loops (slow, correct, reached only by inputs
 // whose scores span more than fp32's exponent range).  Every decision is taken per row from that
 // row's own values, so a row's bits never depend on its neighbours.
@@ -34,9 +39,6 @@
 #include "rocs_internal.h"
 #include "sm100_ptx.cuh"
 
-#ifdef ROCS_DCA_TRACE
-extern "C" void* rocs_dca_trace_buffer = nullptr;
-#endif
 
 namespace rocs {
 namespace {
@@ -63,52 +65,47 @@ struct DcaCfg {
   static_assert(kRowBytes == 128 || kRowBytes == 64, "operand rows");
   static constexpr int kCols = BKV / 2;                      // score columns per softmax thread
   static constexpr int kOutCols = DH / 2;                    // output columns per softmax thread
-  static constexpr int kKvStages = DH == 128 ? 2 : DH == 64 ? 3 : 4;  // per side
+  static constexpr int kKvSlots = DH == 128 ? 5 : DH == 64 ? 6 : 8;  // per side, one K or V block each
   static constexpr int kQBoxBytes = BQ * kRowBytes, kQBytes = kBoxes * kQBoxBytes;
   static constexpr int kKvBoxBytes = BKV * kRowBytes, kKBytes = kBoxes * kKvBoxBytes;
   // operand descriptor of a tile of 8-row groups, rows of kRowBytes
   __device__ static uint64_t desc(uint32_t addr) {
     return kRowBytes == 128 ? smem_desc_sw128(addr, 1024, 16) : smem_desc_sw64(addr, 512, 16);
   }
-  static constexpr int kKvStageBytes = 2 * kKBytes;          // K block + V block
+  // V block as the N x K operand of P V: rows are keys, boxes of output columns kKvBoxBytes apart
+  __device__ static uint64_t desc_v(uint32_t addr) {
+    return kRowBytes == 128 ? smem_desc_sw128(addr, 1024, kBoxes > 1 ? kKvBoxBytes : 16) : smem_desc_sw64(addr, 512, 16);
+  }
   // tensor memory per side: S [0, BKV) fp32, P [BKV, BKV + BKV/2) bf16 pairs, O [.., + DH) fp32
   static constexpr int kPColOffset = BKV, kOColOffset = BKV + BKV / 2;
   static_assert(kOColOffset + DH <= kSideTmemStride, "tensor memory columns of a side");
   static_assert(kCols == 32 || kCols == 64, "score columns per thread");
   // Shared-memory map (byte offsets from the 1024-byte aligned base); per side: one Q tile (freed when
-  // the item's last S is issued, a block before its end) and a ring of K/V stages.
+  // the item's last S is issued, a block before its end) and a ring of K / V slots.
   static constexpr uint32_t kOffQ = 0;                                          // [2 sides][boxes][128][64] bf16
-  static constexpr uint32_t kOffKv = kOffQ + 2 * kQBytes;                       // [2 sides][stages][K | V]
-  static constexpr uint32_t kOffL = kOffKv + 2 * kKvStages * kKvStageBytes;     // partial sums [2 sides][2 halves][128] fp32
+  static constexpr uint32_t kOffKv = kOffQ + 2 * kQBytes;                       // [2 sides][slots]
+  static constexpr uint32_t kOffL = kOffKv + 2 * kKvSlots * kKBytes;     // partial sums [2 sides][2 halves][128] fp32
   static constexpr uint32_t kOffBar = kOffL + 2 * 2 * BQ * 4;
   // barriers, 8 bytes each, [side] innermost where there are two
   static constexpr uint32_t kBarQFull = kOffBar;                    // [2]
   static constexpr uint32_t kBarQEmpty = kBarQFull + 16;            // [2]
-  static constexpr uint32_t kBarKvFull = kBarQEmpty + 16;           // [2][stages]
-  static constexpr uint32_t kBarKvEmpty = kBarKvFull + 16 * kKvStages;
-  static constexpr uint32_t kBarSFull = kBarKvEmpty + 16 * kKvStages;  // [2]
+  static constexpr uint32_t kBarKvFull = kBarQEmpty + 16;           // [2][slots]
+  static constexpr uint32_t kBarKvEmpty = kBarKvFull + 16 * kKvSlots;
+  static constexpr uint32_t kBarSFull = kBarKvEmpty + 16 * kKvSlots;  // [2]
   static constexpr uint32_t kBarSEmpty = kBarSFull + 16;
   static constexpr uint32_t kBarPFull = kBarSEmpty + 16;
   static constexpr uint32_t kBarOFull = kBarPFull + 16;
   static constexpr uint32_t kBarPair = kBarOFull + 16;              // [8]: the two warps that share 32 query rows
   static constexpr uint32_t kBarDrain = kBarPair + 64;              // [2]
-  static constexpr uint32_t kOffTmemPtr = kBarDrain + 16;
+  static constexpr uint32_t kBarInfoFull = kBarDrain + 16;          // [2][2 slots]
+  static constexpr uint32_t kBarInfoEmpty = kBarInfoFull + 32;      // [2][2 slots]
+  static constexpr uint32_t kBarTail = kBarInfoEmpty + 32;          // [2]
+  static constexpr uint32_t kOffInfo = (kBarTail + 16 + 15) / 16 * 16;  // [2][2 slots][2] int4
+  static constexpr uint32_t kOffTmemPtr = kOffInfo + 128;
   static constexpr uint32_t kOffAbort = kOffTmemPtr + 4;
   static constexpr int kSmemBytes = kOffAbort + 12;
   static_assert(kSmemBytes <= 232448, "shared memory of one SM");
 };
-
-#ifndef ROCS_DCA_EMU
-#define ROCS_DCA_EMU 0
-#endif
-// Of every 8 column pairs of a row, this many take 2^x from a cubic on the FMA pipe instead of the
-// exponential unit (which pairs is fixed by the column index, so a row's bits do not depend on its
-// neighbours): 2^x = 2^n 2^r, n = round(x), |r| <= 1/2, 2^r by a polynomial with relative error
-// 7.5e-5, far below the rounding of P to bf16.  Off by default: with the rest of the loop as it is
-// the exponential unit is not what limits the kernel (measured).
-constexpr int kEmuPairs = ROCS_DCA_EMU;
-constexpr float kMagic = 12582912.f;  // 1.5 * 2^23: adding it rounds to an integer kept in the low mantissa bits
-constexpr float kPoly0 = 0.9999280572f, kPoly1 = 0.6932609677f, kPoly2 = 0.2426111251f, kPoly3 = 0.0551716685f;
 
 struct DcaParams {
   const DcaItem* items;
@@ -119,10 +116,9 @@ struct DcaParams {
   const __nv_bfloat16 *Q, *K, *V;  // plain pointers for rows that are computed by hand
   __nv_bfloat16* O;
   uint32_t* status;
-#ifdef ROCS_DCA_TRACE
-  long long* trace;
-#endif
 };
+
+__host__ __device__ constexpr int32_t round16(int32_t x) { return (x + 15) / 16 * 16; }
 
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -152,11 +148,6 @@ __device__ __forceinline__ uint64_t fadd2(uint64_t a, uint64_t b) {
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-__device__ __forceinline__ float fmax_nan(float a, float b) {  // NaN if either input is NaN
-  float d;
-  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
   return d;
 }
 __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
@@ -215,28 +206,20 @@ __device__ __forceinline__ bool mbar_wait_spin(uint32_t bar, uint32_t parity, Ab
   return mbar_wait_paced(bar, parity, abort_flag, status, code);
 }
 
-#ifdef ROCS_DCA_TRACE
-// event stamps of CTA 0: [role 0..3][block 0..kTraceBlocks)[event 0..8)
-constexpr int kTraceBlocks = 96;
-#define TRACE_EV(role, ev) do { if (p.trace && blockIdx.x == 0 && lane == 0 && tr_blk < kTraceBlocks) p.trace[((role) * kTraceBlocks + tr_blk) * 8 + (ev)] = clock64(); } while (0)
-#define TRACE_NEXT() ++tr_blk
-#else
-#define TRACE_EV(role, ev)
-#define TRACE_NEXT()
-#endif
 
 template <int DH, int BKV>
 __global__ void __launch_bounds__(kThreads, 1)
 dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, const DcaParams p) {
   using C = DcaCfg<DH, BKV>;
-  constexpr int kKvStages = C::kKvStages, kBoxes = C::kBoxes, kCols = C::kCols, kOutCols = C::kOutCols;
-  constexpr int kQBytes = C::kQBytes, kKBytes = C::kKBytes, kKvStageBytes = C::kKvStageBytes;
+  constexpr int kKvSlots = C::kKvSlots, kBoxes = C::kBoxes, kCols = C::kCols, kOutCols = C::kOutCols;
+  constexpr int kQBytes = C::kQBytes, kKBytes = C::kKBytes;
   constexpr int kPColOffset = C::kPColOffset, kOColOffset = C::kOColOffset;
   constexpr uint32_t kOffQ = C::kOffQ, kOffKv = C::kOffKv, kOffL = C::kOffL, kBarQFull = C::kBarQFull,
                      kBarQEmpty = C::kBarQEmpty, kBarKvFull = C::kBarKvFull, kBarKvEmpty = C::kBarKvEmpty,
                      kBarSFull = C::kBarSFull, kBarSEmpty = C::kBarSEmpty, kBarPFull = C::kBarPFull,
-                     kBarOFull = C::kBarOFull, kBarPair = C::kBarPair, kBarDrain = C::kBarDrain,
+                     kBarOFull = C::kBarOFull, kBarPair = C::kBarPair, kBarDrain = C::kBarDrain, kBarInfoFull = C::kBarInfoFull,
+                     kBarInfoEmpty = C::kBarInfoEmpty, kBarTail = C::kBarTail, kOffInfo = C::kOffInfo,
                      kOffTmemPtr = C::kOffTmemPtr, kOffAbort = C::kOffAbort;
   extern __shared__ __align__(1024) uint8_t smem[];     // swizzled operand tiles need 1024-byte alignment
   const uint32_t sb = smem_u32(smem);                   // every shared-memory address below is sb + constant
@@ -254,14 +237,17 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     };
     init(kBarQFull, 2, 1);
     init(kBarQEmpty, 2, 1);
-    init(kBarKvFull, 2 * kKvStages, 1);
-    init(kBarKvEmpty, 2 * kKvStages, 1);
+    init(kBarKvFull, 2 * kKvSlots, 1);
+    init(kBarKvEmpty, 2 * kKvSlots, 1);
     init(kBarSFull, 2, 1);
     init(kBarSEmpty, 2, kSoftmaxWarps / 2);
     init(kBarPFull, 2, kSoftmaxWarps / 2);
     init(kBarOFull, 2, 1);
     init(kBarPair, 8, 2);
     init(kBarDrain, 2, 1);
+    init(kBarInfoFull, 4, 1);
+    init(kBarInfoEmpty, 4, kSoftmaxWarps / 2 + 1);
+    init(kBarTail, 2, 1);
     abort_flag->v = 0;
     fence_mbar_init();
   }
@@ -278,167 +264,222 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
   griddep_wait();
   griddep_launch_dependents();
   const int32_t row_width = p.H * DH;  // elements per query / key row over all heads
-  // Each side is a stream of its own: items 2 b + side, 2 b + side + 2 grid, ... of CTA b.
-  const int32_t item0 = 2 * (int32_t)blockIdx.x, item_step = 2 * (int32_t)gridDim.x;
 
   if (warp == kControlWarp0 || warp == kControlWarp0 + 3) {
     // ------------------------------ TMA producers: one warp per side --------------------------
+    // Also the side's item reader: it looks items 2 b + side, 2 b + side + 2 grid, ... of CTA b up in global
+    // memory, one ahead, and hands them to the other warps through two slots in shared memory, so that
+    // nobody else waits for global memory between two items.
     const int side = warp == kControlWarp0 ? 0 : 1;
-    if (elect_one()) {
+    const uint32_t q_full = sb + kBarQFull + 8 * side, q_empty = sb + kBarQEmpty + 8 * side;
+    const uint32_t kv_full = sb + kBarKvFull + 8 * kKvSlots * side, kv_empty = sb + kBarKvEmpty + 8 * kKvSlots * side;
+    const uint32_t info_full = sb + kBarInfoFull + 16 * side, info_empty = sb + kBarInfoEmpty + 16 * side;
+    const uint32_t q_dst = sb + kOffQ + side * kQBytes, kv_dst = sb + kOffKv + side * kKvSlots * kKBytes;
+    int4* info = reinterpret_cast<int4*>(smem + kOffInfo) + side * 4;
+    uint32_t kv_it = 0, n_work = 0, n_item = 0;
+    bool ok = true;
+    auto wait = [&](uint32_t bar, uint32_t parity, uint32_t code) {  // the same answer for the whole warp
+      return __all_sync(0xffffffffu, mbar_wait_paced(bar, parity, abort_flag, p.status, kStatusDca | code)) != 0;
+    };
+    if (lane == 0) {
       prefetch_tensormap(&map_q);
       prefetch_tensormap(&map_k);
       prefetch_tensormap(&map_v);
-      const uint32_t q_full = sb + kBarQFull + 8 * side, q_empty = sb + kBarQEmpty + 8 * side;
-      const uint32_t kv_full = sb + kBarKvFull + 8 * kKvStages * side, kv_empty = sb + kBarKvEmpty + 8 * kKvStages * side;
-      const uint32_t q_dst = sb + kOffQ + side * kQBytes, kv_dst = sb + kOffKv + side * kKvStages * kKvStageBytes;
-      uint32_t kv_it = 0, n_work = 0;
-      bool ok = true;
-      for (int32_t i = item0 + side; i < p.num_items && ok; i += item_step) {
-        const DcaItem item = p.items[i];
-        const int32_t s0 = p.seq_offsets[item.req];
-        const int32_t L = p.seq_offsets[item.req + 1] - s0;
-        if (L == 0) continue;  // nobody touches a barrier for an item without keys
-        if (!mbar_wait_paced(q_empty, (n_work & 1) ^ 1, abort_flag, p.status, kStatusDca | 1)) { ok = false; break; }
-        ++n_work;
+    }
+    // The last block of a sequence may reach past it into the next request's rows (or past the
+    // tensor, where TMA fills zeros).  Scores of such keys are masked to -inf by the softmax warps,
+    // so P is exactly 0 there; the V rows are zeroed here so that 0 x (Inf or NaN of a foreign
+    // request) cannot reach this request's output.  (The products go no further than the next multiple of 16
+    // keys, so at most 15 rows.)  Done once the next item's Q load is out, i.e. after the last S of this item
+    // was issued and while its softmax runs; P V waits for it.
+    int32_t tail_valid = 0;  // valid keys of a block that waits to be zeroed; 0: none
+    uint32_t tail_slot = 0, tail_phase = 0;
+    auto zero_tail = [&]() {
+      if (tail_valid == 0) return true;
+      if (!wait(kv_full + 8 * tail_slot, tail_phase, 4)) return false;
+      uint8_t* v = smem + kOffKv + (side * kKvSlots + tail_slot) * kKBytes;
+      for (int bx = 0; bx < kBoxes; ++bx)
+        for (int idx = tail_valid * (C::kRowBytes / 16) + lane; idx < round16(tail_valid) * (C::kRowBytes / 16); idx += 32)
+          *reinterpret_cast<uint4*>(v + bx * C::kKvBoxBytes + idx * 16) = make_uint4(0u, 0u, 0u, 0u);
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(sb + kBarTail + 8 * side);
+      tail_valid = 0;
+      return true;
+    };
+    const int32_t step = 2 * (int32_t)gridDim.x;
+    int32_t i = 2 * (int32_t)blockIdx.x + side;
+    DcaItem next{-1, 0, 0, 0};
+    int32_t next_s0 = 0, next_L = 0;
+    auto read_next = [&]() {
+      if (i < p.num_items) {
+        next = p.items[i];
+        next_s0 = p.seq_offsets[next.req];
+        next_L = p.seq_offsets[next.req + 1] - next_s0;
+      } else {
+        next.req = -1;
+        next_L = 0;
+      }
+      i += step;
+    };
+    read_next();
+    while (true) {
+      const DcaItem item = next;
+      const int32_t s0 = next_s0, L = next_L;
+      const uint32_t slot = n_item & 1;
+      // (a slot comes free only if the items in front of it can finish, the last one included when this one
+      // has no loads behind which its tail would be zeroed)
+      if (L == 0 && !zero_tail()) { ok = false; break; }
+      if (!wait(info_empty + 8 * slot, ((n_item >> 1) & 1) ^ 1, 12)) { ok = false; break; }
+      if (lane == 0) {
+        info[2 * slot] = make_int4(item.req, item.cand0, item.count * p.n_q, item.head);
+        info[2 * slot + 1] = make_int4(L, s0, 0, 0);
+        mbar_arrive(info_full + 8 * slot);
+      }
+      ++n_item;
+      if (item.req < 0) break;
+      read_next();
+      if (L == 0) continue;  // nobody touches another barrier for an item without keys
+      if (!wait(q_empty, (n_work & 1) ^ 1, 1)) { ok = false; break; }
+      ++n_work;
+      if (elect_one()) {
         mbar_expect_tx(q_full, kQBytes);
 #pragma unroll
         for (int bx = 0; bx < kBoxes; ++bx)
           tma_load_2d(q_dst + bx * C::kQBoxBytes, &map_q, q_full, item.head * DH + bx * C::kBoxCols, item.cand0 * p.n_q);
-        const int32_t nblk = (L + BKV - 1) / BKV;
-        for (int32_t j = 0; j < nblk; ++j, ++kv_it) {
-          const uint32_t s = kv_it % kKvStages;
-          if (!mbar_wait_paced(kv_empty + 8 * s, ((kv_it / kKvStages) & 1) ^ 1, abort_flag, p.status, kStatusDca | 2)) { ok = false; break; }
-          mbar_expect_tx(kv_full + 8 * s, kKvStageBytes);
-#pragma unroll
-          for (int bx = 0; bx < kBoxes; ++bx) {
-            tma_load_2d(kv_dst + s * kKvStageBytes + bx * C::kKvBoxBytes, &map_k, kv_full + 8 * s,
-                        item.head * DH + bx * C::kBoxCols, s0 + j * BKV);
-            tma_load_2d(kv_dst + s * kKvStageBytes + kKBytes + bx * C::kKvBoxBytes, &map_v, kv_full + 8 * s,
-                        item.head * DH + bx * C::kBoxCols, s0 + j * BKV);
-          }
-        }
       }
-      if (!ok) {
-        // let the loads in flight land before the CTA's shared memory goes away
-        for (uint32_t s = 0; s < kKvStages; ++s) {
-          const uint32_t n_issued = kv_it / kKvStages + ((kv_it % kKvStages > s) ? 1 : 0);
-          if (n_issued == 0) continue;
-          const uint64_t t0 = globaltimer_ns();
-          while (!mbar_try_wait_brief(kv_full + 8 * s, (n_issued - 1) & 1) && globaltimer_ns() - t0 < kWaitLimitNs) {}
+      __syncwarp();
+      if (!zero_tail()) { ok = false; break; }
+      const int32_t nblk = (L + BKV - 1) / BKV;
+      auto load_block = [&](const CUtensorMap* map, int32_t j) {
+        const uint32_t s = kv_it % kKvSlots;
+        if (!wait(kv_empty + 8 * s, ((kv_it / kKvSlots) & 1) ^ 1, 2)) return false;
+        if (elect_one()) {
+          mbar_expect_tx(kv_full + 8 * s, kKBytes);
+#pragma unroll
+          for (int bx = 0; bx < kBoxes; ++bx)
+            tma_load_2d(kv_dst + s * kKBytes + bx * C::kKvBoxBytes, map, kv_full + 8 * s, item.head * DH + bx * C::kBoxCols,
+                        s0 + j * BKV);
         }
+        __syncwarp();
+        ++kv_it;
+        return true;
+      };
+      // in the order of their use, which is the order they come free in: K_0, K_1, V_0, K_2, V_1, ...
+      ok = load_block(&map_k, 0);
+      for (int32_t j = 0; j < nblk && ok; ++j) {
+        if (j + 1 < nblk) ok = load_block(&map_k, j + 1);
+        if (ok) ok = load_block(&map_v, j);
+      }
+      if (!ok) break;
+      tail_valid = L % 16 == 0 ? 0 : L % BKV;
+      tail_slot = (kv_it - 1) % kKvSlots;
+      tail_phase = ((kv_it - 1) / kKvSlots) & 1;
+    }
+    if (!ok) {
+      // let the loads in flight land before the CTA's shared memory goes away
+      for (uint32_t s = 0; s < kKvSlots; ++s) {
+        const uint32_t n_issued = kv_it / kKvSlots + ((kv_it % kKvSlots > s) ? 1 : 0);
+        if (n_issued == 0) continue;
+        const uint64_t t0 = globaltimer_ns();
+        while (!mbar_try_wait_brief(kv_full + 8 * s, (n_issued - 1) & 1) && globaltimer_ns() - t0 < kWaitLimitNs) {}
       }
     }
   } else if (warp >= kControlWarp0) {
-    // ------------------------------ MMA issuers: one warp per side ---------------------------
-    const int side = warp - (kControlWarp0 + 1);
-    constexpr uint32_t idesc_s = umma_idesc_bf16(BQ, BKV, false, false);  // S = Q K^T, both K-major
-    constexpr uint32_t idesc_o = umma_idesc_bf16(BQ, C::kBoxCols, false, true);  // O = P V per box of output columns, V is MN-major
-    const uint32_t q_full = sb + kBarQFull + 8 * side, q_empty = sb + kBarQEmpty + 8 * side;
-    const uint32_t kv_full = sb + kBarKvFull + 8 * kKvStages * side, kv_empty = sb + kBarKvEmpty + 8 * kKvStages * side;
-    const uint32_t s_full = sb + kBarSFull + 8 * side, s_empty = sb + kBarSEmpty + 8 * side;
-    const uint32_t p_full = sb + kBarPFull + 8 * side, o_full = sb + kBarOFull + 8 * side;
-    const uint32_t kv_base = sb + kOffKv + side * kKvStages * kKvStageBytes;
-    uint32_t kv_it = 0, n_work = 0;           // n_work: items that had keys (phase of q_full)
-    uint32_t cnt_p = 0, cnt_se = 0;           // phases of p_full and s_empty of this side
-    bool ok = true;
-#ifdef ROCS_DCA_TRACE
-    int tr_blk = 0;
-#endif
-    const uint32_t t_s = tmem_base + side * kSideTmemStride;
-    // Q tile of this side, K block and V block of a stage as shared-memory operand descriptors
-    const uint64_t dq = C::desc(sb + kOffQ + side * kQBytes);
-    auto desc_k = [&](uint32_t stage) { return C::desc(kv_base + stage * kKvStageBytes); };
-    auto desc_v = [&](uint32_t stage) { return C::desc(kv_base + stage * kKvStageBytes + kKBytes); };
-    auto issue_s = [&](uint64_t b_desc) {
+    // ------------------------------ MMA issuers: one thread per side -------------------------
+    // (a whole loop under one elected lane: with the products alone under it, in a loop of the whole warp,
+    // issuing S and P V of a block took 780 cycles instead of the 180 here)
+    if (elect_one()) {
+      const int side = warp - (kControlWarp0 + 1);
+      constexpr uint32_t idesc_o = umma_idesc_bf16(BQ, DH, false, true);    // O = P V, V is MN-major
+      const uint32_t q_full = sb + kBarQFull + 8 * side, q_empty = sb + kBarQEmpty + 8 * side;
+      const uint32_t kv_full = sb + kBarKvFull + 8 * kKvSlots * side, kv_empty = sb + kBarKvEmpty + 8 * kKvSlots * side;
+      const uint32_t s_full = sb + kBarSFull + 8 * side, s_empty = sb + kBarSEmpty + 8 * side;
+      const uint32_t p_full = sb + kBarPFull + 8 * side, o_full = sb + kBarOFull + 8 * side;
+      const uint32_t tail_done = sb + kBarTail + 8 * side;
+      const uint32_t info_full = sb + kBarInfoFull + 16 * side, info_empty = sb + kBarInfoEmpty + 16 * side;
+      const int4* info = reinterpret_cast<const int4*>(smem + kOffInfo) + side * 4;
+      uint32_t kv_it = 0, n_work = 0, n_tail = 0, n_item = 0;  // phases of kv_full, q_full, tail_done, info_full
+      uint32_t cnt_p = 0, cnt_se = 0;                          // phases of p_full and s_empty
+      bool ok = true;
+      const uint32_t t_s = tmem_base + side * kSideTmemStride;
+      // Q tile of this side; slot 0 as a K and as a V block (a slot is kKBytes >> 4 further on)
+      const uint64_t dq = C::desc(sb + kOffQ + side * kQBytes);
+      const uint64_t dk0 = C::desc(sb + kOffKv + side * kKvSlots * kKBytes);
+      const uint64_t dv0 = C::desc_v(sb + kOffKv + side * kKvSlots * kKBytes);
+      // `keys`: of the block, a multiple of 16
+      auto issue_s = [&](uint32_t slot, int32_t keys) {
+        const uint64_t dk = dk0 + slot * (kKBytes >> 4);
+        const uint32_t idesc_s = umma_idesc_bf16(BQ, (uint32_t)keys, false, false);  // S = Q K^T, both K-major
 #pragma unroll
-      for (int k = 0; k < DH / 16; ++k) {  // 16 columns of dh per step: box k / kPerBox, 32 bytes further on inside it
-        constexpr int kPerBox = C::kBoxCols / 16;
-        umma_ss(t_s, dq + (k / kPerBox) * (C::kQBoxBytes >> 4) + 2 * (k % kPerBox),
-                b_desc + (k / kPerBox) * (C::kKvBoxBytes >> 4) + 2 * (k % kPerBox), idesc_s, k != 0 ? 1u : 0u);
-      }
-      umma_commit(s_full);
-    };
-    auto issue_pv = [&](uint64_t b_desc, bool first_block) {
-      // P: 16 keys = 8 columns of bf16 pairs in tensor memory
-      // V: rows are keys (K), one row = a box of head dims (N): 16 keys = 16 rows further on
-#pragma unroll
-      for (int k = 0; k < BKV / 16; ++k)
-#pragma unroll
-        for (int bx = 0; bx < kBoxes; ++bx)  // one box of output columns per product
-          umma_ts(t_s + kOColOffset + bx * C::kBoxCols, t_s + kPColOffset + k * 8,
-                  b_desc + bx * (C::kKvBoxBytes >> 4) + k * (16 * C::kRowBytes / 16), idesc_o, (k != 0 || !first_block) ? 1u : 0u);
-      umma_commit(o_full);
-    };
-    // The last block of a sequence may reach past it into the next request's rows (or past the
-    // tensor, where TMA fills zeros).  Scores of such keys are masked to -inf by the softmax warps,
-    // so P is exactly 0 there; the V rows are zeroed here so that 0 x (Inf or NaN of a foreign
-    // request) cannot reach this request's output.
-    auto zero_v_tail = [&](uint32_t stage, int32_t valid) {
-      uint8_t* v = smem + kOffKv + (side * kKvStages + stage) * kKvStageBytes + kKBytes;
-      for (int bx = 0; bx < kBoxes; ++bx)
-        for (int idx = valid * (C::kRowBytes / 16) + lane; idx < BKV * (C::kRowBytes / 16); idx += 32)
-          *reinterpret_cast<uint4*>(v + bx * C::kKvBoxBytes + idx * 16) = make_uint4(0u, 0u, 0u, 0u);
-      fence_proxy_async_smem();
-      __syncwarp();
-    };
-    for (int32_t i = item0 + side; i < p.num_items && ok; i += item_step) {
-      const DcaItem item = p.items[i];
-      const int32_t L = p.seq_offsets[item.req + 1] - p.seq_offsets[item.req];
-      if (L == 0) continue;
-      const int32_t nblk = (L + BKV - 1) / BKV;
-      const int32_t tail_valid = L - (nblk - 1) * BKV;  // keys of the last block that exist
-      if (!mbar_wait_paced(q_full, n_work & 1, abort_flag, p.status, kStatusDca | 3)) { ok = false; break; }
-      ++n_work;
-      // first key block (the S tile was drained at the end of the previous item)
-      if (!mbar_wait_paced(kv_full + 8 * (kv_it % kKvStages), (kv_it / kKvStages) & 1, abort_flag, p.status, kStatusDca | 4)) { ok = false; break; }
-      if (nblk == 1 && tail_valid < BKV) zero_v_tail(kv_it % kKvStages, tail_valid);
-      tc_fence_after_sync();
-      if (elect_one()) {
-        issue_s(desc_k(kv_it % kKvStages));
-        if (nblk == 1) umma_commit(q_empty);
-      }
-      __syncwarp();
-      for (int32_t j = 0; j < nblk && ok; ++j, ++kv_it) {
-        const uint32_t stage = kv_it % kKvStages;
-        const uint32_t next_stage = (kv_it + 1) % kKvStages;
-        const uint64_t dk_next = desc_k(next_stage), dv = desc_v(stage);
-        TRACE_EV(2 + side, 0);
-        if (j + 1 < nblk) {
-          if (!mbar_wait_paced(kv_full + 8 * next_stage, ((kv_it + 1) / kKvStages) & 1, abort_flag, p.status, kStatusDca | 5)) { ok = false; break; }
-          TRACE_EV(2 + side, 1);
-          if (j + 2 == nblk && tail_valid < BKV) zero_v_tail(next_stage, tail_valid);
+        for (int k = 0; k < DH / 16; ++k) {  // 16 columns of dh per step: box k / kPerBox, 32 bytes further on inside it
+          constexpr int kPerBox = C::kBoxCols / 16;
+          umma_ss(t_s, dq + (k / kPerBox) * (C::kQBoxBytes >> 4) + 2 * (k % kPerBox),
+                  dk + (k / kPerBox) * (C::kKvBoxBytes >> 4) + 2 * (k % kPerBox), idesc_s, k != 0 ? 1u : 0u);
         }
-        // S_{j+1} as soon as the side has pulled S_j into registers
-        if (!mbar_wait_paced(s_empty, cnt_se & 1, abort_flag, p.status, kStatusDca | 11)) { ok = false; break; }
-        ++cnt_se;
-        TRACE_EV(2 + side, 2);
-        if (j + 1 < nblk) {
-          tc_fence_after_sync();
-          if (elect_one()) {
-            issue_s(dk_next);
+        umma_commit(s_full);
+        umma_commit(kv_empty + 8 * slot);
+      };
+      auto issue_pv = [&](uint32_t slot, int32_t keys, bool first_block) {
+        const uint64_t dv = dv0 + slot * (kKBytes >> 4);
+        // P: 16 keys = 8 columns of bf16 pairs in tensor memory; V: rows are keys, 16 keys = 16 rows further on
+#pragma unroll
+        for (int k = 0; k < BKV / 16; ++k)
+          if (k * 16 < keys)
+            umma_ts(t_s + kOColOffset, t_s + kPColOffset + k * 8, dv + k * (16 * C::kRowBytes / 16), idesc_o,
+                    (k != 0 || !first_block) ? 1u : 0u);
+        umma_commit(o_full);
+        umma_commit(kv_empty + 8 * slot);
+      };
+      auto next_slot = [&](uint32_t code) {  // the next block in the order of loading, landed
+        if (!mbar_wait_paced(kv_full + 8 * (kv_it % kKvSlots), (kv_it / kKvSlots) & 1, abort_flag, p.status, kStatusDca | code)) return false;
+        ++kv_it;
+        return true;
+      };
+      while (ok) {
+        const uint32_t slot = n_item & 1;
+        if (!mbar_wait_paced(info_full + 8 * slot, (n_item >> 1) & 1, abort_flag, p.status, kStatusDca | 13)) { ok = false; break; }
+        ++n_item;
+        const int32_t req = info[2 * slot].x, L = info[2 * slot + 1].x;
+        mbar_arrive(info_empty + 8 * slot);
+        if (req < 0) break;
+        if (L == 0) continue;
+        const int32_t nblk = (L + BKV - 1) / BKV;
+        const int32_t tail_keys = round16(L - (nblk - 1) * BKV);  // products of the last block
+        if (!mbar_wait_paced(q_full, n_work & 1, abort_flag, p.status, kStatusDca | 3)) { ok = false; break; }
+        ++n_work;
+        // first key block (the S tile was drained at the end of the previous item)
+        if (!next_slot(4)) { ok = false; break; }
+        tc_fence_after_sync();
+        issue_s((kv_it - 1) % kKvSlots, nblk == 1 ? tail_keys : BKV);
+        if (nblk == 1) umma_commit(q_empty);
+        for (int32_t j = 0; j < nblk; ++j) {
+          if (j + 1 < nblk && !next_slot(5)) { ok = false; break; }
+          // S_{j+1} as soon as the side has pulled S_j into registers
+          if (!mbar_wait_paced(s_empty, cnt_se & 1, abort_flag, p.status, kStatusDca | 11)) { ok = false; break; }
+          ++cnt_se;
+          if (j + 1 < nblk) {
+            tc_fence_after_sync();
+            issue_s((kv_it - 1) % kKvSlots, j + 2 == nblk ? tail_keys : BKV);
             if (j + 2 == nblk) umma_commit(q_empty);  // last S of the item: the Q tile is free
           }
-          __syncwarp();
-          TRACE_EV(2 + side, 3);
+          if (!next_slot(8)) { ok = false; break; }
+          if (j + 1 == nblk && L % 16 != 0) {  // V rows past the sequence are zero
+            if (!mbar_wait_paced(tail_done, n_tail & 1, abort_flag, p.status, kStatusDca | 10)) { ok = false; break; }
+            ++n_tail;
+          }
+          // P_j of this side is in tensor memory
+          if (!mbar_wait_paced(p_full, cnt_p & 1, abort_flag, p.status, kStatusDca | 6)) { ok = false; break; }
+          ++cnt_p;
+          tc_fence_after_sync();
+          issue_pv((kv_it - 1) % kKvSlots, j + 1 == nblk ? tail_keys : BKV, j == 0);
         }
-        // P_j of this side is in tensor memory
-        if (!mbar_wait_paced(p_full, cnt_p & 1, abort_flag, p.status, kStatusDca | 6)) { ok = false; break; }
-        ++cnt_p;
-        TRACE_EV(2 + side, 4);
-        tc_fence_after_sync();
-        if (elect_one()) {
-          issue_pv(dv, j == 0);
-          umma_commit(kv_empty + 8 * stage);  // K_j and V_j are no longer needed
-        }
-        __syncwarp();
-        TRACE_EV(2 + side, 5);
-        TRACE_NEXT();
       }
-    }
-    if (!ok && lane == 0) {
-      umma_commit(sb + kBarDrain + 8 * side);
-      const uint64_t t0 = globaltimer_ns();
-      while (!mbar_try_wait_brief(sb + kBarDrain + 8 * side, 0) && globaltimer_ns() - t0 < kWaitLimitNs) {}
+      if (!ok) {
+        umma_commit(sb + kBarDrain + 8 * side);
+        const uint64_t t0 = globaltimer_ns();
+        while (!mbar_try_wait_brief(sb + kBarDrain + 8 * side, 0) && globaltimer_ns() - t0 < kWaitLimitNs) {}
+      }
     }
   } else {
     // ------------------------------ softmax warps ------------------------------------------
@@ -454,62 +495,49 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const uint32_t p_full = sb + kBarPFull + 8 * side, o_full = sb + kBarOFull + 8 * side;
     const uint32_t my_pair = sb + kBarPair + 8 * (side * 4 + q);
     uint32_t cnt_s = 0, cnt_o = 0, cnt_pair = 0;
-#ifdef ROCS_DCA_TRACE
-    int tr_blk = 0;
-    const int tr_role = warp == 0 ? 0 : warp == 8 ? 1 : -1;
-#define TRACE_SM(ev) do { if (tr_role >= 0) TRACE_EV(tr_role, ev); } while (0)
-#else
-#define TRACE_SM(ev)
-#endif
-    for (int32_t i = item0 + side; i < p.num_items; i += item_step) {
-      const DcaItem item = p.items[i];
-      const int32_t L = p.seq_offsets[item.req + 1] - p.seq_offsets[item.req];
-      const int32_t rows_valid = item.count * p.n_q;
+    const uint32_t info_full = sb + kBarInfoFull + 16 * side, info_empty = sb + kBarInfoEmpty + 16 * side;
+    const int4* info = reinterpret_cast<const int4*>(smem + kOffInfo) + side * 4;
+    for (uint32_t n_item = 0;; ++n_item) {
+      const uint32_t slot = n_item & 1;
+      if (!mbar_wait_spin(info_full + 8 * slot, (n_item >> 1) & 1, abort_flag, p.status, kStatusDca | 13)) break;
+      const int4 item = info[2 * slot];  // request, first candidate, query rows, head
+      const int32_t L = info[2 * slot + 1].x;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(info_empty + 8 * slot);
+      if (item.x < 0) break;
+      const int32_t rows_valid = item.z;
       // this thread's half of the output columns of its row
-      auto out_ptr = [&]() { return p.O + ((int64_t)item.cand0 * p.n_q + row) * row_width + item.head * DH + half * kOutCols; };
+      auto out_ptr = [&]() { return p.O + ((int64_t)item.y * p.n_q + row) * row_width + item.w * DH + half * kOutCols; };
       bool aborted = false;
       if (L > 0) {
         const int32_t nblk = (L + BKV - 1) / BKV;
-        // ---- reference of the row: the maximum of its first block, rounded up to an integer
-        TRACE_SM(0);
+        // ---- reference of the row: the maximum over its first 32 keys, rounded up to an integer
         if (!mbar_wait_spin(s_full, cnt_s & 1, abort_flag, p.status, kStatusDca | 7)) break;
         tc_fence_after_sync();
         float m_ref;
         {
           float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+          uint32_t ov[32];
+          tmem_ld_32x32b_x32(t_row, ov);
+          tmem_ld_wait();
+          if (L < 32) {
 #pragma unroll
-          for (int c = 0; c < BKV; c += 32) {
-            uint32_t ov[32];
-            tmem_ld_32x32b_x32(t_row + c, ov);
-            tmem_ld_wait();
-            if (L < c + 32) {
-#pragma unroll
-              for (int e = 0; e < 32; ++e)
-                if (c + e >= L) ov[e] = 0xff800000u;  // -inf: the key does not exist
-            }
-#pragma unroll
-            for (int e = 0; e < 32; e += 2)  // four short chains of three-input maxima
-              mx4[(e >> 1) & 3] = fmax3(mx4[(e >> 1) & 3], __uint_as_float(ov[e]), __uint_as_float(ov[e + 1]));
+            for (int e = 0; e < 32; ++e)
+              if (e >= L) ov[e] = 0xff800000u;  // -inf: the key does not exist
           }
+#pragma unroll
+          for (int e = 0; e < 32; e += 2)  // four short chains of three-input maxima
+            mx4[(e >> 1) & 3] = fmax3(mx4[(e >> 1) & 3], __uint_as_float(ov[e]), __uint_as_float(ov[e + 1]));
           m_ref = ceilf(fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * p.scale_log2e);
         }
         const uint64_t c2 = pack2(p.scale_log2e, p.scale_log2e), m2 = pack2(-m_ref, -m_ref);
-        // the polynomial path: x = s c - m_ref with m_ref an integer, so n = round(x) comes out of one
-        // fused multiply-add against kMagic - m_ref; scores are clamped from below at x = -126 (2^x is
-        // nothing there) and must stay below x = 126, which is checked per block
-        const float k_off = kMagic - m_ref;
-        const float s_lo = (m_ref - 126.f) / p.scale_log2e;
-        bool by_hand = kEmuPairs > 0 && !(fabsf(m_ref) < 1048576.f);  // kMagic - m_ref must be exact
-        float g_max = -INFINITY;                     // largest raw score that went through the polynomial
         uint64_t sum2 = pack2(0.f, 0.f);
         for (int32_t j = 0; j < nblk; ++j) {
           if (j > 0) {
-            TRACE_SM(0);
             if (!mbar_wait_spin(s_full, cnt_s & 1, abort_flag, p.status, kStatusDca | 7)) { aborted = true; break; }
             tc_fence_after_sync();
           }
           ++cnt_s;
-          TRACE_SM(1);
           uint32_t sv[kCols];  // this thread's scores of the block
 #pragma unroll
           for (int c = 0; c < kCols; c += 32) tmem_ld_32x32b_x32(t_s + c, sv + c);
@@ -523,68 +551,50 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             for (int e = 0; e < kCols; ++e)
               if (e >= valid) sv[e] = 0xff800000u;  // -inf: the key does not exist
           }
-          TRACE_SM(2);
           uint32_t pk[kCols / 4];  // P of half of this thread's keys, bf16 pairs; stored in two halves
           auto store_p = [&](uint32_t taddr) {
             if constexpr (kCols == 64) tmem_st_32x32b_x16(taddr, pk); else tmem_st_32x32b_x8(taddr, pk);
           };
           auto exp_pair = [&](int e) {
-            float p0, p1;
-            if (((e >> 1) & 7) < kEmuPairs) {
-              const uint64_t k2 = pack2(k_off, k_off);
-              const float s0 = __uint_as_float(sv[e]), s1 = __uint_as_float(sv[e + 1]);
-              g_max = fmax3(g_max, s0, s1);
-              const uint64_t s2 = pack2(fmax_nan(s0, s_lo), fmax_nan(s1, s_lo));
-              const uint64_t xf2 = ffma2(s2, c2, k2);                        // kMagic + n
-              const uint64_t w2 = ffma2(xf2, pack2(-1.f, -1.f), k2);          // -(n + m_ref)
-              const uint64_t r2 = ffma2(s2, c2, w2);                         // x - n
-              uint64_t q2 = ffma2(r2, pack2(kPoly3, kPoly3), pack2(kPoly2, kPoly2));
-              q2 = ffma2(q2, r2, pack2(kPoly1, kPoly1));
-              q2 = ffma2(q2, r2, pack2(kPoly0, kPoly0));
-              float q0, q1, f0, f1;
-              unpack2(q2, q0, q1);
-              unpack2(xf2, f0, f1);
-              p0 = __uint_as_float(__float_as_uint(q0) + (__float_as_uint(f0) << 23));  // 2^r scaled by 2^n
-              p1 = __uint_as_float(__float_as_uint(q1) + (__float_as_uint(f1) << 23));
-            } else {
-              float x0, x1;
-              unpack2(ffma2(pack2(__uint_as_float(sv[e]), __uint_as_float(sv[e + 1])), c2, m2), x0, x1);
-              p0 = ex2(x0);
-              p1 = ex2(x1);
-            }
+            float x0, x1;
+            unpack2(ffma2(pack2(__uint_as_float(sv[e]), __uint_as_float(sv[e + 1])), c2, m2), x0, x1);
+            const float p0 = ex2(x0), p1 = ex2(x1);
             sum2 = fadd2(sum2, pack2(p0, p1));
             pk[(e / 2) % (kCols / 4)] = bf16x2_bits(p0, p1);
           };
+          // P V of the previous block has read P_{j-1} (it was issued most of a block ago): from there on this
+          // thread's P columns may be rewritten
+          auto previous_pv_done = [&]() {
+            if (j > 0) {
+              if (!mbar_wait_spin(o_full, (cnt_o & 1) ^ 1, abort_flag, p.status, kStatusDca | 9)) return false;
+              tc_fence_after_sync();
+            }
+            ++cnt_o;
+            return true;
+          };
+          if (valid > 0) {
 #pragma unroll
-          for (int e = 0; e < kCols / 2; e += 2) exp_pair(e);
-          TRACE_SM(3);
-          if (j > 0) {
-            // P V of the previous block has read P_{j-1} (it was issued most of a block ago): from here
-            // on this thread's P columns may be rewritten
-            if (!mbar_wait_spin(o_full, (cnt_o & 1) ^ 1, abort_flag, p.status, kStatusDca | 8)) { aborted = true; break; }
-            tc_fence_after_sync();
+            for (int e = 0; e < kCols / 2; e += 2) exp_pair(e);
+            if (!previous_pv_done()) { aborted = true; break; }
+            store_p(t_p);
+#pragma unroll
+            for (int e = kCols / 2; e < kCols; e += 2) exp_pair(e);
+            store_p(t_p + kCols / 4);
+          } else if (!previous_pv_done()) {  // no key in this half of the last block: P V stops in front of it
+            aborted = true;
+            break;
           }
-          ++cnt_o;
-          TRACE_SM(4);
-          store_p(t_p);
-#pragma unroll
-          for (int e = kCols / 2; e < kCols; e += 2) exp_pair(e);
-          TRACE_SM(5);
-          store_p(t_p + kCols / 4);
-          if (kEmuPairs > 0 && g_max * p.scale_log2e - m_ref > 126.f) by_hand = true;  // 2^n would leave fp32's exponent field
           tmem_st_wait();
           tc_fence_before_sync();
           __syncwarp();
           if (lane == 0) mbar_arrive(p_full);
-          TRACE_SM(6);
-          TRACE_NEXT();
         }
         if (aborted) break;
         float sum_lo, sum_hi;
         unpack2(sum2, sum_lo, sum_hi);
         const float l_run = sum_lo + sum_hi;
         float* l_x = reinterpret_cast<float*>(smem + kOffL);
-        l_x[(side * 2 + half) * BQ + row] = by_hand ? __int_as_float(0x7fc00000) : l_run;  // NaN tells the other half of the row too
+        l_x[(side * 2 + half) * BQ + row] = l_run;
         __syncwarp();
         if (lane == 0) mbar_arrive(my_pair);
         if (!mbar_wait_paced(my_pair, cnt_pair & 1, abort_flag, p.status, kStatusDca | 14) ||
@@ -610,7 +620,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         for (int e = 0; e < kOutCols; ++e) probe = fmaf(__uint_as_float(v[e]), 0.f, probe);
         if (row < rows_valid) {
           __nv_bfloat16* out = out_ptr();
-          if (probe == 0.f && !by_hand) {
+          if (probe == 0.f) {
 #pragma unroll
             for (int e = 0; e < kOutCols; e += 8) {
               uint4 w;
@@ -622,9 +632,9 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             }
           } else {
             // such a row is computed again here, by this thread alone, with its true maximum as reference
-            const int64_t q_row = (int64_t)item.cand0 * p.n_q + row;
-            const int64_t kv0 = ((int64_t)p.seq_offsets[item.req] * p.H + item.head) * DH;
-            row_by_hand<DH>(p.Q + q_row * row_width + item.head * DH, p.K + kv0, p.V + kv0 + half * kOutCols, row_width,
+            const int64_t q_row = (int64_t)item.y * p.n_q + row;
+            const int64_t kv0 = ((int64_t)p.seq_offsets[item.x] * p.H + item.w) * DH;
+            row_by_hand<DH>(p.Q + q_row * row_width + item.w * DH, p.K + kv0, p.V + kv0 + half * kOutCols, row_width,
                             L, p.scale_log2e, out);
           }
         }
@@ -701,9 +711,6 @@ static rocs_status_t launch_dca(const rocs_plan* plan, int32_t n_q, int32_t H, f
   p.V = (const __nv_bfloat16*)V;
   p.O = (__nv_bfloat16*)O;
   p.status = status;
-#ifdef ROCS_DCA_TRACE
-  p.trace = (long long*)rocs_dca_trace_buffer;
-#endif
   auto kernel = dca_umma_kernel<DH, BKV>;
   ROCS_ALLOW_SMEM(kernel, C::kSmemBytes);
   const int grid = std::min((items.num + 1) / 2, sm_count_dca());  // one CTA per SM, two item streams per CTA

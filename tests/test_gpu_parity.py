@@ -280,6 +280,25 @@ def test_dca_bf16_head_dim_32_and_128_ragged_on_tensor_cores(dh):
     assert _run_dca(cfg, wl.offsets_from_counts([3, 50, 9]), wl.offsets_from_counts([70, 33, 257]), scale=0.1) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("dh", [32, 64, 128])
+def test_dca_bf16_short_last_blocks_between_empty_requests(dh):
+    # products of the last key block end at a multiple of 16 keys, the rows of V between are zeroed behind the next
+    # item's loads: every remainder class, items with no keys and with no ragged end in between, one item per side
+    # and long streams; V rows behind each sequence hold NaN, in a request that has no candidates
+    lens = [1, 0, 15, 16, 17, 0, 0, 31, 33, 48, 63, 64, 65, 79, 80, 81, 0, 95, 97, 112, 127, 128, 129, 143, 144, 145, 200, 257]
+    co = wl.offsets_from_counts([c for _ in lens for c in (3, 0)])
+    so = wl.offsets_from_counts([x for n in lens for x in (n, 3)])
+    for H in (1, 16):
+        cfg = wl.CONFIGS[3].with_(R=len(co) - 1, H=H, dh=dh)
+        d = wl.dca_inputs(cfg, co, so)
+        V = wl.bf16_bits_to_f32(d["V"]).copy()
+        want = ref.dca_attention(co, so, d["Q"], d["K"], d["V"])
+        for r in range(1, len(so) - 1, 2):
+            V[so[r]:so[r + 1]] = np.nan
+        O = rocs.dca_attention(_plan(co), to_dev(d["Q"]), to_dev(d["K"]), to_dev(wl.f32_to_bf16_bits(V)), to_dev(so))
+        assert rel_err(to_host_f64(O), want) <= tol_for("bf16")
+
+
 @pytest.mark.parametrize("dh", [32, 128])
 def test_dca_bf16_head_dim_32_and_128_many_tiles_sampled(dh):
     # enough tiles that every SM runs several items on both of its streams (L = 700: 11 or 6 key blocks)
