@@ -598,19 +598,22 @@ rocs_status_t rocs_glm_interaction(const rocs_plan_t* plan, rocs_dtype_t dtype, 
       return ROCS_ERR_WORKSPACE;
     zr = (float*)workspace;
   }
-  if (dtype == ROCS_BF16 && g_path.load() == ROCS_PATH_AUTO && umma_glm_supported(n_r, n_c, d, n_ro, n_co)) {
+  const bool mma = !umma_glm_supported(n_r, n_c, d, n_ro, n_co) && glm_mma_supported(n_r, n_c, d, n_co);
+  if (dtype == ROCS_BF16 && g_path.load() == ROCS_PATH_AUTO && (mma || umma_glm_supported(n_r, n_c, d, n_ro, n_co))) {
     // The candidate kernel's tile list first: that kernel then starts beside the request kernel.
     TileList tiles;
-    rocs_status_t st = (YC || OC) ? plan_tiles(plan, 128 / n_c, stream, &tiles) : ROCS_OK;
+    rocs_status_t st = !YC && !OC ? ROCS_OK
+                       : mma      ? glm_mma_tiles(plan, n_r, n_c, d, stream, &tiles)
+                                  : plan_tiles(plan, 128 / n_c, stream, &tiles);
     if (st != ROCS_OK) return st;
     // Request side once per request (tiny), candidate side on tensor cores.
     st = glm_request_mma_supported(n_r, d, n_ro, n_co)
-                           ? glm_request_mma(plan, n_r, n_c, d, XR, W, n_ro, n_co, YR, OR_, zr, stream)
-                           : simt_glm(dtype, plan, n_r, n_c, d, XR, nullptr, W, n_ro, n_co, YR, nullptr, OR_,
-                                      nullptr, zr, stream);
+             ? glm_request_mma(plan, n_r, n_c, d, XR, W, n_ro, n_co, YR, OR_, zr, stream)
+             : simt_glm(dtype, plan, n_r, n_c, d, XR, nullptr, W, n_ro, n_co, YR, nullptr, OR_, nullptr, zr, stream);
     if (st != ROCS_OK) return st;
     if (!YC && !OC) return ROCS_OK;
-    return umma_glm(plan, n_r, n_c, d, XR, XC, W, n_ro, n_co, YC, OC, zr, stream);
+    return mma ? glm_mma(plan, n_r, n_c, d, XR, XC, W, n_ro, n_co, YC, OC, zr, stream)
+               : umma_glm(plan, n_r, n_c, d, XR, XC, W, n_ro, n_co, YC, OC, zr, stream);
   }
   return simt_glm(dtype, plan, n_r, n_c, d, XR, XC, W, n_ro, n_co, YR, YC, OR_, OC, zr, stream);
 }

@@ -179,6 +179,13 @@ bool umma_dca_supported(int32_t n_q, int32_t H, int32_t dh);
 rocs_status_t umma_dca(const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh, float scale,
                        const void* Q, const void* K, const void* V, const int32_t* seq_offsets,
                        int64_t T, void* O, cudaStream_t stream);
+// Candidate side of the interaction operator (bf16).  glm_mma: warp-level tensor cores, 4 to 16 embeddings per
+// candidate; its tile list can be made in front of the request kernel.  umma_glm: 8, 16 or 32, the faster of the two.
+bool glm_mma_supported(int32_t n_r, int32_t n_c, int32_t d, int32_t n_co);
+rocs_status_t glm_mma_tiles(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, cudaStream_t stream, TileList* out);
+rocs_status_t glm_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, const void* XR, const void* XC,
+                      const void* W, int32_t n_ro, int32_t n_co, void* YC, void* OC, const float* zr_workspace,
+                      cudaStream_t stream);
 bool umma_glm_supported(int32_t n_r, int32_t n_c, int32_t d, int32_t n_ro, int32_t n_co);
 rocs_status_t umma_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, const void* XR,
                        const void* XC, const void* W, int32_t n_ro, int32_t n_co, void* YC,

@@ -469,6 +469,41 @@ def test_glm_general_kernel_tiles(dtype, n_r, n_c, d, n_co):
     assert _run_glm(cfg, co) <= tol_for(dtype)
 
 
+@pytest.mark.parametrize("n_r,n_c,d,n_co,raw", [(32, 16, 128, 8, False), (20, 12, 64, 4, True), (4, 4, 192, 16, True), (44, 8, 256, 3, False),
+                                                  (20, 8, 128, 0, True), (16, 4, 64, 8, False), (100, 16, 64, 16, True),
+                                                  (128, 12, 256, 1, False), (44, 16, 128, 0, True), (24, 12, 128, 8, False)])
+@pytest.mark.parametrize("many", [False, True])
+def test_glm_fragments(n_r, n_c, d, n_co, raw, many):
+    # 4 to 16 embeddings per candidate (one to four candidates per 16-row fragment, unused rows in some), request
+    # columns that end inside a group of 16 and take several passes, fewer fragments than warps; a candidate
+    # and a request full of NaN must show in their own rows only
+    counts = [1, 0, 9, 8, 33, 7, 0, 133] * (30 if many else 1)
+    co = wl.offsets_from_counts(counts + ([3000] if many and n_c < 8 else []))
+    cfg = wl.CONFIGS[4].with_(R=len(co) - 1, n_r=n_r, n_c=n_c, d_emb=d, n_ro=min(2, n_co), n_co=n_co)
+    g = wl.glm_inputs(cfg, co)
+    plan, W = _plan(co), to_dev(g["W"]) if n_co else None
+    N, m = int(co[-1]), np.repeat(np.arange(cfg.R), np.diff(co))
+
+    def run(XR, XC):
+        o = rocs.glm_interaction(plan, to_dev(XR), to_dev(XC), W, cfg.n_ro, cfg.n_co, want_raw=raw)
+        return {k: o[k] for k in ("YC", "OC") if k in o}
+
+    base = run(g["XR"], g["XC"])
+    sample = np.unique(np.concatenate([np.arange(min(N, 70)), np.random.default_rng(1).integers(0, N, 60), [N - 1]]))
+    G, O = ref.glm_interaction(co, g["XR"], g["XC"], g["W"] if n_co else None, cfg.n_ro, cfg.n_co, sample=sample)
+    if raw:
+        assert rel_err(to_host_f64(base["YC"])[sample], G[:, n_r:]) <= tol_for("bf16")
+    if n_co:
+        assert rel_err(to_host_f64(base["OC"])[sample], O[:, cfg.n_ro:]) <= tol_for("bf16")
+    XC, XR = g["XC"].copy(), g["XR"].copy()
+    XC[12], XR[4] = 0x7fc0, 0x7fc0
+    pert = run(XR, XC)
+    keep = (m != 4) & (np.arange(N) != 12)
+    for k in base:
+        assert np.array_equal(_bits(base[k])[keep], _bits(pert[k])[keep])
+        assert bool(torch.isnan(pert[k][12].float()).any())
+
+
 @pytest.mark.parametrize("R", [1, 127, 128, 129, 255, 257, 12000, 12001])
 def test_work_lists_of_many_requests(R):
     # the lists are scanned by 256 threads per block up to 12000 requests and on the host beyond: counts of
