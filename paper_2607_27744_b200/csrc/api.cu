@@ -270,10 +270,16 @@ static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, in
   return st;
 }
 
-rocs_status_t plan_row2req(const rocs_plan* plan, cudaStream_t stream, const int32_t** out) {
+rocs_status_t plan_request_map(const rocs_plan* plan, cudaStream_t stream, RequestMap* out) {
+  *out = RequestMap{};
+  if (plan->N <= kSearchRows) {
+    out->offsets = plan->cand_offsets;
+    out->R = plan->R;
+    return ROCS_OK;
+  }
   DeviceList list;
   const rocs_status_t st = plan_list(plan, 0, 0, stream, &list);
-  *out = static_cast<const int32_t*>(list.dev);
+  out->row2req = static_cast<const int32_t*>(list.dev);
   return st;
 }
 
@@ -397,15 +403,15 @@ size_t rocs_ikbo_linear_workspace(const rocs_plan_t* plan, int32_t d_out) {
 static rocs_status_t linear_dispatch(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_out,
                                      const void* X, int64_t ld_x, const void* W, int64_t ld_w,
                                      const float* bias, const float* add, int64_t ld_add,
-                                     const int32_t* row2req, int act, void* Y, int64_t ld_y,
+                                     const RequestMap& map, int act, void* Y, int64_t ld_y,
                                      bool out_f32, cudaStream_t stream,
                                      bool add_from_previous_launch = false, float2* stat_partials = nullptr,
                                      int64_t add_rows = 0) {
   if (dt == ROCS_BF16 && g_path.load() == ROCS_PATH_AUTO &&
       umma_linear_supported(M, d_in, d_out, ld_x, ld_w, ld_y, out_f32))
-    return umma_linear(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act, Y, ld_y,
+    return umma_linear(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y,
                        out_f32, stream, add_from_previous_launch, stat_partials, add_rows);
-  return simt_linear(dt, M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act, Y, ld_y,
+  return simt_linear(dt, M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y,
                      out_f32, stream);
 }
 
@@ -439,17 +445,17 @@ static rocs_status_t ikbo_linear_impl(const rocs_plan_t* plan, rocs_dtype_t dtyp
     if (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255u))
       return ROCS_ERR_WORKSPACE;
   }
-  const int32_t* row2req = nullptr;
+  RequestMap map;
   if (d_req > 0) {
     const size_t need = z_bytes;
     if (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255u))
       return ROCS_ERR_WORKSPACE;
     // In front of the request half: the candidate kernel may start beside that one and reads the map at once.
-    rocs_status_t st = plan_row2req(plan, stream, &row2req);
+    rocs_status_t st = plan_request_map(plan, stream, &map);
     if (st != ROCS_OK) return st;
     // Request half, once per request (Section 4.1): Z = X^R W_CR^T + bias, fp32.
     st = linear_dispatch(dtype, plan->R, d_req, d_out, XR, ld_xr, W_CR, ld_wcr, bias,
-                                       nullptr, 0, nullptr, ROCS_ACT_NONE, workspace, d_out,
+                                       nullptr, 0, RequestMap{}, ROCS_ACT_NONE, workspace, d_out,
                                        /*out_f32=*/true, stream);
     if (st != ROCS_OK) return st;
     Z = (const float*)workspace;
@@ -468,7 +474,7 @@ static rocs_status_t ikbo_linear_impl(const rocs_plan_t* plan, rocs_dtype_t dtyp
       umma_linear_ws2_supported(plan->N, d_cand, d_out, false))
     partials = reinterpret_cast<float2*>(static_cast<uint8_t*>(workspace) + z_bytes);
   rocs_status_t st = linear_dispatch(dtype, plan->N, d_cand, d_out, XC, ld_xc, W_CC, ld_wcc, bias, Z, d_out,
-                                     row2req, act, Y, ld_y, /*out_f32=*/false, stream,
+                                     map, act, Y, ld_y, /*out_f32=*/false, stream,
                                      request_half_on_umma, partials, plan->R);
   if (st != ROCS_OK || row_stats == nullptr) return st;
   if (partials != nullptr)
@@ -545,7 +551,7 @@ rocs_status_t rocs_linear(rocs_dtype_t dtype, int64_t M, int32_t d_in, int32_t d
   if (!aligned16(X) || !aligned16(W) || !aligned16(Y) || !aligned16(bias) || !row_stride_ok(ld_x, d_in, dtype) ||
       !row_stride_ok(ld_w, d_in, dtype) || !row_stride_ok(ld_y, d_out, dtype))
     return ROCS_ERR_ALIGNMENT;
-  return linear_dispatch(dtype, M, d_in, d_out, X, ld_x, W, ld_w, bias, nullptr, 0, nullptr, act, Y,
+  return linear_dispatch(dtype, M, d_in, d_out, X, ld_x, W, ld_w, bias, nullptr, 0, RequestMap{}, act, Y,
                          ld_y, false, (cudaStream_t)stream_);
 }
 

@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(256) fm_request_kernel(int32_t n_r, int32_t d,
 template <typename T>
 __global__ void __launch_bounds__(128) fm_candidate_simt_kernel(int32_t n_r, int32_t n_c, int32_t d, int32_t k,
                                                                 const T* __restrict__ XC, const T* __restrict__ P,
-                                                                const int32_t* __restrict__ row2req,
+                                                                const RequestMap map,
                                                                 const float* __restrict__ TT, T* __restrict__ FC) {
   extern __shared__ float sm[];
   const int32_t ds = d + 1;
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(128) fm_candidate_simt_kernel(int32_t n_r, int
   float* ht = xc + (size_t)n_c * ds;  // [k, d + 1]
   float* pc = ht + (size_t)k * ds;    // [n_c, k]
   const int64_t i = blockIdx.x;
-  const int32_t r = row2req[i];
+  const int32_t r = map.of(i);
   for (int e = threadIdx.x; e < n_c * d; e += blockDim.x) xc[(e / d) * ds + e % d] = ld_f(XC, i * n_c * d + e);
   for (int e = threadIdx.x; e < n_c * k; e += blockDim.x) pc[e] = ld_f(P, (int64_t)n_r * k + e);
   __syncthreads();
@@ -266,7 +266,7 @@ struct FmParams {
   int64_t N;
   int32_t n_r, n_c, k, num_tiles, stages;
   const __nv_bfloat16* P;        // [n_r + n_c, k]
-  const int32_t* row2req;        // [N]
+  RequestMap map;
   const float* TT;               // [R, k, d]
   __nv_bfloat16* FC;             // [N, n_c, k]
   uint32_t* status;
@@ -376,12 +376,12 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
     // otherwise sit on every candidate's critical path)
     int32_t r_next = 0;
     if (tile_begin < tile_end && (int64_t)tile_begin * kTileCands + warp < p.N)
-      r_next = p.row2req[(int64_t)tile_begin * kTileCands + warp];
+      r_next = p.map.of((int64_t)tile_begin * kTileCands + warp);
     for (int32_t t = tile_begin; t < tile_end; ++t) {
       const int32_t r = r_next;
       {
         const int64_t cand_next = (int64_t)(t + 1) * kTileCands + warp;
-        if (t + 1 < tile_end && cand_next < p.N) r_next = p.row2req[cand_next];
+        if (t + 1 < tile_end && cand_next < p.N) r_next = p.map.of(cand_next);
       }
       if (!mbar_wait(&full[s], phase, abort_flag, p.status, kStatusFm | 2)) break;
       const int64_t cand = (int64_t)t * kTileCands + warp;
@@ -465,7 +465,7 @@ int sm_count_fm() {
 }
 
 template <int D, int KT, bool FULL>
-rocs_status_t launch_fm_mma_as(const rocs_plan* plan, const int32_t* row2req, int32_t n_r, int32_t n_c, int32_t k,
+rocs_status_t launch_fm_mma_as(const rocs_plan* plan, const RequestMap& map, int32_t n_r, int32_t n_c, int32_t k,
                                const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
   const int stage_bytes = D / 64 * kTileCands * n_c * 128;
   constexpr int kFixed = kFragRows * 128 + 2 * kMaxStages * 8 + 16;
@@ -483,7 +483,7 @@ rocs_status_t launch_fm_mma_as(const rocs_plan* plan, const int32_t* row2req, in
   p.num_tiles = (int32_t)((plan->N + kTileCands - 1) / kTileCands);
   p.stages = std::min(kMaxStages, (227 * 1024 - kFixed) / stage_bytes);
   p.P = (const __nv_bfloat16*)P;
-  p.row2req = row2req;
+  p.map = map;
   p.TT = TT;
   p.FC = (__nv_bfloat16*)FC;
   p.status = status;
@@ -507,11 +507,11 @@ rocs_status_t launch_fm_mma_as(const rocs_plan* plan, const int32_t* row2req, in
 }
 
 template <int D>
-rocs_status_t launch_fm_mma(const rocs_plan* plan, const int32_t* row2req, int32_t n_r, int32_t n_c, int32_t k,
+rocs_status_t launch_fm_mma(const rocs_plan* plan, const RequestMap& map, int32_t n_r, int32_t n_c, int32_t k,
                             const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
-  if (k > 16) return launch_fm_mma_as<D, 2, false>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
-  if (n_c < kFragRows) return launch_fm_mma_as<D, 1, false>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
-  return launch_fm_mma_as<D, 1, true>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
+  if (k > 16) return launch_fm_mma_as<D, 2, false>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
+  if (n_c < kFragRows) return launch_fm_mma_as<D, 1, false>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
+  return launch_fm_mma_as<D, 1, true>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
 }
 
 template <typename T>
@@ -525,9 +525,9 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
   const size_t n_rp = (size_t)(n_r + 15) / 16 * 16, kp = (size_t)(k + 15) / 16 * 16;
   const size_t smem_mma = n_rp * ((size_t)(d + 8) * 2 + (kp + 8) * 2) + 2 * kp * (size_t)(d + 8) * 2;
   // in front of the request kernel: the candidate kernel may start beside that one and reads the map at once
-  const int32_t* row2req = nullptr;
+  RequestMap map;
   if (plan->N > 0 && FC) {
-    const rocs_status_t st = plan_row2req(plan, stream, &row2req);
+    const rocs_status_t st = plan_request_map(plan, stream, &map);
     if (st != ROCS_OK) return st;
   }
   if (plan->R > 0 && tensor_core_request && sizeof(T) == 2 && d % 16 == 0 && k % 8 == 0 && smem_mma <= kMaxSmem) {
@@ -543,16 +543,16 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
   if (plan->N == 0 || !FC) return ROCS_OK;
   if (fast_candidates) {
     switch (d) {
-      case 64: return launch_fm_mma<64>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
-      case 128: return launch_fm_mma<128>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
-      case 192: return launch_fm_mma<192>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
-      case 256: return launch_fm_mma<256>(plan, row2req, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 64: return launch_fm_mma<64>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 128: return launch_fm_mma<128>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 192: return launch_fm_mma<192>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 256: return launch_fm_mma<256>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
       default: break;
     }
   }
   ROCS_ALLOW_SMEM(fm_candidate_simt_kernel<T>, kMaxSmem);
   fm_candidate_simt_kernel<T><<<(unsigned)plan->N, 128, smem_c, stream>>>(n_r, n_c, d, k, (const T*)XC, (const T*)P,
-                                                                         row2req, TT, (T*)FC);
+                                                                         map, TT, (T*)FC);
   ROCS_CUDA_TRY(cudaGetLastError());
   return ROCS_OK;
 }

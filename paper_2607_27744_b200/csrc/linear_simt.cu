@@ -1,5 +1,5 @@
 // Linear layer on the CUDA cores (Eq. 4 / Eq. 14):
-//     Y[i, n] = act( sum_k X[i, k] W[n, k] + bias[n] + add[row2req[i], n] )
+//     Y[i, n] = act( sum_k X[i, k] W[n, k] + bias[n] + add[map.of(i), n] )
 // in fp32 FMA on fp32 or bf16 storage: the fp32 path, and bf16 shapes the tensor-core kernels do not take.
 //
 // A block computes a BM x BN tile.  Its threads form KS groups of 64 (8 x 8 threads, TM x TN outputs each)
@@ -71,9 +71,10 @@ template <typename TIn, typename TOut, int TM, int TN, int KS>
 __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kernel(
     int64_t M, int32_t d_in, int32_t d_out, const TIn* __restrict__ X, int64_t ld_x, const TIn* __restrict__ W,
     int64_t ld_w, const float* __restrict__ bias, const float* __restrict__ add, int64_t ld_add,
-    const int32_t* __restrict__ row2req, int act, TOut* __restrict__ Y, int64_t ld_y) {
+    const RequestMap map, int act, TOut* __restrict__ Y, int64_t ld_y) {
   constexpr int BM = 8 * TM, BN = 8 * TN;
   extern __shared__ __align__(16) float sm[];
+  __shared__ int32_t req[BM];  // request of each row of the tile
   const int group = threadIdx.x / kGroup, t = threadIdx.x % kGroup;
   const int tx = t % 8, ty = t / 8;
   const int64_t m0 = (int64_t)blockIdx.x * BM;
@@ -123,6 +124,7 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
         }
     }
   }
+  if (add && threadIdx.x < BM && m0 + threadIdx.x < M) req[threadIdx.x] = map.of(m0 + threadIdx.x);
   cp_async_wait<0>();
   __syncthreads();  // the rings become the groups' partial tiles
   float* part = sm + group * BM * BN;
@@ -139,7 +141,7 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
 #pragma unroll
     for (int g = 1; g < KS; ++g) v += sm[g * BM * BN + e];
     if (bias) v += bias[n];
-    if (add) v += add[(int64_t)(row2req ? row2req[m] : m) * ld_add + n];
+    if (add) v += add[(int64_t)req[e / BN] * ld_add + n];
     if (act == ROCS_ACT_RELU) v = fmaxf(v, 0.f);
     st_f(Y + m * ld_y + n, v);
   }
@@ -148,7 +150,7 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
 template <typename TIn, typename TOut>
 rocs_status_t launch_linear(int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x, const void* W,
                             int64_t ld_w, const float* bias, const float* add, int64_t ld_add,
-                            const int32_t* row2req, int act, void* Y, int64_t ld_y, cudaStream_t stream) {
+                            const RequestMap& map, int act, void* Y, int64_t ld_y, cudaStream_t stream) {
   if (M == 0 || d_out == 0) return ROCS_OK;
   auto tiles = [&](int b) { return ((M + b - 1) / b) * ((d_out + b - 1) / b); };
 #define ROCS_LAUNCH(T_, KS_)                                                                                         \
@@ -157,7 +159,7 @@ rocs_status_t launch_linear(int64_t M, int32_t d_in, int32_t d_out, const void* 
     auto kernel = linear_simt_kernel<TIn, TOut, T_, T_, KS_>;                                                        \
     ROCS_ALLOW_SMEM(kernel, smem);                                                                                   \
     kernel<<<dim3((unsigned)((M + 8 * T_ - 1) / (8 * T_)), (unsigned)((d_out + 8 * T_ - 1) / (8 * T_))), kGroup * KS_, \
-             smem, stream>>>(M, d_in, d_out, (const TIn*)X, ld_x, (const TIn*)W, ld_w, bias, add, ld_add, row2req,   \
+             smem, stream>>>(M, d_in, d_out, (const TIn*)X, ld_x, (const TIn*)W, ld_w, bias, add, ld_add, map,       \
                              act, (TOut*)Y, ld_y);                                                                   \
   } while (0)
   if (tiles(64) >= 296) ROCS_LAUNCH(8, 2);
@@ -172,14 +174,14 @@ rocs_status_t launch_linear(int64_t M, int32_t d_in, int32_t d_out, const void* 
 
 rocs_status_t simt_linear(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x,
                           const void* W, int64_t ld_w, const float* bias, const float* add, int64_t ld_add,
-                          const int32_t* row2req, int act, void* Y, int64_t ld_y, bool out_f32, cudaStream_t stream) {
+                          const RequestMap& map, int act, void* Y, int64_t ld_y, bool out_f32, cudaStream_t stream) {
   if (dt == ROCS_F32)
-    return launch_linear<float, float>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act, Y, ld_y,
+    return launch_linear<float, float>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y,
                                        stream);
   if (out_f32)
-    return launch_linear<__nv_bfloat16, float>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act, Y,
+    return launch_linear<__nv_bfloat16, float>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y,
                                                ld_y, stream);
-  return launch_linear<__nv_bfloat16, __nv_bfloat16>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act,
+  return launch_linear<__nv_bfloat16, __nv_bfloat16>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act,
                                                      Y, ld_y, stream);
 }
 

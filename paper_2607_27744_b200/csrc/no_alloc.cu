@@ -58,12 +58,12 @@ bool stride_ok(int64_t ld, int64_t cols, rocs_dtype_t dt) {
 
 rocs_status_t run_linear(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x,
                          const void* W, int64_t ld_w, const float* bias, const float* add, int64_t ld_add,
-                         const int32_t* row2req, int act, void* Y, int64_t ld_y, bool out_f32,
+                         const RequestMap& map, int act, void* Y, int64_t ld_y, bool out_f32,
                          cudaStream_t stream, int64_t add_rows = 0) {
   if (dt == ROCS_BF16 && umma_linear_supported(M, d_in, d_out, ld_x, ld_w, ld_y, out_f32))
-    return umma_linear(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act, Y, ld_y, out_f32,
+    return umma_linear(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y, out_f32,
                        stream, false, nullptr, add_rows);
-  return simt_linear(dt, M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act, Y, ld_y, out_f32,
+  return simt_linear(dt, M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y, out_f32,
                      stream);
 }
 
@@ -103,10 +103,10 @@ rocs_status_t rocs_ikbo_linear_static(rocs_dtype_t dtype, int32_t R, int64_t N, 
   // 0..R-1, map entries 0..N-1), so nothing left behind by an earlier call is ever consumed.
   static_row2req_kernel<<<(unsigned)((N + 255) / 256), 256, 0, stream>>>(R, N, cand_offsets);
   ROCS_CUDA_TRY(cudaGetLastError());
-  st = run_linear(dtype, R, d_req, d_out, XR, ld_xr, W_CR, ld_wcr, bias, nullptr, 0, nullptr, ROCS_ACT_NONE, Z,
+  st = run_linear(dtype, R, d_req, d_out, XR, ld_xr, W_CR, ld_wcr, bias, nullptr, 0, RequestMap{}, ROCS_ACT_NONE, Z,
                   d_out, /*out_f32=*/true, stream);
   if (st != ROCS_OK) return st;
-  return run_linear(dtype, N, d_cand, d_out, XC, ld_xc, W_CC, ld_wcc, nullptr, Z, d_out, map, act, Y, ld_y,
+  return run_linear(dtype, N, d_cand, d_out, XC, ld_xc, W_CC, ld_wcc, nullptr, Z, d_out, RequestMap{map, nullptr, 0}, act, Y, ld_y,
                     /*out_f32=*/false, stream, R);
 }
 

@@ -94,8 +94,29 @@ inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // Tiles of at most `cands_per_tile` candidates that the batch's requests are cut into.
 int64_t plan_entries(const rocs_plan* plan, int32_t cands_per_tile);
 
-// m_i of Section 4.1, int32 [N] on the device; made on first use.
-rocs_status_t plan_row2req(const rocs_plan* plan, cudaStream_t stream, const int32_t** out);
+// m_i of Section 4.1: a table of all rows, or the offsets to search in; neither: row i is its own request.
+struct RequestMap {
+  const int32_t* row2req = nullptr;  // [N]
+  const int32_t* offsets = nullptr;  // [R + 1]
+  int32_t R = 0;
+#ifdef __CUDACC__
+  __device__ __forceinline__ int32_t of(int64_t row) const {
+    if (row2req != nullptr) return row2req[row];
+    if (offsets == nullptr) return (int32_t)row;
+    int32_t lo = 0, hi = R;  // largest r with offsets[r] <= row
+    while (hi - lo > 1) {
+      const int32_t mid = lo + (hi - lo) / 2;
+      if (offsets[mid] <= row) lo = mid; else hi = mid;
+    }
+    return lo;
+  }
+#endif
+};
+// Up to this many candidates the kernels search for a row's request themselves: the table is a launch of its own
+// in front of them (about 2 us of a 24 us tower on 500 candidates, and host time), the search a handful of
+// cached loads per row; with more rows the loads add up and the launch does not.
+constexpr int64_t kSearchRows = 16384;
+rocs_status_t plan_request_map(const rocs_plan* plan, cudaStream_t stream, RequestMap* out);
 
 // Returns the cached tile list for `cands_per_tile`, building it on first use.
 rocs_status_t plan_tiles(const rocs_plan* plan, int32_t cands_per_tile, cudaStream_t stream,
@@ -106,11 +127,11 @@ rocs_status_t plan_dca_items(const rocs_plan* plan, int32_t cands_per_tile, int3
                              DcaItemList* out);
 
 // ---- general (CUDA-core) kernels: simt_kernels.cu -------------------------------------
-// Y[i, :] = act(add[row2req ? row2req[i] : -, :] + X[i, :] W^T + bias).  out_f32 selects an
+// Y[i, :] = act(add[map.of(i), :] + X[i, :] W^T + bias).  out_f32 selects an
 // fp32 output regardless of the storage type (used for the request half Z).
 rocs_status_t simt_linear(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_out, const void* X,
                           int64_t ld_x, const void* W, int64_t ld_w, const float* bias,
-                          const float* add, int64_t ld_add, const int32_t* row2req, int act,
+                          const float* add, int64_t ld_add, const RequestMap& map, int act,
                           void* Y, int64_t ld_y, bool out_f32, cudaStream_t stream);
 rocs_status_t simt_dca(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh,
                        float scale, const void* Q, const void* K, const void* V,
@@ -141,7 +162,7 @@ bool umma_linear_supported(int64_t M, int32_t d_in, int32_t d_out, int64_t ld_x,
 // set-up with that launch and waits for it only before it reads `add`.
 rocs_status_t umma_linear(int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x,
                           const void* W, int64_t ld_w, const float* bias, const float* add,
-                          int64_t ld_add, const int32_t* row2req, int act, void* Y, int64_t ld_y,
+                          int64_t ld_add, const RequestMap& map, int act, void* Y, int64_t ld_y,
                           bool out_f32, cudaStream_t stream, bool add_from_previous_launch = false,
                           float2* stat_partials = nullptr, int64_t add_rows = 0);
 // Weight-stationary kernel on CTA pairs (cta_group::2) for d_in <= 256 and bf16 output: half a weight
@@ -149,7 +170,7 @@ rocs_status_t umma_linear(int64_t M, int32_t d_in, int32_t d_out, const void* X,
 bool umma_linear_ws2_supported(int64_t M, int32_t d_in, int32_t d_out, bool out_f32);
 rocs_status_t umma_linear_ws2(int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x,
                               const void* W, int64_t ld_w, const float* bias, const float* add,
-                              int64_t ld_add, const int32_t* row2req, int act, void* Y, int64_t ld_y,
+                              int64_t ld_add, const RequestMap& map, int act, void* Y, int64_t ld_y,
                               cudaStream_t stream, bool add_from_previous_launch = false,
                               float2* stat_partials = nullptr, int64_t add_rows = 0);
 // Number of (sum, sum of squares) partials per row the kernel above writes when asked to.

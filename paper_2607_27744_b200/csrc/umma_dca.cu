@@ -261,6 +261,11 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
   const uint32_t tmem_base = *reinterpret_cast<const uint32_t*>(smem + kOffTmemPtr);
   // launched as a programmatic dependent: the set-up above may overlap the end of the kernel in front;
   // global memory is touched only from here on, and the kernel behind this one is released after the wait
+  if (warp == kControlWarp0 && lane == 0) {  // parameters of the launch: no need to wait
+    prefetch_tensormap(&map_q);
+    prefetch_tensormap(&map_k);
+    prefetch_tensormap(&map_v);
+  }
   griddep_wait();
   griddep_launch_dependents();
   const int32_t row_width = p.H * DH;  // elements per query / key row over all heads
@@ -281,11 +286,6 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     auto wait = [&](uint32_t bar, uint32_t parity, uint32_t code) {  // the same answer for the whole warp
       return __all_sync(0xffffffffu, mbar_wait_paced(bar, parity, abort_flag, p.status, kStatusDca | code)) != 0;
     };
-    if (lane == 0) {
-      prefetch_tensormap(&map_q);
-      prefetch_tensormap(&map_k);
-      prefetch_tensormap(&map_v);
-    }
     // The last block of a sequence may reach past it into the next request's rows (or past the
     // tensor, where TMA fills zeros).  Scores of such keys are masked to -inf by the softmax warps,
     // so P is exactly 0 there; the V rows are zeroed here so that 0 x (Inf or NaN of a foreign

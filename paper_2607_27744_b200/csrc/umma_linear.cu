@@ -1,5 +1,5 @@
 // Linear layer on the 5th-generation tensor cores (Eq. 4 / Eq. 14):
-//     Y[i, n] = act( sum_k X[i, k] W[n, k] + bias[n] + add[row2req[i], n] )
+//     Y[i, n] = act( sum_k X[i, k] W[n, k] + bias[n] + add[map.of(i), n] )
 // `add` is the request half Z of the split layer; it is gathered per output row in the epilogue
 // through the candidate->request map (the in-kernel broadcast of Section 4.2.1), so the broadcast
 // tensor never exists.
@@ -45,8 +45,10 @@ struct LinearParams {
   const float* bias;
   const float* add;
   int64_t ld_add;
-  const int32_t* row2req;
+  RequestMap map;
   int32_t act;
+  int32_t x_rows;     // rows of an X tile that are loaded
+  int32_t wait_late;  // `add` is written by the launch in front and nothing else this kernel reads is
   uint32_t* status;
 };
 
@@ -101,14 +103,21 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   // (the candidate half behind the request half) may begin its own set-up; it waits for this grid before
   // it reads our output, and since it is released only after the wait above, everything in front of this
   // kernel is complete by the time it starts.
-  griddep_wait();
-  griddep_launch_dependents();
+  if (warp == 0 && lane == 0) {  // parameters of the launch: no need to wait
+    prefetch_tensormap(&map_x);
+    prefetch_tensormap(&map_w);
+    prefetch_tensormap(&map_y);
+  }
+  // A candidate half in front of which only the request half is still running streams X and W at once; its
+  // epilogue waits.
+  if (!p.wait_late) {
+    griddep_wait();
+    griddep_launch_dependents();
+  }
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------------------
     if (elect_one()) {
-      prefetch_tensormap(&map_x);
-      prefetch_tensormap(&map_w);
       uint32_t it = 0;
       bool ok = true;
       for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
@@ -118,7 +127,7 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           const uint32_t ph = (it / kStages) & 1;
           if (!mbar_wait(&empty[s], ph ^ 1, abort_flag, p.status, kStatusLinear | 1)) { ok = false; break; }
           uint8_t* a = smem + s * Cfg::kStageBytes;
-          mbar_expect_tx(&full[s], Cfg::kStageBytes);
+          mbar_expect_tx(&full[s], p.x_rows * (BK * 2) + Cfg::kBBytes);
           tma_load_2d(a, &map_x, &full[s], kb * BK, m0);
           tma_load_2d(a + Cfg::kABytes, &map_w, &full[s], kb * BK, n0);
         }
@@ -171,13 +180,17 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     uint8_t* my_stage = staging + (warp - 2) * 8192;
     uint32_t lt = 0, stores = 0;
     bool ok = true;
+    if (p.wait_late) {
+      griddep_wait();
+      griddep_launch_dependents();
+    }
     for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++lt) {
       const uint32_t acc = lt & 1;
       const int32_t m0 = (int32_t)(t / n_tiles) * BM, n0 = (int32_t)(t % n_tiles) * BN;
       const int64_t row = (int64_t)m0 + q * 32 + lane;
       const float* add_row = nullptr;
       if (p.add != nullptr && row < p.M)
-        add_row = p.add + (int64_t)(p.row2req ? p.row2req[row] : row) * p.ld_add;
+        add_row = p.add + (int64_t)p.map.of(row) * p.ld_add;
       if (!mbar_wait(&tmem_full[acc], (lt >> 1) & 1, abort_flag, p.status, kStatusLinear | 4)) { ok = false; break; }
       tc_fence_after_sync();
       const uint32_t t_row = tmem_base + acc * BN + ((uint32_t)(q * 32) << 16);
@@ -278,13 +291,17 @@ int sm_count() {
 
 template <int BN, typename OutT>
 rocs_status_t launch(int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x, const void* W,
-                     int64_t ld_w, const float* bias, const float* add, int64_t ld_add, const int32_t* row2req,
-                     int act, void* Y, int64_t ld_y, cudaStream_t stream) {
+                     int64_t ld_w, const float* bias, const float* add, int64_t ld_add, const RequestMap& map,
+                     int act, void* Y, int64_t ld_y, cudaStream_t stream, bool wait_late) {
   using Cfg = LinearCfg<BN>;
   constexpr int CH = 128 / (int)sizeof(OutT);
+  // A batch of fewer rows than a tile loads no more than it has: the loads of a small batch, 64 bytes per clock and
+  // SM whatever they bring, are its time (K = 1024 on one row: 408 cycles per 64-deep block with 128 rows of X and
+  // 64 of W).  The other rows of the operand hold whatever the buffer held; so do their outputs, which are not stored.
+  const int32_t x_rows = (int32_t)std::min<int64_t>(BM, (M + 7) / 8 * 8);
   CUtensorMap map_x, map_w, map_y;
   if (!make_tensor_map_2d(&map_x, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)M, (uint64_t)d_in, (uint64_t)ld_x,
-                          BM, BK, true) ||
+                          (uint32_t)x_rows, BK, true) ||
       !make_tensor_map_2d(&map_w, W, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_out, (uint64_t)d_in,
                           (uint64_t)ld_w, BN, BK, true) ||
       !make_tensor_map_2d(&map_y, Y, sizeof(OutT) == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
@@ -296,7 +313,7 @@ rocs_status_t launch(int64_t M, int32_t d_in, int32_t d_out, const void* X, int6
   ROCS_ALLOW_SMEM(kernel, Cfg::kSmemBytes);
   const int64_t tiles = ((M + BM - 1) / BM) * ((d_out + BN - 1) / BN);
   const int grid = (int)std::min<int64_t>(tiles, sm_count());
-  LinearParams p{M, d_in, d_out, bias, add, ld_add, row2req, act, status};
+  LinearParams p{M, d_in, d_out, bias, add, ld_add, map, act, x_rows, wait_late ? 1 : 0, status};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kThreads);
@@ -325,20 +342,21 @@ bool umma_linear_supported(int64_t M, int32_t d_in, int32_t d_out, int64_t ld_x,
 
 rocs_status_t umma_linear(int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x, const void* W,
                           int64_t ld_w, const float* bias, const float* add, int64_t ld_add,
-                          const int32_t* row2req, int act, void* Y, int64_t ld_y, bool out_f32,
+                          const RequestMap& map, int act, void* Y, int64_t ld_y, bool out_f32,
                           cudaStream_t stream, bool add_from_previous_launch, float2* stat_partials,
                           int64_t add_rows) {
   if (umma_linear_ws2_supported(M, d_in, d_out, out_f32))
-    return umma_linear_ws2(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act, Y, ld_y, stream,
+    return umma_linear_ws2(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y, stream,
                            add_from_previous_launch, stat_partials, add_rows);
   if (stat_partials != nullptr) return ROCS_ERR_UNSUPPORTED;  // the caller asks for them only where the kernel above applies
   if (umma_linear_pair_supported(M, d_in, d_out, out_f32, add != nullptr))
     return umma_linear_pair(M, d_in, d_out, X, ld_x, W, ld_w, bias, act, Y, ld_y, stream);
-#define ROCS_LAUNCH(BN_)                                                                                   \
-  (out_f32 ? launch<BN_, float>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act, Y, ld_y, \
-                                stream)                                                                    \
-           : launch<BN_, __nv_bfloat16>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, row2req, act, Y, \
-                                        ld_y, stream))
+  const bool wait_late = add_from_previous_launch && add != nullptr;
+#define ROCS_LAUNCH(BN_)                                                                                              \
+  (out_f32 ? launch<BN_, float>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y, stream,       \
+                                wait_late)                                                                           \
+           : launch<BN_, __nv_bfloat16>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y, stream, \
+                                        wait_late))
   // Widest tile that still gives every SM something to do: a small batch (the request half at
   // batch size R) is spread over more, narrower tiles instead of leaving most SMs idle.
   const int64_t m_tiles = (M + BM - 1) / BM;

@@ -32,7 +32,7 @@ constexpr uint32_t kStatusPair = 0x300;
 
 struct PairParams {
   int64_t M;
-  int32_t d_in, d_out;
+  int32_t d_in, d_out, bn;  // bn: output columns per tile, 128, 192 or 256
   const float* bias;
   int32_t act;
   uint32_t* status;
@@ -63,7 +63,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   const uint32_t rank = cluster_ctarank();
   const int32_t pair = blockIdx.x / 2, pairs = gridDim.x / 2;
   const int32_t super_tiles = (int32_t)((p.M + 2 * BM - 1) / (2 * BM));
-  const int32_t n_tiles = (p.d_out + BN - 1) / BN;
+  const int32_t n_tiles = (p.d_out + p.bn - 1) / p.bn;
   const int32_t k_blocks = (p.d_in + BK - 1) / BK;
   const int64_t num_tiles = (int64_t)super_tiles * n_tiles;
 
@@ -92,23 +92,26 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   // kernel in front of this one on the stream finishes; nothing below touches global memory before that
   // kernel is complete.  The next kernel on the stream is released only after this wait, so whatever
   // it may assume about its predecessors holds transitively.
+  if (warp == 0 && lane == 0) {  // parameters of the launch: no need to wait
+    prefetch_tensormap(&map_x);
+    prefetch_tensormap(&map_w);
+    prefetch_tensormap(&map_y);
+  }
   griddep_wait();
   griddep_launch_dependents();
 
   if (warp == 0) {
     // ------------------------------ TMA producer (both CTAs) -------------------------------
     if (elect_one()) {
-      prefetch_tensormap(&map_x);
-      prefetch_tensormap(&map_w);
       uint32_t it = 0;
       bool ok = true;
       for (int64_t t = pair; t < num_tiles && ok; t += pairs) {
         const int32_t m0 = (int32_t)(t / n_tiles) * 2 * BM + (int32_t)rank * BM;
-        const int32_t n0 = (int32_t)(t % n_tiles) * BN + (int32_t)rank * (BN / 2);
+        const int32_t n0 = (int32_t)(t % n_tiles) * p.bn + (int32_t)rank * (p.bn / 2);
         for (int32_t kb = 0; kb < k_blocks; ++kb, ++it) {
           const int s = it % kStages;
           if (!mbar_wait(&empty[s], ((it / kStages) & 1) ^ 1, abort_flag, p.status, kStatusPair | 1)) { ok = false; break; }
-          if (rank == 0) mbar_expect_tx(&full[s], 2 * kStageBytes);  // both CTAs' bytes land on the leader's barrier
+          if (rank == 0) mbar_expect_tx(&full[s], 2 * kABytes + p.bn * (BK * 2));  // both CTAs' bytes land on the leader's barrier
           const uint32_t full_leader = map_to_cta(smem_u32(&full[s]), 0);
           uint8_t* st = smem + s * kStageBytes;
           tma_load_2d_pair(st, &map_x, full_leader, kb * BK, m0);
@@ -123,7 +126,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   } else if (warp == 1) {
     // ------------------------------ MMA issuer (leader CTA only) ---------------------------
     if (rank == 0 && elect_one()) {
-      constexpr uint32_t idesc = umma_idesc_bf16(2 * BM, BN, false, false);
+      const uint32_t idesc = umma_idesc_bf16(2 * BM, (uint32_t)p.bn, false, false);
       uint32_t it = 0, lt = 0;
       bool ok = true;
       for (int64_t t = pair; t < num_tiles && ok; t += pairs, ++lt) {
@@ -162,12 +165,12 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     for (int64_t t = pair; t < num_tiles; t += pairs, ++lt) {
       const uint32_t acc = lt & 1;
       const int32_t m0 = (int32_t)(t / n_tiles) * 2 * BM + (int32_t)rank * BM;
-      const int32_t n0 = (int32_t)(t % n_tiles) * BN;
+      const int32_t n0 = (int32_t)(t % n_tiles) * p.bn;
       if (!mbar_wait(&tmem_full[acc], (lt >> 1) & 1, abort_flag, p.status, kStatusPair | 4)) break;
       tc_fence_after_sync();
       if (elect_one()) tma_store_wait_read<0>();  // the previous tile's stores have read this warp's boxes
       __syncwarp();
-      const uint32_t t_row = tmem_base + acc * BN + half * 128 + ((uint32_t)(q * 32) << 16);
+      const uint32_t t_row = tmem_base + acc * BN + half * 64 + ((uint32_t)(q * 32) << 16);
       float sc = 1.f, sh = 0.f;
       if (p.in_stats != nullptr) {
         const int64_t row = (int64_t)m0 + q * 32 + lane;
@@ -182,12 +185,15 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       }
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
-        const int32_t col0 = n0 + half * 128 + c * 64;
+        // chunks of 64 columns: half, half + 2 (the second of them only in tiles that are wide enough)
+        if (half * 64 + c * 128 >= p.bn) break;
+        const bool last = half * 64 + (c + 1) * 128 >= p.bn;
+        const int32_t col0 = n0 + half * 64 + c * 128;
         uint32_t v[64];
-        tmem_ld_32x32b_x32(t_row + c * 64, v);
-        tmem_ld_32x32b_x32(t_row + c * 64 + 32, v + 32);
+        tmem_ld_32x32b_x32(t_row + c * 128, v);
+        tmem_ld_32x32b_x32(t_row + c * 128 + 32, v + 32);
         tmem_ld_wait();
-        if (c == 1) {
+        if (last) {
           tc_fence_before_sync();
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster_relaxed(tmem_empty_leader[acc]);
@@ -280,17 +286,31 @@ bool umma_linear_pair_supported(int64_t M, int32_t d_in, int32_t d_out, bool out
 rocs_status_t umma_linear_pair(int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x, const void* W,
                                int64_t ld_w, const float* bias, int act, void* Y, int64_t ld_y, cudaStream_t stream,
                                const RowNorm* norm) {
+  // Columns per tile: the pairs work in rounds, and a round takes about as long as its loads, 128 + bn / 2 rows per
+  // CTA and K block.  Narrower tiles pay where they fill the rounds better (4866 rows x 1024 columns: two rounds of
+  // 192 columns and not of 256; x 256 columns: one round of 128 on 80 CTAs and not of 256 on 40).
+  const int64_t row_tiles = (M + 2 * BM - 1) / (2 * BM);
+  int32_t bn = BN;
+  int64_t best = INT64_MAX;
+  for (int32_t b = BN; b >= 128; b -= 64) {
+    const int64_t t = row_tiles * ((d_out + b - 1) / b);
+    const int64_t cost = (t + sm_count_pair() / 2 - 1) / (sm_count_pair() / 2) * (128 + b / 2);
+    if (cost < best) {
+      best = cost;
+      bn = b;
+    }
+  }
   CUtensorMap map_x, map_w, map_y;
   if (!make_tensor_map_2d(&map_x, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)M, (uint64_t)d_in, (uint64_t)ld_x,
                           BM, BK, true) ||
       !make_tensor_map_2d(&map_w, W, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_out, (uint64_t)d_in,
-                          (uint64_t)ld_w, BN / 2, BK, true) ||
+                          (uint64_t)ld_w, (uint32_t)bn / 2, BK, true) ||
       !make_tensor_map_2d(&map_y, Y, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)M, (uint64_t)d_out, (uint64_t)ld_y,
                           32, 64, true))
     return ROCS_ERR_CUDA;
   uint32_t* status = device_status_word();
   if (!status) return ROCS_ERR_CUDA;
-  PairParams p{M, d_in, d_out, bias, act, status, nullptr, nullptr, 0, 0.f, 0.f};
+  PairParams p{M, d_in, d_out, bn, bias, act, status, nullptr, nullptr, 0, 0.f, 0.f};
   if (norm != nullptr) {
     p.in_stats = norm->row_stats;
     p.wbar = norm->wbar;
@@ -298,7 +318,7 @@ rocs_status_t umma_linear_pair(int64_t M, int32_t d_in, int32_t d_out, const voi
     p.eps = norm->eps;
     p.inv_d = 1.f / (float)d_in;
   }
-  const int64_t tiles = ((M + 2 * BM - 1) / (2 * BM)) * ((d_out + BN - 1) / BN);
+  const int64_t tiles = row_tiles * ((d_out + bn - 1) / bn);
   const int pairs = (int)std::min<int64_t>(tiles, sm_count_pair() / 2);
   ROCS_ALLOW_SMEM(linear_pair_kernel, kSmemBytes);
   cudaLaunchConfig_t cfg = {};

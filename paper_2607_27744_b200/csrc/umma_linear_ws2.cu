@@ -48,7 +48,7 @@ struct Ws2Params {
   const float* bias;
   const float* add;
   int64_t ld_add;
-  const int32_t* row2req;
+  RequestMap map;
   int32_t act;
   int32_t wait_for_previous;  // launched with programmatic serialization behind the kernel that writes `add`
   float2* stat_partials;      // [M][2 n_slices] (sum, sum of squares) of each row's 128 columns per epilogue warp, or NULL
@@ -113,6 +113,12 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     tmem_alloc_pair(tmem_ptr, 2 * BN);
     tmem_relinquish_pair();
   }
+  if (warp == 0 && lane == 0) {
+    prefetch_tensormap(&map_x);
+    prefetch_tensormap(&map_w);
+    prefetch_tensormap(&map_z);
+    prefetch_tensormap(&map_y);
+  }
   tc_fence_before_sync();
   cluster_sync_all();  // barriers of both CTAs are initialised before anything signals across the pair
   tc_fence_after_sync();
@@ -124,8 +130,6 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   if (warp == 0) {
     // ------------------------------ TMA producer (both CTAs) -------------------------------
     if (elect_one()) {
-      prefetch_tensormap(&map_x);
-      prefetch_tensormap(&map_w);
       const uint32_t w_full_leader = map_to_cta(smem_u32(w_full), 0);
       if (rank == 0) mbar_expect_tx(w_full, 2 * k_blocks * kWBlockBytes);
       for (int32_t kb = 0; kb < k_blocks; ++kb)
@@ -138,7 +142,7 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int64_t r0 = min((int64_t)st_ * 2 * BM + (int64_t)rank * BM + q * 32, p.M - 1);
-          req_next[q] = p.row2req ? p.row2req[r0] : (int32_t)r0;
+          req_next[q] = p.map.of(r0);
         }
       };
       if (has_add && group < super_tiles) fetch_req(group);
@@ -219,7 +223,7 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       bool uniform = false;
       if (has_add) {
         const int64_t rc = max((int64_t)0, min(row, p.M - 1));
-        const int32_t my_req = p.row2req ? p.row2req[rc] : (int32_t)rc;
+        const int32_t my_req = p.map.of(rc);
         const int32_t slab_req = __shfl_sync(0xffffffffu, my_req, 0);
         uniform = __all_sync(0xffffffffu, my_req == slab_req);
         // shared-memory copy when this row belongs to the slab's first request, global otherwise
@@ -346,7 +350,7 @@ bool umma_linear_ws2_supported(int64_t M, int32_t d_in, int32_t d_out, bool out_
 
 rocs_status_t umma_linear_ws2(int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x, const void* W,
                               int64_t ld_w, const float* bias, const float* add, int64_t ld_add,
-                              const int32_t* row2req, int act, void* Y, int64_t ld_y, cudaStream_t stream,
+                              const RequestMap& map, int act, void* Y, int64_t ld_y, cudaStream_t stream,
                               bool add_from_previous_launch, float2* stat_partials, int64_t add_rows) {
   const int32_t k_blocks = (d_in + BK - 1) / BK;
   CUtensorMap map_x, map_w, map_z, map_y;
@@ -374,7 +378,7 @@ rocs_status_t umma_linear_ws2(int64_t M, int32_t d_in, int32_t d_out, const void
   p.groups = std::max(1, std::min(super_tiles, (sm_count_ws2() / 2) / p.n_slices));
   const int fixed = k_blocks * kWBlockBytes + kStagingBytes + kZBufs * kZBufBytes + 512 + 1024;
   p.a_stages = std::min(10, (227 * 1024 - fixed) / kAStageBytes);
-  p.bias = bias; p.add = add; p.ld_add = ld_add; p.row2req = row2req; p.act = act; p.status = status;
+  p.bias = bias; p.add = add; p.ld_add = ld_add; p.map = map; p.act = act; p.status = status;
   p.wait_for_previous = (add_from_previous_launch && add != nullptr) ? 1 : 0;
   p.stat_partials = stat_partials;
   const int smem_bytes = fixed + p.a_stages * kAStageBytes;

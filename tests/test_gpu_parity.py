@@ -121,6 +121,28 @@ def test_linear_general_kernel_tiles(dtype, M, d_in, d_out):
     assert rel_err(to_host_f64(Y), want) <= tol_for(dtype)
 
 
+@pytest.mark.parametrize("M,d_out", [(2048, 256), (4866, 1024), (4866, 256), (2305, 520), (9000, 456)])
+def test_plain_linear_tile_widths(M, d_out):
+    # 128, 192 and 256 columns per tile of the CTA-pair kernel, with and without a partial last tile
+    g = np.random.default_rng(M + d_out)
+    X = wl.store(g.standard_normal((M, 136), dtype=np.float32), "bf16")
+    W = wl.store(g.standard_normal((d_out, 136), dtype=np.float32) * 136 ** -0.5, "bf16")
+    b = g.standard_normal(d_out).astype(np.float32)
+    y = rocs.linear(to_dev(X), to_dev(W), bias=to_dev(b), relu=True)
+    want = ref.ikbo_linear(wl.offsets_from_counts([M]), None, X, W, bias=b, relu=True)
+    assert rel_err(to_host_f64(y), want) <= tol_for("bf16")
+
+
+@pytest.mark.parametrize("N", [1, 7, 9, 127, 129, 500, 511, 16384, 16385])
+def test_linear_few_rows_and_both_request_maps(N):
+    # X tiles of fewer than 128 rows, the candidate half that waits for the request half in its epilogue only
+    # (below 512 rows), the request searched in the offsets (up to 16384 rows) or read from the table
+    counts = [0, N // 3, 1, 0, N - N // 3 - 1, 0] if N > 1 else [0, 1]
+    co = wl.offsets_from_counts(counts)
+    cfg = wl.CONFIGS[2].with_(R=len(counts), d_req=136, d_cand=320 if N < 512 else 72, d_out=192)
+    assert _run_linear(cfg, co, bias=True, relu=True) <= tol_for("bf16")
+
+
 def test_linear_empty_batch():
     co = np.zeros(3, np.int32)
     cfg = wl.CONFIGS[2].with_(R=2, d_req=64, d_cand=64, d_out=64)
