@@ -303,6 +303,33 @@ def test_dca_bf16_head_dim_32_and_128_ragged_on_tensor_cores(dh):
 
 
 @pytest.mark.parametrize("dh", [32, 64, 128])
+@pytest.mark.parametrize("R,n,H,L", [(1, 7, 1, 2048), (2, 300, 2, 1500), (3, 129, 4, 1030), (5, 200, 8, 700), (9, 100, 16, 400),
+                                     (300, 0, 1, 600), (1, 5, 2, 4000)])
+def test_dca_bf16_items_split_along_their_keys(dh, R, n, H, L):
+    # clusters of 8, 4, 2 and 1 CTAs, sequences shorter than the batch's average (sides without keys), a request
+    # without keys and one without candidates, more requests than a warp has lanes, item list and item search;
+    # scores that outgrow the reference of one part only, of all rows but one
+    g = np.random.default_rng(R * 7 + n)
+    counts = [n if n else int(r % 97 == 5) for r in range(R)]
+    lens = [L if r == 0 else int(g.integers(0, 2 * L)) for r in range(R)]
+    if R > 2:
+        counts[1], lens[2] = 0, 0
+    if R > 3:
+        lens[3] = 17
+    co, so = wl.offsets_from_counts(counts), wl.offsets_from_counts(lens)
+    cfg = wl.CONFIGS[3].with_(R=R, H=H, dh=dh)
+    assert _run_dca(cfg, co, so) <= tol_for("bf16")
+    d = wl.dca_inputs(cfg, co, so)
+    if lens[0] > 300 and counts[0] > 4:
+        K = wl.bf16_bits_to_f32(d["K"]).copy()
+        K[290] = wl.bf16_bits_to_f32(d["Q"])[3, 0] * 60.0
+        d["K"] = wl.f32_to_bf16_bits(K)
+        want = ref.dca_attention(co, so, d["Q"], d["K"], d["V"])
+        O = rocs.dca_attention(_plan(co), to_dev(d["Q"]), to_dev(d["K"]), to_dev(d["V"]), to_dev(so))
+        assert rel_err(to_host_f64(O), want) <= tol_for("bf16")
+
+
+@pytest.mark.parametrize("dh", [32, 64, 128])
 def test_dca_bf16_short_last_blocks_between_empty_requests(dh):
     # products of the last key block end at a multiple of 16 keys, the rows of V between are zeroed behind the next
     # item's loads: every remainder class, items with no keys and with no ragged end in between, one item per side
