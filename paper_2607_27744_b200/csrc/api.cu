@@ -7,6 +7,7 @@
 #include <new>
 
 #include "rocs_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace rocs {
 namespace {
@@ -17,7 +18,8 @@ std::atomic<int> g_path{ROCS_PATH_AUTO};
 __global__ void fill_row2req_kernel(int32_t R, int64_t N, const int32_t* __restrict__ off,
                                     int32_t* __restrict__ row2req) {
   // the first layer's kernel may set itself up beside this one; it waits for this grid before it reads anything
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  ptx::griddep_wait_for(off);
+  ptx::griddep_launch_dependents();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   int32_t lo = 0, hi = R;  // largest r with off[r] <= i
@@ -139,6 +141,8 @@ __global__ void __launch_bounds__(kListThreads) expand_list_kernel(int32_t R, in
                                                                    const int32_t* __restrict__ base,
                                                                    void* __restrict__ out) {
   extern __shared__ int32_t pre[];
+  ptx::griddep_wait_for(off, base);
+  ptx::griddep_launch_dependents();
   if (base == nullptr) {
     scan_entries(R, cands_per_tile, off, pre);
     base = pre;
@@ -171,8 +175,11 @@ static rocs_status_t make_list(const rocs_plan* plan, int32_t cands_per_tile, in
   DeviceList list;
   if (plan->N > 0 && cands_per_tile == 0) {
     ROCS_CUDA_TRY(pool_alloc(&list.dev, sizeof(int32_t) * (size_t)plan->N, stream));
-    fill_row2req_kernel<<<(unsigned)((plan->N + 255) / 256), 256, 0, stream>>>(plan->R, plan->N, off,
-                                                                              static_cast<int32_t*>(list.dev));
+    if (launch_dependent(fill_row2req_kernel, dim3((unsigned)((plan->N + 255) / 256)), 256, 0, stream, plan->R, plan->N, off,
+                         static_cast<int32_t*>(list.dev)) != ROCS_OK) {
+      cudaFreeAsync(list.dev, stream);
+      return ROCS_ERR_CUDA;
+    }
   } else if (plan->N > 0) {
     const int32_t R = plan->R;
     const int64_t total = plan_entries(plan, cands_per_tile) * std::max(heads, 1);
@@ -191,19 +198,16 @@ static rocs_status_t make_list(const rocs_plan* plan, int32_t cands_per_tile, in
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(base_dev, base.data(), sizeof(int32_t) * base.size(), cudaMemcpyHostToDevice, stream);
     }
-    if (e == cudaSuccess)
-      expand_list_kernel<<<(unsigned)((total + kListThreads - 1) / kListThreads), kListThreads,
-                           base_dev ? 0 : sizeof(int32_t) * ((size_t)R + 1), stream>>>(
-          R, list.num, cands_per_tile, heads, off, base_dev, list.dev);
+    if (e == cudaSuccess &&
+        launch_dependent(expand_list_kernel, dim3((unsigned)((total + kListThreads - 1) / kListThreads)), kListThreads,
+                         base_dev ? 0 : sizeof(int32_t) * ((size_t)R + 1), stream, R, list.num, cands_per_tile, heads, off,
+                         base_dev, list.dev) != ROCS_OK)
+      e = cudaErrorUnknown;
     if (base_dev) cudaFreeAsync(base_dev, stream);
     if (e != cudaSuccess) {
       cudaFreeAsync(list.dev, stream);
       return ROCS_ERR_CUDA;
     }
-  }
-  if (cudaGetLastError() != cudaSuccess) {
-    if (list.dev) cudaFreeAsync(list.dev, stream);
-    return ROCS_ERR_CUDA;
   }
   *out = list;
   return ROCS_OK;

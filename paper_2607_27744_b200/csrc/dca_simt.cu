@@ -44,6 +44,8 @@ __global__ void __launch_bounds__(kThreads, DHP <= 64 ? 4 : DHP <= 128 ? 2 : 1) 
   float* ks = qs + kRows * S;          // [64][S]
   float* vs = ks + kKeys * S;          // [64][S]
   float* ps = vs + kKeys * S;          // [32][kPStride]
+  ptx::griddep_wait_for(Q, K, V, cand_offsets, items, seq_offsets);
+  ptx::griddep_launch_dependents();
   DcaItem item;
   if (items != nullptr) {
     item = items[blockIdx.x];
@@ -203,10 +205,8 @@ rocs_status_t launch(const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh, 
   auto kernel = dca_simt_kernel<T, DHP>;
   ROCS_ALLOW_SMEM(kernel, smem);
   const dim3 grid((unsigned)items.num, (unsigned)std::min<int64_t>(((int64_t)cands * n_q + kRows - 1) / kRows, 65535));
-  kernel<<<grid, kThreads, smem, stream>>>(n_q, H, dh, scale, (const T*)Q, (const T*)K, (const T*)V, plan->R, cands,
-                                           plan->cand_offsets, items.dev, seq_offsets, (T*)O);
-  ROCS_CUDA_TRY(cudaGetLastError());
-  return ROCS_OK;
+  return launch_dependent(kernel, grid, kThreads, smem, stream, n_q, H, dh, scale, (const T*)Q, (const T*)K, (const T*)V,
+                          plan->R, cands, plan->cand_offsets, (const DcaItem*)items.dev, seq_offsets, (T*)O);
 }
 
 template <typename T>

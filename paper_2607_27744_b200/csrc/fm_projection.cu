@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(256) fm_request_kernel(int32_t n_r, int32_t d,
   const int32_t r = blockIdx.x;
   // the candidate kernel may start now: it streams X^C on its own and waits for this grid only
   // before it reads TT
+  ptx::griddep_wait_for(XR, P);
   ptx::griddep_launch_dependents();
   rows_to_shared(XR + (int64_t)r * n_r * d, xr, n_r, d, ds);
   for (int e = threadIdx.x; e < n_r * k; e += blockDim.x) pr[e] = ld_f(P, e);
@@ -102,7 +103,10 @@ __global__ void __launch_bounds__(128) fm_candidate_simt_kernel(int32_t n_r, int
   float* ht = xc + (size_t)n_c * ds;  // [k, d + 1]
   float* pc = ht + (size_t)k * ds;    // [n_c, k]
   const int64_t i = blockIdx.x;
-  const int32_t r = map.of(i);
+  RequestMap requests = map;
+  ptx::griddep_wait_for(XC, P, TT, requests.row2req, requests.offsets);
+  ptx::griddep_launch_dependents();
+  const int32_t r = requests.of(i);
   for (int e = threadIdx.x; e < n_c * d; e += blockDim.x) xc[(e / d) * ds + e % d] = ld_f(XC, i * n_c * d + e);
   for (int e = threadIdx.x; e < n_c * k; e += blockDim.x) pc[e] = ld_f(P, (int64_t)n_r * k + e);
   __syncthreads();
@@ -181,6 +185,7 @@ __global__ void __launch_bounds__(256) fm_request_mma_kernel(int32_t n_r, int32_
   uint8_t* tl = th + (size_t)kp * x_row;     // [kp][d + 8] bf16: what the rounding left
   const int32_t r = blockIdx.x;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  ptx::griddep_wait_for(XR, P);
   ptx::griddep_launch_dependents();
 
   const int32_t vpr = d / 8, n_vec = n_r * vpr;
@@ -532,13 +537,14 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
   }
   if (plan->R > 0 && tensor_core_request && sizeof(T) == 2 && d % 16 == 0 && k % 8 == 0 && smem_mma <= kMaxSmem) {
     ROCS_ALLOW_SMEM(fm_request_mma_kernel, kMaxSmem);
-    fm_request_mma_kernel<<<plan->R, 256, smem_mma, stream>>>(n_r, d, k, (const __nv_bfloat16*)XR,
-                                                              (const __nv_bfloat16*)P, TT, (__nv_bfloat16*)FR);
-    ROCS_CUDA_TRY(cudaGetLastError());
+    const rocs_status_t st = launch_dependent(fm_request_mma_kernel, dim3((unsigned)plan->R), 256, smem_mma, stream, n_r, d, k,
+                                              (const __nv_bfloat16*)XR, (const __nv_bfloat16*)P, TT, (__nv_bfloat16*)FR);
+    if (st != ROCS_OK) return st;
   } else if (plan->R > 0) {
     ROCS_ALLOW_SMEM(fm_request_kernel<T>, kMaxSmem);
-    fm_request_kernel<T><<<plan->R, 256, smem_r, stream>>>(n_r, d, k, (const T*)XR, (const T*)P, TT, (T*)FR);
-    ROCS_CUDA_TRY(cudaGetLastError());
+    const rocs_status_t st = launch_dependent(fm_request_kernel<T>, dim3((unsigned)plan->R), 256, smem_r, stream, n_r, d, k,
+                                              (const T*)XR, (const T*)P, TT, (T*)FR);
+    if (st != ROCS_OK) return st;
   }
   if (plan->N == 0 || !FC) return ROCS_OK;
   if (fast_candidates) {
@@ -551,10 +557,8 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
     }
   }
   ROCS_ALLOW_SMEM(fm_candidate_simt_kernel<T>, kMaxSmem);
-  fm_candidate_simt_kernel<T><<<(unsigned)plan->N, 128, smem_c, stream>>>(n_r, n_c, d, k, (const T*)XC, (const T*)P,
-                                                                         map, TT, (T*)FC);
-  ROCS_CUDA_TRY(cudaGetLastError());
-  return ROCS_OK;
+  return launch_dependent(fm_candidate_simt_kernel<T>, dim3((unsigned)plan->N), 128, smem_c, stream, n_r, n_c, d, k,
+                          (const T*)XC, (const T*)P, map, (const float*)TT, (T*)FC);
 }
 
 }  // namespace

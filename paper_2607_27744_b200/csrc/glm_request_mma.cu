@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(kThreads) glm_request_mma_kernel(
   const int32_t r = blockIdx.x;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   // the candidate kernel launched behind this one may start: it waits for this grid before it reads ZR
+  ptx::griddep_wait_for(XR, W);
   ptx::griddep_launch_dependents();
 
   // X^R_r as it is (bf16), 16 bytes per load, four loads in flight per thread
@@ -146,11 +147,9 @@ rocs_status_t glm_request_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, i
   if (plan->R == 0) return ROCS_OK;
   const size_t smem = request_smem(n_r, d, n_ro, n_co);
   ROCS_ALLOW_SMEM(glm_request_mma_kernel, kMaxDynamicSmem);
-  glm_request_mma_kernel<<<plan->R, kThreads, smem, stream>>>(n_r, n_c, d, (const __nv_bfloat16*)XR,
-                                                             (const __nv_bfloat16*)W, n_ro, n_co,
-                                                             (__nv_bfloat16*)YR, (__nv_bfloat16*)OR_, zr);
-  ROCS_CUDA_TRY(cudaGetLastError());
-  return ROCS_OK;
+  return launch_dependent(glm_request_mma_kernel, dim3((unsigned)plan->R), kThreads, smem, stream, n_r, n_c, d,
+                          (const __nv_bfloat16*)XR, (const __nv_bfloat16*)W, n_ro, n_co, (__nv_bfloat16*)YR,
+                          (__nv_bfloat16*)OR_, zr);
 }
 
 }  // namespace rocs

@@ -11,6 +11,7 @@
 #include <algorithm>
 
 #include "rocs_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace rocs {
 namespace {
@@ -66,6 +67,8 @@ group_norm_rows_kernel(int kind, int64_t M, const T* __restrict__ X, int64_t ld_
                        const T* __restrict__ beta, float eps, T* __restrict__ Y, int64_t ld_y) {
   constexpr int E = Vec<T>::kElems;
   constexpr int d = NV * 32 * E;
+  ptx::griddep_wait_for(X, gamma, beta);
+  ptx::griddep_launch_dependents();
   const int lane = threadIdx.x % 32;
   const int64_t warp = (int64_t)blockIdx.x * kWarpsPerBlock + threadIdx.x / 32;
   const int64_t n_warps = (int64_t)gridDim.x * kWarpsPerBlock;
@@ -118,6 +121,8 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 group_norm_general_kernel(int kind, int64_t M, int32_t d, const T* __restrict__ X, int64_t ld_x,
                           const T* __restrict__ gamma, const T* __restrict__ beta, float eps, T* __restrict__ Y,
                           int64_t ld_y) {
+  ptx::griddep_wait_for(X, gamma, beta);
+  ptx::griddep_launch_dependents();
   const int lane = threadIdx.x % 32;
   const int64_t warp = (int64_t)blockIdx.x * kWarpsPerBlock + threadIdx.x / 32;
   const int64_t n_warps = (int64_t)gridDim.x * kWarpsPerBlock;
@@ -163,23 +168,21 @@ rocs_status_t launch_norm(int kind, int64_t M, int32_t d, const void* X, int64_t
   const int threads = kWarpsPerBlock * 32;
   const bool vec_ok = d % (32 * E) == 0 && ld_x % E == 0 && ld_y % E == 0;
   const int nv = vec_ok ? d / (32 * E) : 0;
-#define ROCS_NORM_LAUNCH(NV_)                                                                                      \
-  group_norm_rows_kernel<T, NV_><<<grid, threads, 0, stream>>>(kind, M, (const T*)X, ld_x, (const T*)gamma,        \
-                                                               (const T*)beta, eps, (T*)Y, ld_y)
+#define ROCS_NORM_LAUNCH(kernel)                                                                              \
+  return launch_dependent(kernel, dim3((unsigned)grid), threads, 0, stream, kind, M, (const T*)X, ld_x,       \
+                          (const T*)gamma, (const T*)beta, eps, (T*)Y, ld_y)
   switch (nv) {
-    case 1: ROCS_NORM_LAUNCH(1); break;
-    case 2: ROCS_NORM_LAUNCH(2); break;
-    case 3: ROCS_NORM_LAUNCH(3); break;
-    case 4: ROCS_NORM_LAUNCH(4); break;
-    case 6: ROCS_NORM_LAUNCH(6); break;
-    case 8: ROCS_NORM_LAUNCH(8); break;
-    default:
-      group_norm_general_kernel<T><<<grid, threads, 0, stream>>>(kind, M, d, (const T*)X, ld_x, (const T*)gamma,
-                                                                 (const T*)beta, eps, (T*)Y, ld_y);
+    case 1: ROCS_NORM_LAUNCH((group_norm_rows_kernel<T, 1>));
+    case 2: ROCS_NORM_LAUNCH((group_norm_rows_kernel<T, 2>));
+    case 3: ROCS_NORM_LAUNCH((group_norm_rows_kernel<T, 3>));
+    case 4: ROCS_NORM_LAUNCH((group_norm_rows_kernel<T, 4>));
+    case 6: ROCS_NORM_LAUNCH((group_norm_rows_kernel<T, 6>));
+    case 8: ROCS_NORM_LAUNCH((group_norm_rows_kernel<T, 8>));
+    default: break;
   }
 #undef ROCS_NORM_LAUNCH
-  ROCS_CUDA_TRY(cudaGetLastError());
-  return ROCS_OK;
+  return launch_dependent(group_norm_general_kernel<T>, dim3((unsigned)grid), threads, 0, stream, kind, M, d, (const T*)X,
+                          ld_x, (const T*)gamma, (const T*)beta, eps, (T*)Y, ld_y);
 }
 
 }  // namespace

@@ -18,6 +18,7 @@
 // independent of the other rows' values (Eq. 1).
 #include "rocs_internal.h"
 #include "simt_util.cuh"
+#include "sm100_ptx.cuh"
 
 namespace rocs {
 namespace {
@@ -75,6 +76,9 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
   constexpr int BM = 8 * TM, BN = 8 * TN;
   extern __shared__ __align__(16) float sm[];
   __shared__ int32_t req[BM];  // request of each row of the tile
+  RequestMap requests = map;
+  ptx::griddep_wait_for(X, W, bias, add, requests.row2req, requests.offsets);
+  ptx::griddep_launch_dependents();
   const int group = threadIdx.x / kGroup, t = threadIdx.x % kGroup;
   const int tx = t % 8, ty = t / 8;
   const int64_t m0 = (int64_t)blockIdx.x * BM;
@@ -124,7 +128,7 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
         }
     }
   }
-  if (add && threadIdx.x < BM && m0 + threadIdx.x < M) req[threadIdx.x] = map.of(m0 + threadIdx.x);
+  if (add && threadIdx.x < BM && m0 + threadIdx.x < M) req[threadIdx.x] = requests.of(m0 + threadIdx.x);
   cp_async_wait<0>();
   __syncthreads();  // the rings become the groups' partial tiles
   float* part = sm + group * BM * BN;
@@ -153,21 +157,19 @@ rocs_status_t launch_linear(int64_t M, int32_t d_in, int32_t d_out, const void* 
                             const RequestMap& map, int act, void* Y, int64_t ld_y, cudaStream_t stream) {
   if (M == 0 || d_out == 0) return ROCS_OK;
   auto tiles = [&](int b) { return ((M + b - 1) / b) * ((d_out + b - 1) / b); };
-#define ROCS_LAUNCH(T_, KS_)                                                                                         \
-  do {                                                                                                               \
-    constexpr int smem = smem_bytes<8 * T_, 8 * T_, KS_>();                                                          \
-    auto kernel = linear_simt_kernel<TIn, TOut, T_, T_, KS_>;                                                        \
-    ROCS_ALLOW_SMEM(kernel, smem);                                                                                   \
-    kernel<<<dim3((unsigned)((M + 8 * T_ - 1) / (8 * T_)), (unsigned)((d_out + 8 * T_ - 1) / (8 * T_))), kGroup * KS_, \
-             smem, stream>>>(M, d_in, d_out, (const TIn*)X, ld_x, (const TIn*)W, ld_w, bias, add, ld_add, map,       \
-                             act, (TOut*)Y, ld_y);                                                                   \
+#define ROCS_LAUNCH(T_, KS_)                                                                                      \
+  do {                                                                                                            \
+    constexpr int smem = smem_bytes<8 * T_, 8 * T_, KS_>();                                                       \
+    auto kernel = linear_simt_kernel<TIn, TOut, T_, T_, KS_>;                                                     \
+    ROCS_ALLOW_SMEM(kernel, smem);                                                                                \
+    const dim3 grid((unsigned)((M + 8 * T_ - 1) / (8 * T_)), (unsigned)((d_out + 8 * T_ - 1) / (8 * T_)));        \
+    return launch_dependent(kernel, grid, kGroup * KS_, smem, stream, M, d_in, d_out, (const TIn*)X, ld_x,        \
+                            (const TIn*)W, ld_w, bias, add, ld_add, map, act, (TOut*)Y, ld_y);                    \
   } while (0)
   if (tiles(64) >= 296) ROCS_LAUNCH(8, 2);
   else if (tiles(32) >= 148) ROCS_LAUNCH(4, 4);
   else ROCS_LAUNCH(2, 8);
 #undef ROCS_LAUNCH
-  ROCS_CUDA_TRY(cudaGetLastError());
-  return ROCS_OK;
 }
 
 }  // namespace

@@ -85,6 +85,26 @@ namespace rocs {
       _done.fetch_or(_bit, std::memory_order_release);                                                     \
     }                                                                                                      \
   } while (0)
+// Launches a kernel as a programmatic dependent of the one in front of it on the stream.  The kernel must wait for
+// that one (griddep_wait) before it touches global memory, and may then release the next (in this order: what is
+// released relies on everything in front of its predecessor being complete).
+template <typename... P, typename... A>
+inline rocs_status_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream,
+                                      A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+  return ROCS_OK;
+}
+
 constexpr int kMaxDynamicSmem = 227 * 1024;  // per block on sm_100
 
 inline size_t elem_size(rocs_dtype_t dt) { return dt == ROCS_BF16 ? 2 : 4; }

@@ -4,12 +4,15 @@
 // are added up here in a fixed order.  Also: the same sums straight from a stored tensor (for layers
 // whose kernel does not emit partials) and the row sums of a weight matrix (W 1, LayerNorm's shift).
 #include "rocs_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace rocs {
 namespace {
 
 __global__ void stats_from_partials_kernel(int64_t M, int32_t P, const float2* __restrict__ partials,
                                            float2* __restrict__ row_stats) {
+  ptx::griddep_wait_for(partials);
+  ptx::griddep_launch_dependents();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= M) return;
   float s = 0.f, q = 0.f;
@@ -32,6 +35,8 @@ __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 v) { return
 template <typename T>
 __global__ void stats_direct_kernel(int64_t M, int32_t d, const T* __restrict__ Y, int64_t ld, float2* __restrict__ out,
                                     int32_t as_weight_sums, float* __restrict__ wbar) {
+  ptx::griddep_wait_for(Y);
+  ptx::griddep_launch_dependents();
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   if (row >= M) return;
   const int lane = threadIdx.x % 32;
@@ -56,9 +61,8 @@ __global__ void stats_direct_kernel(int64_t M, int32_t d, const T* __restrict__ 
 rocs_status_t row_stats_from_partials(int64_t M, int32_t P, const float2* partials, float2* row_stats,
                                       cudaStream_t stream) {
   if (M == 0) return ROCS_OK;
-  stats_from_partials_kernel<<<(unsigned)((M + 255) / 256), 256, 0, stream>>>(M, P, partials, row_stats);
-  ROCS_CUDA_TRY(cudaGetLastError());
-  return ROCS_OK;
+  return launch_dependent(stats_from_partials_kernel, dim3((unsigned)((M + 255) / 256)), 256, 0, stream, M, P, partials,
+                          row_stats);
 }
 
 static rocs_status_t launch_direct(rocs_dtype_t dt, int64_t M, int32_t d, const void* Y, int64_t ld, float2* out,
@@ -66,11 +70,10 @@ static rocs_status_t launch_direct(rocs_dtype_t dt, int64_t M, int32_t d, const 
   if (M == 0) return ROCS_OK;
   const unsigned blocks = (unsigned)((M + 7) / 8);
   if (dt == ROCS_BF16)
-    stats_direct_kernel<__nv_bfloat16><<<blocks, 256, 0, stream>>>(M, d, (const __nv_bfloat16*)Y, ld, out, as_weight_sums, wbar);
-  else
-    stats_direct_kernel<float><<<blocks, 256, 0, stream>>>(M, d, (const float*)Y, ld, out, as_weight_sums, wbar);
-  ROCS_CUDA_TRY(cudaGetLastError());
-  return ROCS_OK;
+    return launch_dependent(stats_direct_kernel<__nv_bfloat16>, dim3(blocks), 256, 0, stream, M, d, (const __nv_bfloat16*)Y, ld,
+                            out, as_weight_sums, wbar);
+  return launch_dependent(stats_direct_kernel<float>, dim3(blocks), 256, 0, stream, M, d, (const float*)Y, ld, out,
+                          as_weight_sums, wbar);
 }
 
 rocs_status_t row_stats_direct(rocs_dtype_t dt, int64_t M, int32_t d, const void* Y, int64_t ld_y, float2* row_stats,

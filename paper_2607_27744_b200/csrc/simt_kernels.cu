@@ -35,8 +35,9 @@ __global__ void __launch_bounds__(256) glm_request_simt_kernel(
   float* g = xr + (size_t)n_r * ds;            // [n_r, n_r]
   float* w = g + (size_t)n_r * n_r;            // [n_ro + n_co, n_r]: the request columns of W
   const int32_t r = blockIdx.x;
-  // a candidate kernel launched behind this one as a programmatic dependent may start now: it streams
-  // its own operands and waits for this grid only before it reads ZR
+  // the candidate kernel launched behind this one may start now: it streams its own operands and waits for this
+  // grid only before it reads ZR
+  ptx::griddep_wait_for(XR, W);
   ptx::griddep_launch_dependents();
   rows_to_shared(XR + (int64_t)r * n_r * d, xr, n_r, d, ds);
   if (W)
@@ -236,26 +237,16 @@ static rocs_status_t launch_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c,
   }
   if (plan->R > 0) {
     ROCS_ALLOW_SMEM(glm_request_simt_kernel<T>, kMaxSmem);
-    glm_request_simt_kernel<T><<<plan->R, 256, smem_r, stream>>>(
-        n_r, n_c, d, (const T*)XR, (const T*)W, n_ro, n_co, (T*)YR, (T*)OR_, zr);
-    ROCS_CUDA_TRY(cudaGetLastError());
+    const rocs_status_t st = launch_dependent(glm_request_simt_kernel<T>, dim3((unsigned)plan->R), 256, smem_r, stream, n_r, n_c, d,
+                                              (const T*)XR, (const T*)W, n_ro, n_co, (T*)YR, (T*)OR_, zr);
+    if (st != ROCS_OK) return st;
   }
   if (candidate_side) {
     auto kernel = glm_candidate_simt_kernel<T>;
     ROCS_ALLOW_SMEM(kernel, kMaxSmemC);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)tiles.num);
-    cfg.blockDim = dim3(kGlmThreads);
-    cfg.dynamicSmemBytes = smem_c(cands);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, plan->R, cands, plan->cand_offsets, (const Tile*)tiles.dev, n_r, n_c,
-                                     d, (const T*)XR, (const T*)XC, (const T*)W, n_ro, n_co, w_shared, (const float*)zr, (T*)YC,
-                                     (T*)OC));
+    return launch_dependent(kernel, dim3((unsigned)tiles.num), kGlmThreads, smem_c(cands), stream, plan->R, cands,
+                            plan->cand_offsets, (const Tile*)tiles.dev, n_r, n_c, d, (const T*)XR, (const T*)XC, (const T*)W,
+                            n_ro, n_co, w_shared, (const float*)zr, (T*)YC, (T*)OC);
   }
   return ROCS_OK;
 }

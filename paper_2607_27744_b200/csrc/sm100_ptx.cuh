@@ -121,6 +121,13 @@ __device__ __forceinline__ bool elect_one() {
 // predecessor still runs; it must call griddep_wait() before touching anything the predecessor
 // writes.  The predecessor releases such a dependent early with griddep_launch_dependents().
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The same in front of reads through the given pointers.  A load through a const __restrict__ pointer may be moved
+// over any fence, since nothing in the kernel writes there; it cannot be moved over the place its address comes from.
+template <typename... P>
+__device__ __forceinline__ void griddep_wait_for(P&... p) {
+  griddep_wait();
+  (([](auto& q) { asm volatile("" : "+l"(q) : : "memory"); }(p)), ...);
+}
 __device__ __forceinline__ void griddep_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
