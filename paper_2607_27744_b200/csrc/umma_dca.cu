@@ -382,7 +382,11 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
       const uint32_t slot = n_item & 1;
       // (a slot comes free only if the items in front of it can finish, the last one included when this one
       // has no loads behind which its tail would be zeroed)
-      if (L == 0 && !zero_tail()) { ok = false; break; }
+      if (L == 0 && tail_valid != 0) {
+        // not before that item's last S, as in the ordinary case: the issuer is then past the tail in front of it,
+        // and two arrivals never meet one wait
+        if (!wait(q_empty, (n_work & 1) ^ 1, 1) || !zero_tail()) { ok = false; break; }
+      }
       if (!wait(info_empty + 8 * slot, ((n_item >> 1) & 1) ^ 1, 12)) { ok = false; break; }
       if (lane == 0) {
         info[2 * slot] = make_int4(item.req, item.cand0, item.count * p.n_q, item.head);

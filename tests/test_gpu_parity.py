@@ -348,6 +348,25 @@ def test_dca_bf16_short_last_blocks_between_empty_requests(dh):
         assert rel_err(to_host_f64(O), want) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("dh", [32, 64, 128])
+@pytest.mark.parametrize("heads", [1, 4, 64])
+def test_dca_bf16_streams_that_end_with_short_ragged_items(dh, heads):
+    # the last item of a side's stream is loaded whole while the one in front of it is still at work; both end
+    # inside a group of 16 keys.  Items taken by position (few or very many) and claimed; repeated, since what goes
+    # wrong is a hand-over that comes too early
+    R = 200
+    co = wl.offsets_from_counts([3] * R)
+    so = wl.offsets_from_counts([150 + (r * 37) % 90 if r < R // 2 else 1 + (r * 7) % 60 for r in range(R)])
+    cfg = wl.CONFIGS[3].with_(R=R, H=heads, dh=dh)
+    d = wl.dca_inputs(cfg, co, so)
+    Q, K, V, sod, plan = to_dev(d["Q"]), to_dev(d["K"]), to_dev(d["V"]), to_dev(so), _plan(co)
+    want = ref.dca_attention(co, so, d["Q"], d["K"], d["V"])
+    for _ in range(300):
+        O = rocs.dca_attention(plan, Q, K, V, sod)
+    assert rocs.last_device_status() == 0
+    assert rel_err(to_host_f64(O), want) <= tol_for("bf16")
+
+
 @pytest.mark.parametrize("dh", [32, 128])
 def test_dca_bf16_head_dim_32_and_128_many_tiles_sampled(dh):
     # enough tiles that every SM runs several items on both of its streams (L = 700: 11 or 6 key blocks)
