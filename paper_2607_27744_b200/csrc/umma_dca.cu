@@ -82,8 +82,14 @@ struct DcaCfg {
   __device__ static uint64_t desc_v(uint32_t addr) {
     return kRowBytes == 128 ? smem_desc_sw128(addr, 1024, kBoxes > 1 ? kKvBoxBytes : 16) : smem_desc_sw64(addr, 512, 16);
   }
-  // tensor memory per side: S [0, BKV) fp32, P [BKV, BKV + BKV/2) bf16 pairs, O [.., + DH) fp32
-  static constexpr int kPColOffset = BKV, kOColOffset = BKV + BKV / 2;
+  // tensor memory per side: S [0, BKV) fp32, P (one or two buffers of BKV / 2) bf16 pairs, O [.., + DH) fp32.
+  // Two P buffers where they fit (dh = 128): P_j then replaces P_{j-2}, whose P V was issued in front of S_j, so the
+  // arrival of S_j says that it is done and the wait in the middle of a block goes.  That wait also kept a fast warp
+  // from announcing P_{j+1} before a slow one had announced P_j: each buffer has a barrier of its own instead (P_{j+2}
+  // comes after S_{j+2}, which is issued when every warp has read S_{j+1}, i.e. has announced P_j).
+  // 821 candidates x 32 query tokens, 4 heads of 128, 500..1500 keys: 86 us with one buffer, 79 us with two.
+  static constexpr int kPBuffers = BKV + BKV + DH <= kSideTmemStride ? 2 : 1;
+  static constexpr int kPColOffset = BKV, kOColOffset = BKV + kPBuffers * (BKV / 2);
   static_assert(kOColOffset + DH <= kSideTmemStride, "tensor memory columns of a side");
   static_assert(kCols == 32 || kCols == 64, "score columns per thread");
   // Shared-memory map (byte offsets from the 1024-byte aligned base); per side: one Q tile (freed when
@@ -99,8 +105,8 @@ struct DcaCfg {
   static constexpr uint32_t kBarKvEmpty = kBarKvFull + 16 * kKvSlots;
   static constexpr uint32_t kBarSFull = kBarKvEmpty + 16 * kKvSlots;  // [2]
   static constexpr uint32_t kBarSEmpty = kBarSFull + 16;
-  static constexpr uint32_t kBarPFull = kBarSEmpty + 16;
-  static constexpr uint32_t kBarOFull = kBarPFull + 16;
+  static constexpr uint32_t kBarPFull = kBarSEmpty + 16;            // [2][2 buffers]
+  static constexpr uint32_t kBarOFull = kBarPFull + 32;
   static constexpr uint32_t kBarPair = kBarOFull + 16;              // [8]: the two warps that share 32 query rows
   static constexpr uint32_t kBarDrain = kBarPair + 64;              // [2]
   static constexpr uint32_t kBarInfoFull = kBarDrain + 16;          // [2][2 slots]
@@ -285,7 +291,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     init(kBarKvEmpty, 2 * kKvSlots, 1);
     init(kBarSFull, 2, 1);
     init(kBarSEmpty, 2, kSoftmaxWarps / 2);
-    init(kBarPFull, 2, kSoftmaxWarps / 2);
+    init(kBarPFull, 4, kSoftmaxWarps / 2);
     init(kBarOFull, 2, 1);
     init(kBarPair, 8, 2);
     init(kBarDrain, 2, 1);
@@ -452,7 +458,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
       const uint32_t q_full = sb + kBarQFull + 8 * side, q_empty = sb + kBarQEmpty + 8 * side;
       const uint32_t kv_full = sb + kBarKvFull + 8 * kKvSlots * side, kv_empty = sb + kBarKvEmpty + 8 * kKvSlots * side;
       const uint32_t s_full = sb + kBarSFull + 8 * side, s_empty = sb + kBarSEmpty + 8 * side;
-      const uint32_t p_full = sb + kBarPFull + 8 * side, o_full = sb + kBarOFull + 8 * side;
+      const uint32_t p_full = sb + kBarPFull + 16 * side, o_full = sb + kBarOFull + 8 * side;
       const uint32_t tail_done = sb + kBarTail + 8 * side;
       const uint32_t info_full = sb + kBarInfoFull + 16 * side, info_empty = sb + kBarInfoEmpty + 16 * side;
       const int4* info = reinterpret_cast<const int4*>(smem + kOffInfo) + side * 4;
@@ -477,15 +483,15 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         umma_commit(s_full);
         umma_commit(kv_empty + 8 * slot);
       };
-      auto issue_pv = [&](uint32_t slot, int32_t keys, bool first_block) {
+      auto issue_pv = [&](uint32_t slot, uint32_t buf, int32_t keys, int32_t j, bool last) {
         const uint64_t dv = dv0 + slot * (kKBytes >> 4);
+        const uint32_t t_p = t_s + kPColOffset + buf * (BKV / 2);
         // P: 16 keys = 8 columns of bf16 pairs in tensor memory; V: rows are keys, 16 keys = 16 rows further on
 #pragma unroll
         for (int k = 0; k < BKV / 16; ++k)
           if (k * 16 < keys)
-            umma_ts(t_s + kOColOffset, t_s + kPColOffset + k * 8, dv + k * (16 * C::kRowBytes / 16), idesc_o,
-                    (k != 0 || !first_block) ? 1u : 0u);
-        umma_commit(o_full);
+            umma_ts(t_s + kOColOffset, t_p + k * 8, dv + k * (16 * C::kRowBytes / 16), idesc_o, (k | j) != 0 ? 1u : 0u);
+        if (C::kPBuffers == 1 || last) umma_commit(o_full);
         umma_commit(kv_empty + 8 * slot);
       };
       auto next_slot = [&](uint32_t code) {  // the next block in the order of loading, landed
@@ -526,10 +532,11 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             ++n_tail;
           }
           // P_j of this side is in tensor memory
-          if (!mbar_wait_paced(p_full, cnt_p & 1, abort_flag, p.status, kStatusDca | 6)) { ok = false; break; }
+          const uint32_t buf = cnt_p & (C::kPBuffers - 1);
+          if (!mbar_wait_paced(p_full + 8 * buf, (cnt_p / C::kPBuffers) & 1, abort_flag, p.status, kStatusDca | 6)) { ok = false; break; }
           ++cnt_p;
           tc_fence_after_sync();
-          issue_pv((kv_it - 1) % kKvSlots, j + 1 == nblk ? tail_keys : BKV, j == 0);
+          issue_pv((kv_it - 1) % kKvSlots, buf, j + 1 == nblk ? tail_keys : BKV, j, j + 1 == nblk);
         }
       }
       if (!ok) {
@@ -549,7 +556,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const uint32_t t_p = t_row + kPColOffset + half * (kCols / 2);
     const uint32_t t_o = t_row + kOColOffset + half * kOutCols;
     const uint32_t s_full = sb + kBarSFull + 8 * side, s_empty = sb + kBarSEmpty + 8 * side;
-    const uint32_t p_full = sb + kBarPFull + 8 * side, o_full = sb + kBarOFull + 8 * side;
+    const uint32_t p_full = sb + kBarPFull + 16 * side, o_full = sb + kBarOFull + 8 * side;
     const uint32_t my_pair = sb + kBarPair + 8 * (side * 4 + q);
     uint32_t cnt_s = 0, cnt_o = 0, cnt_pair = 0;
     const uint32_t info_full = sb + kBarInfoFull + 16 * side, info_empty = sb + kBarInfoEmpty + 16 * side;
@@ -622,6 +629,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           // P V of the previous block has read P_{j-1} (it was issued most of a block ago): from there on this
           // thread's P columns may be rewritten
           auto previous_pv_done = [&]() {
+            if (C::kPBuffers == 2) return true;
             if (j > 0) {
               if (!mbar_wait_spin(o_full, (cnt_o & 1) ^ 1, abort_flag, p.status, kStatusDca | 9)) return false;
               tc_fence_after_sync();
@@ -629,14 +637,15 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             ++cnt_o;
             return true;
           };
+          const uint32_t buf = (cnt_s - 1) & (C::kPBuffers - 1), t_pj = t_p + buf * (BKV / 2);
           if (valid > 0) {
 #pragma unroll
             for (int e = 0; e < kCols / 2; e += 2) exp_pair(e);
             if (!previous_pv_done()) { aborted = true; break; }
-            store_p(t_p);
+            store_p(t_pj);
 #pragma unroll
             for (int e = kCols / 2; e < kCols; e += 2) exp_pair(e);
-            store_p(t_p + kCols / 4);
+            store_p(t_pj + kCols / 4);
           } else if (!previous_pv_done()) {  // no key in this half of the last block: P V stops in front of it
             aborted = true;
             break;
@@ -644,9 +653,10 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           tmem_st_wait();
           tc_fence_before_sync();
           __syncwarp();
-          if (lane == 0) mbar_arrive(p_full);
+          if (lane == 0) mbar_arrive(p_full + 8 * buf);
         }
         if (aborted) break;
+        if (C::kPBuffers == 2) ++cnt_o;  // one arrival per item
         float sum_lo, sum_hi;
         unpack2(sum2, sum_lo, sum_hi);
         const float l_run = sum_lo + sum_hi;
