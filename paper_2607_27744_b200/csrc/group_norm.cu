@@ -3,11 +3,11 @@
 // separate tensors and separate calls).
 //   LayerNorm:  y = (x - mean) / sqrt(var + eps) * gamma + beta     (biased variance)
 //   RMSNorm:    y = x / sqrt(mean(x^2) + eps) * gamma
-// Pure streaming work (read once, write once): one warp per row, the row held in registers as
-// 16-byte vectors (coalesced 512-byte warp accesses), statistics in fp32 by warp shuffles, the
+// Pure streaming work (read once, write once), bound by memory: a row on 4 to 32 lanes of one
+// warp, held in registers as 16-byte vectors, statistics in fp32 by shuffles among them, the
 // variance taken around the mean from the registers (no E[x^2] - E[x]^2 cancellation).  Rows
-// wider than the register variant allows, or with a width that is no multiple of one warp's
-// 16-byte vectors, run on a two-pass variant that re-reads the row (from L1/L2).
+// of more than 256 vectors or a width that is no whole number of them run on a kernel that
+// re-reads the row element by element (from L1/L2).
 #include <algorithm>
 
 #include "rocs_internal.h"
@@ -60,41 +60,60 @@ struct Vec<__nv_bfloat16> {
   }
 };
 
-// d == NV * 32 * Vec<T>::kElems: lane l owns vectors l, l + 32, ...
-template <typename T, int NV>
+// Rows of whole 16-byte vectors, at most NV * G of them (FULL: exactly): G lanes per row, lane l of them owns vectors
+// l, l + G, ...; a warp has 32 / G rows at a time.  Lanes without a row or a vector add nothing.
+template <typename T, int NV, int G, bool FULL>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
-group_norm_rows_kernel(int kind, int64_t M, const T* __restrict__ X, int64_t ld_x, const T* __restrict__ gamma,
+group_norm_rows_kernel(int kind, int64_t M, int32_t d_arg, const T* __restrict__ X, int64_t ld_x, const T* __restrict__ gamma,
                        const T* __restrict__ beta, float eps, T* __restrict__ Y, int64_t ld_y) {
   constexpr int E = Vec<T>::kElems;
-  constexpr int d = NV * 32 * E;
+  constexpr int kRows = 32 / G;
   ptx::griddep_wait_for(X, gamma, beta);
   ptx::griddep_launch_dependents();
-  const int lane = threadIdx.x % 32;
+  const int d = FULL ? NV * G * E : d_arg;
+  const float inv_d = 1.f / (float)d;
+  const int lane = threadIdx.x % G, sub = threadIdx.x % 32 / G;
   const int64_t warp = (int64_t)blockIdx.x * kWarpsPerBlock + threadIdx.x / 32;
   const int64_t n_warps = (int64_t)gridDim.x * kWarpsPerBlock;
-  for (int64_t row = warp; row < M; row += n_warps) {
+  auto group_sum = [](float v) {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  for (int64_t first = warp * kRows; first < M; first += n_warps * kRows) {
+    const int64_t row = first + sub;
+    const bool have = kRows == 1 || row < M;
     float x[NV][E];
     float s = 0.f;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      Vec<T>::load(X + row * ld_x + (v * 32 + lane) * E, x[v]);
+      const int col = (v * G + lane) * E;
+      if (have && (FULL || col < d)) {
+        Vec<T>::load(X + row * ld_x + col, x[v]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) x[v][e] = 0.f;
+      }
 #pragma unroll
       for (int e = 0; e < E; ++e) s += x[v][e];
     }
     float mean = 0.f;
-    if (kind == ROCS_NORM_LAYER) mean = warp_sum(s) * (1.f / d);
+    if (kind == ROCS_NORM_LAYER) mean = group_sum(s) * inv_d;
     float sq = 0.f;
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
+    for (int v = 0; v < NV; ++v) {
+      if (!FULL && (v * G + lane) * E >= d) continue;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         x[v][e] -= mean;
         sq = fmaf(x[v][e], x[v][e], sq);
       }
-    const float inv = rsqrtf(warp_sum(sq) * (1.f / d) + eps);
+    }
+    const float inv = rsqrtf(group_sum(sq) * inv_d + eps);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      const int col = (v * 32 + lane) * E;
+      const int col = (v * G + lane) * E;
+      if (!have || (!FULL && col >= d)) continue;
       float g[E], b[E];
 #pragma unroll
       for (int e = 0; e < E; ++e) {
@@ -163,25 +182,35 @@ rocs_status_t launch_norm(int kind, int64_t M, int32_t d, const void* X, int64_t
                           const void* beta, float eps, void* Y, int64_t ld_y, cudaStream_t stream) {
   if (M == 0) return ROCS_OK;
   constexpr int E = Vec<T>::kElems;
-  const int64_t want = (M + kWarpsPerBlock - 1) / kWarpsPerBlock;
-  const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count_norm() * 8);  // 64 resident warps per SM
   const int threads = kWarpsPerBlock * 32;
-  const bool vec_ok = d % (32 * E) == 0 && ld_x % E == 0 && ld_y % E == 0;
-  const int nv = vec_ok ? d / (32 * E) : 0;
-#define ROCS_NORM_LAUNCH(kernel)                                                                              \
-  return launch_dependent(kernel, dim3((unsigned)grid), threads, 0, stream, kind, M, (const T*)X, ld_x,       \
-                          (const T*)gamma, (const T*)beta, eps, (T*)Y, ld_y)
-  switch (nv) {
-    case 1: ROCS_NORM_LAUNCH((group_norm_rows_kernel<T, 1>));
-    case 2: ROCS_NORM_LAUNCH((group_norm_rows_kernel<T, 2>));
-    case 3: ROCS_NORM_LAUNCH((group_norm_rows_kernel<T, 3>));
-    case 4: ROCS_NORM_LAUNCH((group_norm_rows_kernel<T, 4>));
-    case 6: ROCS_NORM_LAUNCH((group_norm_rows_kernel<T, 6>));
-    case 8: ROCS_NORM_LAUNCH((group_norm_rows_kernel<T, 8>));
-    default: break;
-  }
+  auto blocks = [&](int rows_per_warp) {  // 64 resident warps per SM at most
+    const int64_t per_block = (int64_t)kWarpsPerBlock * rows_per_warp;
+    return dim3((unsigned)std::min<int64_t>((M + per_block - 1) / per_block, (int64_t)sm_count_norm() * 8));
+  };
+  // Lanes per row and vectors per lane by the width: the fewest that hold the row, so that few lanes idle.  A width that
+  // is no multiple of a warp's 512 bytes on the element-wise kernel below took 34.1 us at [51922, 384] bf16 where
+  // three vectors on 16 lanes take 13.2 (6.0 TB/s), 20.0 against 8.8 at [40000, 200] and 12.8 against 4.0 at [40000, 64].
+  // Two rows in flight per lane group measured 5.4 us for 5.9 at [40000, 128] and 11.2 for 10.4 at [46262, 256]: not taken.
+  const int vecs = d % E == 0 && ld_x % E == 0 && ld_y % E == 0 ? d / E : 0;
+#define ROCS_NORM_LAUNCH(NV_, G_, FULL_)                                                                              \
+  return launch_dependent(group_norm_rows_kernel<T, NV_, G_, FULL_>, blocks(32 / G_), threads, 0, stream, kind, M, d, \
+                          (const T*)X, ld_x, (const T*)gamma, (const T*)beta, eps, (T*)Y, ld_y)
+#define ROCS_NORM_WIDTH(NV_, G_)                            \
+  if (vecs == NV_ * G_) ROCS_NORM_LAUNCH(NV_, G_, true);    \
+  if (vecs > 0 && vecs < NV_ * G_) ROCS_NORM_LAUNCH(NV_, G_, false)
+  ROCS_NORM_WIDTH(1, 4);
+  ROCS_NORM_WIDTH(1, 8);
+  ROCS_NORM_WIDTH(1, 16);
+  ROCS_NORM_WIDTH(1, 32);
+  ROCS_NORM_WIDTH(3, 16);
+  ROCS_NORM_WIDTH(2, 32);
+  ROCS_NORM_WIDTH(3, 32);
+  ROCS_NORM_WIDTH(4, 32);
+  ROCS_NORM_WIDTH(6, 32);
+  ROCS_NORM_WIDTH(8, 32);
+#undef ROCS_NORM_WIDTH
 #undef ROCS_NORM_LAUNCH
-  return launch_dependent(group_norm_general_kernel<T>, dim3((unsigned)grid), threads, 0, stream, kind, M, d, (const T*)X,
+  return launch_dependent(group_norm_general_kernel<T>, blocks(1), threads, 0, stream, kind, M, d, (const T*)X,
                           ld_x, (const T*)gamma, (const T*)beta, eps, (T*)Y, ld_y);
 }
 

@@ -27,6 +27,18 @@ def test_rows_against_the_oracle(kind, dtype, d):
     assert rel_err(to_host_f64(y), want) <= tol_for(dtype)
 
 
+# lanes per row and vectors per lane: 4, 8, 16 and 32 lanes, full and one vector short or over, and rows beyond them
+@pytest.mark.parametrize("kind", [rocs.NORM_LAYER, rocs.NORM_RMS])
+@pytest.mark.parametrize("dtype,d", [("bf16", d) for d in (8, 32, 40, 64, 72, 128, 200, 264, 384, 392, 712, 1160, 2040, 2056)] +
+                         [("f32", d) for d in (4, 60, 132, 1020, 1028)])
+@pytest.mark.parametrize("M", [1, 1237])
+def test_rows_of_any_number_of_vectors(kind, dtype, d, M):
+    x, gamma, beta = _inputs(M, d, dtype, d % 7)
+    y = rocs.group_norm(to_dev(x), to_dev(gamma), to_dev(beta), eps=1e-5, kind=kind)
+    want = ref.group_norm(x, gamma, beta, 1e-5, kind)
+    assert rel_err(to_host_f64(y), want) <= tol_for(dtype)
+
+
 def test_no_scale_no_shift_strided_rows_and_in_place():
     x, _, _ = _inputs(300, 512, "bf16", 3)
     buf = torch.zeros((300, 640), dtype=torch.bfloat16, device="cuda")
