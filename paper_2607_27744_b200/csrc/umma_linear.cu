@@ -22,21 +22,25 @@ namespace {
 
 using namespace ptx;
 
-constexpr int BM = 128;           // rows per tile = TMEM lanes
+constexpr int BM = 128;           // rows of an MMA = TMEM lanes
 constexpr int BK = 64;            // 64 bf16 = one 128-byte swizzle row
 constexpr int kThreads = 192;
 constexpr int kEpiWarps = 4;
 constexpr uint32_t kStatusLinear = 0x100;
 
-template <int BN>
+// TM x BN outputs per tile.  With TM < 128 the MMA still has 128 rows: those behind the tile's hold whatever lies behind
+// its slot of X in shared memory, and their outputs are not stored.
+template <int TM, int BN>
 struct LinearCfg {
-  static constexpr int kStages = BN == 256 ? 4 : 6;
-  static constexpr int kABytes = BM * BK * 2;
+  static constexpr int kABytes = TM * BK * 2;
   static constexpr int kBBytes = BN * BK * 2;
-  static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kStagingBytes = kEpiWarps * 2 * 4096;  // per warp: two 32-row x 128-byte buffers
-  static constexpr int kTmemCols = 2 * BN >= 32 ? 2 * BN : 32;
-  static constexpr int kSmemBytes = kStages * kStageBytes + kStagingBytes + 256 /*barriers*/ + 1024 /*align*/;
+  static constexpr int kStages = BN == 256 ? 4 : TM + BN >= 192 ? 6 : TM + BN >= 128 ? 8 : 12;
+  static constexpr int kOffB = kStages * kABytes;  // slots of X, then of W
+  static constexpr int kOffStaging = kOffB + kStages * kBBytes;
+  static constexpr int kStagingBytes = kEpiWarps * 2 * 4096;  // per warp: two buffers of 32 rows x 128 bytes at most
+  static constexpr int kTmemCols = 2 * BN;
+  static constexpr int kSmemBytes = kOffStaging + kStagingBytes + 512 /*barriers*/ + 1024 /*align*/;
+  static_assert(kOffB - kABytes + BM * BK * 2 <= kOffStaging + kStagingBytes, "rows behind the last slot");
 };
 
 struct LinearParams {
@@ -52,17 +56,18 @@ struct LinearParams {
   uint32_t* status;
 };
 
-template <int BN, typename OutT>
+template <int TM, int BN, typename OutT>
 __global__ void __launch_bounds__(kThreads, 1)
 linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                    const __grid_constant__ CUtensorMap map_y, const LinearParams p) {
-  using Cfg = LinearCfg<BN>;
+  using Cfg = LinearCfg<TM, BN>;
   constexpr int kStages = Cfg::kStages;
-  constexpr int CH = 128 / (int)sizeof(OutT);  // output columns per 128-byte staging row
+  constexpr int CH = BN * (int)sizeof(OutT) < 128 ? BN : 128 / (int)sizeof(OutT);  // output columns per staging row
+  constexpr int kChunks16 = CH * (int)sizeof(OutT) / 16;                           // 16-byte chunks of a staging row
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* staging = smem + kStages * Cfg::kStageBytes;
+  uint8_t* staging = smem + Cfg::kOffStaging;
   uint64_t* full = reinterpret_cast<uint64_t*>(staging + Cfg::kStagingBytes);
   uint64_t* empty = full + kStages;
   uint64_t* tmem_full = empty + kStages;
@@ -72,7 +77,7 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   AbortFlag* abort_flag = reinterpret_cast<AbortFlag*>(tmem_ptr + 1);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int32_t m_tiles = (int32_t)((p.M + BM - 1) / BM);
+  const int32_t m_tiles = (int32_t)((p.M + TM - 1) / TM);
   const int32_t n_tiles = (p.d_out + BN - 1) / BN;
   const int32_t k_blocks = (p.d_in + BK - 1) / BK;
   const int64_t num_tiles = (int64_t)m_tiles * n_tiles;
@@ -121,15 +126,14 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       uint32_t it = 0;
       bool ok = true;
       for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
-        const int32_t m0 = (int32_t)(t / n_tiles) * BM, n0 = (int32_t)(t % n_tiles) * BN;
+        const int32_t m0 = (int32_t)(t / n_tiles) * TM, n0 = (int32_t)(t % n_tiles) * BN;
         for (int32_t kb = 0; kb < k_blocks; ++kb, ++it) {
           const int s = it % kStages;
           const uint32_t ph = (it / kStages) & 1;
           if (!mbar_wait(&empty[s], ph ^ 1, abort_flag, p.status, kStatusLinear | 1)) { ok = false; break; }
-          uint8_t* a = smem + s * Cfg::kStageBytes;
           mbar_expect_tx(&full[s], p.x_rows * (BK * 2) + Cfg::kBBytes);
-          tma_load_2d(a, &map_x, &full[s], kb * BK, m0);
-          tma_load_2d(a + Cfg::kABytes, &map_w, &full[s], kb * BK, n0);
+          tma_load_2d(smem + s * Cfg::kABytes, &map_x, &full[s], kb * BK, m0);
+          tma_load_2d(smem + Cfg::kOffB + s * Cfg::kBBytes, &map_w, &full[s], kb * BK, n0);
         }
       }
       if (!ok) {
@@ -158,9 +162,8 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           const int s = it % kStages;
           if (!mbar_wait(&full[s], (it / kStages) & 1, abort_flag, p.status, kStatusLinear | 3)) { ok = false; break; }
           tc_fence_after_sync();
-          const uint32_t a_addr = smem_u32(smem + s * Cfg::kStageBytes);
-          const uint64_t a_desc = smem_desc_sw128(a_addr, 1024, 16);
-          const uint64_t b_desc = smem_desc_sw128(a_addr + Cfg::kABytes, 1024, 16);
+          const uint64_t a_desc = smem_desc_sw128(smem_u32(smem + s * Cfg::kABytes), 1024, 16);
+          const uint64_t b_desc = smem_desc_sw128(smem_u32(smem + Cfg::kOffB + s * Cfg::kBBytes), 1024, 16);
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)  // +32 bytes = 16 bf16 along K, in 16-byte units
             umma_ss(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
@@ -186,15 +189,21 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     }
     for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++lt) {
       const uint32_t acc = lt & 1;
-      const int32_t m0 = (int32_t)(t / n_tiles) * BM, n0 = (int32_t)(t % n_tiles) * BN;
+      const int32_t m0 = (int32_t)(t / n_tiles) * TM, n0 = (int32_t)(t % n_tiles) * BN;
       const int64_t row = (int64_t)m0 + q * 32 + lane;
+      const bool mine = TM == BM || q * 32 < TM;  // rows of the tile among this warp's
       const float* add_row = nullptr;
-      if (p.add != nullptr && row < p.M)
+      if (p.add != nullptr && mine && row < p.M)
         add_row = p.add + (int64_t)p.map.of(row) * p.ld_add;
       if (!mbar_wait(&tmem_full[acc], (lt >> 1) & 1, abort_flag, p.status, kStatusLinear | 4)) { ok = false; break; }
       tc_fence_after_sync();
       const uint32_t t_row = tmem_base + acc * BN + ((uint32_t)(q * 32) << 16);
       constexpr int kChunks = BN / CH;
+      if (!mine) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tmem_empty[acc]);
+        continue;
+      }
 #pragma unroll 1
       for (int c = 0; c < kChunks; ++c) {
         const int32_t col0 = n0 + c * CH;
@@ -238,9 +247,10 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         uint8_t* buf = my_stage + (stores & 1) * 4096;
         if (elect_one()) tma_store_wait_read<1>();
         __syncwarp();
-        uint8_t* row_ptr = buf + lane * 128;
+        uint8_t* row_ptr = buf + lane * (kChunks16 * 16);
+        const int swizzle = kChunks16 == 8 ? lane & 7 : lane / 2 & 3;  // of 128- and 64-byte rows
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {  // eight 16-byte chunks per 128-byte row, XOR-swizzled by row
+        for (int j = 0; j < kChunks16; ++j) {  // 16-byte chunks, XOR-swizzled by row
           uint4 w;
           if constexpr (sizeof(OutT) == 2) {
             __nv_bfloat162 h0 = __floats2bfloat162_rn(f[8 * j + 0], f[8 * j + 1]);
@@ -257,7 +267,7 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             w.z = __float_as_uint(f[4 * j + 2]);
             w.w = __float_as_uint(f[4 * j + 3]);
           }
-          *reinterpret_cast<uint4*>(row_ptr + ((j ^ (lane & 7)) << 4)) = w;
+          *reinterpret_cast<uint4*>(row_ptr + ((j ^ swizzle) << 4)) = w;
         }
         fence_proxy_async_smem();
         __syncwarp();
@@ -289,29 +299,30 @@ int sm_count() {
   return n;
 }
 
-template <int BN, typename OutT>
+template <int TM, int BN, typename OutT>
 rocs_status_t launch(int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x, const void* W,
                      int64_t ld_w, const float* bias, const float* add, int64_t ld_add, const RequestMap& map,
                      int act, void* Y, int64_t ld_y, cudaStream_t stream, bool wait_late) {
-  using Cfg = LinearCfg<BN>;
-  constexpr int CH = 128 / (int)sizeof(OutT);
+  using Cfg = LinearCfg<TM, BN>;
+  constexpr int CH = BN * (int)sizeof(OutT) < 128 ? BN : 128 / (int)sizeof(OutT);
   // A batch of fewer rows than a tile loads no more than it has: the loads of a small batch, 64 bytes per clock and
   // SM whatever they bring, are its time (K = 1024 on one row: 408 cycles per 64-deep block with 128 rows of X and
   // 64 of W).  The other rows of the operand hold whatever the buffer held; so do their outputs, which are not stored.
-  const int32_t x_rows = (int32_t)std::min<int64_t>(BM, (M + 7) / 8 * 8);
+  const int32_t x_rows = (int32_t)std::min<int64_t>(TM, (M + 7) / 8 * 8);
   CUtensorMap map_x, map_w, map_y;
   if (!make_tensor_map_2d(&map_x, X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)M, (uint64_t)d_in, (uint64_t)ld_x,
                           (uint32_t)x_rows, BK, true) ||
       !make_tensor_map_2d(&map_w, W, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_out, (uint64_t)d_in,
                           (uint64_t)ld_w, BN, BK, true) ||
       !make_tensor_map_2d(&map_y, Y, sizeof(OutT) == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
-                          sizeof(OutT), (uint64_t)M, (uint64_t)d_out, (uint64_t)ld_y, 32, CH, true))
+                          sizeof(OutT), (uint64_t)M, (uint64_t)d_out, (uint64_t)ld_y, 32, CH, CH * sizeof(OutT) == 128,
+                          CH * sizeof(OutT) == 64))
     return ROCS_ERR_CUDA;
   uint32_t* status = device_status_word();
   if (!status) return ROCS_ERR_CUDA;
-  auto kernel = linear_umma_kernel<BN, OutT>;
+  auto kernel = linear_umma_kernel<TM, BN, OutT>;
   ROCS_ALLOW_SMEM(kernel, Cfg::kSmemBytes);
-  const int64_t tiles = ((M + BM - 1) / BM) * ((d_out + BN - 1) / BN);
+  const int64_t tiles = ((M + TM - 1) / TM) * ((d_out + BN - 1) / BN);
   const int grid = (int)std::min<int64_t>(tiles, sm_count());
   LinearParams p{M, d_in, d_out, bias, add, ld_add, map, act, x_rows, wait_late ? 1 : 0, status};
   cudaLaunchConfig_t cfg = {};
@@ -352,20 +363,37 @@ rocs_status_t umma_linear(int64_t M, int32_t d_in, int32_t d_out, const void* X,
   if (umma_linear_pair_supported(M, d_in, d_out, out_f32, add != nullptr))
     return umma_linear_pair(M, d_in, d_out, X, ld_x, W, ld_w, bias, act, Y, ld_y, stream);
   const bool wait_late = add_from_previous_launch && add != nullptr;
-#define ROCS_LAUNCH(BN_)                                                                                              \
-  (out_f32 ? launch<BN_, float>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y, stream,       \
-                                wait_late)                                                                           \
-           : launch<BN_, __nv_bfloat16>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y, stream, \
-                                        wait_late))
-  // Widest tile that still gives every SM something to do: a small batch (the request half at
-  // batch size R) is spread over more, narrower tiles instead of leaving most SMs idle.
-  const int64_t m_tiles = (M + BM - 1) / BM;
+#define ROCS_LAUNCH(TM_, BN_)                                                                                         \
+  (out_f32 ? launch<TM_, BN_, float>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y, stream,  \
+                                     wait_late)                                                                      \
+           : launch<TM_, BN_, __nv_bfloat16>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y, \
+                                             stream, wait_late))
+  // Few tiles: the one that loads least (its rows of X and of W) among those that give every tile an SM of its own.
+  // An SM loads 64 bytes per clock, which is the time of such a layer, down to about 240 cycles per K block (the
+  // products of 128 rows, however few are used, and their hand-over).  In a chain of the same layer, with 128 x 64
+  // tiles and with these: 500 x 1024 -> 1024 4.80 and 4.48 us (64 x 64), 500 x 1024 -> 256 4.63 and 4.09 (32 x 32),
+  // 741 x 512 -> 512 3.69 and 3.40, 96 x 512 -> 1024 3.54 and 3.04, 128 x 256 -> 256 2.90 and 2.43.  Measured and not
+  // taken: a tile's K blocks split over a cluster of 2 to 8 CTAs (5.64, 6.6, 4.86, 4.24, 4.26: clusters start later
+  // and hold up the next launch), the two loads of a K block issued by two warps (4.53, 4.15, 3.43, 3.09, 2.49).
   const int sms = sm_count();
-  int bn = d_out > 128 ? 256 : (d_out > 64 ? 128 : 64);
-  while (bn > 64 && m_tiles * ((d_out + bn - 1) / bn) < sms) bn /= 2;
-  if (bn == 256) return ROCS_LAUNCH(256);
-  if (bn == 128) return ROCS_LAUNCH(128);
-  return ROCS_LAUNCH(64);
+  auto tiles = [&](int tm, int bn) { return ((M + tm - 1) / tm) * ((d_out + bn - 1) / bn); };
+  int tm = 128, bn = 64;
+  int64_t least = INT64_MAX;
+  for (int t = 32; t <= 128; t *= 2)
+    for (int b = 32; b <= 64; b *= 2) {
+      const int64_t rows = std::min<int64_t>(t, (M + 7) / 8 * 8) + b;
+      if (tiles(t, b) <= sms && rows < least) { least = rows; tm = t; bn = b; }
+    }
+  if (least != INT64_MAX) {
+    if (bn == 32) return tm == 32 ? ROCS_LAUNCH(32, 32) : tm == 64 ? ROCS_LAUNCH(64, 32) : ROCS_LAUNCH(128, 32);
+    return tm == 32 ? ROCS_LAUNCH(32, 64) : tm == 64 ? ROCS_LAUNCH(64, 64) : ROCS_LAUNCH(128, 64);
+  }
+  // Otherwise the widest tile that still gives every SM something to do.
+  bn = d_out > 128 ? 256 : (d_out > 64 ? 128 : 64);
+  while (bn > 64 && tiles(128, bn) < sms) bn /= 2;
+  if (bn == 256) return ROCS_LAUNCH(128, 256);
+  if (bn == 128) return ROCS_LAUNCH(128, 128);
+  return ROCS_LAUNCH(128, 64);
 #undef ROCS_LAUNCH
 }
 

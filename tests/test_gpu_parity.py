@@ -143,6 +143,31 @@ def test_linear_few_rows_and_both_request_maps(N):
     assert _run_linear(cfg, co, bias=True, relu=True) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("M", [1, 9, 127, 130, 500])
+@pytest.mark.parametrize("d_in,d_out", [(256, 64), (264, 8), (520, 132), (1024, 60), (1048, 256), (2056, 68), (136, 1100)])
+def test_plain_linear_small_tiles(M, d_in, d_out):
+    # 32, 64 and 128 rows by 32 and 64 columns per tile, ragged last tiles in every dimension
+    g = np.random.default_rng(17 * M + d_in)
+    X = wl.store(g.standard_normal((M, d_in), dtype=np.float32), "bf16")
+    W = wl.store(g.standard_normal((d_out, d_in), dtype=np.float32) * d_in ** -0.5, "bf16")
+    b = g.standard_normal(d_out).astype(np.float32)
+    ld = rocs.padded_ld(d_out, rocs.BF16)
+    y = torch.zeros((M, ld), dtype=torch.bfloat16, device="cuda")
+    rocs.linear(to_dev(X), to_dev(W), bias=to_dev(b), relu=True, out=y[:, :d_out])
+    want = ref.ikbo_linear(wl.offsets_from_counts([M]), None, X, W, bias=b, relu=True)
+    assert rel_err(to_host_f64(y[:, :d_out]), want) <= tol_for("bf16")
+    assert torch.all(y[:, d_out:] == 0)
+
+
+@pytest.mark.parametrize("N", [1, 40, 129, 300])
+def test_linear_halves_in_small_tiles(N):
+    # the request half in fp32 tiles of 32 columns, the candidate half waiting for it in its epilogue only
+    counts = [0, N // 3, 1, 0, N - N // 3 - 1, 0] if N > 1 else [0, 1]
+    co = wl.offsets_from_counts(counts)
+    cfg = wl.CONFIGS[2].with_(R=len(counts), d_req=1032, d_cand=520, d_out=200)
+    assert _run_linear(cfg, co, bias=True, relu=True) <= tol_for("bf16")
+
+
 def test_linear_empty_batch():
     co = np.zeros(3, np.int32)
     cfg = wl.CONFIGS[2].with_(R=2, d_req=64, d_cand=64, d_out=64)
