@@ -271,7 +271,8 @@ struct FmParams {
   int64_t N;
   int32_t n_r, n_c, k, num_tiles, stages;
   const __nv_bfloat16* P;        // [n_r + n_c, k]
-  RequestMap map;
+  const int32_t* offsets;        // [R + 1]
+  int32_t R;
   const float* TT;               // [R, k, d]
   __nv_bfloat16* FC;             // [N, n_c, k]
   uint32_t* status;
@@ -377,16 +378,17 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
     int32_t cached_req = -1;
     int s = 0;
     uint32_t phase = 0;
-    // the request of this warp's candidate, fetched one tile ahead of its use (the load would
+    // the request of this warp's candidate, found one tile ahead of its use (the load would
     // otherwise sit on every candidate's critical path)
     int32_t r_next = 0;
+    RequestWalk walk{p.offsets, p.R};
     if (tile_begin < tile_end && (int64_t)tile_begin * kTileCands + warp < p.N)
-      r_next = p.map.of((int64_t)tile_begin * kTileCands + warp);
+      r_next = walk.of((int64_t)tile_begin * kTileCands + warp);
     for (int32_t t = tile_begin; t < tile_end; ++t) {
       const int32_t r = r_next;
       {
         const int64_t cand_next = (int64_t)(t + 1) * kTileCands + warp;
-        if (t + 1 < tile_end && cand_next < p.N) r_next = p.map.of(cand_next);
+        if (t + 1 < tile_end && cand_next < p.N) r_next = walk.of(cand_next);
       }
       if (!mbar_wait(&full[s], phase, abort_flag, p.status, kStatusFm | 2)) break;
       const int64_t cand = (int64_t)t * kTileCands + warp;
@@ -470,7 +472,7 @@ int sm_count_fm() {
 }
 
 template <int D, int KT, bool FULL>
-rocs_status_t launch_fm_mma_as(const rocs_plan* plan, const RequestMap& map, int32_t n_r, int32_t n_c, int32_t k,
+rocs_status_t launch_fm_mma_as(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t k,
                                const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
   const int stage_bytes = D / 64 * kTileCands * n_c * 128;
   constexpr int kFixed = kFragRows * 128 + 2 * kMaxStages * 8 + 16;
@@ -488,7 +490,8 @@ rocs_status_t launch_fm_mma_as(const rocs_plan* plan, const RequestMap& map, int
   p.num_tiles = (int32_t)((plan->N + kTileCands - 1) / kTileCands);
   p.stages = std::min(kMaxStages, (227 * 1024 - kFixed) / stage_bytes);
   p.P = (const __nv_bfloat16*)P;
-  p.map = map;
+  p.offsets = plan->cand_offsets;
+  p.R = plan->R;
   p.TT = TT;
   p.FC = (__nv_bfloat16*)FC;
   p.status = status;
@@ -512,11 +515,11 @@ rocs_status_t launch_fm_mma_as(const rocs_plan* plan, const RequestMap& map, int
 }
 
 template <int D>
-rocs_status_t launch_fm_mma(const rocs_plan* plan, const RequestMap& map, int32_t n_r, int32_t n_c, int32_t k,
+rocs_status_t launch_fm_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t k,
                             const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
-  if (k > 16) return launch_fm_mma_as<D, 2, false>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
-  if (n_c < kFragRows) return launch_fm_mma_as<D, 1, false>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
-  return launch_fm_mma_as<D, 1, true>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
+  if (k > 16) return launch_fm_mma_as<D, 2, false>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+  if (n_c < kFragRows) return launch_fm_mma_as<D, 1, false>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+  return launch_fm_mma_as<D, 1, true>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
 }
 
 template <typename T>
@@ -529,12 +532,6 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
   if (smem_r > kMaxSmem || smem_c > kMaxSmem) return ROCS_ERR_UNSUPPORTED;
   const size_t n_rp = (size_t)(n_r + 15) / 16 * 16, kp = (size_t)(k + 15) / 16 * 16;
   const size_t smem_mma = n_rp * ((size_t)(d + 8) * 2 + (kp + 8) * 2) + 2 * kp * (size_t)(d + 8) * 2;
-  // in front of the request kernel: the candidate kernel may start beside that one and reads the map at once
-  RequestMap map;
-  if (plan->N > 0 && FC) {
-    const rocs_status_t st = plan_request_map(plan, stream, &map);
-    if (st != ROCS_OK) return st;
-  }
   if (plan->R > 0 && tensor_core_request && sizeof(T) == 2 && d % 16 == 0 && k % 8 == 0 && smem_mma <= kMaxSmem) {
     ROCS_ALLOW_SMEM(fm_request_mma_kernel, kMaxSmem);
     const rocs_status_t st = launch_dependent(fm_request_mma_kernel, dim3((unsigned)plan->R), 256, smem_mma, stream, n_r, d, k,
@@ -549,13 +546,16 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
   if (plan->N == 0 || !FC) return ROCS_OK;
   if (fast_candidates) {
     switch (d) {
-      case 64: return launch_fm_mma<64>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
-      case 128: return launch_fm_mma<128>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
-      case 192: return launch_fm_mma<192>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
-      case 256: return launch_fm_mma<256>(plan, map, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 64: return launch_fm_mma<64>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 128: return launch_fm_mma<128>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 192: return launch_fm_mma<192>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 256: return launch_fm_mma<256>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
       default: break;
     }
   }
+  RequestMap map;
+  const rocs_status_t st = plan_request_map(plan, stream, &map);
+  if (st != ROCS_OK) return st;
   ROCS_ALLOW_SMEM(fm_candidate_simt_kernel<T>, kMaxSmem);
   return launch_dependent(fm_candidate_simt_kernel<T>, dim3((unsigned)plan->N), 128, smem_c, stream, n_r, n_c, d, k,
                           (const T*)XC, (const T*)P, map, (const float*)TT, (T*)FC);

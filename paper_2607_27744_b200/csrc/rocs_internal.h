@@ -132,6 +132,30 @@ struct RequestMap {
   }
 #endif
 };
+// The same for a thread whose rows ascend.  The end of the request behind is loaded with a request's own, long before
+// it is compared with: no load is waited for unless a request is skipped, which takes a search.  For the streaming
+// interaction kernel in place of a table, which is a launch of its own: plan and projected interaction of 112 requests
+// x 454 candidates 31.8 us with the table, 24.4 us with this (a load of the next end when it is needed: 24.7 us).
+struct RequestWalk {
+  const int32_t* offsets;  // [R + 1]
+  int32_t R;
+  int32_t r = -1, end = 0, next_end = -1;
+#ifdef __CUDACC__
+  __device__ __forceinline__ int32_t of(int64_t row) {
+    if (row >= end) {
+      if (row < next_end) {
+        ++r;
+        end = next_end;
+      } else {
+        r = RequestMap{nullptr, offsets, R}.of(row);
+        end = offsets[r + 1];
+      }
+      next_end = offsets[min(r + 2, R)];
+    }
+    return r;
+  }
+#endif
+};
 // Up to this many candidates the kernels search for a row's request themselves: the table is a launch of its own
 // in front of them (about 2 us of a 24 us tower on 500 candidates, and host time), the search a handful of
 // cached loads per row; with more rows the loads add up and the launch does not.
