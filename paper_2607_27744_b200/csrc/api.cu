@@ -15,19 +15,23 @@ namespace {
 std::atomic<int> g_path{ROCS_PATH_AUTO};
 
 // m_i of Section 4.1 from the segment offsets: one thread per candidate, binary search.
+// beside: the kernel in front may still run.  It waited for everything in front of itself before it released this one
+// and touches neither the offsets nor the table; this grid completes behind it, so that the next need wait for this
+// one only.
 __global__ void fill_row2req_kernel(int32_t R, int64_t N, const int32_t* __restrict__ off,
-                                    int32_t* __restrict__ row2req) {
-  // the first layer's kernel may set itself up beside this one; it waits for this grid before it reads anything
-  ptx::griddep_wait_for(off);
+                                    int32_t* __restrict__ row2req, bool beside) {
+  if (!beside) ptx::griddep_wait_for(off);
   ptx::griddep_launch_dependents();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  int32_t lo = 0, hi = R;  // largest r with off[r] <= i
-  while (hi - lo > 1) {
-    const int32_t mid = lo + (hi - lo) / 2;
-    if (off[mid] <= i) lo = mid; else hi = mid;
+  if (i < N) {
+    int32_t lo = 0, hi = R;  // largest r with off[r] <= i
+    while (hi - lo > 1) {
+      const int32_t mid = lo + (hi - lo) / 2;
+      if (off[mid] <= i) lo = mid; else hi = mid;
+    }
+    row2req[i] = lo;
   }
-  row2req[i] = lo;
+  if (beside) ptx::griddep_wait();
 }
 
 bool row_stride_ok(int64_t ld, int64_t min_cols, rocs_dtype_t dt) {
@@ -170,13 +174,13 @@ int64_t plan_entries(const rocs_plan* plan, int32_t cands_per_tile) {
 // Allocates and fills one list of the plan (key as in rocs_plan::lists) in the order of `stream`, from the
 // offsets at `off`.
 static rocs_status_t make_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, const int32_t* off,
-                               cudaStream_t stream, DeviceList* out) {
+                               cudaStream_t stream, DeviceList* out, bool beside = false) {
   static_assert(sizeof(Tile) == 16 && sizeof(DcaItem) == 16, "list entries");
   DeviceList list;
   if (plan->N > 0 && cands_per_tile == 0) {
     ROCS_CUDA_TRY(pool_alloc(&list.dev, sizeof(int32_t) * (size_t)plan->N, stream));
     if (launch_dependent(fill_row2req_kernel, dim3((unsigned)((plan->N + 255) / 256)), 256, 0, stream, plan->R, plan->N, off,
-                         static_cast<int32_t*>(list.dev)) != ROCS_OK) {
+                         static_cast<int32_t*>(list.dev), beside) != ROCS_OK) {
       cudaFreeAsync(list.dev, stream);
       return ROCS_ERR_CUDA;
     }
@@ -246,7 +250,7 @@ static unsigned long long capture_of(cudaStream_t stream) {  // 0: the stream is
 }
 
 static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, cudaStream_t stream,
-                               DeviceList* out) {
+                               DeviceList* out, bool beside = false) {
   const unsigned long long capture = capture_of(stream);
   std::lock_guard<std::mutex> lock(plan->mu);
   if (capture != 0 && capture != plan->capture) {
@@ -269,12 +273,12 @@ static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, in
     *out = it->second;
     return ROCS_OK;
   }
-  const rocs_status_t st = make_list(plan, cands_per_tile, heads, plan->cand_offsets, stream, out);
+  const rocs_status_t st = make_list(plan, cands_per_tile, heads, plan->cand_offsets, stream, out, beside);
   if (st == ROCS_OK) plan->lists[key] = *out;
   return st;
 }
 
-rocs_status_t plan_request_map(const rocs_plan* plan, cudaStream_t stream, RequestMap* out) {
+rocs_status_t plan_request_map(const rocs_plan* plan, cudaStream_t stream, RequestMap* out, bool beside) {
   *out = RequestMap{};
   if (plan->N <= kSearchRows) {
     out->offsets = plan->cand_offsets;
@@ -282,7 +286,7 @@ rocs_status_t plan_request_map(const rocs_plan* plan, cudaStream_t stream, Reque
     return ROCS_OK;
   }
   DeviceList list;
-  const rocs_status_t st = plan_list(plan, 0, 0, stream, &list);
+  const rocs_status_t st = plan_list(plan, 0, 0, stream, &list, beside);
   out->row2req = static_cast<const int32_t*>(list.dev);
   return st;
 }
@@ -454,13 +458,13 @@ static rocs_status_t ikbo_linear_impl(const rocs_plan_t* plan, rocs_dtype_t dtyp
     const size_t need = z_bytes;
     if (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255u))
       return ROCS_ERR_WORKSPACE;
-    // In front of the request half: the candidate kernel may start beside that one and reads the map at once.
-    rocs_status_t st = plan_request_map(plan, stream, &map);
-    if (st != ROCS_OK) return st;
     // Request half, once per request (Section 4.1): Z = X^R W_CR^T + bias, fp32.
-    st = linear_dispatch(dtype, plan->R, d_req, d_out, XR, ld_xr, W_CR, ld_wcr, bias,
+    rocs_status_t st = linear_dispatch(dtype, plan->R, d_req, d_out, XR, ld_xr, W_CR, ld_wcr, bias,
                                        nullptr, 0, RequestMap{}, ROCS_ACT_NONE, workspace, d_out,
                                        /*out_f32=*/true, stream);
+    if (st != ROCS_OK) return st;
+    // The map beside it, on the SMs that it leaves idle; the candidate kernel waits for both before it reads either.
+    st = plan_request_map(plan, stream, &map, /*beside=*/plan->R > 0);
     if (st != ROCS_OK) return st;
     Z = (const float*)workspace;
     bias = nullptr;

@@ -50,7 +50,7 @@ struct Ws2Params {
   int64_t ld_add;
   RequestMap map;
   int32_t act;
-  int32_t wait_for_previous;  // launched with programmatic serialization behind the kernel that writes `add`
+  int32_t wait_for_previous;  // nothing but `add` and the map is written by the launches right in front
   float2* stat_partials;      // [M][2 n_slices] (sum, sum of squares) of each row's 128 columns per epilogue warp, or NULL
   uint32_t* status;
 };
@@ -123,6 +123,10 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   cluster_sync_all();  // barriers of both CTAs are initialised before anything signals across the pair
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_ptr;
+  // The set-up above may overlap the end of the kernel in front.  Behind the request half alone, the weights and the
+  // rows are streamed at once; that kernel is waited for where its rows are read.  (Launched plainly where there is
+  // no request half, 20000 x 256 -> 512 in a chain: 12.3 us, 9.2 us like this.)
+  if (!p.wait_for_previous) griddep_wait();
   // A kernel launched behind this one as a programmatic dependent (the next layer) may set itself up as
   // SMs become free; it waits for this whole grid before it touches global memory.
   griddep_launch_dependents();
@@ -145,8 +149,8 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
           req_next[q] = p.map.of(r0);
         }
       };
-      if (has_add && group < super_tiles) fetch_req(group);
       bool previous_done = !p.wait_for_previous;
+      if (has_add && previous_done && group < super_tiles) fetch_req(group);
       for (int32_t st = group; st < super_tiles && ok; st += p.groups, ++lt) {
         const int32_t m0 = st * 2 * BM + (int32_t)rank * BM;
         // X first: the MMA needs it now; the request rows are only needed by this tile's epilogue
@@ -160,9 +164,10 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         if (has_add) {
           const uint32_t zb = lt % kZBufs;
           if (!mbar_wait(&z_empty[zb], ((lt / kZBufs) & 1) ^ 1, abort_flag, p.status, kStatusWs2 | 5)) { ok = false; break; }
-          if (!previous_done) {  // the request half must have finished before its rows are read
+          if (!previous_done) {  // the request half and the map must have finished before they are read
             griddep_wait();
             previous_done = true;
+            fetch_req(st);
           }
           mbar_expect_tx(&z_full[zb], kZBufBytes);
 #pragma unroll
@@ -215,6 +220,7 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     const uint32_t tmem_empty_leader[2] = {map_to_cta(smem_u32(&tmem_empty[0]), 0),
                                            map_to_cta(smem_u32(&tmem_empty[1]), 0)};
     uint32_t lt = 0;
+    if (p.wait_for_previous) griddep_wait();
     for (int32_t st = group; st < super_tiles; st += p.groups, ++lt) {
       const uint32_t acc = lt & 1;
       const int32_t m0 = st * 2 * BM + (int32_t)rank * BM;
@@ -392,7 +398,7 @@ rocs_status_t umma_linear_ws2(int64_t M, int32_t d_in, int32_t d_out, const void
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = p.wait_for_previous ? 1 : 0;
+  cfg.numAttrs = 1;
   ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, linear_ws2_kernel, map_x, map_w, map_z, map_y, p));
   return ROCS_OK;
 }
