@@ -182,8 +182,9 @@ __global__ void __launch_bounds__(kGlmThreads) glm_candidate_simt_kernel(
     T* out = YC + (int64_t)tile.cand0 * n_c * n;
     for (int32_t e = tid; e < rows * n; e += kGlmThreads) st_f(out, e, yc[e]);
   }
+  // Launched beside the request kernel: its ZR is read from here on, and whoever waits for this grid counts on both.
+  ptx::griddep_wait();
   if (!compress) return;
-  ptx::griddep_wait();  // launched beside the request kernel: its ZR is read from here on
   const float* zr = ZR + (int64_t)tile.req * n_co * n;
   T* out = OC + (int64_t)tile.cand0 * n_co * n;
   for (int32_t e = tid; e < tile.count * n; e += kGlmThreads) {
