@@ -299,6 +299,13 @@ rocs_status_t plan_tiles(const rocs_plan* plan, int32_t cands_per_tile, cudaStre
   return st;
 }
 
+rocs_status_t plan_tile_runs(const rocs_plan* plan, int32_t cands_per_tile, cudaStream_t stream, TileList* out) {
+  const int64_t total = plan_entries(plan, cands_per_tile);
+  if (plan->R > kMaxTileWalkRequests || total > kMaxTileWalk) return plan_tiles(plan, cands_per_tile, stream, out);
+  *out = TileList{nullptr, (int32_t)total};
+  return ROCS_OK;
+}
+
 rocs_status_t plan_dca_items(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, cudaStream_t stream,
                              DcaItemList* out) {
   if (cands_per_tile < 1 || heads < 1) return ROCS_ERR_INVALID_ARG;
@@ -618,7 +625,7 @@ rocs_status_t rocs_glm_interaction(const rocs_plan_t* plan, rocs_dtype_t dtype, 
     TileList tiles;
     rocs_status_t st = !YC && !OC ? ROCS_OK
                        : mma      ? glm_mma_tiles(plan, n_r, n_c, d, stream, &tiles)
-                                  : plan_tiles(plan, 128 / n_c, stream, &tiles);
+                                  : plan_tile_runs(plan, 128 / n_c, stream, &tiles);
     if (st != ROCS_OK) return st;
     // Request side once per request (tiny), candidate side on tensor cores.
     st = glm_request_mma_supported(n_r, d, n_ro, n_co)

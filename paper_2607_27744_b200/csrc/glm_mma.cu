@@ -39,12 +39,12 @@ constexpr int kGroups = 2;  // 16-column groups of the request block per pass
 constexpr uint32_t kStatusGlmMma = 0x800;
 
 struct GlmMmaParams {
-  const Tile* tiles;
-  int32_t num_tiles;
+  const Tile* tiles;       // the list, or null
+  const int32_t* offsets;  // [R + 1]
+  int32_t R, tile_cands, num_tiles;
   int32_t n_r, n_c, d, n_ro, n_co;
   int32_t frags, frag_cands;  // fragments per tile, whole candidates per fragment
   int32_t stages, stage_bytes, tx_bytes, slab_bytes, xr_bytes, xr_slab_bytes;
-  int32_t zr_from_previous_launch;
   const __nv_bfloat16* W;  // [n_ro + n_co, n]
   const float* ZR;         // [R, n_co, n]
   __nv_bfloat16* YC;       // [N, n_c, n] or null
@@ -96,7 +96,8 @@ __device__ __forceinline__ void product(Acc& acc, const uint32_t (&frag)[4], con
 }
 
 // CO8: blocks of 8 compressed outputs (0: no compression).
-template <int CO8, bool RAW>
+// WALK: the tiles are found in the offsets, otherwise read from the list.
+template <int CO8, bool RAW, bool WALK>
 __global__ void __launch_bounds__(kThreads, 1)
 glm_mma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant__ CUtensorMap map_xc,
                const GlmMmaParams p) {
@@ -131,6 +132,8 @@ glm_mma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant
   const int32_t slabs = p.d / 64;
   const int32_t t_begin = (int32_t)((int64_t)blockIdx.x * p.num_tiles / gridDim.x);
   const int32_t t_end = (int32_t)((int64_t)(blockIdx.x + 1) * p.num_tiles / gridDim.x);
+  TileWalk walk{p.offsets, p.R, p.tile_cands};
+  if constexpr (WALK) walk.start(t_begin, lane);
 
   if (warp == kWarps) {
     // ------------------------------ TMA producer ------------------------------------------
@@ -140,10 +143,10 @@ glm_mma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant
       int s = 0;
       uint32_t phase = 0, it = 0, n_req = 0;
       int32_t req = -1;
-      Tile next = t_begin < t_end ? p.tiles[t_begin] : Tile{};
+      Tile next = !WALK && t_begin < t_end ? p.tiles[t_begin] : Tile{};
       for (int32_t t = t_begin; t < t_end; ++t, ++it) {
-        const Tile tile = next;
-        if (t + 1 < t_end) next = p.tiles[t + 1];
+        const Tile tile = WALK ? walk.take(t + 1 < t_end) : next;
+        if (!WALK && t + 1 < t_end) next = p.tiles[t + 1];
         if (tile.req != req) {
           const uint32_t x = n_req & 1;
           if (!mbar_wait(&xr_empty[x], ((n_req >> 1) & 1) ^ 1, abort_flag, p.status, kStatusGlmMma | 1)) break;
@@ -199,15 +202,15 @@ glm_mma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant
       }
     }
   }
-  bool zr_ready = !p.zr_from_previous_launch;
+  bool zr_ready = false;
   int s = 0;
   uint32_t phase = 0, n_req = 0;
   int32_t req = -1;
   uint32_t xr_slot = 0;
-  Tile next = t_begin < t_end ? p.tiles[t_begin] : Tile{};
+  Tile next = !WALK && t_begin < t_end ? p.tiles[t_begin] : Tile{};
   for (int32_t t = t_begin; t < t_end; ++t) {
-    const Tile tile = next;
-    if (t + 1 < t_end) next = p.tiles[t + 1];
+    const Tile tile = WALK ? walk.take(t + 1 < t_end) : next;
+    if (!WALK && t + 1 < t_end) next = p.tiles[t + 1];
     if (tile.req != req) {
       __syncwarp();
       if (req >= 0 && lane == 0) mbar_arrive(&xr_empty[xr_slot]);
@@ -331,6 +334,7 @@ glm_mma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant
     if (lane == 0) mbar_arrive(&empty[s]);
     if (++s == p.stages) { s = 0; phase ^= 1; }
   }
+  if (!zr_ready) griddep_wait();  // complete only behind the request kernel, for whoever waits for this grid
 }
 
 int sm_count_glm_mma() {
@@ -373,7 +377,7 @@ bool glm_mma_supported(int32_t n_r, int32_t n_c, int32_t d, int32_t n_co) {
 }
 
 rocs_status_t glm_mma_tiles(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, cudaStream_t stream, TileList* out) {
-  return plan_tiles(plan, layout(n_r, n_c, d).tile_cands, stream, out);
+  return plan_tile_runs(plan, layout(n_r, n_c, d).tile_cands, stream, out);
 }
 
 rocs_status_t glm_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, const void* XR, const void* XC,
@@ -384,7 +388,7 @@ rocs_status_t glm_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d
   if (!compress && YC == nullptr) return ROCS_OK;
   const Layout L = layout(n_r, n_c, d);
   TileList tl;
-  const rocs_status_t st = plan_tiles(plan, L.tile_cands, stream, &tl);
+  const rocs_status_t st = plan_tile_runs(plan, L.tile_cands, stream, &tl);
   if (st != ROCS_OK) return st;
   if (tl.num == 0) return ROCS_OK;
   CUtensorMap map_xr, map_xc;
@@ -397,6 +401,9 @@ rocs_status_t glm_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d
   if (!status) return ROCS_ERR_CUDA;
   GlmMmaParams p{};
   p.tiles = tl.dev;
+  p.offsets = plan->cand_offsets;
+  p.R = plan->R;
+  p.tile_cands = L.tile_cands;
   p.num_tiles = tl.num;
   p.n_r = n_r; p.n_c = n_c; p.d = d; p.n_ro = n_ro; p.n_co = n_co;
   p.frags = L.frags; p.frag_cands = L.frag_cands;
@@ -406,8 +413,7 @@ rocs_status_t glm_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d
   p.YC = (__nv_bfloat16*)YC; p.OC = (__nv_bfloat16*)OC;
   p.status = status;
   // The request kernel runs directly in front on the same stream and releases its dependents at once:
-  // this kernel streams X^C beside it and waits for it only before it reads ZR.
-  p.zr_from_previous_launch = compress ? 1 : 0;
+  // this kernel streams X^C beside it and waits for it only before it reads ZR, if it does.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)std::min(tl.num, sm_count_glm_mma()));
   cfg.blockDim = dim3(kThreads);
@@ -417,13 +423,18 @@ rocs_status_t glm_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = p.zr_from_previous_launch ? 1 : 0;
-#define ROCS_GLM_LAUNCH(C_, R_)                                                  \
+  cfg.numAttrs = 1;
+#define ROCS_GLM_LAUNCH_AS(...)                                                  \
   do {                                                                           \
-    auto kernel = glm_mma_kernel<C_, R_>;                                        \
+    auto kernel = glm_mma_kernel<__VA_ARGS__>;                                   \
     ROCS_ALLOW_SMEM(kernel, kMaxDynamicSmem);                                    \
     ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, map_xr, map_xc, p));          \
     return ROCS_OK;                                                              \
+  } while (0)
+#define ROCS_GLM_LAUNCH(C_, R_)                                                  \
+  do {                                                                           \
+    if (tl.dev == nullptr) ROCS_GLM_LAUNCH_AS(C_, R_, true);                     \
+    ROCS_GLM_LAUNCH_AS(C_, R_, false);                                           \
   } while (0)
   if (!compress) ROCS_GLM_LAUNCH(0, true);
   if (n_co <= 8 && YC) ROCS_GLM_LAUNCH(1, true);
@@ -431,6 +442,7 @@ rocs_status_t glm_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d
   if (YC) ROCS_GLM_LAUNCH(2, true);
   ROCS_GLM_LAUNCH(2, false);
 #undef ROCS_GLM_LAUNCH
+#undef ROCS_GLM_LAUNCH_AS
 }
 
 }  // namespace rocs

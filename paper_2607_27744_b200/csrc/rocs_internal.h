@@ -156,6 +156,62 @@ struct RequestWalk {
   }
 #endif
 };
+// A run of consecutive interaction tiles found in the offsets and walked like the above, in place of the plan's list.
+// Making the list is a launch in front of the request kernel, which a small batch feels and a large one does not: a
+// block of 8 requests x 697 candidates (attention's list made in its kernel too) 40.0 us with lists and 35.4 without,
+// one of 2 x 17 36.4 and 26.0; 128 x 1024 candidates (16384 tiles) 127.0 us with the list and 130.7 walked, the walk
+// being on every warp's path from tile to tile.  (One kernel for both ran the list in 136.4 us for 132.0: two instantiations.)
+constexpr int32_t kMaxTileWalk = 2400;         // tiles: 16 per CTA, for about half of what the launch costs
+constexpr int32_t kMaxTileWalkRequests = 512;  // the first tile takes two loads per 32 requests
+struct TileWalk {
+  const int32_t* offsets;  // [R + 1]
+  int32_t R, per;          // requests, candidates per tile
+  Tile next = {0, 0, 0, 0};
+  int32_t end = 0, next_end = 0;
+#ifdef __CUDACC__
+  // Finds tile t; all lanes of a warp take part.
+  __device__ __forceinline__ void start(int32_t t, int lane) {
+    const int32_t chunk = (R + 31) / 32, r0 = min(lane * chunk, R), r1 = min(r0 + chunk, R);
+    int32_t sum = 0;
+    for (int32_t r = r0; r < r1; ++r) sum += (offsets[r + 1] - offsets[r] + per - 1) / per;
+    int32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += up;
+    }
+    const uint32_t hit = __ballot_sync(0xffffffffu, incl - sum <= t && t < incl);
+    if (hit == 0) return;
+    const int src = __ffs(hit) - 1;
+    int32_t r = __shfl_sync(0xffffffffu, r0, src), local = t - __shfl_sync(0xffffffffu, incl - sum, src), first, n;
+    while (true) {
+      first = offsets[r];
+      end = offsets[r + 1];
+      n = (end - first + per - 1) / per;
+      if (local < n) break;
+      local -= n;
+      ++r;
+    }
+    next_end = offsets[min(r + 2, R)];
+    const int32_t c = first + local * per;
+    next = Tile{r, c, min(per, end - c), 0};
+  }
+  // The tile at hand; moves on to the next one if there is `more`.
+  __device__ __forceinline__ Tile take(bool more) {
+    const Tile t = next;
+    if (!more) return t;
+    next.cand0 += per;
+    while (next.cand0 >= end) {  // the end of a request: on to the next that has candidates
+      ++next.req;
+      next.cand0 = end;
+      end = next_end;
+      next_end = offsets[min(next.req + 2, R)];
+    }
+    next.count = min(per, end - next.cand0);
+    return t;
+  }
+#endif
+};
 // Up to this many candidates the kernels search for a row's request themselves: the table is a launch of its own
 // in front of them (about 2 us of a 24 us tower on 500 candidates, and host time), the search a handful of
 // cached loads per row; with more rows the loads add up and the launch does not.
@@ -165,6 +221,8 @@ constexpr int64_t kSearchRows = 16384;
 // 46262 candidates of 96 requests: 97.1 us behind it, 96.0 beside it).  The kernel behind must wait before it reads the map.
 rocs_status_t plan_request_map(const rocs_plan* plan, cudaStream_t stream, RequestMap* out, bool beside = false);
 
+// The tiles of a launch whose CTAs take contiguous runs of them: `out` without a list where they can be walked.
+rocs_status_t plan_tile_runs(const rocs_plan* plan, int32_t cands_per_tile, cudaStream_t stream, TileList* out);
 // Returns the cached tile list for `cands_per_tile`, building it on first use.
 rocs_status_t plan_tiles(const rocs_plan* plan, int32_t cands_per_tile, cudaStream_t stream,
                          TileList* out);

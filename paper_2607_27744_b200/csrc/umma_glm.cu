@@ -35,19 +35,20 @@ constexpr uint32_t kStatusGlm = 0x200;
 constexpr int kAccStride = 256;  // TMEM columns per accumulator
 
 struct GlmParams {
-  const Tile* tiles;
-  int32_t num_tiles;
+  const Tile* tiles;       // the list, or null
+  const int32_t* offsets;  // [R + 1]
+  int32_t R, num_tiles;
   int32_t n_r, n_r_pad, n_c, d, n_ro, n_co;
   int32_t stages, stage_bytes, group_staging_bytes, yc_stride;
   const __nv_bfloat16* W;  // [n_ro + n_co, n] or null
   const float* ZR;         // [R, n_co, n] or null
-  int32_t zr_from_previous_launch;  // launched as a programmatic dependent of the kernel that writes ZR
   __nv_bfloat16* YC;       // [N, n_c, n] or null
   __nv_bfloat16* OC;       // [N, n_co, n] or null
   uint32_t* status;
 };
 
-template <int NC>
+// WALK: the tiles are found in the offsets, otherwise read from the list.
+template <int NC, bool WALK>
 __global__ void __launch_bounds__(kThreads, 1)
 glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant__ CUtensorMap map_xc,
                 const GlmParams p) {
@@ -93,6 +94,8 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_ptr;
+  TileWalk walk{p.offsets, p.R, 128 / NC};
+  if (WALK && warp != 1) walk.start(t_begin, lane);
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------------------
@@ -102,7 +105,7 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
       uint32_t it = 0;
       bool ok = true;
       for (int32_t t = t_begin; t < t_end; ++t, ++it) {
-        const Tile tile = p.tiles[t];
+        const Tile tile = WALK ? walk.take(t + 1 < t_end) : p.tiles[t];
         const int s = it % p.stages;
         if (!mbar_wait(&empty[s], ((it / p.stages) & 1) ^ 1, abort_flag, p.status, kStatusGlm | 1)) { ok = false; break; }
         uint8_t* st = smem + s * p.stage_bytes;
@@ -160,7 +163,7 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
     uint8_t* yc_w = staging + g * p.group_staging_bytes + q * 32 * p.yc_stride;
     uint8_t* my = yc_w + lane * p.yc_stride;
     const bool compress = p.W != nullptr && p.OC != nullptr;
-    bool zr_ready = !p.zr_from_previous_launch;
+    bool zr_ready = false;
     // A fragments of W_CC for mma.m16n8k16 (rows = outputs o, padded to 16; cols = a, padded to
     // 16 per K step): a0 = (g8, 2t..), a1 = (g8+8, 2t..), a2 = (g8, 2t+8..), a3 = (g8+8, 2t+8..)
     constexpr int KS = (NC + 15) / 16;
@@ -184,8 +187,10 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
     }
     uint32_t it = 0;
     for (int32_t t = t_begin; t < t_end; ++t, ++it) {
+      Tile tile;
+      if (WALK) tile = walk.take(t + 1 < t_end);
       if ((int)(it & 1) != g) continue;
-      const Tile tile = p.tiles[t];
+      if (!WALK) tile = p.tiles[t];
       if (!mbar_wait(&tmem_full[g], (it >> 1) & 1, abort_flag, p.status, kStatusGlm | 4)) break;
       tc_fence_after_sync();
       const uint32_t t_row = tmem_base + g * kAccStride + ((uint32_t)(q * 32) << 16);
@@ -306,6 +311,7 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
       }
       __syncwarp();  // the row buffer is rewritten by this warp's next tile
     }
+    if (!zr_ready) griddep_wait();  // complete only behind the request kernel, for whoever waits for this grid
   }
 
   tc_fence_before_sync();
@@ -365,7 +371,7 @@ rocs_status_t umma_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t 
                        const float* zr_workspace, cudaStream_t stream) {
   if (plan->N == 0) return ROCS_OK;
   TileList tl;
-  rocs_status_t st = plan_tiles(plan, 128 / n_c, stream, &tl);
+  rocs_status_t st = plan_tile_runs(plan, 128 / n_c, stream, &tl);
   if (st != ROCS_OK) return st;
   if (tl.num == 0) return ROCS_OK;
   const GlmLayout L = glm_layout(n_r, n_c, d, n_co);
@@ -379,6 +385,8 @@ rocs_status_t umma_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t 
   if (!status) return ROCS_ERR_CUDA;
   GlmParams p{};
   p.tiles = tl.dev;
+  p.offsets = plan->cand_offsets;
+  p.R = plan->R;
   p.num_tiles = tl.num;
   p.n_r = n_r; p.n_r_pad = L.n_r_pad; p.n_c = n_c; p.d = d; p.n_ro = n_ro; p.n_co = n_co;
   p.stages = L.stages; p.stage_bytes = L.stage_bytes; p.group_staging_bytes = L.group_staging_bytes;
@@ -388,8 +396,7 @@ rocs_status_t umma_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t 
   p.status = status;
   const int grid = std::min(tl.num, sm_count_glm());
   // The request kernel runs directly in front on the same stream and releases its dependents at once:
-  // this kernel sets itself up and streams X^C beside it and waits for it only before it reads ZR.
-  p.zr_from_previous_launch = (zr_workspace != nullptr && W != nullptr && OC != nullptr) ? 1 : 0;
+  // this kernel sets itself up and streams X^C beside it and waits for it only before it reads ZR, if it does.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kThreads);
@@ -399,11 +406,16 @@ rocs_status_t umma_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t 
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = p.zr_from_previous_launch ? 1 : 0;
+  cfg.numAttrs = 1;
 #define ROCS_GLM_LAUNCH(NC_)                                                                                  \
   do {                                                                                                        \
-    ROCS_ALLOW_SMEM(glm_umma_kernel<NC_>, kMaxSmem);                                                          \
-    ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, glm_umma_kernel<NC_>, map_xr, map_xc, p));                         \
+    if (tl.dev == nullptr) {                                                                                  \
+      ROCS_ALLOW_SMEM((glm_umma_kernel<NC_, true>), kMaxSmem);                                                \
+      ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, glm_umma_kernel<NC_, true>, map_xr, map_xc, p));                 \
+    } else {                                                                                                  \
+      ROCS_ALLOW_SMEM((glm_umma_kernel<NC_, false>), kMaxSmem);                                               \
+      ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, glm_umma_kernel<NC_, false>, map_xr, map_xc, p));                \
+    }                                                                                                         \
   } while (0)
   if (n_c == 8) ROCS_GLM_LAUNCH(8);
   else if (n_c == 16) ROCS_GLM_LAUNCH(16);

@@ -5,8 +5,8 @@
 // tensor never exists.
 //
 // One persistent CTA per SM, 6 warps:
-//   warp 0   TMA producer: 128 x 64 tiles of X and BN x 64 tiles of W into a shared-memory ring
-//   warp 1   issues tcgen05.mma (128 x BN x 16, bf16 -> fp32) into one of two TMEM accumulators
+//   warp 0   TMA producer: TM x 64 tiles of X and BN x 64 tiles of W into a shared-memory ring
+//   warp 1   issues tcgen05.mma (128 x BN x 16, bf16 -> fp32) into one of two TMEM accumulators (TM rows of it used)
 //   warps 2-5 epilogue: TMEM -> registers, + Z[m_i] (+ bias), ReLU, round to the output type,
 //            128-byte-swizzled staging in shared memory, TMA store (clipped at the edges)
 // The two accumulators let the epilogue of tile t overlap the main loop of tile t + 1.

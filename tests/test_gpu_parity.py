@@ -608,6 +608,15 @@ def test_work_lists_of_many_requests(R):
     assert _run_dca(wl.CONFIGS[3].with_(R=R, H=2, dh=32), co, so) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("R", [1, 31, 33, 200, 512])
+@pytest.mark.parametrize("n_c", [8, 12])
+def test_glm_tiles_walked_in_the_offsets(R, n_c):
+    # runs of tiles that begin and end inside requests, behind partial last tiles and runs of empty requests
+    g = np.random.default_rng(R)
+    co = wl.offsets_from_counts([int(c) for c in g.choice([0, 0, 1, 7, 16, 17, 40], R - 1)] + [23])
+    assert _run_glm(wl.CONFIGS[5].with_(R=R, n_r=8, n_c=n_c, d_emb=64, n_ro=2, n_co=4), co) <= tol_for("bf16")
+
+
 def test_glm_config4_full_size_sampled():
     cfg = wl.CONFIGS[4]
     co = wl.cand_offsets(cfg)
