@@ -12,11 +12,12 @@
 // (16 x d x 16 each) run on mma.sync m16n8k16 straight out of the swizzled tile:
 //   step 1   H^T = T^T + P_C^T X^C_i    accumulators start at T^T (fp32); X^C_i is the K x N
 //                                       operand, read with ldmatrix.trans
-//   step 2   FC_i = X^C_i H             H rounded to bf16 once: the accumulator layout of step 1
-//                                       is the B-operand layout of step 2, so it never leaves
-//                                       registers; X^C_i is the M x K operand, read with ldmatrix
+//   step 2   FC_i = X^C_i H             the accumulator layout of step 1 is the B-operand layout of
+//                                       step 2, so H never leaves registers; X^C_i is the M x K
+//                                       operand, read with ldmatrix
 // A general kernel (any shape, fp32 or bf16 storage, fp32 FMA) covers everything else.
 #include <algorithm>
+#include <type_traits>
 
 #include "rocs_internal.h"
 #include "simt_util.cuh"
@@ -128,9 +129,12 @@ __global__ void __launch_bounds__(128) fm_candidate_simt_kernel(int32_t n_r, int
 // ---------------------------------------------------------------------------------------------
 // Candidate side, bf16 streaming kernel: n_c up to 16, even k up to 32, d a multiple of 64 up to 256.
 // The fragments hold 16 candidate rows: of a candidate with fewer the rest are the next candidate's, which
-// step 1 masks to zero (0 x NaN of a neighbour must not arise) and step 2 computes and drops.  Bound by HBM.
-// 18 399 candidates of 12 embeddings x 128, k = 16: the general kernel (a block per candidate) took 284 us, a
-// whole pass through this one 34 us, most of it host work.
+// step 1 masks to zero (0 x NaN of a neighbour must not arise) and step 2 computes and drops.
+// 16 embeddings and 8 or 16 columns (FULL) round H to bf16 and are bound by HBM.  Every other shape takes H as a bf16 pair
+// (value and remainder) through two products in step 2, and is bound by the products: error of FC against 64 bits on 128
+// requests x 1024 candidates, 32 + 12 embeddings x 128, k = 16, 1.6568e-3 as with fp32 FMA throughout (all of it the
+// rounding of FC) at 128.6 us; 1.8657e-3 at 81.8 us with H rounded; three parts, every bit of H, 157.7 us.
+// 18 400 candidates of 12 embeddings x 128, k = 16: 27.4 us; the general kernel, a block per candidate, 284 us.
 // ---------------------------------------------------------------------------------------------
 constexpr int kFragRows = 16;      // rows of a candidate's fragments
 constexpr int kTileCands = 8;      // candidates per tile = compute warps per CTA
@@ -278,6 +282,22 @@ struct FmParams {
   uint32_t* status;
 };
 
+// Two fp32 values as bf16 pairs that add up to them.  Rounded value and rounded remainder: 17 bits.
+__device__ __forceinline__ void split_bf16(float a, float b, uint32_t (&part)[2]) {
+  part[0] = pack_bf16(a, b);
+  part[1] = pack_bf16(a - __uint_as_float(part[0] << 16), b - __uint_as_float(part[0] & 0xffff0000u));
+}
+// Upper halves of the values, of what is left and of what is left then: every bit.  An infinity is infinite in every part.
+__device__ __forceinline__ void split_bf16(float a, float b, uint32_t (&part)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
+    part[i] = __byte_perm(ua, ub, 0x7632);
+    a = fabsf(a) == INFINITY ? a : a - __uint_as_float(ua & 0xffff0000u);
+    b = fabsf(b) == INFINITY ? b : b - __uint_as_float(ub & 0xffff0000u);
+  }
+}
+
 // KT: blocks of 16 projection columns.  With one, the request's T stays in registers while consecutive
 // candidates share it; with two it would not fit beside H and comes from L1 for every candidate.
 template <int D, int KT, bool FULL>
@@ -406,10 +426,8 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
         __nv_bfloat16* fc = p.FC + cand * n_c * p.k;
 #pragma unroll
         for (int kt = 0; kt < KT; ++kt) {
-          // step 1: H^T (16 x D) = T^T + P_C^T X^C, rounded to bf16 as the K x N operand of step 2
-          uint32_t hb[kPairs][2][2];  // [k-step][projection columns 0-7 | 8-15][b0, b1]
-#pragma unroll
-          for (int cp = 0; cp < kPairs; ++cp) {
+          // step 1: H^T (16 x D) = T^T + P_C^T X^C, whose accumulator is the K x N operand of step 2 as it stands
+          auto step1 = [&](int cp, float (&f)[2][4]) {
             const int chunk = 2 * cp + lsel;  // 16-byte chunk along d
             uint32_t xb[4];
             ldmatrix_x4_trans(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xb);
@@ -419,7 +437,6 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
               xb[2] &= keep_lo;
               xb[3] &= keep_hi;
             }
-            float f[2][4];
             if constexpr (KT == 1) {
 #pragma unroll
               for (int e = 0; e < 8; ++e) f[e / 4][e % 4] = tfrag[cp][e / 4][e % 4];
@@ -428,20 +445,59 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
             }
             mma_bf16(f[0], pa[kt], xb[0], xb[1]);
             mma_bf16(f[1], pa[kt], xb[2], xb[3]);
-            hb[cp][0][0] = pack_bf16(f[0][0], f[0][1]);
-            hb[cp][0][1] = pack_bf16(f[1][0], f[1][1]);
-            hb[cp][1][0] = pack_bf16(f[0][2], f[0][3]);
-            hb[cp][1][1] = pack_bf16(f[1][2], f[1][3]);
-          }
+          };
           // step 2: FC (16 x 16) = X^C H
           float out[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll
-          for (int cp = 0; cp < kPairs; ++cp) {
+          auto rows_of = [&](int cp, uint32_t (&xa)[4]) {
             const int chunk = 2 * cp + lsel;
-            uint32_t xa[4];
             ldmatrix_x4(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xa);
-            mma_bf16(out[0], xa, hb[cp][0][0], hb[cp][0][1]);
-            mma_bf16(out[1], xa, hb[cp][1][0], hb[cp][1][1]);
+          };
+          if constexpr (FULL) {
+            uint32_t hb[kPairs][2][2];  // [k-step][projection columns 0-7 | 8-15][b0, b1]
+#pragma unroll
+            for (int cp = 0; cp < kPairs; ++cp) {
+              float f[2][4];
+              step1(cp, f);
+              hb[cp][0][0] = pack_bf16(f[0][0], f[0][1]);
+              hb[cp][0][1] = pack_bf16(f[1][0], f[1][1]);
+              hb[cp][1][0] = pack_bf16(f[0][2], f[0][3]);
+              hb[cp][1][1] = pack_bf16(f[1][2], f[1][3]);
+            }
+#pragma unroll
+            for (int cp = 0; cp < kPairs; ++cp) {
+              uint32_t xa[4];
+              rows_of(cp, xa);
+              mma_bf16(out[0], xa, hb[cp][0][0], hb[cp][0][1]);
+              mma_bf16(out[1], xa, hb[cp][1][0], hb[cp][1][1]);
+            }
+          } else {
+            auto product = [&](auto parts) {
+              constexpr int kParts = decltype(parts)::value;
+#pragma unroll
+              for (int cp = 0; cp < kPairs; ++cp) {
+                float f[2][4];
+                uint32_t xa[4];
+                step1(cp, f);
+                rows_of(cp, xa);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                  uint32_t b0[kParts], b1[kParts];
+                  split_bf16(f[0][2 * h], f[0][2 * h + 1], b0);
+                  split_bf16(f[1][2 * h], f[1][2 * h + 1], b1);
+#pragma unroll
+                  for (int i = 0; i < kParts; ++i) mma_bf16(out[h], xa, b0[i], b1[i]);
+                }
+              }
+            };
+            product(std::integral_constant<int, 2>());
+            bool nan = false;  // in this candidate's rows: what the next one's hold must not decide
+#pragma unroll
+            for (int e = 0; e < 8; ++e) nan = nan || (g + 8 * (e / 2 % 2) < n_c && isnan(out[e / 4][e % 4]));
+            if (__any_sync(0xffffffffu, nan)) {  // perhaps of an infinity, or of a value that rounds to one
+#pragma unroll
+              for (int e = 0; e < 8; ++e) out[e / 4][e % 4] = 0.f;
+              product(std::integral_constant<int, 3>());
+            }
           }
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
@@ -518,8 +574,9 @@ template <int D>
 rocs_status_t launch_fm_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t k,
                             const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
   if (k > 16) return launch_fm_mma_as<D, 2, false>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
-  if (n_c < kFragRows) return launch_fm_mma_as<D, 1, false>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
-  return launch_fm_mma_as<D, 1, true>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+  if (n_c == kFragRows && (k == 8 || k == 16))
+    return launch_fm_mma_as<D, 1, true>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+  return launch_fm_mma_as<D, 1, false>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
 }
 
 template <typename T>
