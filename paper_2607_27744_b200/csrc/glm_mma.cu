@@ -5,9 +5,12 @@
 //
 // Takes what the tcgen05 kernel (umma_glm.cu) does not: 4 or 12 embeddings per candidate, request sides that are
 // no multiple of 8.  Bound by the fixed latencies of its short chains (mma.sync, ldmatrix) with four warps per
-// scheduler.  100 requests x 184 candidates, 20 + 12 embeddings x 128 with compression to 4: 29 us; the general
-// kernel 286 us.  Where both apply the tcgen05 kernel is the faster (128 x 1024 candidates, 32 + 16 embeddings
-// with compression: 127 us, this one 145 us with 15 compute warps, 161 us with 8 that take two fragments each).
+// scheduler.  100 requests x 184 candidates, 20 + 12 embeddings x 128 with compression to 4: 36.6 us; the general
+// kernel 286 us.  The compression takes the fp32 block as a bf16 pair (value and remainder) through two products, as
+// exact as that kernel: error of OC against 64 bits 1.6573e-3 on 128 requests x 1024 candidates, 32 + 12 embeddings x
+// 128 to 8, at 192 us; 1.9116e-3 and 140 us with the block rounded first.  The tcgen05 kernel rounds it: where both
+// apply it is the faster also without the pair (128 x 1024 candidates, 32 + 16 embeddings with compression: 127 us,
+// this one 145 us with 15 compute warps, 161 us with 8 that take two fragments each).
 //
 // A persistent CTA takes a contiguous run of tiles (tiles never cross a request); a producer warp streams the
 // tiles through a TMA ring and each request's X^R, once per run of tiles of that request, through two slots.
@@ -18,11 +21,11 @@
 // Rows are permuted inside a fragment (and inside 16 rows of X^R) so that a thread ends up with four
 // neighbouring columns, in either order, and the eight rows of an ldmatrix block differ modulo 8 (no bank
 // conflicts under the 128-byte swizzle).  Outputs leave as 8-byte stores that fill whole 32-byte sectors.
-// With compression the products are formed transposed, so that an accumulator, rounded to bf16 (the value a
-// caller would read back), is the K x N operand of OC = ZR + W_CC YC as it stands; W_CC is repeated for every
-// candidate of the fragment and the other candidates' rows are masked out of YC, not multiplied by zero (a NaN
-// of one candidate must not reach another).  The raw block, if wanted too, is turned by movmatrix.
+// With compression the products are formed transposed, so that an accumulator, split into bf16 parts, is the K x N
+// operand of OC = ZR + W_CC YC as it stands; W_CC is repeated for every candidate of the fragment, and the other
+// candidates' rows are masked out of both operands (a NaN of one candidate must not reach another).  The raw block, if wanted too, is turned by movmatrix.
 #include <algorithm>
+#include <type_traits>
 
 #include "rocs_internal.h"
 #include "sm100_ptx.cuh"
@@ -66,6 +69,24 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], 
 __device__ __forceinline__ uint32_t pack(float lo, float hi) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h);
+}
+// Two fp32 values as bf16 pairs that add up to them.  Rounded value and rounded remainder: 17 bits.
+__device__ __forceinline__ void split(float a, float b, uint32_t (&part)[2]) {
+  part[0] = pack(a, b);
+  part[1] = pack(a - __uint_as_float(part[0] << 16), b - __uint_as_float(part[0] & 0xffff0000u));
+}
+// Upper halves of the values, of what is left and of what is left then: every bit.  An infinity is infinite in every part,
+// and what is left of a value is never 0 unless the value is, so that products with an infinity stay what they are.
+__device__ __forceinline__ void split(float a, float b, uint32_t (&part)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
+    part[i] = __byte_perm(ua, ub, 0x7632);
+    const float ra = a - __uint_as_float(ua & 0xffff0000u), rb = b - __uint_as_float(ub & 0xffff0000u);
+    const uint32_t least = 0x10000u;  // the smallest positive bf16
+    a = fabsf(a) == INFINITY || a == 0.f ? a : ra == 0.f ? __uint_as_float((ua & 0x80000000u) | least) : ra;
+    b = fabsf(b) == INFINITY || b == 0.f ? b : rb == 0.f ? __uint_as_float((ub & 0x80000000u) | least) : rb;
+  }
 }
 __device__ __forceinline__ uint32_t transpose8x8(uint32_t v) {
   uint32_t r;
@@ -258,22 +279,19 @@ glm_mma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant
           for (int h = 0; h < 2; ++h)
             store_raw(h, pack(acc.v[0][2 * h], acc.v[0][2 * h + 1]), pack(acc.v[1][2 * h], acc.v[1][2 * h + 1]));
         } else {
-          // yt[j][h]: columns of index 8 j + g of YC, fragment rows of index 8 h + 2 tq, + 1
-          uint32_t yt[2][2];
-#pragma unroll
-          for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) yt[j][h] = pack(acc.v[h][2 * j], acc.v[h][2 * j + 1]);
+          // of yt[j][h]: columns of index 8 j + g of YC, fragment rows of index 8 h + 2 tq, + 1
           if constexpr (RAW) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-              const uint32_t first = transpose8x8(yt[0][h]), second = transpose8x8(yt[1][h]);
+              const uint32_t first = transpose8x8(pack(acc.v[h][0], acc.v[h][1])),
+                             second = transpose8x8(pack(acc.v[h][2], acc.v[h][3]));
               store_raw(h, first, second);
             }
           }
-          for (int c = 0; c < last; ++c) {
+          auto compress = [&](int c, float (&o)[2][4], auto parts) {  // candidate c of the fragment
+            constexpr int kParts = decltype(parts)::value;
             const uint32_t k0 = k_cand[0] == c ? 0xffffffffu : 0u, k1 = k_cand[1] == c ? 0xffffffffu : 0u;
-            float o[2][4];
+            const uint32_t w[4] = {wa[0] & k0, wa[1] & k0, wa[2] & k1, wa[3] & k1};
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
               const float4 zb = b < CO8 ? z[b < CO8 ? b : 0] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -283,9 +301,24 @@ glm_mma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant
               o[1][2 * b + 1] = swap ? zb.y : zb.w;
             }
 #pragma unroll
-            for (int j = 0; j < 2; ++j) mma_bf16(o[j], wa, yt[j][0] & k0, yt[j][1] & k1);
-            __nv_bfloat16* oc = p.OC + (cand + c) * p.n_co * n + col;
+            for (int j = 0; j < 2; ++j) {
+              uint32_t yt[2][kParts];
+              split(acc.v[0][2 * j], acc.v[0][2 * j + 1], yt[0]);
+              split(acc.v[1][2 * j], acc.v[1][2 * j + 1], yt[1]);
+#pragma unroll
+              for (int i = 0; i < kParts; ++i) mma_bf16(o[j], w, yt[0][i] & k0, yt[1][i] & k1);
+            }
+          };
+          for (int c = 0; c < last; ++c) {
+            float o[2][4];
+            compress(c, o, std::integral_constant<int, 2>());
             const bool in = in_cols && (!self || col_cand == c);
+            bool nan = false;  // in this candidate's outputs: what the fragment's others hold must not decide
+#pragma unroll
+            for (int e = 0; e < 4 * CO8; ++e) nan = nan || (in && g + 8 * (e / 4) < p.n_co && isnan(o[e / 2 % 2][2 * (e / 4) + e % 2]));
+            if (__any_sync(0xffffffffu, nan))  // perhaps of an infinity, or of a value that rounds to one
+              compress(c, o, std::integral_constant<int, 3>());
+            __nv_bfloat16* oc = p.OC + (cand + c) * p.n_co * n + col;
 #pragma unroll
             for (int b = 0; b < CO8; ++b)
               if (in && g + 8 * b < p.n_co)

@@ -597,6 +597,34 @@ def test_glm_fragments(n_r, n_c, d, n_co, raw, many):
         assert bool(torch.isnan(pert[k][12].float()).any())
 
 
+@pytest.mark.parametrize("n_r,n_c,d,n_co,raw", [(20, 12, 128, 4, False), (16, 4, 64, 8, True), (44, 8, 256, 3, False), (100, 16, 64, 16, True)])
+def test_glm_fragments_are_as_exact_as_fp32_arithmetic(n_r, n_c, d, n_co, raw):
+    # Both kernels compress the fp32 products and round the result to bf16 once.  Sums of fp32 in another order differ by
+    # some 2^-20, against the 2^-9 of that rounding: the errors against fp64 are the same up to which way close values are
+    # rounded (well below 1 % of the norm over these thousands of values; products rounded first would add about 20 %).
+    co = wl.offsets_from_counts([1, 0, 9, 8, 33, 7, 0, 133])
+    cfg = wl.CONFIGS[4].with_(R=len(co) - 1, n_r=n_r, n_c=n_c, d_emb=d, n_ro=2, n_co=n_co)
+    g = wl.glm_inputs(cfg, co)
+    want = ref.glm_interaction(co, g["XR"], g["XC"], g["W"], cfg.n_ro, n_co)[1][:, cfg.n_ro:]
+    plan = _plan(co)
+
+    def run(XC, W):
+        return to_host_f64(rocs.glm_interaction(plan, to_dev(g["XR"]), to_dev(XC), to_dev(W), 2, n_co, want_raw=raw)["OC"])
+
+    XC, W = g["XC"].copy(), g["W"].copy()
+    XC[60, 1, 5] = 0x7f80                          # infinities show in the same values either way
+    W[cfg.n_ro + n_co - 1, n_r + n_c - 1] = 0xff80
+    err, kinds = [], []
+    for path in PATHS:
+        rocs.set_path(path)
+        got = run(g["XC"], g["W"])
+        err.append(np.linalg.norm(got - want) / np.linalg.norm(want))
+        kinds.append([np.where(np.isnan(o), 2, np.where(np.isinf(o), np.sign(o), 0)) for o in (run(XC, g["W"]), run(g["XC"], W))])
+    assert err[0] <= 1.01 * err[1]
+    for auto, general in zip(*kinds):
+        assert np.array_equal(auto, general) and np.any(auto[60] != 0)
+
+
 @pytest.mark.parametrize("R", [1, 127, 128, 129, 255, 257, 12000, 12001])
 def test_work_lists_of_many_requests(R):
     # the lists are scanned by 256 threads per block up to 12000 requests and on the host beyond: counts of
