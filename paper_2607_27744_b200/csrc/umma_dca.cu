@@ -190,7 +190,8 @@ __device__ __forceinline__ void tmem_st_32x32b_x8(uint32_t taddr, const uint32_t
 }
 
 // One query row of one head, half of its DH output columns, unnormalised, in plain fp32 with the row's true maximum
-// m as reference and l as sum: q and k point at the head's DH values of the row / of the first key, v at the
+// m as reference and l as sum (a score of -inf has weight 0 whatever the maximum: these keys may be a part of the row's
+// only, and the others' scores finite): q and k point at the head's DH values of the row / of the first key, v at the
 // DH / 2 columns wanted; consecutive keys are `stride` elements apart.  Inlined on purpose: as a called
 // function it forces the caller's hot loop to keep its registers where the calling convention wants
 // them, and the loop spills.
@@ -208,7 +209,7 @@ __device__ __forceinline__ void row_by_hand(const __nv_bfloat16* q, const __nv_b
   l = 0.f;
   for (int d = 0; d < DH / 2; ++d) acc[d] = 0.f;
   for (int32_t j = 0; j < L; ++j) {
-    const float pj = exp2f(score(j) - m);
+    const float s = score(j), pj = s == -INFINITY ? 0.f : exp2f(s - m);
     l += pj;
     for (int d = 0; d < DH / 2; ++d) acc[d] = fmaf(pj, __bfloat162float(v[(int64_t)j * stride + d]), acc[d]);
   }
@@ -828,7 +829,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           const uint32_t part = map_to_cta(sb + C::part_offset(side) + row * (C::kPartStride * 4), c);
           const float4 both = ld_cluster_f4(part + DH * 4);  // reference and sum of either half of the columns
           const float m = col < DH / 2 ? both.x : both.z, l_part = col < DH / 2 ? both.y : both.w;
-          if (m == -INFINITY && l_part == 0.f) continue;  // a side without keys
+          if (m == -INFINITY && l_part == 0.f) continue;  // a side without keys, or whose scores are all -inf
           const float m_new = fmaxf(M, m);
           const float a = M == -INFINITY ? 0.f : exp2f(M - m_new), b = exp2f(m - m_new);
           const float4 o = ld_cluster_f4(part + col * 4);

@@ -511,6 +511,32 @@ def test_dca_config5_full_size_sampled():
     assert _run_dca(cfg, co, so, sample=sample) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("L", [200, 1500])   # one part per item; split over sides and CTAs
+@pytest.mark.parametrize("dh", [32, 64, 128])
+@pytest.mark.parametrize("where", ["head", "tail", "most", "all"])
+def test_dca_bf16_scores_of_minus_infinity(L, dh, where):
+    # a key whose score is -inf has weight 0, also where all keys of a part score so; a row of nothing else is NaN
+    co, so = wl.offsets_from_counts([40, 0, 3]), wl.offsets_from_counts([L, 5, L - 37])
+    cfg = wl.CONFIGS[3].with_(R=3, H=2, dh=dh)
+    d = wl.dca_inputs(cfg, co, so)
+    Q, K, V = to_dev(d["Q"]), to_dev(d["K"]), to_dev(d["V"])
+    Q[..., 0] = Q[..., 0].abs() + 0.5
+    for r in (0, 2):
+        n = int(so[r + 1] - so[r])
+        keys = {"head": slice(0, n // 2), "tail": slice(n // 3, n), "most": slice(0, n - 1), "all": slice(0, n)}[where]
+        K[int(so[r]):int(so[r + 1])][keys, :, 0] = float("-inf")
+    got = rocs.dca_attention(_plan(co), Q, K, V, to_dev(so)).double()
+    if where == "all":
+        assert bool(torch.isnan(got).all())
+        return
+    want = torch.empty_like(got)
+    for r in (0, 2):
+        c, k = slice(int(co[r]), int(co[r + 1])), slice(int(so[r]), int(so[r + 1]))
+        p = torch.softmax(torch.einsum("nqhd,khd->nqhk", Q[c].double(), K[k].double()) * dh ** -0.5, -1)
+        want[c] = torch.einsum("nqhk,khd->nqhd", p, V[k].double())
+    assert rel_err(got.cpu().numpy(), want.cpu().numpy()) <= tol_for("bf16")
+
+
 # ------------------------------------------------------------------ interaction -------------
 def _run_glm(cfg, co, sample=None, path=rocs.PATH_AUTO):
     rocs.set_path(path)
