@@ -811,7 +811,10 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     tmem_dealloc(tmem_base, kTmemCols);
   }
   if constexpr (SPLIT) {
-    // O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s over the parts s of the item, M the largest reference
+    // O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s over the parts s of the item, M the largest reference.  Every
+    // weight is 2^-kScaleDown of that, in both sums: up to 16 parts that are finite each, perhaps close to 2^128, have
+    // a finite sum.
+    constexpr float kScaleDown = 5.f;
     cluster_sync_all();
     const int4* info = reinterpret_cast<const int4*>(smem + kOffInfo);  // slot 0 of side A: the item
     const int4 item = info[0];
@@ -831,7 +834,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           const float m = col < DH / 2 ? both.x : both.z, l_part = col < DH / 2 ? both.y : both.w;
           if (m == -INFINITY && l_part == 0.f) continue;  // a side without keys, or whose scores are all -inf
           const float m_new = fmaxf(M, m);
-          const float a = M == -INFINITY ? 0.f : exp2f(M - m_new), b = exp2f(m - m_new);
+          const float a = M == -INFINITY ? 0.f : exp2f(M - m_new), b = exp2f(m - m_new - kScaleDown);
           const float4 o = ld_cluster_f4(part + col * 4);
           acc.x = acc.x * a + o.x * b;
           acc.y = acc.y * a + o.y * b;

@@ -537,6 +537,22 @@ def test_dca_bf16_scores_of_minus_infinity(L, dh, where):
     assert rel_err(got.cpu().numpy(), want.cpu().numpy()) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("dh", [32, 64, 128])
+@pytest.mark.parametrize("log2_weight", [126, 123])
+def test_dca_bf16_split_items_whose_parts_add_up_past_fp32(dh, log2_weight):
+    # The last key of every 128 weighs 2^126 against the reference 1 of its part: three of them are within fp32 in each of
+    # 4 parts (8 at width 128), a dozen are not.  The rows are the mean of these keys' values.
+    co, so = wl.offsets_from_counts([40, 3]), wl.offsets_from_counts([1536, 1536])
+    Q = torch.zeros((43, 1, 2, dh), dtype=torch.bfloat16, device="cuda")
+    K = torch.zeros((3072, 2, dh), dtype=torch.bfloat16, device="cuda")
+    V = (torch.randn((3072, 2, dh), generator=torch.Generator().manual_seed(3)) * 0.05).to(torch.bfloat16).cuda()
+    Q[..., 0] = 1.0
+    K[127::128, :, 0] = log2_weight
+    got = rocs.dca_attention(_plan(co), Q, K, V, to_dev(so), scale=float(np.log(2.0)))
+    want = torch.stack([V[127:1536:128].double().mean(0)] * 40 + [V[1536 + 127::128].double().mean(0)] * 3)[:, None]
+    assert rel_err(to_host_f64(got), want.cpu().numpy()) <= tol_for("bf16")
+
+
 # ------------------------------------------------------------------ interaction -------------
 def _run_glm(cfg, co, sample=None, path=rocs.PATH_AUTO):
     rocs.set_path(path)
