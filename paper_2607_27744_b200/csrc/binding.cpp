@@ -10,10 +10,10 @@
 
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <algorithm>
-#include <stdexcept>
 
 #include "../../include/rocs.h"
 
@@ -67,6 +67,12 @@ struct Arg {
     return ROCS_F32;
   }
   size_t bytes() const { return t ? (size_t)t->numel() : 0; }  // of a uint8 workspace
+  void need_dims(int64_t n) const {
+    if ((*this)->dim() != n) {
+      PyErr_Format(PyExc_ValueError, "expected a tensor of %d dimensions, got %d", (int)n, (int)t->dim());
+      throw PyRaised{};
+    }
+  }
 };
 
 // The caller's tensor, or a new one with `like`'s device.
@@ -198,7 +204,7 @@ PyObject* ikbo_linear_stats(PyObject* const* a) {
 PyObject* weight_row_sums(PyObject* const* a) {
   const Arg W(a[0]);
   Out out(a[1]);
-  require(W->dim() == 2);
+  W.need_dims(2);
   out.or_empty({W.size(0)}, W, at::kFloat);
   const rocs_dtype_t dt = W.dtype();
   const int64_t ld = W.ld();
@@ -214,7 +220,7 @@ PyObject* weight_row_sums(PyObject* const* a) {
 // X, row_stats, W, wbar, bias, eps, kind, relu, out
 PyObject* linear_normed(PyObject* const* a) {
   const Arg X(a[0]), stats(a[1]), W(a[2]), wbar(a[3]), bias(a[4]);
-  require(X->dim() == 2);
+  X.need_dims(2);
   const int64_t M = X.size(0);
   const int32_t d_in = (int32_t)X.size(1), d_out = (int32_t)W.size(0);
   require(stats->scalar_type() == at::kFloat && stats->dim() == 2 && stats.size(0) == M && stats.size(1) == 2 &&
@@ -239,7 +245,7 @@ PyObject* linear_normed(PyObject* const* a) {
 // X, W, bias, relu, out
 PyObject* linear(PyObject* const* a) {
   const Arg X(a[0]), W(a[1]), bias(a[2]);
-  require(X->dim() == 2);
+  X.need_dims(2);
   const int64_t M = X.size(0);
   const int32_t d_in = (int32_t)X.size(1), d_out = (int32_t)W.size(0);
   Out out(a[4]);
@@ -260,7 +266,7 @@ PyObject* linear(PyObject* const* a) {
 PyObject* dca_attention(PyObject* const* a) {
   const PlanArg plan(a);
   const Arg Q(a[3]), K(a[4]), V(a[5]), seq(a[6]);
-  require(Q->dim() == 4);
+  Q.need_dims(4);
   require(Q.size(0) == plan.N && Q->is_contiguous() && K->is_contiguous() && V->is_contiguous());
   require(seq->scalar_type() == at::kInt && seq->is_cuda() && seq->numel() == plan.R + 1);
   const int32_t n_q = (int32_t)Q.size(1), H = (int32_t)Q.size(2), dh = (int32_t)Q.size(3);
@@ -284,7 +290,8 @@ PyObject* dca_attention(PyObject* const* a) {
 PyObject* glm_interaction(PyObject* const* a) {
   const PlanArg plan(a);
   const Arg XR(a[3]), XC(a[4]), W(a[5]), YR(a[8]), YC(a[9]), OR_(a[10]), OC(a[11]);
-  require(XR->dim() == 3 && XC->dim() == 3);
+  XR.need_dims(3);
+  XC.need_dims(3);
   require(XR.size(0) == plan.R && XC.size(0) == plan.N && XR->is_contiguous() && XC->is_contiguous());
   const int32_t n_r = (int32_t)XR.size(1), d = (int32_t)XR.size(2), n_c = (int32_t)XC.size(1);
   const int32_t n_ro = i32(a[6]), n_co = i32(a[7]);
@@ -306,7 +313,8 @@ PyObject* glm_interaction(PyObject* const* a) {
 PyObject* glm_fm_projection(PyObject* const* a) {
   const PlanArg plan(a);
   const Arg XR(a[3]), XC(a[4]), P(a[5]), FR(a[6]), FC(a[7]);
-  require(XR->dim() == 3 && XC->dim() == 3);
+  XR.need_dims(3);
+  XC.need_dims(3);
   require(XR.size(0) == plan.R && XC.size(0) == plan.N && XR->is_contiguous() && XC->is_contiguous());
   const int32_t n_r = (int32_t)XR.size(1), d = (int32_t)XR.size(2), n_c = (int32_t)XC.size(1);
   require(P->dim() == 2 && P.size(0) == n_r + n_c && P->is_contiguous() && P->scalar_type() == XC->scalar_type());
@@ -364,9 +372,11 @@ PyObject* set_error_type(PyObject* const* a) {
   Py_RETURN_NONE;
 }
 
-// Argument count, and C++ exceptions as Python ones.
+// Argument count, and C++ exceptions as the Python ones that torch raises for them (running out of memory has a type of
+// its own, which callers catch to score a smaller batch).
 template <PyObject* (*F)(PyObject* const*), Py_ssize_t N>
 PyObject* entry(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
   if (n != N) {
     PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", N, n);
     return nullptr;
@@ -375,10 +385,8 @@ PyObject* entry(PyObject*, PyObject* const* args, Py_ssize_t n) {
     return F(args);
   } catch (const PyRaised&) {
     return nullptr;
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
-    return nullptr;
   }
+  END_HANDLE_TH_ERRORS
 }
 
 #define ENTRY(name, n) {#name, (PyCFunction)(void (*)(void))entry<name, n>, METH_FASTCALL, nullptr}

@@ -53,3 +53,21 @@ def test_binding_fails_loudly_without_the_library(monkeypatch, tmp_path):
     monkeypatch.setattr(binding, "LIB_PATH", str(tmp_path / "missing.so"))
     with pytest.raises(RuntimeError, match="no fallback"):
         binding.lib()
+
+
+@pytest.mark.parametrize("call,error", [
+    (lambda plan, x: binding.ikbo_linear(plan, None, x(4), None, x(3, 8)), IndexError),       # rows of one dimension
+    (lambda plan, x: binding.linear(x(4), x(3, 8)), ValueError),
+    (lambda plan, x: binding.linear_normed(x(2, 2, 8), x(2, 2), x(3, 8)), ValueError),
+    (lambda plan, x: binding.weight_row_sums(x(8)), ValueError),
+    (lambda plan, x: binding.dca_attention(plan, x(4, 1, 8), x(2, 1, 8), x(2, 1, 8), x(2)), ValueError),
+    (lambda plan, x: binding.group_norm(x(4)), AssertionError),
+    (lambda plan, x: binding.linear(x(4, 8).half(), x(3, 8).half()), TypeError),
+    (lambda plan, x: binding.linear(None, x(3, 8)), AttributeError),
+    (lambda plan, x: binding.linear(x(4, 8), x(3, 8)), AssertionError),                       # not on a GPU
+])
+def test_malformed_arguments_raise_what_python_would(lib, call, error):
+    import torch
+    plan = type("P", (), {"handle": None, "R": 1, "N": 4})
+    with pytest.raises(error):
+        call(plan, torch.zeros)

@@ -798,6 +798,13 @@ def test_calls_captured_in_a_graph_replay(warm):
 
 
 # ------------------------------------------------------------------ ABI errors --------------
+def test_an_output_that_does_not_fit_raises_torchs_own_error():
+    X = torch.zeros((1, 64), dtype=torch.bfloat16, device="cuda").expand(1 << 31, 64)
+    W = torch.zeros((4096, 64), dtype=torch.bfloat16, device="cuda")
+    with pytest.raises(torch.OutOfMemoryError):
+        rocs.linear(X, W)
+
+
 def test_error_codes_on_bad_arguments():
     co = wl.offsets_from_counts([4, 4])
     d_co = to_dev(co)
