@@ -54,7 +54,8 @@ struct Arg {
     if (t == nullptr) raise(PyExc_AttributeError, "a required tensor is None");
     return t;
   }
-  void* ptr() const { return t ? const_cast<void*>(t->const_data_ptr()) : nullptr; }
+  const void* ptr() const { return t ? t->const_data_ptr() : nullptr; }
+  void* mut() const { return t ? t->mutable_data_ptr() : nullptr; }  // written to: a lazy clone gets memory of its own first
   int64_t size(int64_t d) const { return (*this)->size(d); }
   // row stride of a row-major 2-D CUDA tensor
   int64_t ld() const {
@@ -169,7 +170,7 @@ PyObject* ikbo_linear(PyObject* const* a) {
   check(call([&] {
           return rocs_ikbo_linear(plan.handle, dt, d_req, d_cand, d_out, XR.ptr(), ld_xr, XC.ptr(), ld_xc,
                                   d_req ? W_CR.ptr() : nullptr, ld_wcr, W_CC.ptr(), ld_wcc,
-                                  static_cast<const float*>(bias.ptr()), ac, out.given.ptr(), ld_y, ws.given.ptr(),
+                                  static_cast<const float*>(bias.ptr()), ac, out.given.mut(), ld_y, ws.given.mut(),
                                   ws.given.bytes(), st);
         }),
         "rocs_ikbo_linear");
@@ -193,7 +194,7 @@ PyObject* ikbo_linear_stats(PyObject* const* a) {
   check(call([&] {
           return rocs_ikbo_linear_stats(plan.handle, dt, d_req, d_cand, d_out, XR.ptr(), ld_xr, XC.ptr(), ld_xc, W_CR.ptr(),
                                         ld_wcr, W_CC.ptr(), ld_wcc, static_cast<const float*>(bias.ptr()), ac,
-                                        out.given.ptr(), ld_y, static_cast<float*>(stats.given.ptr()), ws.given.ptr(),
+                                        out.given.mut(), ld_y, static_cast<float*>(stats.given.mut()), ws.given.mut(),
                                         ws.given.bytes(), st);
         }),
         "rocs_ikbo_linear_stats");
@@ -211,7 +212,7 @@ PyObject* weight_row_sums(PyObject* const* a) {
   void* st = stream();
   check(call([&] {
           return rocs_weight_row_sums(dt, (int32_t)W.size(0), (int32_t)W.size(1), W.ptr(), ld,
-                                      static_cast<float*>(out.given.ptr()), st);
+                                      static_cast<float*>(out.given.mut()), st);
         }),
         "rocs_weight_row_sums");
   return out.release();
@@ -236,7 +237,7 @@ PyObject* linear_normed(PyObject* const* a) {
   check(call([&] {
           return rocs_linear_normed(dt, kind, M, d_in, d_out, X.ptr(), ld_x, static_cast<const float*>(stats.ptr()), eps,
                                     W.ptr(), ld_w, static_cast<const float*>(wbar.ptr()),
-                                    static_cast<const float*>(bias.ptr()), ac, out.given.ptr(), ld_y, st);
+                                    static_cast<const float*>(bias.ptr()), ac, out.given.mut(), ld_y, st);
         }),
         "rocs_linear_normed");
   return out.release();
@@ -256,7 +257,7 @@ PyObject* linear(PyObject* const* a) {
   void* st = stream();
   check(call([&] {
           return rocs_linear(dt, M, d_in, d_out, X.ptr(), ld_x, W.ptr(), ld_w, static_cast<const float*>(bias.ptr()), ac,
-                             out.given.ptr(), ld_y, st);
+                             out.given.mut(), ld_y, st);
         }),
         "rocs_linear");
   return out.release();
@@ -280,7 +281,7 @@ PyObject* dca_attention(PyObject* const* a) {
   void* st = stream();
   check(call([&] {
           return rocs_dca_attention(plan.handle, dt, n_q, H, dh, scale, Q.ptr(), K.ptr(), V.ptr(), T,
-                                    static_cast<const int32_t*>(seq.ptr()), out.given.ptr(), ws.given.ptr(), need, st);
+                                    static_cast<const int32_t*>(seq.ptr()), out.given.mut(), ws.given.mut(), need, st);
         }),
         "rocs_dca_attention");
   return out.release();
@@ -302,8 +303,8 @@ PyObject* glm_interaction(PyObject* const* a) {
   const rocs_dtype_t dt = XC.dtype();
   void* st = stream();
   check(call([&] {
-          return rocs_glm_interaction(plan.handle, dt, n_r, n_c, d, XR.ptr(), XC.ptr(), W.ptr(), n_ro, n_co, YR.ptr(), YC.ptr(),
-                                      OR_.ptr(), OC.ptr(), ws.given.ptr(), ws.given.bytes(), st);
+          return rocs_glm_interaction(plan.handle, dt, n_r, n_c, d, XR.ptr(), XC.ptr(), W.ptr(), n_ro, n_co, YR.mut(), YC.mut(),
+                                      OR_.mut(), OC.mut(), ws.given.mut(), ws.given.bytes(), st);
         }),
         "rocs_glm_interaction");
   Py_RETURN_NONE;
@@ -324,8 +325,8 @@ PyObject* glm_fm_projection(PyObject* const* a) {
   const rocs_dtype_t dt = XC.dtype();
   void* st = stream();
   check(call([&] {
-          return rocs_glm_fm_projection(plan.handle, dt, n_r, n_c, d, k, XR.ptr(), XC.ptr(), P.ptr(), FR.ptr(), FC.ptr(),
-                                        ws.given.ptr(), ws.given.bytes(), st);
+          return rocs_glm_fm_projection(plan.handle, dt, n_r, n_c, d, k, XR.ptr(), XC.ptr(), P.ptr(), FR.mut(), FC.mut(),
+                                        ws.given.mut(), ws.given.bytes(), st);
         }),
         "rocs_glm_fm_projection");
   Py_RETURN_NONE;
@@ -344,7 +345,7 @@ PyObject* group_norm(PyObject* const* a) {
   void* st = stream();
   check(call([&] {
           return rocs_group_norm(dt, kind, X.size(0), (int32_t)X.size(1), X.ptr(), ld_x, gamma.ptr(), beta.ptr(), eps,
-                                 out.given.ptr(), ld_y, st);
+                                 out.given.mut(), ld_y, st);
         }),
         "rocs_group_norm");
   return out.release();
@@ -361,7 +362,7 @@ PyObject* ikbo_linear_static(PyObject* const* a) {
           return rocs_ikbo_linear_static(dt, (int32_t)(off->numel() - 1), XC.size(0), static_cast<const int32_t*>(off.ptr()),
                                          (int32_t)XR.size(1), (int32_t)XC.size(1), (int32_t)W_CC.size(0), XR.ptr(), ld_xr,
                                          XC.ptr(), ld_xc, W_CR.ptr(), ld_wcr, W_CC.ptr(), ld_wcc,
-                                         static_cast<const float*>(bias.ptr()), ac, out.ptr(), ld_y, st);
+                                         static_cast<const float*>(bias.ptr()), ac, out.mut(), ld_y, st);
         }),
         "rocs_ikbo_linear_static");
   return Py_NewRef(a[5]);

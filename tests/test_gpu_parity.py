@@ -798,6 +798,26 @@ def test_calls_captured_in_a_graph_replay(warm):
 
 
 # ------------------------------------------------------------------ ABI errors --------------
+def test_outputs_that_are_lazy_clones_leave_their_source_alone():
+    co = wl.offsets_from_counts([3, 5])
+    plan = _plan(co)
+    def t(*shape):
+        return torch.randn(shape, device="cuda").to(torch.bfloat16)
+    source = torch.full((8 * 64,), 7.0, dtype=torch.bfloat16, device="cuda")
+    def out(*shape):
+        return torch._lazy_clone(source)[:int(np.prod(shape))].view(shape)
+    W, stats = t(64, 64), torch._lazy_clone(torch.zeros((8, 2), device="cuda"))
+    rocs.linear(t(8, 64), W, out=out(8, 64))
+    rocs.ikbo_linear(plan, t(2, 64), t(8, 64), W, W, out=out(8, 64))
+    rocs.ikbo_linear_stats(plan, t(2, 64), t(8, 64), W, W, out=out(8, 64), row_stats=stats)
+    rocs.ikbo_linear_static(to_dev(co), t(2, 64), t(8, 64), W, W, out(8, 64))
+    rocs.group_norm(t(8, 64), out=out(8, 64))
+    rocs.dca_attention(plan, t(8, 1, 2, 32), t(6, 2, 32), t(6, 2, 32), to_dev(np.array([0, 4, 6], np.int32)), out=out(8, 1, 2, 32))
+    rocs.glm_interaction(plan, t(2, 2, 64), t(8, 2, 64), None, outs={"YR": out(2, 2, 4), "YC": out(8, 2, 4)})
+    rocs.glm_fm_projection(plan, t(2, 2, 64), t(8, 2, 64), t(4, 8), outs={"FR": out(2, 2, 8), "FC": out(8, 2, 8)})
+    assert bool((source == 7.0).all())
+
+
 def test_an_output_that_does_not_fit_raises_torchs_own_error():
     X = torch.zeros((1, 64), dtype=torch.bfloat16, device="cuda").expand(1 << 31, 64)
     W = torch.zeros((4096, 64), dtype=torch.bfloat16, device="cuda")
