@@ -15,9 +15,11 @@ namespace {
 std::atomic<int> g_path{ROCS_PATH_AUTO};
 
 // m_i of Section 4.1 from the segment offsets: one thread per candidate, binary search.
-// beside: the kernel in front may still run.  It waited for everything in front of itself before it released this one
-// and touches neither the offsets nor the table; this grid completes behind it, so that the next need wait for this
-// one only.
+// beside: kernels in front may still run, of this call and of other threads' calls that share the stream.  One of them,
+// the request half, waited for everything in front of itself before it released the next: the offsets, and all that ever
+// used the table's memory, are complete.  (The memory is taken in front of the request half: taken behind it, it could be
+// that of another thread's plan whose last kernel still reads it.)  This grid completes behind the kernels in front, so
+// that the next need wait for this one only.
 __global__ void fill_row2req_kernel(int32_t R, int64_t N, const int32_t* __restrict__ off,
                                     int32_t* __restrict__ row2req, bool beside) {
   if (!beside) ptx::griddep_wait_for(off);
@@ -171,16 +173,20 @@ int64_t plan_entries(const rocs_plan* plan, int32_t cands_per_tile) {
   return entries;
 }
 
+static rocs_status_t fill_table(const rocs_plan* plan, const int32_t* off, int32_t* table, cudaStream_t stream, bool beside) {
+  return launch_dependent(fill_row2req_kernel, dim3((unsigned)((plan->N + 255) / 256)), 256, 0, stream, plan->R, plan->N, off,
+                          table, beside);
+}
+
 // Allocates and fills one list of the plan (key as in rocs_plan::lists) in the order of `stream`, from the
 // offsets at `off`.
 static rocs_status_t make_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, const int32_t* off,
-                               cudaStream_t stream, DeviceList* out, bool beside = false) {
+                               cudaStream_t stream, DeviceList* out) {
   static_assert(sizeof(Tile) == 16 && sizeof(DcaItem) == 16, "list entries");
   DeviceList list;
   if (plan->N > 0 && cands_per_tile == 0) {
     ROCS_CUDA_TRY(pool_alloc(&list.dev, sizeof(int32_t) * (size_t)plan->N, stream));
-    if (launch_dependent(fill_row2req_kernel, dim3((unsigned)((plan->N + 255) / 256)), 256, 0, stream, plan->R, plan->N, off,
-                         static_cast<int32_t*>(list.dev), beside) != ROCS_OK) {
+    if (fill_table(plan, off, static_cast<int32_t*>(list.dev), stream, false) != ROCS_OK) {
       cudaFreeAsync(list.dev, stream);
       return ROCS_ERR_CUDA;
     }
@@ -249,10 +255,12 @@ static unsigned long long capture_of(cudaStream_t stream) {  // 0: the stream is
   return id;
 }
 
-static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, cudaStream_t stream,
-                               DeviceList* out, bool beside = false) {
-  const unsigned long long capture = capture_of(stream);
-  std::lock_guard<std::mutex> lock(plan->mu);
+// The list that a call on `stream` may read, if there is one (out->dev stays null otherwise), and the key under which
+// one that is made on the stream is kept.  Under a capture that the plan does not live in there always is one.  The caller
+// holds plan->mu.
+static rocs_status_t find_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, unsigned long long capture,
+                               cudaStream_t stream, rocs_plan::ListKey* key, bool* found, DeviceList* out) {
+  *found = true;
   if (capture != 0 && capture != plan->capture) {
     // A graph that outlives this call: it must hold a list that exists now, not one that its own replays would
     // allocate.  Any list made outside a capture will do, since the graph is launched behind the plan.
@@ -267,18 +275,27 @@ static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, in
   }
   unsigned long long id = 0;
   if (plan->capture == 0) ROCS_CUDA_TRY(cudaStreamGetId(stream, &id));
-  const auto key = std::make_tuple(id, cands_per_tile, heads);
-  auto it = plan->lists.find(key);
-  if (it != plan->lists.end()) {
-    *out = it->second;
-    return ROCS_OK;
-  }
-  const rocs_status_t st = make_list(plan, cands_per_tile, heads, plan->cand_offsets, stream, out, beside);
+  *key = std::make_tuple(id, cands_per_tile, heads);
+  auto it = plan->lists.find(*key);
+  *found = it != plan->lists.end();
+  if (*found) *out = it->second;
+  return ROCS_OK;
+}
+
+static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, cudaStream_t stream,
+                               DeviceList* out) {
+  const unsigned long long capture = capture_of(stream);
+  std::lock_guard<std::mutex> lock(plan->mu);
+  rocs_plan::ListKey key;
+  bool found;
+  rocs_status_t st = find_list(plan, cands_per_tile, heads, capture, stream, &key, &found, out);
+  if (st != ROCS_OK || found) return st;
+  st = make_list(plan, cands_per_tile, heads, plan->cand_offsets, stream, out);
   if (st == ROCS_OK) plan->lists[key] = *out;
   return st;
 }
 
-rocs_status_t plan_request_map(const rocs_plan* plan, cudaStream_t stream, RequestMap* out, bool beside) {
+rocs_status_t plan_request_map(const rocs_plan* plan, cudaStream_t stream, RequestMap* out) {
   *out = RequestMap{};
   if (plan->N <= kSearchRows) {
     out->offsets = plan->cand_offsets;
@@ -286,7 +303,45 @@ rocs_status_t plan_request_map(const rocs_plan* plan, cudaStream_t stream, Reque
     return ROCS_OK;
   }
   DeviceList list;
-  const rocs_status_t st = plan_list(plan, 0, 0, stream, &list, beside);
+  const rocs_status_t st = plan_list(plan, 0, 0, stream, &list);
+  out->row2req = static_cast<const int32_t*>(list.dev);
+  return st;
+}
+
+rocs_status_t plan_request_map_begin(const rocs_plan* plan, cudaStream_t stream, RequestMap* out, void** memory) {
+  *memory = nullptr;
+  if (plan->N <= kSearchRows) return plan_request_map(plan, stream, out);
+  *out = RequestMap{};
+  const unsigned long long capture = capture_of(stream);
+  {
+    std::lock_guard<std::mutex> lock(plan->mu);
+    rocs_plan::ListKey key;
+    bool found;
+    DeviceList list;
+    const rocs_status_t st = find_list(plan, 0, 0, capture, stream, &key, &found, &list);
+    out->row2req = static_cast<const int32_t*>(list.dev);
+    if (st != ROCS_OK || found) return st;
+  }
+  ROCS_CUDA_TRY(pool_alloc(memory, sizeof(int32_t) * (size_t)plan->N, stream));
+  return ROCS_OK;
+}
+
+rocs_status_t plan_request_map_fill(const rocs_plan* plan, cudaStream_t stream, void* memory, RequestMap* out) {
+  const unsigned long long capture = capture_of(stream);
+  std::lock_guard<std::mutex> lock(plan->mu);
+  rocs_plan::ListKey key;
+  bool found = false;
+  DeviceList list;
+  rocs_status_t st = find_list(plan, 0, 0, capture, stream, &key, &found, &list);
+  if (st == ROCS_OK && !found) {
+    st = fill_table(plan, plan->cand_offsets, static_cast<int32_t*>(memory), stream, /*beside=*/true);
+    if (st == ROCS_OK) {
+      list.dev = memory;
+      plan->lists[key] = list;
+      memory = nullptr;
+    }
+  }
+  if (memory != nullptr) cudaFreeAsync(memory, stream);  // not used: a call of another thread was in front of this one
   out->row2req = static_cast<const int32_t*>(list.dev);
   return st;
 }
@@ -465,13 +520,15 @@ static rocs_status_t ikbo_linear_impl(const rocs_plan_t* plan, rocs_dtype_t dtyp
     const size_t need = z_bytes;
     if (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255u))
       return ROCS_ERR_WORKSPACE;
-    // Request half, once per request (Section 4.1): Z = X^R W_CR^T + bias, fp32.
-    rocs_status_t st = linear_dispatch(dtype, plan->R, d_req, d_out, XR, ld_xr, W_CR, ld_wcr, bias,
-                                       nullptr, 0, RequestMap{}, ROCS_ACT_NONE, workspace, d_out,
-                                       /*out_f32=*/true, stream);
+    // Request half, once per request (Section 4.1): Z = X^R W_CR^T + bias, fp32.  The map, where a table of it has to be
+    // made, beside it on the SMs that it leaves idle; the candidate kernel waits for both before it reads either.
+    void* table = nullptr;
+    rocs_status_t st = plan_request_map_begin(plan, stream, &map, &table);
     if (st != ROCS_OK) return st;
-    // The map beside it, on the SMs that it leaves idle; the candidate kernel waits for both before it reads either.
-    st = plan_request_map(plan, stream, &map, /*beside=*/plan->R > 0);
+    st = linear_dispatch(dtype, plan->R, d_req, d_out, XR, ld_xr, W_CR, ld_wcr, bias, nullptr, 0, RequestMap{}, ROCS_ACT_NONE,
+                         workspace, d_out, /*out_f32=*/true, stream);
+    if (st != ROCS_OK && table != nullptr) cudaFreeAsync(table, stream);
+    if (st == ROCS_OK && table != nullptr) st = plan_request_map_fill(plan, stream, table, &map);
     if (st != ROCS_OK) return st;
     Z = (const float*)workspace;
     bias = nullptr;

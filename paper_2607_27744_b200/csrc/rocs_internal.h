@@ -58,7 +58,8 @@ struct rocs_plan {
   // Device lists, made on first use and kept per stream (its id, which is never reused): a list is only
   // ever read on the stream whose order puts its making in front of the reader, or by a graph captured later.
   // Key: stream id, candidates per tile (0: the candidate -> request map), heads (0: no head dimension).
-  mutable std::map<std::tuple<unsigned long long, int32_t, int32_t>, rocs::DeviceList> lists;
+  using ListKey = std::tuple<unsigned long long, int32_t, int32_t>;
+  mutable std::map<ListKey, rocs::DeviceList> lists;
   int device = 0;
   cudaStream_t stream = nullptr;  // stream the plan was created on; its memory is freed there
   unsigned long long capture = 0; // the capture the plan was created in, and lives in; 0: none
@@ -216,10 +217,13 @@ struct TileWalk {
 // in front of them (about 2 us of a 24 us tower on 500 candidates, and host time), the search a handful of
 // cached loads per row; with more rows the loads add up and the launch does not.
 constexpr int64_t kSearchRows = 16384;
-// beside: the launch in front on the stream is one of this library's kernels, which waits for everything in front of
-// itself at once and uses no list of the plan; a table that has to be made is made while it runs (normalised tower on
-// 46262 candidates of 96 requests: 97.1 us behind it, 96.0 beside it).  The kernel behind must wait before it reads the map.
-rocs_status_t plan_request_map(const rocs_plan* plan, cudaStream_t stream, RequestMap* out, bool beside = false);
+rocs_status_t plan_request_map(const rocs_plan* plan, cudaStream_t stream, RequestMap* out);
+// The same around a launch that waits for everything in front of itself before it releases the next (a request half):
+// begin in front of it, and behind it, where begin gave memory for a table, fill.  The table is made while that kernel runs
+// (normalised tower on 46262 candidates of 96 requests: 97.1 us behind it, 96.0 beside it).  The kernel behind must wait
+// before it reads the map.
+rocs_status_t plan_request_map_begin(const rocs_plan* plan, cudaStream_t stream, RequestMap* out, void** memory);
+rocs_status_t plan_request_map_fill(const rocs_plan* plan, cudaStream_t stream, void* memory, RequestMap* out);
 
 // The tiles of a launch whose CTAs take contiguous runs of them: `out` without a list where they can be walked.
 rocs_status_t plan_tile_runs(const rocs_plan* plan, int32_t cands_per_tile, cudaStream_t stream, TileList* out);

@@ -5,6 +5,8 @@ Error metric for every output tensor: max_i |gpu_i - ref_i| / max_i |ref_i|, whi
 the full-size configurations compare a stratified sample of candidates (segment ends, the
 smallest requests, uniform draws) because the oracle is slow by design.
 """
+from concurrent.futures import ThreadPoolExecutor
+
 import numpy as np
 import pytest
 import torch
@@ -761,6 +763,35 @@ def test_candidate_isolation_is_bit_exact(path):
 
 
 # ------------------------------------------------------------------ streams and graphs -------
+@pytest.mark.parametrize("d_cand,d_out", [(128, 512), (320, 128)])   # candidate halves that release early and late
+def test_threads_that_share_a_stream_have_request_tables_of_their_own(d_cand, d_out):
+    # plans of different segments, made and dropped at once by each thread: the memory of one table is the next one's, and
+    # other threads' launches come between a call's request half and its table
+    g = np.random.default_rng(11)
+    W = torch.randn((d_out, 64 + d_cand), device="cuda").to(torch.bfloat16)
+    batches = []
+    for R in (3, 40, 700, 2500):
+        co = wl.offsets_from_counts(np.diff(np.sort(np.concatenate([[0, 20000], g.integers(0, 20001, R - 1)]))).tolist())
+        XR, XC = torch.randn((R, 64), device="cuda").to(torch.bfloat16), torch.randn((20000, d_cand), device="cuda").to(torch.bfloat16)
+        Z = XR.double() @ W[:, :64].double().T
+        want = Z.repeat_interleave(to_dev(np.diff(co)), 0) + XC.double() @ W[:, 64:].double().T
+        batches.append((to_dev(co), torch.from_numpy(co), XR, XC, want))
+    torch.cuda.synchronize()
+
+    def score(batch):
+        cod, host, XR, XC, want = batch
+        outs = []
+        for _ in range(12):
+            plan = rocs.plan_create(cod, host)
+            outs.append(rocs.ikbo_linear(plan, XR, XC, W[:, :64], W[:, 64:]))
+            plan.close()
+        return max(float((y.double() - want).abs().max() / want.abs().max()) for y in outs)
+
+    with ThreadPoolExecutor(len(batches)) as pool:
+        for _ in range(4):
+            assert max(pool.map(score, batches)) <= tol_for("bf16")
+
+
 @pytest.mark.parametrize("warm", [False, True])
 def test_calls_captured_in_a_graph_replay(warm):
     # a plan made outside the capture, its lists made or not yet made when the capture begins; and a plan that
