@@ -87,8 +87,11 @@ namespace rocs {
     }                                                                                                      \
   } while (0)
 // Launches a kernel as a programmatic dependent of the one in front of it on the stream.  The kernel must wait for
-// that one (griddep_wait) before it touches global memory, and may then release the next (in this order: what is
-// released relies on everything in front of its predecessor being complete).
+// that one (griddep_wait) before it touches global memory, and may then release the next, in this order: what is
+// released relies on everything in front of its predecessor being complete.  A kernel may read, or write, before its
+// wait what was complete, or free, in front of a kernel of the same call that kept to this order (the request half or
+// request kernel in front of a candidate kernel).  The request table made beside a request half releases first; nothing
+// but that call's candidate half relies on it, and on the request half only.  Every grid waits before it completes.
 template <typename... P, typename... A>
 inline rocs_status_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream,
                                       A&&... args) {

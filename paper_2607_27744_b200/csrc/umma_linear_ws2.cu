@@ -126,10 +126,12 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   // The set-up above may overlap the end of the kernel in front.  Behind the request half alone, the weights and the
   // rows are streamed at once; that kernel is waited for where its rows are read.  (Launched plainly where there is
   // no request half, 20000 x 256 -> 512 in a chain: 12.3 us, 9.2 us like this.)
-  if (!p.wait_for_previous) griddep_wait();
   // A kernel launched behind this one as a programmatic dependent (the next layer) may set itself up as
-  // SMs become free; it waits for this whole grid before it touches global memory.
-  griddep_launch_dependents();
+  // SMs become free, once everything in front of this one is complete.
+  if (!p.wait_for_previous) {
+    griddep_wait();
+    griddep_launch_dependents();
+  }
 
   if (warp == 0) {
     // ------------------------------ TMA producer (both CTAs) -------------------------------
@@ -220,7 +222,10 @@ linear_ws2_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     const uint32_t tmem_empty_leader[2] = {map_to_cta(smem_u32(&tmem_empty[0]), 0),
                                            map_to_cta(smem_u32(&tmem_empty[1]), 0)};
     uint32_t lt = 0;
-    if (p.wait_for_previous) griddep_wait();
+    if (p.wait_for_previous) {
+      griddep_wait();
+      griddep_launch_dependents();
+    }
     for (int32_t st = group; st < super_tiles; st += p.groups, ++lt) {
       const uint32_t acc = lt & 1;
       const int32_t m0 = st * 2 * BM + (int32_t)rank * BM;
