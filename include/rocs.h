@@ -88,6 +88,11 @@ rocs_status_t rocs_set_path(rocs_path_t path);
  * Each is made on the stream of the first call that needs it (one allocation + one launch), kept
  * for that stream's later calls, and freed in stream order on `stream`; use the plan on that
  * stream, or order other streams behind it (and it behind them before the plan is destroyed).
+ * Stream capture: a captured call on a plan created outside the capture reads lists that exist
+ * when it is captured; the plan, and cand_offsets, must outlive every replay of that graph, and
+ * the graph be launched behind the plan's creation.  A plan created inside a capture has its
+ * lists in that graph's memory: destroy it inside the same capture (calls outside the capture
+ * are allowed while it lives, and make lists of their own).
  * Errors: INVALID_ARG, SEGMENTS, CUDA.
  */
 rocs_status_t rocs_plan_create(rocs_plan_t** out, int32_t R, int64_t N,

@@ -241,6 +241,7 @@ static rocs_status_t make_list_now(const rocs_plan* plan, int32_t cands_per_tile
     if (cudaStreamSynchronize(own) != cudaSuccess) st = ROCS_ERR_CUDA;
     cudaStreamDestroy(own);
   }
+  out->common = true;
   cudaThreadExchangeStreamCaptureMode(&mode);
   return st;
 }
@@ -255,29 +256,47 @@ static unsigned long long capture_of(cudaStream_t stream) {  // 0: the stream is
   return id;
 }
 
-// The list that a call on `stream` may read, if there is one (out->dev stays null otherwise), and the key under which
-// one that is made on the stream is kept.  Under a capture that the plan does not live in there always is one.  The caller
-// holds plan->mu.
+// The list that a call on `stream` may read, if there is one (`found`), and where one that is made on the stream is kept.
+// Under a capture that the plan was not created in there always is one.  The caller holds plan->mu.
+struct ListPlace {
+  std::map<rocs_plan::ListKey, DeviceList>* lists;
+  rocs_plan::ListKey key;
+  bool common;
+  void keep(DeviceList& list) const {
+    list.common = common;
+    (*lists)[key] = list;
+  }
+};
 static rocs_status_t find_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, unsigned long long capture,
-                               cudaStream_t stream, rocs_plan::ListKey* key, bool* found, DeviceList* out) {
+                               cudaStream_t stream, ListPlace* place, bool* found, DeviceList* out) {
   *found = true;
-  if (capture != 0 && capture != plan->capture) {
-    // A graph that outlives this call: it must hold a list that exists now, not one that its own replays would
-    // allocate.  Any list made outside a capture will do, since the graph is launched behind the plan.
+  if (capture == 0 || capture != plan->capture) {
+    // what was complete when it was made serves everybody; a graph that outlives this call, and is launched behind the
+    // plan, also takes a list made on the plan's stream, and otherwise one made now and not one that its own replays
+    // would allocate
     for (const auto& kv : plan->lists)
-      if (std::get<1>(kv.first) == cands_per_tile && std::get<2>(kv.first) == heads) {
+      if (std::get<1>(kv.first) == cands_per_tile && std::get<2>(kv.first) == heads && kv.second.common &&
+          (capture != 0 || std::get<0>(kv.first) == 0)) {
         *out = kv.second;
         return ROCS_OK;
       }
-    const rocs_status_t st = make_list_now(plan, cands_per_tile, heads, out);
-    if (st == ROCS_OK) plan->lists[std::make_tuple(0ull, cands_per_tile, heads)] = *out;
-    return st;
+    if (capture != 0) {
+      const rocs_status_t st = make_list_now(plan, cands_per_tile, heads, out);
+      if (st == ROCS_OK) plan->lists[std::make_tuple(0ull, cands_per_tile, heads)] = *out;
+      return st;
+    }
   }
-  unsigned long long id = 0;
-  if (plan->capture == 0) ROCS_CUDA_TRY(cudaStreamGetId(stream, &id));
-  *key = std::make_tuple(id, cands_per_tile, heads);
-  auto it = plan->lists.find(*key);
-  *found = it != plan->lists.end();
+  unsigned long long id = (unsigned long long)reinterpret_cast<uintptr_t>(stream);
+  place->lists = &plan->captured;
+  place->common = false;
+  if (capture == 0) {
+    ROCS_CUDA_TRY(cudaStreamGetId(stream, &id));
+    place->lists = &plan->lists;
+    place->common = plan->capture == 0 && stream == plan->stream;
+  }
+  place->key = std::make_tuple(id, cands_per_tile, heads);
+  auto it = place->lists->find(place->key);
+  *found = it != place->lists->end();
   if (*found) *out = it->second;
   return ROCS_OK;
 }
@@ -286,12 +305,12 @@ static rocs_status_t plan_list(const rocs_plan* plan, int32_t cands_per_tile, in
                                DeviceList* out) {
   const unsigned long long capture = capture_of(stream);
   std::lock_guard<std::mutex> lock(plan->mu);
-  rocs_plan::ListKey key;
+  ListPlace place;
   bool found;
-  rocs_status_t st = find_list(plan, cands_per_tile, heads, capture, stream, &key, &found, out);
+  rocs_status_t st = find_list(plan, cands_per_tile, heads, capture, stream, &place, &found, out);
   if (st != ROCS_OK || found) return st;
   st = make_list(plan, cands_per_tile, heads, plan->cand_offsets, stream, out);
-  if (st == ROCS_OK) plan->lists[key] = *out;
+  if (st == ROCS_OK) place.keep(*out);
   return st;
 }
 
@@ -315,10 +334,10 @@ rocs_status_t plan_request_map_begin(const rocs_plan* plan, cudaStream_t stream,
   const unsigned long long capture = capture_of(stream);
   {
     std::lock_guard<std::mutex> lock(plan->mu);
-    rocs_plan::ListKey key;
+    ListPlace place;
     bool found;
     DeviceList list;
-    const rocs_status_t st = find_list(plan, 0, 0, capture, stream, &key, &found, &list);
+    const rocs_status_t st = find_list(plan, 0, 0, capture, stream, &place, &found, &list);
     out->row2req = static_cast<const int32_t*>(list.dev);
     if (st != ROCS_OK || found) return st;
   }
@@ -329,15 +348,15 @@ rocs_status_t plan_request_map_begin(const rocs_plan* plan, cudaStream_t stream,
 rocs_status_t plan_request_map_fill(const rocs_plan* plan, cudaStream_t stream, void* memory, RequestMap* out) {
   const unsigned long long capture = capture_of(stream);
   std::lock_guard<std::mutex> lock(plan->mu);
-  rocs_plan::ListKey key;
+  ListPlace place;
   bool found = false;
   DeviceList list;
-  rocs_status_t st = find_list(plan, 0, 0, capture, stream, &key, &found, &list);
+  rocs_status_t st = find_list(plan, 0, 0, capture, stream, &place, &found, &list);
   if (st == ROCS_OK && !found) {
     st = fill_table(plan, plan->cand_offsets, static_cast<int32_t*>(memory), stream, /*beside=*/true);
     if (st == ROCS_OK) {
       list.dev = memory;
-      plan->lists[key] = list;
+      place.keep(list);
       memory = nullptr;
     }
   }
@@ -459,8 +478,12 @@ rocs_status_t rocs_plan_destroy(rocs_plan_t* plan) {
   if (!plan) return ROCS_OK;
   rocs_status_t st = ROCS_OK;
   // Freed in stream order behind whatever the caller enqueued on the plan's stream.
-  for (auto& kv : plan->lists)
-    if (kv.second.dev && cudaFreeAsync(kv.second.dev, plan->stream) != cudaSuccess) st = ROCS_ERR_CUDA;
+  for (const auto* lists : {&plan->captured, &plan->lists})
+    for (const auto& kv : *lists)
+      if (kv.second.dev && cudaFreeAsync(kv.second.dev, plan->stream) != cudaSuccess) {
+        cudaGetLastError();  // of a graph that has not run, or has ended already: not the next call's error
+        st = ROCS_ERR_CUDA;
+      }
   delete plan;
   return st;
 }

@@ -32,6 +32,7 @@ struct TileList {
 struct DeviceList {
   void* dev = nullptr;
   int32_t num = 0;
+  bool common = false;  // complete, or made on the plan's stream: for whoever is ordered behind the plan
 };
 
 // One unit of work of the attention kernels: one head of `count` consecutive candidates of a request.
@@ -55,14 +56,18 @@ struct rocs_plan {
   const int32_t* cand_offsets = nullptr;  // device, borrowed
   std::vector<int32_t> offsets_host;      // [R+1]
   mutable std::mutex mu;
-  // Device lists, made on first use and kept per stream (its id, which is never reused): a list is only
-  // ever read on the stream whose order puts its making in front of the reader, or by a graph captured later.
+  // Device lists, made on first use and kept per stream (its id, which is never reused; 0: complete when it was made):
+  // a list is only ever read on the stream whose order puts its making in front of the reader, or, if it is a common one,
+  // by a graph captured later.
   // Key: stream id, candidates per tile (0: the candidate -> request map), heads (0: no head dimension).
   using ListKey = std::tuple<unsigned long long, int32_t, int32_t>;
   mutable std::map<ListKey, rocs::DeviceList> lists;
+  // The same of calls inside the capture that the plan was created in (by stream: ids cannot be asked for there).  They
+  // are memory of the graph, which exists while it runs, and serve no call outside it.
+  mutable std::map<ListKey, rocs::DeviceList> captured;
   int device = 0;
   cudaStream_t stream = nullptr;  // stream the plan was created on; its memory is freed there
-  unsigned long long capture = 0; // the capture the plan was created in, and lives in; 0: none
+  unsigned long long capture = 0; // the capture the plan was created in; 0: none
 };
 
 namespace rocs {

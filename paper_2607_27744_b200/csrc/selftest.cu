@@ -1,4 +1,4 @@
-// Self-test of the bounded waits (not part of the public header): a kernel that waits on a barrier
+// Self-tests (not part of the public header).  Bounded waits: a kernel that waits on a barrier
 // nobody ever arrives on, through the same wait routines the tensor-core kernels use, with a limit
 // given by the caller.  The wait must give up, record its code in the device status word and let the
 // kernel return, so that the context stays usable; rocs_last_device_status then reports
@@ -46,4 +46,11 @@ extern "C" rocs_status_t rocs_selftest_wait_expires(int flavour, uint32_t limit_
                                                                gave_up_dev);
   ROCS_CUDA_TRY(cudaGetLastError());
   return ROCS_OK;
+}
+
+// Number of device lists that a plan keeps: of eager calls and of graphs captured later (0), of calls inside the capture it
+// was created in (1).  Tests ask whether the calls they make reach the code that makes and finds lists.
+extern "C" int rocs_selftest_plan_lists(const rocs_plan_t* plan, int captured) {
+  std::lock_guard<std::mutex> lock(plan->mu);
+  return (int)(captured ? plan->captured : plan->lists).size();
 }

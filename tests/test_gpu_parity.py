@@ -5,6 +5,7 @@ Error metric for every output tensor: max_i |gpu_i - ref_i| / max_i |ref_i|, whi
 the full-size configurations compare a stratified sample of candidates (segment ends, the
 smallest requests, uniform draws) because the oracle is slow by design.
 """
+import ctypes
 from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
@@ -826,6 +827,118 @@ def test_calls_captured_in_a_graph_replay(warm):
             assert all(np.array_equal(_bits(t), w) for t, w in zip(outs, want))
     again = layers(plan)   # and the plan still serves calls outside the graph
     assert all(np.array_equal(_bits(t), w) for t, w in zip(again, want))
+
+
+def _lists(plan, captured=False):
+    fn = rocs.lib().rocs_selftest_plan_lists
+    fn.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    return fn(plan.handle, int(captured))
+
+
+class _ListedBatch:
+    """A batch whose calls all need a list of the plan: the request table of more than 16384 candidates, the attention
+    items of more than 256 requests (fp32: 128) and the interaction tiles of more than 512 (fp32: 128)."""
+    LISTS = 5   # one for bf16 linear, attention and interaction each, two for the fp32 ones
+
+    def __init__(self):
+        g = np.random.default_rng(4)
+        self.co = wl.offsets_from_counts(g.integers(0, 68, 600).tolist())
+        so = wl.offsets_from_counts(g.integers(1, 40, 600).tolist())
+        cfg = wl.CONFIGS[5].with_(R=600, d_req=64, d_cand=64, d_out=128, H=2, dh=32, n_r=8, n_c=8, d_emb=64, n_ro=4, n_co=4)
+        assert int(self.co[-1]) > 16384
+        lin, att, gi = wl.linear_inputs(cfg, self.co), wl.dca_inputs(cfg, self.co, so), wl.glm_inputs(cfg, self.co)
+        self.W, self.XR, self.XC = to_dev(lin["W"]), to_dev(lin["XR"]), to_dev(lin["XC"])
+        self.Q, self.K, self.V, self.so = to_dev(att["Q"]), to_dev(att["K"]), to_dev(att["V"]), to_dev(so)
+        self.GR, self.GC, self.GW = to_dev(gi["XR"]), to_dev(gi["XC"]), to_dev(gi["W"])
+        self.f = [t.float() for t in (self.Q, self.K, self.V, self.GR, self.GC)]
+        self.cod, self.host = to_dev(self.co), torch.from_numpy(self.co)
+        torch.cuda.synchronize()
+
+    def plan(self):
+        return rocs.plan_create(self.cod, self.host)
+
+    def layers(self, plan):
+        Q, K, V, GR, GC = self.f
+        return [rocs.ikbo_linear(plan, self.XR, self.XC, self.W[:, :64], self.W[:, 64:], relu=True),
+                rocs.dca_attention(plan, self.Q, self.K, self.V, self.so),
+                rocs.glm_interaction(plan, self.GR, self.GC, self.GW, 4, 4)["OC"],
+                rocs.dca_attention(plan, Q, K, V, self.so),
+                rocs.glm_interaction(plan, GR, GC, None)["YC"]]
+
+
+def _same(outs, want):
+    return all(np.array_equal(_bits(t), w) for t, w in zip(outs, want))
+
+
+@pytest.mark.parametrize("before", ["nothing", "plan's stream", "another stream"])
+def test_captured_calls_find_lists_made_outside(before):
+    # what the plan holds when the capture begins: nothing, lists made on its stream (the graph may read them), lists made
+    # on a stream that the graph's is not ordered behind (it must not)
+    b = _ListedBatch()
+    want = [_bits(t) for t in b.layers(b.plan())]
+    plan = b.plan()
+    if before == "plan's stream":
+        b.layers(plan)
+    elif before == "another stream":
+        with torch.cuda.stream(torch.cuda.Stream()):
+            b.layers(plan)
+    had = _lists(plan)
+    assert had == (0 if before == "nothing" else b.LISTS)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        outs = b.layers(plan)
+    assert _lists(plan) == had + (0 if before == "plan's stream" else b.LISTS)
+    for _ in range(3):
+        for t in outs:
+            t.zero_()
+        graph.replay()
+        assert _same(outs, want)
+    assert _same(b.layers(plan), want)     # what was complete when it was made serves eager calls too
+    assert _lists(plan) == had + (0 if before == "plan's stream" else b.LISTS)
+
+
+@pytest.mark.parametrize("closed_inside", [True, False])
+def test_a_plan_created_inside_a_capture(closed_inside):
+    # its lists are the graph's memory; eager calls on it, if it stays open, make lists of their own
+    b = _ListedBatch()
+    want = [_bits(t) for t in b.layers(b.plan())]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        plan = b.plan()
+        outs = b.layers(plan)
+        assert _lists(plan) == 0 and _lists(plan, captured=True) == b.LISTS
+        if closed_inside:
+            plan.close()
+    if not closed_inside:
+        assert _same(b.layers(plan), want)
+        assert _lists(plan) == b.LISTS
+    for _ in range(3 if closed_inside else 1):
+        for t in outs:
+            t.zero_()
+        graph.replay()
+        assert _same(outs, want)
+    if not closed_inside:
+        assert _same(b.layers(plan), want)
+        torch.cuda.synchronize()
+        plan.close()
+    assert rocs.last_device_status() == 0
+
+
+def test_one_plan_on_two_streams():
+    # lists of either stream's own, made at the same time; results are those of one stream
+    b = _ListedBatch()
+    want = [_bits(t) for t in b.layers(b.plan())]
+    plan, streams = b.plan(), [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    outs = []
+    for _ in range(4):
+        for s in streams:
+            with torch.cuda.stream(s):
+                outs.append(b.layers(plan))
+    torch.cuda.synchronize()
+    assert _lists(plan) == 2 * b.LISTS
+    assert all(_same(o, want) for o in outs)
 
 
 # ------------------------------------------------------------------ ABI errors --------------
