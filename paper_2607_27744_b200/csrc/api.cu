@@ -94,11 +94,12 @@ uint32_t* device_status_word() {
 // also takes a staged copy to the device and an allocation for it (plan + query projection + attention of
 // 3 requests x 574 candidates: 49.5 us that way, 42.3 us this way; plan + interaction of 128 x 1024
 // candidates: 159.6 and 156.4 us).  All blocks read the same R offsets, from L2; beyond kMaxScan requests
-// (the 48 KB of shared memory a block has without asking for more) the host adds up.
+// (the 48 KB of shared memory a block has without asking for more) one block adds up for all, into global
+// memory in front of them: under a capture a copy from the host would read this call's host memory at every replay.
 constexpr int kListThreads = 256;
 constexpr int32_t kMaxScan = 12000;
 
-// Prefix sums of the entries per request in shared memory; all threads of the block take part.
+// Prefix sums of the entries per request in the block's memory; all threads of the block take part.
 __device__ void scan_entries(int32_t R, int32_t cands_per_tile, const int32_t* __restrict__ off, int32_t* pre) {
   __shared__ int32_t warp_sum[kListThreads / 32];
   for (int32_t r = threadIdx.x; r < R; r += kListThreads) pre[r] = (off[r + 1] - off[r] + cands_per_tile - 1) / cands_per_tile;
@@ -166,6 +167,13 @@ __global__ void __launch_bounds__(kListThreads) expand_list_kernel(int32_t R, in
     static_cast<DcaItem*>(out)[i] = DcaItem{req, c, count, h};
 }
 
+__global__ void __launch_bounds__(kListThreads) scan_entries_kernel(int32_t R, int32_t cands_per_tile,
+                                                                    const int32_t* __restrict__ off, int32_t* base) {
+  ptx::griddep_wait_for(off);
+  ptx::griddep_launch_dependents();
+  scan_entries(R, cands_per_tile, off, base);
+}
+
 int64_t plan_entries(const rocs_plan* plan, int32_t cands_per_tile) {
   int64_t entries = 0;
   for (int32_t r = 0; r < plan->R; ++r)
@@ -199,14 +207,10 @@ static rocs_status_t make_list(const rocs_plan* plan, int32_t cands_per_tile, in
     int32_t* base_dev = nullptr;
     cudaError_t e = cudaSuccess;
     if (R > kMaxScan) {
-      std::vector<int32_t> base((size_t)R + 1, 0);
-      for (int32_t r = 0; r < R; ++r)
-        base[r + 1] = base[r] + (int32_t)(((int64_t)plan->offsets_host[r + 1] - plan->offsets_host[r] + cands_per_tile - 1) /
-                                          cands_per_tile);
-      e = pool_alloc((void**)&base_dev, sizeof(int32_t) * base.size(), stream);
-      // Pageable source: the copy is staged before the call returns, so `base` may go away.
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(base_dev, base.data(), sizeof(int32_t) * base.size(), cudaMemcpyHostToDevice, stream);
+      e = pool_alloc((void**)&base_dev, sizeof(int32_t) * ((size_t)R + 1), stream);
+      if (e == cudaSuccess &&
+          launch_dependent(scan_entries_kernel, dim3(1), kListThreads, 0, stream, R, cands_per_tile, off, base_dev) != ROCS_OK)
+        e = cudaErrorUnknown;
     }
     if (e == cudaSuccess &&
         launch_dependent(expand_list_kernel, dim3((unsigned)((total + kListThreads - 1) / kListThreads)), kListThreads,

@@ -925,6 +925,35 @@ def test_a_plan_created_inside_a_capture(closed_inside):
     assert rocs.last_device_status() == 0
 
 
+def test_a_graph_of_more_requests_than_a_block_adds_up_keeps_nothing_of_the_host():
+    # the plan lives inside the capture and its lists are made at every replay, when the calls' host memory is long reused
+    R = 12001
+    g = np.random.default_rng(9)
+    co, so = wl.offsets_from_counts(g.integers(0, 4, R).tolist()), wl.offsets_from_counts(g.integers(0, 5, R).tolist())
+    cfg = wl.CONFIGS[5].with_(R=R, H=2, dh=32, n_r=8, n_c=8, d_emb=64, n_ro=0, n_co=0)
+    att, gi = wl.dca_inputs(cfg, co, so), wl.glm_inputs(cfg, co)
+    Q, K, V, sod, GR, GC = (to_dev(a) for a in (att["Q"], att["K"], att["V"], so, gi["XR"], gi["XC"]))
+    cod, host = to_dev(co), torch.from_numpy(co)
+
+    def layers(plan):
+        return [rocs.dca_attention(plan, Q, K, V, sod), rocs.glm_interaction(plan, GR, GC, None)["YC"]]
+
+    want = [_bits(t) for t in layers(rocs.plan_create(cod, host))]
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        plan = rocs.plan_create(cod, host)
+        outs = layers(plan)
+        plan.close()
+    for _ in range(3):
+        junk = [np.full(R + 1, 7, np.int32) for _ in range(200)]
+        for t in outs:
+            t.zero_()
+        graph.replay()
+        assert _same(outs, want)
+        del junk
+
+
 def test_one_plan_on_two_streams():
     # lists of either stream's own, made at the same time; results are those of one stream
     b = _ListedBatch()
