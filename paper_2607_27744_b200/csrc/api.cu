@@ -98,6 +98,7 @@ uint32_t* device_status_word() {
 // memory in front of them: under a capture a copy from the host would read this call's host memory at every replay.
 constexpr int kListThreads = 256;
 constexpr int32_t kMaxScan = 12000;
+constexpr int32_t kAddUpRequests = 64;  // requests that are walked sooner than a number is looked up
 
 // Prefix sums of the entries per request in the block's memory; all threads of the block take part.
 __device__ void scan_entries(int32_t R, int32_t cands_per_tile, const int32_t* __restrict__ off, int32_t* pre) {
@@ -174,11 +175,25 @@ __global__ void __launch_bounds__(kListThreads) scan_entries_kernel(int32_t R, i
   scan_entries(R, cands_per_tile, off, base);
 }
 
-int64_t plan_entries(const rocs_plan* plan, int32_t cands_per_tile) {
+static int64_t add_up_entries(const rocs_plan* plan, int32_t cands_per_tile) {
+  const uint32_t per = (uint32_t)cands_per_tile;  // counts are below 2^31: no sum here leaves 32 bits
   int64_t entries = 0;
   for (int32_t r = 0; r < plan->R; ++r)
-    entries += ((int64_t)plan->offsets_host[r + 1] - plan->offsets_host[r] + cands_per_tile - 1) / cands_per_tile;
+    entries += ((uint32_t)(plan->offsets_host[r + 1] - plan->offsets_host[r]) + per - 1) / per;
   return entries;
+}
+// The caller holds plan->mu.
+static int64_t entries_locked(const rocs_plan* plan, int32_t cands_per_tile) {
+  if (plan->R <= kAddUpRequests) return add_up_entries(plan, cands_per_tile);
+  const auto known = plan->entries.find(cands_per_tile);
+  if (known != plan->entries.end()) return known->second;
+  return plan->entries[cands_per_tile] = add_up_entries(plan, cands_per_tile);
+}
+
+int64_t plan_entries(const rocs_plan* plan, int32_t cands_per_tile) {
+  if (plan->R <= kAddUpRequests) return add_up_entries(plan, cands_per_tile);
+  std::lock_guard<std::mutex> lock(plan->mu);
+  return entries_locked(plan, cands_per_tile);
 }
 
 static rocs_status_t fill_table(const rocs_plan* plan, const int32_t* off, int32_t* table, cudaStream_t stream, bool beside) {
@@ -187,7 +202,7 @@ static rocs_status_t fill_table(const rocs_plan* plan, const int32_t* off, int32
 }
 
 // Allocates and fills one list of the plan (key as in rocs_plan::lists) in the order of `stream`, from the
-// offsets at `off`.
+// offsets at `off`.  The caller holds plan->mu.
 static rocs_status_t make_list(const rocs_plan* plan, int32_t cands_per_tile, int32_t heads, const int32_t* off,
                                cudaStream_t stream, DeviceList* out) {
   static_assert(sizeof(Tile) == 16 && sizeof(DcaItem) == 16, "list entries");
@@ -200,7 +215,7 @@ static rocs_status_t make_list(const rocs_plan* plan, int32_t cands_per_tile, in
     }
   } else if (plan->N > 0) {
     const int32_t R = plan->R;
-    const int64_t total = plan_entries(plan, cands_per_tile) * std::max(heads, 1);
+    const int64_t total = entries_locked(plan, cands_per_tile) * std::max(heads, 1);
     if (total > 0x7fffffffLL) return ROCS_ERR_UNSUPPORTED;
     list.num = (int32_t)total;
     ROCS_CUDA_TRY(pool_alloc(&list.dev, sizeof(Tile) * (size_t)total, stream));
@@ -378,8 +393,9 @@ rocs_status_t plan_tiles(const rocs_plan* plan, int32_t cands_per_tile, cudaStre
 }
 
 rocs_status_t plan_tile_runs(const rocs_plan* plan, int32_t cands_per_tile, cudaStream_t stream, TileList* out) {
+  if (plan->R > kMaxTileWalkRequests) return plan_tiles(plan, cands_per_tile, stream, out);
   const int64_t total = plan_entries(plan, cands_per_tile);
-  if (plan->R > kMaxTileWalkRequests || total > kMaxTileWalk) return plan_tiles(plan, cands_per_tile, stream, out);
+  if (total > kMaxTileWalk) return plan_tiles(plan, cands_per_tile, stream, out);
   *out = TileList{nullptr, (int32_t)total};
   return ROCS_OK;
 }

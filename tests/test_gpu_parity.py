@@ -6,6 +6,7 @@ the full-size configurations compare a stratified sample of candidates (segment 
 smallest requests, uniform draws) because the oracle is slow by design.
 """
 import ctypes
+import time
 from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
@@ -952,6 +953,29 @@ def test_a_graph_of_more_requests_than_a_block_adds_up_keeps_nothing_of_the_host
         graph.replay()
         assert _same(outs, want)
         del junk
+
+
+def test_calls_on_a_kept_plan_do_not_walk_its_requests():
+    # the host's share of a call (it returns without waiting for the device) on 200000 requests: a walk over the offsets is
+    # some 180 us, and an interaction took two; without, a call is some 10 us
+    R = 200000
+    co = torch.arange(R + 1, dtype=torch.int32)
+    so = torch.arange(R + 1, dtype=torch.int32, device="cuda")
+    bf = dict(dtype=torch.bfloat16, device="cuda")
+    XR, XC, Q = torch.zeros((R, 8, 64), **bf), torch.zeros((R, 8, 64), **bf), torch.zeros((R, 1, 1, 32), **bf)
+    plan = rocs.plan_create(co.cuda(), co)
+    raw, att = {"YC": torch.empty((R, 8, 16), **bf)}, torch.empty_like(Q)
+    calls = {"interaction": lambda: rocs.glm_interaction(plan, XR, XC, None, want_request_side=False, outs=raw),
+             "attention": lambda: rocs.dca_attention(plan, Q, Q[:, 0], Q[:, 0], so, out=att)}
+    for name, call in calls.items():
+        took = []
+        for _ in range(21):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            call()
+            took.append(time.perf_counter() - t0)
+        assert sorted(took)[10] < 150e-6, (name, sorted(took)[10])
+    torch.cuda.synchronize()
 
 
 def test_one_plan_on_two_streams():
