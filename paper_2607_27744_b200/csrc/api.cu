@@ -50,25 +50,28 @@ __device__ uint32_t g_device_status;
 // threshold every batch would pay the driver's allocation path again.
 static cudaError_t pool_alloc(void** ptr, size_t bytes, cudaStream_t stream) {
   static std::mutex mu;
-  static std::map<int, cudaMemPool_t> pools;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
+  static std::map<unsigned long long, cudaMemPool_t> pools;  // by context: a reset takes its pool along
+  unsigned long long context = context_id();
+  cudaError_t e;
+  if (context == 0) {  // the thread's first CUDA call
+    if ((e = cudaFree(nullptr)) != cudaSuccess) return e;
+    context = context_id();
+  }
   cudaMemPool_t pool = nullptr;
   {
     std::lock_guard<std::mutex> lock(mu);
-    auto it = pools.find(dev);
+    auto it = pools.find(context);
     if (it == pools.end()) {
       cudaMemPoolProps props = {};
       props.allocType = cudaMemAllocationTypePinned;
       props.handleTypes = cudaMemHandleTypeNone;
       props.location.type = cudaMemLocationTypeDevice;
-      props.location.id = dev;
+      if ((e = cudaGetDevice(&props.location.id)) != cudaSuccess) return e;
       e = cudaMemPoolCreate(&pool, &props);
       if (e != cudaSuccess) return e;
       uint64_t keep = 1ull << 30;
       cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-      pools[dev] = pool;
+      pools[context] = pool;
     } else {
       pool = it->second;
     }
@@ -77,14 +80,8 @@ static cudaError_t pool_alloc(void** ptr, size_t bytes, cudaStream_t stream) {
 }
 
 uint32_t* device_status_word() {
-  static std::atomic<uint32_t*> found[64];  // the word's address on each device: fixed while the library is loaded
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-  uint32_t* p = dev < 64 ? found[dev].load(std::memory_order_acquire) : nullptr;
-  if (p == nullptr) {
-    if (cudaGetSymbolAddress((void**)&p, g_device_status) != cudaSuccess) return nullptr;
-    if (dev < 64) found[dev].store(p, std::memory_order_release);
-  }
+  uint32_t* p = nullptr;
+  if (cudaGetSymbolAddress((void**)&p, g_device_status) != cudaSuccess) return nullptr;
   return p;
 }
 

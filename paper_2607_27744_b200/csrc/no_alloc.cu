@@ -23,19 +23,23 @@ constexpr size_t kStaticBytes = kStaticZFloats * sizeof(float) + kStaticMapEntri
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
 std::mutex g_mu;
-void* g_scratch_addr[64] = {};  // device address of g_static_scratch, per device ordinal
+struct {
+  unsigned long long context;
+  void* addr;
+} g_scratch_addr[64] = {};  // device address of g_static_scratch in a context, per device ordinal
 
-// Resolves (once per device, with that device current) where the array lives on the device.
+// Resolves (once per context, with its device current) where the array lives on the device.
 rocs_status_t scratch_address(void** out) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return ROCS_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_mu);
-  if (!g_scratch_addr[dev]) {
+  const unsigned long long context = context_id();
+  if (context == 0 || g_scratch_addr[dev].context != context) {
     void* p = nullptr;
     if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) return ROCS_ERR_CUDA;
-    g_scratch_addr[dev] = p;
+    g_scratch_addr[dev] = {context_id(), p};
   }
-  *out = g_scratch_addr[dev];
+  *out = g_scratch_addr[dev].addr;
   return ROCS_OK;
 }
 

@@ -1,7 +1,6 @@
-// Host helper: builds TMA tensor maps with cuTensorMapEncodeTiled, resolved at run time through
-// cudaGetDriverEntryPoint so that librocs.so has no link-time dependency on libcuda.
-#include <mutex>
-
+// Host helpers on the driver API: TMA tensor maps with cuTensorMapEncodeTiled, the id of the current context with
+// cuCtxGetId, both resolved at run time through cudaGetDriverEntryPoint so that librocs.so has no link-time dependency
+// on libcuda.
 #include "rocs_internal.h"
 #include "sm100_ptx.cuh"
 
@@ -12,20 +11,28 @@ using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+using GetContextIdFn = CUresult (*)(CUcontext, unsigned long long*);
+
+template <typename F>
+F driver_function(const char* name) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) return nullptr;
+  return reinterpret_cast<F>(p);
+}
+
 EncodeTiledFn encode_tiled() {
-  static EncodeTiledFn fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  });
+  static const EncodeTiledFn fn = driver_function<EncodeTiledFn>("cuTensorMapEncodeTiled");
   return fn;
 }
 
 }  // namespace
+
+unsigned long long context_id() {
+  static const GetContextIdFn fn = driver_function<GetContextIdFn>("cuCtxGetId");
+  unsigned long long id = 0;
+  return fn != nullptr && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
 
 bool make_tensor_map_2d(CUtensorMap* map, const void* base, CUtensorMapDataType dtype, uint32_t elem_bytes,
                         uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows, uint32_t box_cols,
