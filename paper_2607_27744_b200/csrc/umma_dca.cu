@@ -38,8 +38,10 @@
 // fp32 holds 2^x up to x = 128, so a row overflows only if a later score exceeds that maximum by about
 // 88 nats; such a row shows Inf/NaN in its sums at the end of the item and is then
 // computed again by its two threads alone in plain fp32 loops (slow, correct, reached only by inputs
-// whose scores span more than fp32's exponent range).  Every decision is taken per row from that
-// row's own values, so a row's bits never depend on its neighbours.
+// whose scores span more than fp32's exponent range).  Every decision inside a row is taken from that row's own values,
+// so in a batch of given shape a row's bits do not depend on its neighbours' values.  They do depend on the shape: whether
+// items are split, and over how many CTAs, follows from the number of items and the average sequence, and a split has
+// references and an order of summation of its own.
 #include <algorithm>
 
 #include "rocs_internal.h"
@@ -438,7 +440,7 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     // a side that is done before.  In SPLIT every side has its part of the CTA's item and no other.
     auto claim_next = [&]() {
       int32_t c = -1;
-      if (!SPLIT && lane == 0) c = claim_cta(claims, abort_flag, p.status, kStatusDca | 14);
+      if (!SPLIT && lane == 0) c = claim_cta(claims, abort_flag, p.status, kStatusDca | 16);
       i = __shfl_sync(0xffffffffu, c, 0);
     };
     if (!SPLIT && side == 1) claim_next();  // the CTA's own item goes to side A
