@@ -880,12 +880,15 @@ static rocs_status_t launch_dca(const rocs_plan* plan, int32_t n_q, int32_t H, f
   if (num > 0x7fffffffLL) return ROCS_ERR_UNSUPPORTED;
   if (num == 0) return ROCS_OK;
   // Items that fit the SMs once are split along their keys (SPLIT): over the two sides of a CTA, and over the CTAs
-  // of the largest cluster of which every item still gets one at the same time (a cluster stays inside one of the
-  // chip's partitions of 16 to 20 SMs), two key blocks per side at least.  Short sequences are not worth it.
+  // of the largest cluster of which every item still gets one at the same time, two key blocks per side at least.  Short
+  // sequences are not worth it.  How many clusters run at once differs from chip to chip (a cluster stays inside one of
+  // its partitions, of which each chip has other SMs: 74 pairs, 33 of 4 and 15 of 8 on one), and an item more than that
+  // takes a second round: 16 items of 4096 keys 26.1 us over clusters of 8 there, 14.6 us over 4.  The numbers below are a
+  // little less, and constants, so that results do not depend on which GPU they were computed.
   const int64_t blocks = (T + plan->R - 1) / plan->R / BKV + 1;  // of an average sequence
   const bool split = num <= sms && blocks >= 3;
   int32_t cluster = 1;
-  const int32_t most[4] = {sms, 70, 32, 16};
+  const int32_t most[4] = {sms, 70, 32, 14};
   for (int i = 1; i < 4 && split; ++i)
     if (num <= most[i] && (4 << i) <= blocks) cluster = 1 << i;
   // Requests that a producer warp looks through itself, at every item; the list is a launch in front.  Projection and
