@@ -100,7 +100,7 @@ constexpr int32_t kAddUpRequests = 64;  // requests that are walked sooner than 
 // Prefix sums of the entries per request in the block's memory; all threads of the block take part.
 __device__ void scan_entries(int32_t R, int32_t cands_per_tile, const int32_t* __restrict__ off, int32_t* pre) {
   __shared__ int32_t warp_sum[kListThreads / 32];
-  for (int32_t r = threadIdx.x; r < R; r += kListThreads) pre[r] = (off[r + 1] - off[r] + cands_per_tile - 1) / cands_per_tile;
+  for (int32_t r = threadIdx.x; r < R; r += kListThreads) pre[r] = tiles_of(off[r + 1] - off[r], cands_per_tile);
   __syncthreads();
   const int32_t chunk = (R + kListThreads - 1) / kListThreads;
   const int32_t r0 = min((int32_t)threadIdx.x * chunk, R), r1 = min(r0 + chunk, R);
@@ -152,10 +152,10 @@ __global__ void __launch_bounds__(kListThreads) expand_list_kernel(int32_t R, in
     scan_entries(R, cands_per_tile, off, pre);
     base = pre;
   }
-  const int32_t i = blockIdx.x * kListThreads + threadIdx.x;
-  if (i >= total) return;
+  const uint32_t i = blockIdx.x * (uint32_t)kListThreads + threadIdx.x;  // the last block of nearly 2^31 entries reaches past them
+  if (i >= (uint32_t)total) return;
   int32_t req, local, per_head;
-  find_entry(R, max(heads, 1), base, i, req, local, per_head);
+  find_entry(R, max(heads, 1), base, (int32_t)i, req, local, per_head);
   const int32_t h = local / per_head, t = local % per_head;
   const int32_t c = off[req] + t * cands_per_tile;
   const int32_t count = min(cands_per_tile, off[req + 1] - c);
@@ -173,10 +173,8 @@ __global__ void __launch_bounds__(kListThreads) scan_entries_kernel(int32_t R, i
 }
 
 static int64_t add_up_entries(const rocs_plan* plan, int32_t cands_per_tile) {
-  const uint32_t per = (uint32_t)cands_per_tile;  // counts are below 2^31: no sum here leaves 32 bits
   int64_t entries = 0;
-  for (int32_t r = 0; r < plan->R; ++r)
-    entries += ((uint32_t)(plan->offsets_host[r + 1] - plan->offsets_host[r]) + per - 1) / per;
+  for (int32_t r = 0; r < plan->R; ++r) entries += tiles_of(plan->offsets_host[r + 1] - plan->offsets_host[r], cands_per_tile);
   return entries;
 }
 // The caller holds plan->mu.

@@ -125,6 +125,11 @@ inline size_t elem_size(rocs_dtype_t dt) { return dt == ROCS_BF16 ? 2 : 4; }
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// Tiles of at most `per` of n candidates.  Unsigned: a request may have all of nearly 2^31.
+__host__ __device__ inline int32_t tiles_of(int32_t n, int32_t per) {
+  return (int32_t)(((uint32_t)n + (uint32_t)per - 1u) / (uint32_t)per);
+}
+
 // Tiles of at most `cands_per_tile` candidates that the batch's requests are cut into; the plan keeps the number.
 int64_t plan_entries(const rocs_plan* plan, int32_t cands_per_tile);
 
@@ -187,7 +192,7 @@ struct TileWalk {
   __device__ __forceinline__ void start(int32_t t, int lane) {
     const int32_t chunk = (R + 31) / 32, r0 = min(lane * chunk, R), r1 = min(r0 + chunk, R);
     int32_t sum = 0;
-    for (int32_t r = r0; r < r1; ++r) sum += (offsets[r + 1] - offsets[r] + per - 1) / per;
+    for (int32_t r = r0; r < r1; ++r) sum += tiles_of(offsets[r + 1] - offsets[r], per);
     int32_t incl = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -201,7 +206,7 @@ struct TileWalk {
     while (true) {
       first = offsets[r];
       end = offsets[r + 1];
-      n = (end - first + per - 1) / per;
+      n = tiles_of(end - first, per);
       if (local < n) break;
       local -= n;
       ++r;

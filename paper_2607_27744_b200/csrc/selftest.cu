@@ -54,3 +54,6 @@ extern "C" int rocs_selftest_plan_lists(const rocs_plan_t* plan, int captured) {
   std::lock_guard<std::mutex> lock(plan->mu);
   return (int)(captured ? plan->captured : plan->lists).size();
 }
+
+// Tiles of a request as the kernels count them.
+extern "C" int32_t rocs_selftest_tiles_of(int32_t n, int32_t per) { return rocs::tiles_of(n, per); }

@@ -3,6 +3,8 @@
 #include <cuda_bf16.h>
 #include <cstdint>
 
+#include "rocs_internal.h"
+
 namespace rocs {
 
 // Copies `rows` dense rows of `d` elements (fp32 or bf16, global memory) into shared memory as fp32
@@ -71,7 +73,7 @@ __device__ __forceinline__ FoundTile find_tile_in_block(int32_t R, int32_t per, 
   __shared__ FoundTile found;
   const int32_t t = threadIdx.x, lane = t % 32;
   const int32_t c0 = t < R ? off[t] : 0, n = t < R ? off[t + 1] - c0 : 0;
-  const int32_t tiles = (n + per - 1) / per, entries = tiles * heads;
+  const int32_t tiles = tiles_of(n, per), entries = tiles * heads;
   int32_t incl = entries;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {

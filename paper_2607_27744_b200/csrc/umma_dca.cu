@@ -224,7 +224,7 @@ __device__ __forceinline__ DcaItem find_item(const int32_t* __restrict__ off, in
   for (int32_t r0 = 0; r0 < R; r0 += 32) {
     const int32_t r = r0 + lane;
     const int32_t c0 = r < R ? off[r] : 0, n = r < R ? off[r + 1] - c0 : 0;
-    const int32_t tiles = (n + per - 1) / per, entries = tiles * heads;
+    const int32_t tiles = tiles_of(n, per), entries = tiles * heads;
     int32_t incl = entries;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {

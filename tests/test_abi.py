@@ -55,6 +55,12 @@ def test_binding_fails_loudly_without_the_library(monkeypatch, tmp_path):
         binding.lib()
 
 
+@pytest.mark.parametrize("per", [1, 7, 32, 128])
+@pytest.mark.parametrize("n", [0, 1, 31, 32, 33, 2**31 - 128, 2**31 - 1])
+def test_tiles_of_a_request_of_any_legal_size(lib, n, per):
+    assert lib.rocs_selftest_tiles_of(n, per) == -(-n // per)
+
+
 @pytest.mark.parametrize("call,error", [
     (lambda plan, x: binding.ikbo_linear(plan, None, x(4), None, x(3, 8)), IndexError),       # rows of one dimension
     (lambda plan, x: binding.linear(x(4), x(3, 8)), ValueError),
