@@ -27,8 +27,8 @@
  *     ROCS_BF16: bf16 storage, fp32 accumulation (tensor cores where the shape allows),
  *     softmax in fp32, results rounded to bf16 (nearest even).  ROCS_F32: fp32 storage
  *     and plain fp32 FMA arithmetic.
- *   - Results are run-to-run bitwise deterministic, and a candidate's output bits do not
- *     depend on any other candidate's inputs (the GLM invariant, Eq. 1).
+ *   - Results are run-to-run bitwise deterministic, and in a batch of given shape a candidate's
+ *     output bits do not depend on any other candidate's inputs (the GLM invariant, Eq. 1).
  */
 #ifndef ROCS_H_
 #define ROCS_H_

@@ -23,7 +23,8 @@
 // conflicts under the 128-byte swizzle).  Outputs leave as 8-byte stores that fill whole 32-byte sectors.
 // With compression the products are formed transposed, so that an accumulator, split into bf16 parts, is the K x N
 // operand of OC = ZR + W_CC YC as it stands; W_CC is repeated for every candidate of the fragment, and the other
-// candidates' rows are masked out of both operands (a NaN of one candidate must not reach another).  The raw block, if wanted too, is turned by movmatrix.
+// candidates' rows are masked out of both operands (a NaN of one candidate must not reach another).  The raw block, if
+// wanted too, is turned by movmatrix.
 #include <algorithm>
 #include <type_traits>
 

@@ -180,6 +180,10 @@ struct RequestWalk {
 // block of 8 requests x 697 candidates (attention's list made in its kernel too) 40.0 us with lists and 35.4 without,
 // one of 2 x 17 36.4 and 26.0; 128 x 1024 candidates (16384 tiles) 127.0 us with the list and 130.7 walked, the walk
 // being on every warp's path from tile to tile.  (One kernel for both ran the list in 136.4 us for 132.0: two instantiations.)
+// Plan and interaction with compression, 32 + 16 embeddings x 128, walked and with the list: 64 requests with 627 / 1230 /
+// 2432 / 4826 / 9628 tiles 14.0 / 18.6 / 27.5 / 43.9 / 85.9 us and 17.0 / 20.6 / 28.6 / 44.3 / 82.0 us.  About 2200 tiles of
+// 256 / 512 / 768 / 1024 requests 28.3 / 30.9 / 34.0 / 42.1 and 28.8 / 30.8 / 34.5 / 39.0; with 12 embeddings 39.1 / 44.0 /
+// - / 62.5 and 39.5 / 42.5 / - / 53.7.
 constexpr int32_t kMaxTileWalk = 2400;         // tiles: 16 per CTA, for about half of what the launch costs
 constexpr int32_t kMaxTileWalkRequests = 512;  // the first tile takes two loads per 32 requests
 struct TileWalk {
@@ -231,14 +235,17 @@ struct TileWalk {
   }
 #endif
 };
-// Up to this many candidates the kernels search for a row's request themselves: the table is a launch of its own
-// in front of them (about 2 us of a 24 us tower on 500 candidates, and host time), the search a handful of
-// cached loads per row; with more rows the loads add up and the launch does not.
+// Up to this many candidates the kernels search for a row's request themselves: the table is a launch of its own (and
+// host time), the search a handful of cached loads per row and slice of 256 columns; with more rows the loads add up and the
+// launch does not.  Plan and split layer 512|256, about 400 candidates per request, searched and with the table: to 1024
+// columns 2048 / 8192 / 16384 / 32768 candidates 11.5 / 15.1 / 20.9 / 33.6 us and 15.6 / 15.1 / 18.4 / 27.4 us, to 512 columns
+// 8192 / 12000 / 16384 candidates 11.4 / 15.3 / 16.2 and 15.1 / 15.1 / 15.3, to 256 columns 16384 candidates 11.3 and 15.1.
+// The line is between the widths' crossings (8500, 12000 and beyond 16384).
 constexpr int64_t kSearchRows = 16384;
 rocs_status_t plan_request_map(const rocs_plan* plan, cudaStream_t stream, RequestMap* out);
 // The same around a launch that waits for everything in front of itself before it releases the next (a request half):
 // begin in front of it, and behind it, where begin gave memory for a table, fill.  The table is made while that kernel runs
-// (normalised tower on 46262 candidates of 96 requests: 97.1 us behind it, 96.0 beside it).  The kernel behind must wait
+// (normalised tower on 46262 candidates of 96 requests: 106.4 us behind it, 105.0 beside it).  The kernel behind must wait
 // before it reads the map.
 rocs_status_t plan_request_map_begin(const rocs_plan* plan, cudaStream_t stream, RequestMap* out, void** memory);
 rocs_status_t plan_request_map_fill(const rocs_plan* plan, cudaStream_t stream, void* memory, RequestMap* out);

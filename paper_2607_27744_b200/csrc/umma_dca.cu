@@ -30,7 +30,7 @@
 // a cluster of 1 to 8 CTAs takes one item (SPLIT), each of its 2 to 16 sides a run of the item's key blocks with a
 // reference of its own.  The sides leave their unnormalised outputs, references and sums in shared memory and the
 // cluster adds them up, each CTA a share of the rows, through distributed shared memory.  1721 candidates of 3
-// requests x 8 heads, 1000 to 2048 keys (112 items): whole pass with the projection 32.7 us unsplit, 22.2 us split.
+// requests x 8 heads, 1000 to 2048 keys (120 items): whole pass with the projection 32.7 us unsplit, 22.2 us split.
 //
 // Reference of the softmax: the maximum over the row's FIRST 32 keys, rounded up to an integer, found
 // by both threads of the row (each scans those columns, so they agree bit for bit without
@@ -891,9 +891,11 @@ static rocs_status_t launch_dca(const rocs_plan* plan, int32_t n_q, int32_t H, f
   const int32_t most[4] = {sms, 70, 32, 14};
   for (int i = 1; i < 4 && split; ++i)
     if (num <= most[i] && (4 << i) <= blocks) cluster = 1 << i;
-  // Requests that a producer warp looks through itself, at every item; the list is a launch in front.  Projection and
-  // attention of 64 requests x 900 candidates 294.6 us with the list and 290.6 without, of 30 x 27 candidates 22.8 and
-  // 18.2, of 40 x 24 candidates with 32 query tokens 78.8 and 78.9.
+  // Requests that a producer warp looks through itself, at every item; the list is a launch in front.  What looking
+  // costs grows with the requests times the items.  Plan and attention, 8 heads of 64, 200 to 400 keys, without and with
+  // the list: 27 candidates of each of 64 / 256 / 288 / 512 requests 15.9 / 44.4 / 54.1 / 105 us and 18.4 / 46.2 / 52.2 /
+  // 90 us; 150 candidates of 128 / 256 requests 40.2 / 81.7 and 43.3 / 77.3; 600 candidates of 64 / 128 / 256 requests
+  // 60.8 / 115.0 / 242 and 62.7 / 114.6 / 220.  The line is where small requests cross.
   constexpr int32_t kMaxFind = 256;
   DcaItemList items;
   if (plan->R > kMaxFind) {

@@ -796,8 +796,8 @@ def test_threads_that_share_a_stream_have_request_tables_of_their_own(d_cand, d_
 
 @pytest.mark.parametrize("warm", [False, True])
 def test_calls_captured_in_a_graph_replay(warm):
-    # a plan made outside the capture, its lists made or not yet made when the capture begins; and a plan that
-    # lives inside the capture
+    # a plan made outside the capture, used or not yet used when the capture begins; and a plan that lives inside the
+    # capture.  Every call of this batch finds its work in the offsets; batches that need lists are below
     cfg = wl.CONFIGS[5].with_(R=5, d_req=64, d_cand=64, d_out=128, n_ro=4, n_co=4)
     co, so = wl.offsets_from_counts([30, 0, 700, 1, 9]), wl.offsets_from_counts([40, 10, 200, 5, 64])
     lin, att, g = wl.linear_inputs(cfg, co), wl.dca_inputs(cfg, co, so), wl.glm_inputs(cfg, co)
