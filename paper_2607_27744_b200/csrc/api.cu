@@ -53,8 +53,9 @@ static cudaError_t pool_alloc(void** ptr, size_t bytes, cudaStream_t stream) {
   static std::map<unsigned long long, cudaMemPool_t> pools;  // by context: a reset takes its pool along
   unsigned long long context = context_id();
   cudaError_t e;
-  if (context == 0) {  // the thread's first CUDA call
-    if ((e = cudaFree(nullptr)) != cudaSuccess) return e;
+  if (context == 0) {  // the thread's first CUDA call: this makes the device's context its own
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaSetDevice(dev)) != cudaSuccess) return e;
     context = context_id();
   }
   cudaMemPool_t pool = nullptr;
