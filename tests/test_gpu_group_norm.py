@@ -79,3 +79,14 @@ def test_empty_and_errors():
     with pytest.raises(rocs.RocsError) as e:
         rocs.group_norm(X, eps=-1.0)
     assert e.value.code == -1
+
+
+@pytest.mark.parametrize("kind,bound", [(rocs.NORM_LAYER, 6.0e-8), (rocs.NORM_RMS, 5.5e-8)])
+def test_fp32_rows_are_divided_by_their_width(kind, bound):
+    # the fp32 reciprocal of 1000 is 4.75e-8 off and would move every value by half of that: 6.3e-8 and 5.8e-8 in all, beside
+    # the 5.8e-8 and 5.2e-8 of the sums, the root and the rounding of the values
+    X = torch.randn((4000, 1000), generator=torch.Generator().manual_seed(1)).cuda()
+    x = X.double()
+    mean = x.mean(1, keepdim=True) if kind == rocs.NORM_LAYER else 0.0
+    want = (x - mean) / (((x - mean) ** 2).mean(1, keepdim=True) + 1e-5).sqrt()
+    assert float((rocs.group_norm(X, kind=kind).double() - want).norm() / want.norm()) <= bound
