@@ -5,10 +5,10 @@
 //
 // Takes what the tcgen05 kernel (umma_glm.cu) does not: 4 or 12 embeddings per candidate, request sides that are
 // no multiple of 8.  Bound by the fixed latencies of its short chains (mma.sync, ldmatrix) with four warps per
-// scheduler.  100 requests x 184 candidates, 20 + 12 embeddings x 128 with compression to 4: 36.6 us; the general
+// scheduler.  100 requests x 184 candidates, 20 + 12 embeddings x 128 with compression to 4: 32.4 us; the general
 // kernel 286 us.  The compression takes the fp32 block as a bf16 pair (value and remainder) through two products, as
 // exact as that kernel: error of OC against 64 bits 1.6573e-3 on 128 requests x 1024 candidates, 32 + 12 embeddings x
-// 128 to 8, at 192 us; 1.9116e-3 and 140 us with the block rounded first.  The tcgen05 kernel rounds it: where both
+// 128 to 8, at 187 us; 1.9116e-3 and 140 us with the block rounded first.  The tcgen05 kernel rounds it: where both
 // apply it is the faster also without the pair (128 x 1024 candidates, 32 + 16 embeddings with compression: 127 us,
 // this one 145 us with 15 compute warps, 161 us with 8 that take two fragments each).
 //
@@ -74,7 +74,11 @@ __device__ __forceinline__ uint32_t pack(float lo, float hi) {
 // Two fp32 values as bf16 pairs that add up to them.  Rounded value and rounded remainder: 17 bits.
 __device__ __forceinline__ void split(float a, float b, uint32_t (&part)[2]) {
   part[0] = pack(a, b);
-  part[1] = pack(a - __uint_as_float(part[0] << 16), b - __uint_as_float(part[0] & 0xffff0000u));
+  float ra, rb;  // one packed subtraction
+  asm("{\n.reg .b64 v, h;\nmov.b64 v, {%2, %3};\nmov.b64 h, {%4, %5};\nadd.rn.f32x2 v, v, h;\nmov.b64 {%0, %1}, v;\n}"
+      : "=f"(ra), "=f"(rb)
+      : "f"(a), "f"(b), "f"(-__uint_as_float(part[0] << 16)), "f"(-__uint_as_float(part[0] & 0xffff0000u)));
+  part[1] = pack(ra, rb);
 }
 // Upper halves of the values, of what is left and of what is left then: every bit.  An infinity is infinite in every part,
 // and what is left of a value is never 0 unless the value is, so that products with an infinity stay what they are.
@@ -266,7 +270,10 @@ glm_mma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant
       };
       // One 16-column group: columns from col0.  self: the columns are the fragment's own rows, of
       // which each candidate keeps its own.
-      auto emit = [&](const Acc& acc, const float4 (&z)[CO8 > 0 ? CO8 : 1], int32_t col0, bool self) {
+      // parts: bf16 parts of a value in the compression.  redo: the candidates to do (a bit each; ~0: all, and the raw block).
+      // nan: those with a NaN among their outputs.
+      uint32_t nan = 0;
+      auto emit = [&](const Acc& acc, const float4 (&z)[CO8 > 0 ? CO8 : 1], int32_t col0, bool self, auto parts, uint32_t redo) {
         const int32_t last = min(p.frag_cands, tile.count - cand_first);
         const int64_t cand = tile.cand0 + cand_first;
         const int32_t col = self ? own_col : col0 + 4 * tq;
@@ -281,7 +288,8 @@ glm_mma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant
             store_raw(h, pack(acc.v[0][2 * h], acc.v[0][2 * h + 1]), pack(acc.v[1][2 * h], acc.v[1][2 * h + 1]));
         } else {
           // of yt[j][h]: columns of index 8 j + g of YC, fragment rows of index 8 h + 2 tq, + 1
-          if constexpr (RAW) {
+          constexpr int kParts = decltype(parts)::value;
+          if (RAW && kParts == 2) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
               const uint32_t first = transpose8x8(pack(acc.v[h][0], acc.v[h][1])),
@@ -289,10 +297,11 @@ glm_mma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant
               store_raw(h, first, second);
             }
           }
-          auto compress = [&](int c, float (&o)[2][4], auto parts) {  // candidate c of the fragment
-            constexpr int kParts = decltype(parts)::value;
+          for (int c = 0; c < last; ++c) {
+            if ((redo >> c & 1u) == 0u) continue;
             const uint32_t k0 = k_cand[0] == c ? 0xffffffffu : 0u, k1 = k_cand[1] == c ? 0xffffffffu : 0u;
             const uint32_t w[4] = {wa[0] & k0, wa[1] & k0, wa[2] & k1, wa[3] & k1};
+            float o[2][4];
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
               const float4 zb = b < CO8 ? z[b < CO8 ? b : 0] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -309,16 +318,12 @@ glm_mma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant
 #pragma unroll
               for (int i = 0; i < kParts; ++i) mma_bf16(o[j], w, yt[0][i] & k0, yt[1][i] & k1);
             }
-          };
-          for (int c = 0; c < last; ++c) {
-            float o[2][4];
-            compress(c, o, std::integral_constant<int, 2>());
             const bool in = in_cols && (!self || col_cand == c);
-            bool nan = false;  // in this candidate's outputs: what the fragment's others hold must not decide
+            float sum = 0.f;
 #pragma unroll
-            for (int e = 0; e < 4 * CO8; ++e) nan = nan || (in && g + 8 * (e / 4) < p.n_co && isnan(o[e / 2 % 2][2 * (e / 4) + e % 2]));
-            if (__any_sync(0xffffffffu, nan))  // perhaps of an infinity, or of a value that rounds to one
-              compress(c, o, std::integral_constant<int, 3>());
+            for (int b = 0; b < CO8; ++b)
+              if (in && g + 8 * b < p.n_co) sum += (o[0][2 * b] + o[0][2 * b + 1]) + (o[1][2 * b] + o[1][2 * b + 1]);
+            if (isnan(sum)) nan |= 1u << c;
             __nv_bfloat16* oc = p.OC + (cand + c) * p.n_co * n + col;
 #pragma unroll
             for (int b = 0; b < CO8; ++b)
@@ -329,39 +334,47 @@ glm_mma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant
         }
       };
       // request columns in passes of kGroups groups of 16, the fragment's own block in the first of them
-      for (int32_t col0 = 0; col0 < n_r; col0 += 16 * kGroups) {
-        // in front of the products, which hide the latency (with the loads behind them they took half of the time)
-        float4 z[kGroups][CO8 > 0 ? CO8 : 1], z_own[CO8 > 0 ? CO8 : 1];
-        if constexpr (COMPRESS) {
+      auto columns = [&](auto parts, uint32_t redo) {
+        for (int32_t col0 = 0; col0 < n_r; col0 += 16 * kGroups) {
+          // in front of the products, which hide the latency (with the loads behind them they took half of the time)
+          float4 z[kGroups][CO8 > 0 ? CO8 : 1], z_own[CO8 > 0 ? CO8 : 1];
+          if constexpr (COMPRESS) {
 #pragma unroll
-          for (int q = 0; q < kGroups; ++q) load_z(z[q], col0 + 16 * q + 4 * tq, col0 + 16 * q + 4 * tq < n_r);
-          load_z(z_own, own_col, col0 == 0 && col_cand >= 0);
+            for (int q = 0; q < kGroups; ++q) load_z(z[q], col0 + 16 * q + 4 * tq, col0 + 16 * q + 4 * tq < n_r);
+            load_z(z_own, own_col, col0 == 0 && col_cand >= 0);
+          }
+          Acc acc[kGroups] = {}, own = {};
+          const bool second = col0 + 16 < n_r;
+          auto step = [&](int32_t sl, int k, bool first) {
+            const int chunk = 2 * k + lk;
+            uint32_t xf[4], xq[kGroups][4];
+            ldsm_x4(xc_row + sl * p.slab_bytes + ((chunk ^ xc_sw) << 4), xf);
+            const uint32_t at = xr_row + col0 * 128 + sl * p.xr_slab_bytes + ((chunk ^ xr_sw) << 4);
+            ldsm_x4(at, xq[0]);
+            if (second) ldsm_x4(at + 2048, xq[1]);
+            product<COMPRESS>(acc[0], xf, xq[0]);
+            if (second) product<COMPRESS>(acc[1], xf, xq[1]);
+            if (first) product<COMPRESS>(own, xf, xf);
+          };
+          if (col0 == 0) {
+            for (int32_t sl = 0; sl < slabs; ++sl)
+#pragma unroll
+              for (int k = 0; k < 4; ++k) step(sl, k, true);
+          } else {
+            for (int32_t sl = 0; sl < slabs; ++sl)
+#pragma unroll
+              for (int k = 0; k < 4; ++k) step(sl, k, false);
+          }
+          emit(acc[0], z[0], col0, false, parts, redo);
+          if (second) emit(acc[1], z[1], col0 + 16, false, parts, redo);
+          if (col0 == 0) emit(own, z_own, n_r, true, parts, redo);
         }
-        Acc acc[kGroups] = {}, own = {};
-        const bool second = col0 + 16 < n_r;
-        auto step = [&](int32_t sl, int k, bool first) {
-          const int chunk = 2 * k + lk;
-          uint32_t xf[4], xq[kGroups][4];
-          ldsm_x4(xc_row + sl * p.slab_bytes + ((chunk ^ xc_sw) << 4), xf);
-          const uint32_t at = xr_row + col0 * 128 + sl * p.xr_slab_bytes + ((chunk ^ xr_sw) << 4);
-          ldsm_x4(at, xq[0]);
-          if (second) ldsm_x4(at + 2048, xq[1]);
-          product<COMPRESS>(acc[0], xf, xq[0]);
-          if (second) product<COMPRESS>(acc[1], xf, xq[1]);
-          if (first) product<COMPRESS>(own, xf, xf);
-        };
-        if (col0 == 0) {
-          for (int32_t sl = 0; sl < slabs; ++sl)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) step(sl, k, true);
-        } else {
-          for (int32_t sl = 0; sl < slabs; ++sl)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) step(sl, k, false);
-        }
-        emit(acc[0], z[0], col0, false);
-        if (second) emit(acc[1], z[1], col0 + 16, false);
-        if (col0 == 0) emit(own, z_own, n_r, true);
+      };
+      columns(std::integral_constant<int, 2>(), ~0u);
+      if constexpr (COMPRESS) {
+        // Perhaps of an infinity, or of a value that rounds to one.  Decided from a candidate's own outputs, for it alone.
+        const uint32_t redo = __reduce_or_sync(0xffffffffu, nan);
+        if (redo != 0u) columns(std::integral_constant<int, 3>(), redo);
       }
     }
     __syncwarp();
