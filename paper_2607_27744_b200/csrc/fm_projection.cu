@@ -133,12 +133,18 @@ __global__ void __launch_bounds__(128) fm_candidate_simt_kernel(int32_t n_r, int
 // 16 embeddings and 8 or 16 columns (FULL) round H to bf16 and are bound by HBM.  Every other shape takes H as a bf16 pair
 // (value and remainder) through two products in step 2, and is bound by the products: error of FC against 64 bits on 128
 // requests x 1024 candidates, 32 + 12 embeddings x 128, k = 16, 1.6568e-3 as with fp32 FMA throughout (all of it the
-// rounding of FC) at 128.6 us; 1.8657e-3 at 81.8 us with H rounded; three parts, every bit of H, 157.7 us.
-// 18 400 candidates of 12 embeddings x 128, k = 16: 27.4 us; the general kernel, a block per candidate, 284 us.
+// rounding of FC) at 120.3 us; 1.8657e-3 at 81.8 us with H rounded; three parts, every bit of H, about 30 us more.
+// 18 400 candidates of 12 embeddings x 128, k = 16: 26.9 us; the general kernel, a block per candidate, 284 us.
 // ---------------------------------------------------------------------------------------------
 constexpr int kFragRows = 16;      // rows of a candidate's fragments
-constexpr int kTileCands = 8;      // candidates per tile = compute warps per CTA
-constexpr int kFmThreads = (kTileCands + 1) * 32;
+// Candidates per tile = compute warps per CTA.  Two per scheduler are enough for a stream that HBM bounds; the chains of the
+// pair's products want more of them: as many as leave them their registers (11 and the producer are three per scheduler, at
+// 168 registers, 15 four at 128).  With 8: 128.4 us for the batch above, 223 for 183 us on 128 x 512 candidates of 12
+// embeddings x 256, 54.2 for 49.9 on 64 x 512 of 16 x 64 to 24 columns.
+template <int D, bool FULL>
+constexpr int tile_cands() {
+  return FULL ? 8 : D == 64 ? 15 : 11;
+}
 constexpr int kMaxStages = 12;
 constexpr uint32_t kStatusFm = 0x600;
 
@@ -301,13 +307,15 @@ __device__ __forceinline__ void split_bf16(float a, float b, uint32_t (&part)[3]
 // KT: blocks of 16 projection columns.  With one, the request's T stays in registers while consecutive
 // candidates share it; with two it would not fit beside H and comes from L1 for every candidate.
 template <int D, int KT, bool FULL>
-__global__ void __launch_bounds__(kFmThreads, 1)
+__global__ void __launch_bounds__((tile_cands<D, FULL>() + 1) * 32, 1)
 fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmParams p) {
   constexpr int kSlabs = D / 64;
   constexpr int kPairs = D / 16;  // pairs of 8-column groups = k-steps of step 2
   extern __shared__ __align__(1024) uint8_t smem[];
   const int32_t n_c = FULL ? kFragRows : p.n_c;
-  const int32_t slab_bytes = kTileCands * n_c * 128;  // 64 columns of the tile, 128-byte swizzled rows
+  constexpr int kTileCands = tile_cands<D, FULL>();
+  // 64 columns of the tile, 128-byte swizzled rows, to the 1024 bytes that the swizzle repeats in
+  const int32_t slab_bytes = (kTileCands * n_c * 128 + 1023) / 1024 * 1024;
   const int32_t stage_bytes = kSlabs * slab_bytes;
   // behind the stages: rows that the last candidate's fragments read past the tile
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.stages * stage_bytes + (FULL ? 0 : kFragRows * 128));
@@ -341,7 +349,7 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
       uint32_t phase = 0, it = 0;
       for (int32_t t = tile_begin; t < tile_end; ++t, ++it) {
         if (!mbar_wait(&empty[s], phase ^ 1, abort_flag, p.status, kStatusFm | 1)) break;
-        mbar_expect_tx(&full[s], stage_bytes);
+        mbar_expect_tx(&full[s], kSlabs * kTileCands * n_c * 128);
 #pragma unroll
         for (int sl = 0; sl < kSlabs; ++sl)
           tma_load_2d(smem + s * stage_bytes + sl * slab_bytes, &map_xc, &full[s], sl * 64, t * kTileCands * n_c);
@@ -530,7 +538,8 @@ int sm_count_fm() {
 template <int D, int KT, bool FULL>
 rocs_status_t launch_fm_mma_as(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t k,
                                const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
-  const int stage_bytes = D / 64 * kTileCands * n_c * 128;
+  constexpr int kTileCands = tile_cands<D, FULL>();
+  const int stage_bytes = D / 64 * ((kTileCands * n_c * 128 + 1023) / 1024 * 1024);
   constexpr int kFixed = kFragRows * 128 + 2 * kMaxStages * 8 + 16;
   CUtensorMap map_xc;
   if (!make_tensor_map_2d(&map_xc, XC, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)plan->N * n_c, D, D,
@@ -558,7 +567,7 @@ rocs_status_t launch_fm_mma_as(const rocs_plan* plan, int32_t n_r, int32_t n_c, 
   // releases its dependents at once); nothing else this kernel reads is written by that launch.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)std::min(p.num_tiles, sm_count_fm()));
-  cfg.blockDim = dim3(kFmThreads);
+  cfg.blockDim = dim3((kTileCands + 1) * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
