@@ -686,7 +686,7 @@ rocs_status_t rocs_dca_attention(const rocs_plan_t* plan, rocs_dtype_t dtype, in
   cudaStream_t stream = (cudaStream_t)stream_;
   if (dtype == ROCS_BF16 && g_path.load() == ROCS_PATH_AUTO && umma_dca_supported(n_q, H, dh))
     return umma_dca(plan, n_q, H, dh, scale, Q, K, V, seq_offsets, T, O, stream);
-  return simt_dca(dtype, plan, n_q, H, dh, scale, Q, K, V, seq_offsets, O, stream);
+  return simt_dca(dtype, plan, n_q, H, dh, scale, Q, K, V, seq_offsets, T, O, stream);
 }
 
 size_t rocs_glm_interaction_workspace(const rocs_plan_t* plan, int32_t n_r, int32_t n_c, int32_t n_co) {

@@ -3,7 +3,8 @@
 //
 // One block per (tile of 32 query rows of one request, head): the tile's queries stay in shared memory,
 // the request's keys and values come through it in blocks of 64, read once per tile and in place (never
-// copied per candidate).  128 threads as 8 x 16; a thread owns 4 query rows and, of a block, 4 keys for
+// copied per candidate).  A group of 128 threads as 8 x 16, two groups with every other block where a request has several;
+// a thread owns 4 query rows and, of a block, 4 keys for
 // the scores and DHP / 16 columns for the output, so eight 16-byte shared-memory reads feed 64 FMAs.  The
 // running maximum and normaliser of a row live in the 16 neighbouring lanes that share it.  K_{j+1} is
 // fetched while the softmax and P V of block j run, V_{j+1} while the scores of block j + 1 do.
@@ -24,26 +25,33 @@
 namespace rocs {
 namespace {
 
-constexpr int kRows = 32, kKeys = 64, kThreads = 128;
-constexpr int kPStride = kKeys + 4;
+constexpr int kRows = 32, KEYS = 64, kGroup = 128;
 
-template <int DHP>
+template <int DHP, int KS>
 constexpr int smem_floats() {
-  return (kRows + 2 * kKeys) * (DHP + 4) + kRows * kPStride;
+  constexpr int S = DHP + 4, group = 2 * KEYS * S + kRows * (KEYS + 4);
+  constexpr int part = kRows * S;  // what a group leaves for the first one, over its keys and values
+  static_assert(KS == 1 || part <= 2 * KEYS * S, "a part fits the group's keys and values");
+  return kRows * S + KS * group;
 }
 
-template <typename T, int DHP>
-__global__ void __launch_bounds__(kThreads, DHP <= 64 ? 4 : DHP <= 128 ? 2 : 1) dca_simt_kernel(
+// KS groups of 128 threads take the blocks of keys in turn.
+template <typename T, int DHP, int KS>
+__global__ void __launch_bounds__(kGroup* KS, KS == 1 ? (DHP <= 64 ? 4 : DHP <= 128 ? 2 : 1) : KS == 2 && DHP <= 64 ? 2 : 1) dca_simt_kernel(
     int32_t n_q, int32_t H, int32_t dh, float scale, const T* __restrict__ Q, const T* __restrict__ K,
     const T* __restrict__ V, int32_t R, int32_t cands_per_tile, const int32_t* __restrict__ cand_offsets,
     const DcaItem* __restrict__ items, const int32_t* __restrict__ seq_offsets, T* __restrict__ O) {
   constexpr int S = DHP + 4;           // row stride in floats: 16-byte reads of 8 rows hit 8 different bank groups
   constexpr int C = DHP / 16;          // output columns per thread
+  constexpr int J = KEYS / 16;         // keys of a block per thread
+  constexpr int kPStride = KEYS + 4;
+  constexpr int kThreads = kGroup * KS;
   extern __shared__ __align__(16) float sm[];
+  const int tid = threadIdx.x % kGroup, group = threadIdx.x / kGroup, tx = tid % 16, ty = tid / 16;
   float* qs = sm;                      // [32][S]
-  float* ks = qs + kRows * S;          // [64][S]
-  float* vs = ks + kKeys * S;          // [64][S]
-  float* ps = vs + kKeys * S;          // [32][kPStride]
+  float* ks = qs + kRows * S + group * (2 * KEYS * S + kRows * kPStride);  // [KEYS][S]
+  float* vs = ks + KEYS * S;           // [KEYS][S]
+  float* ps = vs + KEYS * S;           // [32][kPStride]
   ptx::griddep_wait_for(Q, K, V, cand_offsets, items, seq_offsets);
   ptx::griddep_launch_dependents();
   DcaItem item;
@@ -53,7 +61,9 @@ __global__ void __launch_bounds__(kThreads, DHP <= 64 ? 4 : DHP <= 128 ? 2 : 1) 
     const FoundTile f = find_tile_in_block<kThreads>(R, cands_per_tile, H, cand_offsets, blockIdx.x);
     item = DcaItem{f.req, f.cand0, f.count, f.head};
   }
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+  auto group_sync = [&]() {
+    if constexpr (KS == 1) __syncthreads(); else asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kGroup) : "memory");
+  };
   const int64_t hd = (int64_t)H * dh;
   const int32_t s0 = seq_offsets[item.req];
   const int32_t L = seq_offsets[item.req + 1] - s0;
@@ -74,47 +84,48 @@ __global__ void __launch_bounds__(kThreads, DHP <= 64 ? 4 : DHP <= 128 ? 2 : 1) 
 #pragma unroll
       for (int c = 0; c < C; ++c) acc[i][c] = 0.f;
     }
-    if (L > 0) {
-      rows_to_shared_async<T, DHP>(Q + q0, hd, rows, kRows, dh, qs, S, tid, kThreads);
-      rows_to_shared_async<T, DHP>(kg, hd, min(kKeys, L), kKeys, dh, ks, S, tid, kThreads);
-      cp_async_commit();
-      rows_to_shared_async<T, DHP>(vg, hd, min(kKeys, L), kKeys, dh, vs, S, tid, kThreads);
-      cp_async_commit();
-    }
-    for (int32_t j0 = 0; j0 < L; j0 += kKeys) {
-      const int32_t next = L - j0 - kKeys;  // keys behind this block
-      cp_async_wait<1>();                   // K_j (and Q) have landed, V_j may still be on its way
+    const int32_t first = group * KEYS;
+    if (L > 0) rows_to_shared_async<T, DHP>(Q + q0, hd, rows, kRows, dh, qs, S, threadIdx.x, kThreads);
+    if (first < L) rows_to_shared_async<T, DHP>(kg + first * hd, hd, min(KEYS, L - first), KEYS, dh, ks, S, tid, kGroup);
+    cp_async_commit();
+    if (first < L) rows_to_shared_async<T, DHP>(vg + first * hd, hd, min(KEYS, L - first), KEYS, dh, vs, S, tid, kGroup);
+    cp_async_commit();
+    if constexpr (KS > 1) {  // everybody's share of Q
+      cp_async_wait<1>();
       __syncthreads();
-      float s[4][4];
+    }
+    for (int32_t j0 = first; j0 < L; j0 += KS * KEYS) {
+      const int32_t next = L - j0 - KS * KEYS;  // keys from the group's next block on
+      cp_async_wait<1>();                       // K_j (and Q) have landed, V_j may still be on its way
+      group_sync();
+      float s[4][J];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
+        for (int j = 0; j < J; ++j) s[i][j] = 0.f;
 #pragma unroll 4
       for (int e = 0; e < DHP; e += 4) {
-        float4 a[4], b[4];
+        float4 a[4], b[J];
 #pragma unroll
         for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(qs + (ty * 4 + i) * S + e);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(ks + (tx + 16 * j) * S + e);
+        for (int j = 0; j < J; ++j) b[j] = *reinterpret_cast<const float4*>(ks + (tx + 16 * j) * S + e);
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int c = 0; c < 4; ++c)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            s[i][j] = fmaf(a[i].x, b[j].x, s[i][j]);
-            s[i][j] = fmaf(a[i].y, b[j].y, s[i][j]);
-            s[i][j] = fmaf(a[i].z, b[j].z, s[i][j]);
-            s[i][j] = fmaf(a[i].w, b[j].w, s[i][j]);
-          }
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < J; ++j) s[i][j] = fmaf(lane_of(a[i], c), lane_of(b[j], c), s[i][j]);
       }
-      __syncthreads();  // K_j is read: its buffer takes K_{j+1}
-      if (next > 0) rows_to_shared_async<T, DHP>(kg + (int64_t)(j0 + kKeys) * hd, hd, min(kKeys, next), kKeys, dh, ks, S, tid, kThreads);
+      group_sync();  // K_j is read: its buffer takes the group's next
+      if (next > 0)
+        rows_to_shared_async<T, DHP>(kg + (int64_t)(j0 + KS * KEYS) * hd, hd, min(KEYS, next), KEYS, dh, ks, S, tid, kGroup);
       cp_async_commit();
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         float mx = -INFINITY;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < J; ++j) {
           s[i][j] = j0 + tx + 16 * j < L ? s[i][j] * scale : -INFINITY;
           mx = fmaxf(mx, s[i][j]);
         }
@@ -124,8 +135,9 @@ __global__ void __launch_bounds__(kThreads, DHP <= 64 ? 4 : DHP <= 128 ? 2 : 1) 
         const float corr = m[i] == -INFINITY ? 0.f : expf(m[i] - m_new);
         float sum = 0.f;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float p = j0 + tx + 16 * j < L ? expf(s[i][j] - m_new) : 0.f;
+        for (int j = 0; j < J; ++j) {
+          // (scores that are all -inf so far have no weight: finite ones may follow, or be another group's)
+          const float p = j0 + tx + 16 * j < L && (mx != -INFINITY || s[i][j] != -INFINITY) ? expf(s[i][j] - m_new) : 0.f;
           sum += p;
           ps[(ty * 4 + i) * kPStride + tx + 16 * j] = p;
         }
@@ -137,9 +149,9 @@ __global__ void __launch_bounds__(kThreads, DHP <= 64 ? 4 : DHP <= 128 ? 2 : 1) 
         for (int c = 0; c < C; ++c) acc[i][c] *= corr;
       }
       cp_async_wait<1>();  // V_j
-      __syncthreads();     // V_j for everybody; the P rows of a warp are its own
+      group_sync();        // V_j for everybody; the P rows of a warp are its own
 #pragma unroll 2
-      for (int k = 0; k < kKeys; k += 4) {
+      for (int k = 0; k < KEYS; k += 4) {
         float4 a[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(ps + (ty * 4 + i) * kPStride + k);
@@ -165,35 +177,91 @@ __global__ void __launch_bounds__(kThreads, DHP <= 64 ? 4 : DHP <= 128 ? 2 : 1) 
           }
         }
       }
-      __syncthreads();  // V_j is read: its buffer takes V_{j+1}
-      if (next > 0) rows_to_shared_async<T, DHP>(vg + (int64_t)(j0 + kKeys) * hd, hd, min(kKeys, next), kKeys, dh, vs, S, tid, kThreads);
+      group_sync();  // V_j is read: its buffer takes the group's next
+      if (next > 0)
+        rows_to_shared_async<T, DHP>(vg + (int64_t)(j0 + KS * KEYS) * hd, hd, min(KEYS, next), KEYS, dh, vs, S, tid, kGroup);
       cp_async_commit();
     }
+    constexpr int W = C == 2 ? 2 : 4;  // neighbouring columns
+    if constexpr (KS > 1) {
+      // the groups' parts, added up by the first in the order of the groups: row by row S floats, maximum and
+      // normaliser behind the columns
+      cp_async_wait<0>();
+      if (group > 0) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int row = ty * 4 + i;
-      if (row >= rows) continue;
-      const float inv = L > 0 ? 1.f / l[i] : 0.f;
-      T* out = O + q0 + (int64_t)row * hd;
-      constexpr int W = C == 2 ? 2 : 4;  // neighbouring columns
+        for (int i = 0; i < 4; ++i) {
+          float* part = ks + (ty * 4 + i) * S;
 #pragma unroll
-      for (int c = 0; c < C; c += W) {
-        const int col = c * 16 + tx * W;
-        if (col < dh) {                  // dh is a multiple of 4 (8 for bf16): whole groups
+          for (int c = 0; c < C; c += W)
 #pragma unroll
-          for (int w = 0; w < W; w += 2) store_pair(out + col + w, acc[i][c + w] * inv, acc[i][c + w + 1] * inv);
+            for (int w = 0; w < W; ++w) part[c * 16 + tx * W + w] = acc[i][c + w];
+          if (tx == 0) {
+            part[DHP] = m[i];
+            part[DHP + 1] = l[i];
+          }
+        }
+      }
+      __syncthreads();
+      if (group == 0) {
+#pragma unroll
+        for (int g = 1; g < KS; ++g) {
+          const float* other = ks + g * (2 * KEYS * S + kRows * kPStride);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float* part = other + (ty * 4 + i) * S;
+            const float m_o = part[DHP], l_o = part[DHP + 1], m_new = fmaxf(m[i], m_o);
+            // a part whose scores are all -inf, or that has no keys, adds nothing
+            const float a = m[i] == -INFINITY ? 0.f : expf(m[i] - m_new), b = m_o == -INFINITY ? 0.f : expf(m_o - m_new);
+            l[i] = l[i] * a + l_o * b;
+            m[i] = m_new;
+#pragma unroll
+            for (int c = 0; c < C; c += W)
+#pragma unroll
+              for (int w = 0; w < W; ++w) acc[i][c + w] = acc[i][c + w] * a + part[c * 16 + tx * W + w] * b;
+          }
         }
       }
     }
+    if (group == 0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int row = ty * 4 + i;
+        if (row >= rows) continue;
+        const float inv = L > 0 ? 1.f / l[i] : 0.f;
+        T* out = O + q0 + (int64_t)row * hd;
+#pragma unroll
+        for (int c = 0; c < C; c += W) {
+          const int col = c * 16 + tx * W;
+          if (col < dh) {                  // dh is a multiple of 4 (8 for bf16): whole groups
+#pragma unroll
+            for (int w = 0; w < W; w += 2) store_pair(out + col + w, acc[i][c + w] * inv, acc[i][c + w + 1] * inv);
+          }
+        }
+      }
+    }
+    if constexpr (KS > 1) __syncthreads();  // the next rows' operands come where the parts are
   }
 }
 
-template <typename T, int DHP>
+template <typename T, int DHP, int KS>
 rocs_status_t launch(const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh, float scale, const void* Q,
-                     const void* K, const void* V, const int32_t* seq_offsets, void* O, cudaStream_t stream) {
+                     const void* K, const void* V, const int32_t* seq_offsets, void* O, const DcaItemList& items,
+                     int32_t cands, cudaStream_t stream) {
+  constexpr int smem = smem_floats<DHP, KS>() * (int)sizeof(float);
+  static_assert(smem <= kMaxDynamicSmem - 256, "shared memory of an SM, less what the search for the tile takes");
+  auto kernel = dca_simt_kernel<T, DHP, KS>;
+  ROCS_ALLOW_SMEM(kernel, smem);
+  const dim3 grid((unsigned)items.num, (unsigned)std::min<int64_t>(((int64_t)cands * n_q + kRows - 1) / kRows, 65535));
+  return launch_dependent(kernel, grid, kGroup * KS, smem, stream, n_q, H, dh, scale, (const T*)Q, (const T*)K, (const T*)V,
+                          plan->R, cands, plan->cand_offsets, (const DcaItem*)items.dev, seq_offsets, (T*)O);
+}
+
+template <typename T>
+rocs_status_t dispatch(const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh, float scale, const void* Q,
+                       const void* K, const void* V, const int32_t* seq_offsets, int64_t T_rows, void* O, cudaStream_t stream) {
   const int32_t cands = std::max(1, kRows / n_q);
   DcaItemList items;
-  if (plan->R > kThreads) {
+  if (plan->R > kGroup) {
     const rocs_status_t st = plan_dca_items(plan, cands, H, stream, &items);
     if (st != ROCS_OK) return st;
   } else {
@@ -201,33 +269,35 @@ rocs_status_t launch(const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh, 
     if (total > 0x7fffffffLL) return ROCS_ERR_UNSUPPORTED;
     items.num = (int32_t)total;
   }
-  constexpr int smem = smem_floats<DHP>() * (int)sizeof(float);
-  auto kernel = dca_simt_kernel<T, DHP>;
-  ROCS_ALLOW_SMEM(kernel, smem);
-  const dim3 grid((unsigned)items.num, (unsigned)std::min<int64_t>(((int64_t)cands * n_q + kRows - 1) / kRows, 65535));
-  return launch_dependent(kernel, grid, kThreads, smem, stream, n_q, H, dh, scale, (const T*)Q, (const T*)K, (const T*)V,
-                          plan->R, cands, plan->cand_offsets, (const DcaItem*)items.dev, seq_offsets, (T*)O);
-}
-
-template <typename T>
-rocs_status_t dispatch(const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh, float scale, const void* Q,
-                       const void* K, const void* V, const int32_t* seq_offsets, void* O, cudaStream_t stream) {
+#define ROCS_LAUNCH(DHP_, KS_) return launch<T, DHP_, KS_>(plan, n_q, H, dh, scale, Q, K, V, seq_offsets, O, items, cands, stream)
+  // Two groups share the blocks of a request that has more than one.  One group and two, 1 x 25 candidates x 2 heads of 64
+  // over 72..144 keys 9.9 and 8.5 us, 1 x 288 x 16 heads of 32 over 58..116 8.4 and 6.9 us, 24 x 109 x 8 heads of 64 over
+  // 64..384 the same; four groups with blocks of 32 keys 9.3, 7.8 and 83 us for 69: an SM's FMAs are then the limit.
+  const int64_t keys = T_rows / plan->R;  // of an average request
+  const bool two = keys > KEYS;
   // smallest compiled width that holds the head: columns beyond dh are zeros in shared memory
-  if (dh <= 32) return launch<T, 32>(plan, n_q, H, dh, scale, Q, K, V, seq_offsets, O, stream);
-  if (dh <= 64) return launch<T, 64>(plan, n_q, H, dh, scale, Q, K, V, seq_offsets, O, stream);
-  if (dh <= 128) return launch<T, 128>(plan, n_q, H, dh, scale, Q, K, V, seq_offsets, O, stream);
-  return launch<T, 256>(plan, n_q, H, dh, scale, Q, K, V, seq_offsets, O, stream);
+  if (dh <= 32) {
+    if (two) ROCS_LAUNCH(32, 2);
+    ROCS_LAUNCH(32, 1);
+  }
+  if (dh <= 64) {
+    if (two) ROCS_LAUNCH(64, 2);
+    ROCS_LAUNCH(64, 1);
+  }
+  if (dh <= 128) ROCS_LAUNCH(128, 1);
+  ROCS_LAUNCH(256, 1);
+#undef ROCS_LAUNCH
 }
 
 }  // namespace
 
 rocs_status_t simt_dca(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh, float scale,
-                       const void* Q, const void* K, const void* V, const int32_t* seq_offsets, void* O,
+                       const void* Q, const void* K, const void* V, const int32_t* seq_offsets, int64_t T, void* O,
                        cudaStream_t stream) {
   if (dh > 256) return ROCS_ERR_UNSUPPORTED;
   if (plan->N == 0) return ROCS_OK;
-  if (dt == ROCS_F32) return dispatch<float>(plan, n_q, H, dh, scale, Q, K, V, seq_offsets, O, stream);
-  return dispatch<__nv_bfloat16>(plan, n_q, H, dh, scale, Q, K, V, seq_offsets, O, stream);
+  if (dt == ROCS_F32) return dispatch<float>(plan, n_q, H, dh, scale, Q, K, V, seq_offsets, T, O, stream);
+  return dispatch<__nv_bfloat16>(plan, n_q, H, dh, scale, Q, K, V, seq_offsets, T, O, stream);
 }
 
 }  // namespace rocs

@@ -12,7 +12,8 @@
 // read fall with it (8 x 8 outputs: 16 FMAs per 16-byte read, 4 x 4: 8, 2 x 2: 4) and what bounds the large
 // shapes is the FMA pipe and those reads, while a small batch (the request half at R rows) is bound by the
 // length of its K chain on a few SMs.  Measured, fp32: 24 requests x 768 -> 1024 with 2613 candidates x
-// 256 -> 1024 behind it, 61 us for both (one 64 x 64 tile of 16-wide synchronous slices for every shape:
+// 256 -> 1024 behind it, 46 us for both (56 us with the request rows of the epilogue read one at a time and a part's rows
+// on the same banks; one 64 x 64 tile of 16-wide synchronous slices for every shape:
 // 160 us, half of it the 16 blocks of the request half).
 // Every output is produced by a sequence that depends on the shape only, so results are deterministic and
 // independent of the other rows' values (Eq. 1).
@@ -28,7 +29,7 @@ constexpr int kGroup = 64, kStages = 3;
 
 template <int BM, int BN, int KS>
 constexpr int smem_bytes() {
-  constexpr int ring = KS * kStages * (BM + BN) * kRow, tiles = KS * BM * BN;
+  constexpr int ring = KS * kStages * (BM + BN) * kRow, tiles = KS * BM * (BN + 8);
   return (ring > tiles ? ring : tiles) * (int)sizeof(float);
 }
 
@@ -39,11 +40,15 @@ __device__ __forceinline__ void st_f(__nv_bfloat16* p, float v) { *p = __float2b
 // 16 columns from k0 of `rows` rows starting at row0 of a matrix, zeros outside it.
 __device__ __forceinline__ void load_slice(const float* __restrict__ src, int64_t ld, int64_t row0, int64_t n_rows,
                                            int rows, int32_t k0, int32_t d, float* dst, int t) {
-  for (int v = t; v < rows * (kBk / 4); v += kGroup) {
-    const int r = v / (kBk / 4), k = k0 + (v % (kBk / 4)) * 4;
-    const int left = row0 + r < n_rows ? min(max(d - k, 0), 4) : 0;
-    cp_async_16((uint32_t)__cvta_generic_to_shared(dst + r * kRow + (v % (kBk / 4)) * 4),
-                src + (left > 0 ? (row0 + r) * ld + k : 0), left * 4);
+  // thread t has the same four columns of every 16th row
+  const int k = k0 + t % 4 * 4, in_row = min(max(d - k, 0), 4);
+  const float* from = src + (row0 + t / 4) * ld + k;
+  const uint32_t to = (uint32_t)__cvta_generic_to_shared(dst + t / 4 * kRow + t % 4 * 4);
+  const int64_t left_rows = n_rows - row0 - t / 4;
+#pragma unroll
+  for (int r = 0; r < rows; r += kGroup / 4) {
+    const int left = r < left_rows ? in_row : 0;
+    cp_async_16(to + r * kRow * 4, left > 0 ? from + r * ld : src, left * 4);
   }
 }
 __device__ __forceinline__ void load_slice(const __nv_bfloat16* __restrict__ src, int64_t ld, int64_t row0,
@@ -118,36 +123,79 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
 #pragma unroll
       for (int j = 0; j < TN; ++j) b[j] = *reinterpret_cast<const float4*>(b_s + j * 8 * kRow + k);
 #pragma unroll
-      for (int i = 0; i < TM; ++i)
+      for (int c = 0; c < 4; ++c)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) {
-          acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
-          acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
-          acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
-          acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
-        }
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(lane_of(a[i], c), lane_of(b[j], c), acc[i][j]);
     }
   }
   if (add && threadIdx.x < BM && m0 + threadIdx.x < M) req[threadIdx.x] = requests.of(m0 + threadIdx.x);
   cp_async_wait<0>();
   __syncthreads();  // the rings become the groups' partial tiles
-  float* part = sm + group * BM * BN;
+  constexpr int PS = BN + 8;  // row stride of a partial tile: the 8 x 4 threads of a warp hit 32 different banks
+  float* part = sm + group * BM * PS;
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < TN; ++j) part[(ty + 8 * i) * BN + tx + 8 * j] = acc[i][j];
+    for (int j = 0; j < TN; ++j) part[(ty + 8 * i) * PS + tx + 8 * j] = acc[i][j];
   __syncthreads();
-  for (int e = threadIdx.x; e < BM * BN; e += kGroup * KS) {
-    const int64_t m = m0 + e / BN;
-    const int32_t n = n0 + e % BN;
-    if (m >= M || n >= d_out) continue;
-    float v = sm[e];
+  // Four neighbouring columns of kRowsEach rows per thread.  The request rows are all asked for before the first is
+  // used: one at a time, every row of a tile waited for the L2 cache.
+  constexpr int kPerRow = BN / 4, kThreads = kGroup * KS, kRowStep = kThreads / kPerRow, kRowsEach = BM / kRowStep;
+  static_assert(kThreads % kPerRow == 0 && (BM % kRowStep == 0 || kRowStep > BM), "rows of a tile over the threads");
+  const int32_t c4 = threadIdx.x % kPerRow * 4, r0 = threadIdx.x / kPerRow, n = n0 + c4;
+  const int32_t cols = min(d_out - n, 4);
+  if (r0 >= BM || cols <= 0) return;
+  constexpr int kEach = kRowsEach > 0 ? kRowsEach : 1;
+  float4 z[kEach];
 #pragma unroll
-    for (int g = 1; g < KS; ++g) v += sm[g * BM * BN + e];
-    if (bias) v += bias[n];
-    if (add) v += add[(int64_t)req[e / BN] * ld_add + n];
-    if (act == ROCS_ACT_RELU) v = fmaxf(v, 0.f);
-    st_f(Y + m * ld_y + n, v);
+  for (int u = 0; u < kEach; ++u) {
+    const int32_t r = r0 + u * kRowStep;
+    z[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (add && m0 + r < M) {
+      const float* from = add + (int64_t)req[r] * ld_add + n;
+      if (cols == 4 && ld_add % 4 == 0) {
+        z[u] = *reinterpret_cast<const float4*>(from);
+      } else {
+        z[u].x = from[0];
+        if (cols > 1) z[u].y = from[1];
+        if (cols > 2) z[u].z = from[2];
+        if (cols > 3) z[u].w = from[3];
+      }
+    }
+  }
+  float b4[4] = {0.f, 0.f, 0.f, 0.f};
+  if (bias)
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (c < cols) b4[c] = bias[n + c];
+#pragma unroll
+  for (int u = 0; u < kEach; ++u) {
+    const int32_t r = r0 + u * kRowStep;
+    if (m0 + r >= M) break;
+    float4 v4 = *reinterpret_cast<const float4*>(sm + r * PS + c4);
+#pragma unroll
+    for (int g = 1; g < KS; ++g) {
+      const float4 o = *reinterpret_cast<const float4*>(sm + (g * BM + r) * PS + c4);
+      v4.x += o.x; v4.y += o.y; v4.z += o.z; v4.w += o.w;
+    }
+    float v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (bias) v[c] += b4[c];
+      if (add) v[c] += lane_of(z[u], c);
+      if (act == ROCS_ACT_RELU) v[c] = fmaxf(v[c], 0.f);
+    }
+    TOut* out = Y + (m0 + r) * ld_y + n;  // rows start on 16-byte boundaries and n is a multiple of 4
+    if (cols == 4) {
+      store_pair(out, v[0], v[1]);
+      store_pair(out + 2, v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (c < cols) st_f(out + c, v[c]);
+    }
   }
 }
 

@@ -269,7 +269,7 @@ rocs_status_t simt_linear(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_ou
                           void* Y, int64_t ld_y, bool out_f32, cudaStream_t stream);
 rocs_status_t simt_dca(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh,
                        float scale, const void* Q, const void* K, const void* V,
-                       const int32_t* seq_offsets, void* O, cudaStream_t stream);
+                       const int32_t* seq_offsets, int64_t T, void* O, cudaStream_t stream);
 rocs_status_t simt_glm(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d,
                        const void* XR, const void* XC, const void* W, int32_t n_ro, int32_t n_co,
                        void* YR, void* YC, void* OR_, void* OC, float* zr_workspace,

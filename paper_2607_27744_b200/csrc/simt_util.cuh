@@ -140,11 +140,17 @@ template <typename T>
 __device__ __forceinline__ void dense_rows_to_shared_async(const T* __restrict__ src, int rows, int d,
                                                            float* __restrict__ dst, int stride, int tid, int threads) {
   constexpr int kVec = 16 / (int)sizeof(T);
-  const int per_row = d / kVec;
+  const int per_row = d / kVec, dr = threads / per_row, dc = threads - dr * per_row;
+  int r = tid / per_row, c = tid - r * per_row;
 #pragma unroll 4
   for (int v = tid; v < rows * per_row; v += threads) {
-    const int r = v / per_row;
-    float* to = dst + r * stride + (v - r * per_row) * kVec;
+    float* to = dst + r * stride + c * kVec;
+    r += dr;
+    c += dc;
+    if (c >= per_row) {
+      c -= per_row;
+      ++r;
+    }
     if constexpr (sizeof(T) == 4) {
       cp_async_16((uint32_t)__cvta_generic_to_shared(to), src + (int64_t)v * kVec, 16);
     } else {
@@ -155,6 +161,9 @@ __device__ __forceinline__ void dense_rows_to_shared_async(const T* __restrict__
     }
   }
 }
+
+// Component c (a constant after unrolling) of a vector.
+__device__ __forceinline__ float lane_of(const float4& v, int c) { return c == 0 ? v.x : c == 1 ? v.y : c == 2 ? v.z : v.w; }
 
 __device__ __forceinline__ void store_pair(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
 __device__ __forceinline__ void store_pair(__nv_bfloat16* p, float a, float b) {

@@ -441,6 +441,26 @@ def test_dca_general_kernel_edges(dtype, dh, n_q):
     assert _run_dca(cfg, co, so) <= tol_for(dtype)
 
 
+@pytest.mark.parametrize("dh", [20, 64])
+@pytest.mark.parametrize("L", [64, 65, 128, 129, 300])
+def test_dca_general_kernel_groups_of_keys(L, dh):
+    # one group of threads or two per tile, the second without keys, with a part of a block, with another number of
+    # blocks than the first; between requests with few keys or none; a first block whose scores are all -inf
+    lengths = np.array([L, 3, 0, 2 * L - 70 if L > 64 else 63, L], np.int32)
+    so = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    co = wl.offsets_from_counts([5, 1, 2, 33, 4])
+    cfg = wl.CONFIGS[1].with_(R=5, H=2, dh=dh)
+    d = wl.dca_inputs(cfg, co, so)
+    d["Q"][-4:, ..., 0] = 1.0
+    d["K"][so[4]:so[4] + 64, :, 0] = -np.inf
+    O = rocs.dca_attention(_plan(co), to_dev(d["Q"]), to_dev(d["K"]), to_dev(d["V"]), to_dev(so))
+    want = ref.dca_attention(co, so, d["Q"], d["K"], d["V"])
+    if L == 64:  # of these rows every score is -inf
+        assert bool(torch.isnan(O[-4:]).all())
+        O, want = O[:-4], want[:-4]
+    assert rel_err(to_host_f64(O), want) <= tol_for("f32")
+
+
 def test_dca_bf16_64_query_tokens_per_candidate():
     # two candidates fill a 128-row tile (Section 4.3.2 names query tiles of 32 and 64 tokens)
     co = wl.offsets_from_counts([5, 1, 12, 2])
@@ -605,6 +625,17 @@ def test_glm_general_kernel_tiles(dtype, n_r, n_c, d, n_co):
     # remainders in every 4 x 4 group, a compression block too large for shared memory
     co = wl.offsets_from_counts([1, 0, 9, 33, 2] if n_c < 100 else [1, 0, 3])
     cfg = wl.CONFIGS[4].with_(R=len(co) - 1, dtype=dtype, n_r=n_r, n_c=n_c, d_emb=d, n_ro=min(2, n_co), n_co=n_co)
+    assert _run_glm(cfg, co) <= tol_for(dtype)
+
+
+@pytest.mark.parametrize("R", [1, 3, 128, 129])
+@pytest.mark.parametrize("per", [1, 31, 600])
+@pytest.mark.parametrize("dtype,n_r,n_c,d,n_co", [("f32", 32, 2, 128, 8), ("f32", 24, 8, 36, 5), ("bf16", 30, 2, 64, 4), ("f32", 9, 3, 8, 0)])
+def test_glm_general_kernel_batch_sizes(dtype, n_r, n_c, d, n_co, per, R):
+    # tiles of one candidate up to 64 rows, lanes that share a product or not, the request side in the same launch or
+    # (more requests than the blocks look through, or more tiles) in one of its own
+    co = wl.offsets_from_counts([per if R < 100 else 1 + r % 5 for r in range(R)])
+    cfg = wl.CONFIGS[4].with_(R=R, dtype=dtype, n_r=n_r, n_c=n_c, d_emb=d, n_ro=min(3, n_co), n_co=n_co)
     assert _run_glm(cfg, co) <= tol_for(dtype)
 
 
