@@ -16,8 +16,9 @@ __global__ void stats_from_partials_kernel(int64_t M, int32_t P, const float2* _
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= M) return;
   float s = 0.f, q = 0.f;
+#pragma unroll 8
   for (int32_t k = 0; k < P; ++k) {
-    const float2 v = partials[i * P + k];
+    const float2 v = partials[k * M + i];
     s += v.x;
     q += v.y;
   }
