@@ -559,6 +559,26 @@ static rocs_status_t ikbo_linear_impl(const rocs_plan_t* plan, rocs_dtype_t dtyp
     const size_t need = z_bytes;
     if (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255u))
       return ROCS_ERR_WORKSPACE;
+    // Both halves in one launch where the batch allows it: otherwise the candidate half waits for the request half in its
+    // epilogue, and the request half holds SMs that the candidate half then starts late on.
+    if (dtype == ROCS_BF16 && d_cand > 0 && g_path.load() == ROCS_PATH_AUTO) {
+      bool taken = false;
+      rocs_status_t st = ROCS_OK;
+      if (row_stats == nullptr) {
+        st = umma_linear_both(plan, d_req, d_cand, d_out, XR, ld_xr, XC, ld_xc, W_CR, ld_wcr, W_CC, ld_wcc, bias, act, Y, ld_y,
+                              stream, &taken);
+        if (taken) return st;
+      }
+      float2* partials = row_stats ? reinterpret_cast<float2*>(static_cast<uint8_t*>(workspace) + z_bytes) : nullptr;
+      st = umma_linear_ws2_both(plan, d_req, d_cand, d_out, XR, ld_xr, XC, ld_xc, W_CR, ld_wcr, W_CC, ld_wcc, bias, act, Y, ld_y,
+                                partials, stream, &taken);
+      if (taken && st == ROCS_OK && row_stats != nullptr)
+        st = row_stats_from_partials(plan->N, umma_linear_ws2_stat_partials(d_out), partials, reinterpret_cast<float2*>(row_stats),
+                                     stream);
+      if (taken) return st;
+    }
+    if (row_stats == nullptr && dtype == ROCS_F32 && d_cand > 0 && simt_linear_both_supported(plan->N, d_req, d_out))
+      return simt_linear_both(plan, d_req, d_cand, d_out, XR, ld_xr, XC, ld_xc, W_CR, ld_wcr, W_CC, ld_wcc, bias, act, Y, ld_y, stream);
     // Request half, once per request (Section 4.1): Z = X^R W_CR^T + bias, fp32.  The map, where a table of it has to be
     // made, beside it on the SMs that it leaves idle; the candidate kernel waits for both before it reads either.
     void* table = nullptr;

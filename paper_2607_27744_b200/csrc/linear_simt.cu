@@ -27,9 +27,9 @@ namespace {
 constexpr int kBk = 16, kRow = kBk + 4;  // k per slice; floats per shared-memory row
 constexpr int kGroup = 64, kStages = 3;
 
-template <int BM, int BN, int KS>
+template <int BM, int BN, int KS, bool BOTH>
 constexpr int smem_bytes() {
-  constexpr int ring = KS * kStages * (BM + BN) * kRow, tiles = KS * BM * (BN + 8);
+  constexpr int ring = KS * kStages * (BM + BN) * kRow, tiles = (BOTH ? 2 : 1) * KS * BM * (BN + 8);
   return (ring > tiles ? ring : tiles) * (int)sizeof(float);
 }
 
@@ -73,11 +73,18 @@ __device__ __forceinline__ void load_slice(const __nv_bfloat16* __restrict__ src
   }
 }
 
-template <typename TIn, typename TOut, int TM, int TN, int KS>
+// The request half of a split layer in the same launch (BOTH): rows of X are gathered by request, its sums kept apart.
+struct RequestHalf {
+  const float *X, *W;
+  int64_t ld_x, ld_w;
+  int32_t d_in;
+};
+
+template <typename TIn, typename TOut, int TM, int TN, int KS, bool BOTH>
 __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kernel(
     int64_t M, int32_t d_in, int32_t d_out, const TIn* __restrict__ X, int64_t ld_x, const TIn* __restrict__ W,
     int64_t ld_w, const float* __restrict__ bias, const float* __restrict__ add, int64_t ld_add,
-    const RequestMap map, int act, TOut* __restrict__ Y, int64_t ld_y) {
+    const RequestMap map, int act, TOut* __restrict__ Y, int64_t ld_y, const RequestHalf half) {
   constexpr int BM = 8 * TM, BN = 8 * TN;
   extern __shared__ __align__(16) float sm[];
   __shared__ int32_t req[BM];  // request of each row of the tile
@@ -91,8 +98,22 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
   const int32_t slices = (d_in + kBk - 1) / kBk;
   const int32_t mine = (slices - group + KS - 1) / KS;  // slices group, group + KS, ...
   float* ring = sm + group * kStages * (BM + BN) * kRow;
+  // BOTH: the group's slices of the request half come behind those
+  const int32_t all = BOTH ? mine + ((half.d_in + kBk - 1) / kBk - group + KS - 1) / KS : mine;
+  if constexpr (BOTH) {
+    if (threadIdx.x < BM) req[threadIdx.x] = requests.of(min(m0 + threadIdx.x, M - 1));
+    __syncthreads();
+  }
   auto fetch = [&](int32_t it) {
-    if (it < mine) {
+    if (BOTH && it >= mine && it < all) {
+      float* st = ring + (it % kStages) * (BM + BN) * kRow;
+      const int32_t k = (group + (it - mine) * KS) * kBk + t % 4 * 4, in_row = min(max(half.d_in - k, 0), 4);
+#pragma unroll
+      for (int r = 0; r < BM; r += kGroup / 4)
+        cp_async_16((uint32_t)__cvta_generic_to_shared(st + (r + t / 4) * kRow + t % 4 * 4),
+                    in_row > 0 ? half.X + req[r + t / 4] * half.ld_x + k : half.X, in_row * 4);
+      load_slice(half.W, half.ld_w, n0, d_out, BN, k - t % 4 * 4, half.d_in, st + BM * kRow, t);
+    } else if (it < mine) {
       float* st = ring + (it % kStages) * (BM + BN) * kRow;
       const int32_t k0 = (group + it * KS) * kBk;
       load_slice(X, ld_x, m0, M, BM, k0, d_in, st, t);
@@ -102,14 +123,15 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
   };
   auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kGroup) : "memory"); };
 
-  float acc[TM][TN];
+  float acc[TM][TN], acc_r[BOTH ? TM : 1][TN];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
-#pragma unroll
-  for (int s = 0; s < kStages - 1; ++s) fetch(s);
-  for (int32_t it = 0; it < mine; ++it) {
+    for (int j = 0; j < TN; ++j) {
+      acc[i][j] = 0.f;
+      acc_r[BOTH ? i : 0][j] = 0.f;
+    }
+  auto multiply = [&](int32_t it, auto& sums) {
     cp_async_wait<kStages - 2>();
     group_sync();  // slice `it` has landed for the group, and everybody is done with slice it - 1
     fetch(it + kStages - 1);
@@ -127,9 +149,14 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
 #pragma unroll
         for (int i = 0; i < TM; ++i)
 #pragma unroll
-          for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(lane_of(a[i], c), lane_of(b[j], c), acc[i][j]);
+          for (int j = 0; j < TN; ++j) sums[i][j] = fmaf(lane_of(a[i], c), lane_of(b[j], c), sums[i][j]);
     }
-  }
+  };
+#pragma unroll
+  for (int s = 0; s < kStages - 1; ++s) fetch(s);
+  for (int32_t it = 0; it < mine; ++it) multiply(it, acc);
+  if constexpr (BOTH)
+    for (int32_t it = mine; it < all; ++it) multiply(it, acc_r);
   if (add && threadIdx.x < BM && m0 + threadIdx.x < M) req[threadIdx.x] = requests.of(m0 + threadIdx.x);
   cp_async_wait<0>();
   __syncthreads();  // the rings become the groups' partial tiles
@@ -138,7 +165,10 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < TN; ++j) part[(ty + 8 * i) * PS + tx + 8 * j] = acc[i][j];
+    for (int j = 0; j < TN; ++j) {
+      part[(ty + 8 * i) * PS + tx + 8 * j] = acc[i][j];
+      if constexpr (BOTH) part[(KS * BM + ty + 8 * i) * PS + tx + 8 * j] = acc_r[i][j];
+    }
   __syncthreads();
   // Four neighbouring columns of kRowsEach rows per thread.  The request rows are all asked for before the first is
   // used: one at a time, every row of a tile waited for the L2 cache.
@@ -181,9 +211,18 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
       v4.x += o.x; v4.y += o.y; v4.z += o.z; v4.w += o.w;
     }
     float v[4] = {v4.x, v4.y, v4.z, v4.w};
+    if constexpr (BOTH) {
+#pragma unroll
+      for (int g = 0; g < KS; ++g) {
+        const float4 o = *reinterpret_cast<const float4*>(sm + ((KS + g) * BM + r) * PS + c4);
+        z[u].x += o.x; z[u].y += o.y; z[u].z += o.z; z[u].w += o.w;
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[c] += lane_of(z[u], c) + b4[c];
+    }
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      if (bias) v[c] += b4[c];
+      if (!BOTH && bias) v[c] += b4[c];
       if (add) v[c] += lane_of(z[u], c);
       if (act == ROCS_ACT_RELU) v[c] = fmaxf(v[c], 0.f);
     }
@@ -202,21 +241,26 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
 template <typename TIn, typename TOut>
 rocs_status_t launch_linear(int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x, const void* W,
                             int64_t ld_w, const float* bias, const float* add, int64_t ld_add,
-                            const RequestMap& map, int act, void* Y, int64_t ld_y, cudaStream_t stream) {
+                            const RequestMap& map, int act, void* Y, int64_t ld_y, cudaStream_t stream,
+                            const RequestHalf* half = nullptr) {
   if (M == 0 || d_out == 0) return ROCS_OK;
   auto tiles = [&](int b) { return ((M + b - 1) / b) * ((d_out + b - 1) / b); };
-#define ROCS_LAUNCH(T_, KS_)                                                                                      \
+#define ROCS_LAUNCH(T_, KS_, BOTH_)                                                                               \
   do {                                                                                                            \
-    constexpr int smem = smem_bytes<8 * T_, 8 * T_, KS_>();                                                       \
-    auto kernel = linear_simt_kernel<TIn, TOut, T_, T_, KS_>;                                                     \
+    constexpr int smem = smem_bytes<8 * T_, 8 * T_, KS_, BOTH_>();                                                \
+    auto kernel = linear_simt_kernel<TIn, TOut, T_, T_, KS_, BOTH_>;                                              \
     ROCS_ALLOW_SMEM(kernel, smem);                                                                                \
     const dim3 grid((unsigned)((M + 8 * T_ - 1) / (8 * T_)), (unsigned)((d_out + 8 * T_ - 1) / (8 * T_)));        \
     return launch_dependent(kernel, grid, kGroup * KS_, smem, stream, M, d_in, d_out, (const TIn*)X, ld_x,        \
-                            (const TIn*)W, ld_w, bias, add, ld_add, map, act, (TOut*)Y, ld_y);                    \
+                            (const TIn*)W, ld_w, bias, add, ld_add, map, act, (TOut*)Y, ld_y,                     \
+                            half ? *half : RequestHalf{});                                                        \
   } while (0)
-  if (tiles(64) >= 296) ROCS_LAUNCH(8, 2);
-  else if (tiles(32) >= 148) ROCS_LAUNCH(4, 4);
-  else ROCS_LAUNCH(2, 8);
+  if constexpr (sizeof(TIn) == 4) {
+    if (half != nullptr) ROCS_LAUNCH(2, 8, true);
+  }
+  if (tiles(64) >= 296) ROCS_LAUNCH(8, 2, false);
+  else if (tiles(32) >= 148) ROCS_LAUNCH(4, 4, false);
+  else ROCS_LAUNCH(2, 8, false);
 #undef ROCS_LAUNCH
 }
 
@@ -233,6 +277,21 @@ rocs_status_t simt_linear(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_ou
                                                ld_y, stream);
   return launch_linear<__nv_bfloat16, __nv_bfloat16>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act,
                                                      Y, ld_y, stream);
+}
+
+// The request half is computed for every candidate: worth it while that is less than a launch.  In a chain, two launches and
+// one: 25 x 80 | 64 -> 64 3.6 and 2.5 us (5.7 and 2.8 with the host in front), 48 x 128 | 64 -> 512 4.2 and 5.1 (5.7 and 5.3),
+// 27 x 64 | 256 -> 512 4.5 and 4.9 (5.6 and 4.9), 341 x 112 | 256 -> 512 9.4 and 11.7.
+bool simt_linear_both_supported(int64_t N, int32_t d_req, int32_t d_out) {
+  constexpr int64_t kMost = 1 << 22;
+  return N > 0 && N <= kSearchRows && N * d_req * d_out <= kMost && ((N + 31) / 32) * ((d_out + 31) / 32) < 148;
+}
+rocs_status_t simt_linear_both(const rocs_plan* plan, int32_t d_req, int32_t d_cand, int32_t d_out, const void* XR, int64_t ld_xr,
+                               const void* XC, int64_t ld_xc, const void* W_CR, int64_t ld_wcr, const void* W_CC, int64_t ld_wcc,
+                               const float* bias, int act, void* Y, int64_t ld_y, cudaStream_t stream) {
+  const RequestHalf half{(const float*)XR, (const float*)W_CR, ld_xr, ld_wcr, d_req};
+  return launch_linear<float, float>(plan->N, d_cand, d_out, XC, ld_xc, W_CC, ld_wcc, bias, nullptr, 0,
+                                     RequestMap{nullptr, plan->cand_offsets, plan->R}, act, Y, ld_y, stream, &half);
 }
 
 }  // namespace rocs

@@ -267,6 +267,11 @@ rocs_status_t simt_linear(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_ou
                           int64_t ld_x, const void* W, int64_t ld_w, const float* bias,
                           const float* add, int64_t ld_add, const RequestMap& map, int act,
                           void* Y, int64_t ld_y, bool out_f32, cudaStream_t stream);
+// Both halves of an fp32 split layer in one launch, for few candidates.
+bool simt_linear_both_supported(int64_t N, int32_t d_req, int32_t d_out);
+rocs_status_t simt_linear_both(const rocs_plan* plan, int32_t d_req, int32_t d_cand, int32_t d_out, const void* XR, int64_t ld_xr,
+                               const void* XC, int64_t ld_xc, const void* W_CR, int64_t ld_wcr, const void* W_CC, int64_t ld_wcc,
+                               const float* bias, int act, void* Y, int64_t ld_y, cudaStream_t stream);
 rocs_status_t simt_dca(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh,
                        float scale, const void* Q, const void* K, const void* V,
                        const int32_t* seq_offsets, int64_t T, void* O, cudaStream_t stream);
@@ -299,6 +304,10 @@ rocs_status_t umma_linear(int64_t M, int32_t d_in, int32_t d_out, const void* X,
                           int64_t ld_add, const RequestMap& map, int act, void* Y, int64_t ld_y,
                           bool out_f32, cudaStream_t stream, bool add_from_previous_launch = false,
                           float2* stat_partials = nullptr, int64_t add_rows = 0);
+// Both halves of a split layer in one launch, for few candidates; `taken` says whether the batch is one of those.
+rocs_status_t umma_linear_both(const rocs_plan* plan, int32_t d_req, int32_t d_cand, int32_t d_out, const void* XR, int64_t ld_xr,
+                               const void* XC, int64_t ld_xc, const void* W_CR, int64_t ld_wcr, const void* W_CC, int64_t ld_wcc,
+                               const float* bias, int act, void* Y, int64_t ld_y, cudaStream_t stream, bool* taken);
 // Weight-stationary kernel on CTA pairs (cta_group::2) for d_in <= 256 and bf16 output: half a weight
 // slice per SM, TMA-store epilogue (umma_linear picks it when it applies).
 bool umma_linear_ws2_supported(int64_t M, int32_t d_in, int32_t d_out, bool out_f32);
@@ -307,6 +316,11 @@ rocs_status_t umma_linear_ws2(int64_t M, int32_t d_in, int32_t d_out, const void
                               int64_t ld_add, const RequestMap& map, int act, void* Y, int64_t ld_y,
                               cudaStream_t stream, bool add_from_previous_launch = false,
                               float2* stat_partials = nullptr, int64_t add_rows = 0);
+// The same with the request half in its launch, where the rows of each CTA pair are of few requests (`taken`).
+rocs_status_t umma_linear_ws2_both(const rocs_plan* plan, int32_t d_req, int32_t d_cand, int32_t d_out, const void* XR,
+                                   int64_t ld_xr, const void* XC, int64_t ld_xc, const void* W_CR, int64_t ld_wcr, const void* W_CC,
+                                   int64_t ld_wcc, const float* bias, int act, void* Y, int64_t ld_y, float2* stat_partials,
+                                   cudaStream_t stream, bool* taken);
 // Number of (sum, sum of squares) partials per row the kernel above writes when asked to.
 inline int32_t umma_linear_ws2_stat_partials(int32_t d_out) { return 2 * ((d_out + 255) / 256); }
 // K-ring GEMM on CTA pairs for wide plain layers (no request term, bf16 output, many rows).

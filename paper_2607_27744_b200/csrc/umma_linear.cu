@@ -10,9 +10,14 @@
 //   warps 2-5 epilogue: TMEM -> registers, + Z[m_i] (+ bias), ReLU, round to the output type,
 //            128-byte-swizzled staging in shared memory, TMA store (clipped at the edges)
 // The two accumulators let the epilogue of tile t overlap the main loop of tile t + 1.
+// A split layer on few candidates is one launch (BOTH): a tile computes the request half of its own requests, at most TM
+// consecutive rows of X^R, into the second accumulator, from where it goes through shared memory to the candidates' rows.  In a
+// chain, two launches and one: 500 candidates of one request, 512|256 -> 1024, 6.6 and 5.5 us; 926 of 28, 736|200 -> 512,
+// 11.0 and 6.9; 12 of one, 96|200 -> 512, 4.1 and 3.0 (and a launch less for the host, 5.4 and 3.5 us).
 // Tiles are ordered with the output-column index fastest, so CTAs working at the same time share
 // the same rows of X in L2.  M tiles may span several requests: each row looks up its own request.
 #include <algorithm>
+#include <type_traits>
 
 #include "rocs_internal.h"
 #include "sm100_ptx.cuh"
@@ -40,6 +45,9 @@ struct LinearCfg {
   static constexpr int kStagingBytes = kEpiWarps * 2 * 4096;  // per warp: two buffers of 32 rows x 128 bytes at most
   static constexpr int kTmemCols = 2 * BN;
   static constexpr int kSmemBytes = kOffStaging + kStagingBytes + 512 /*barriers*/ + 1024 /*align*/;
+  static constexpr int kZStride = BN + 4;  // BOTH: floats per request row, eight rows hit eight different bank groups
+  static constexpr int kZBytes = TM * kZStride * 4;
+  static_assert(BN > 64 || kSmemBytes + kZBytes <= kMaxDynamicSmem, "shared memory of an SM");
   static_assert(kOffB - kABytes + BM * BK * 2 <= kOffStaging + kStagingBytes, "rows behind the last slot");
 };
 
@@ -56,10 +64,21 @@ struct LinearParams {
   uint32_t* status;
 };
 
-template <int TM, int BN, typename OutT>
+// The request half of a split layer in the same launch: one tile per CTA.
+constexpr int kMaxTilesBoth = 192;
+struct RequestHalf {
+  int32_t k_blocks;                // 64-wide blocks of d_req
+  int32_t rows;                    // rows of X^R that a tile loads
+  int32_t first[kMaxTilesBoth];    // the first of them, by row tile
+};
+struct NoRequestHalf {};
+
+template <int TM, int BN, typename OutT, bool BOTH>
 __global__ void __launch_bounds__(kThreads, 1)
 linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-                   const __grid_constant__ CUtensorMap map_y, const LinearParams p) {
+                   const __grid_constant__ CUtensorMap map_y, const LinearParams p, const __grid_constant__ CUtensorMap map_xr,
+                   const __grid_constant__ CUtensorMap map_wr,
+                   const __grid_constant__ std::conditional_t<BOTH, RequestHalf, NoRequestHalf> rh) {
   using Cfg = LinearCfg<TM, BN>;
   constexpr int kStages = Cfg::kStages;
   constexpr int CH = BN * (int)sizeof(OutT) < 128 ? BN : 128 / (int)sizeof(OutT);  // output columns per staging row
@@ -68,7 +87,8 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* staging = smem + Cfg::kOffStaging;
-  uint64_t* full = reinterpret_cast<uint64_t*>(staging + Cfg::kStagingBytes);
+  float* z_rows = reinterpret_cast<float*>(staging + Cfg::kStagingBytes);  // BOTH: [rh.rows][kZStride]
+  uint64_t* full = reinterpret_cast<uint64_t*>(staging + Cfg::kStagingBytes + (BOTH ? Cfg::kZBytes : 0));
   uint64_t* empty = full + kStages;
   uint64_t* tmem_full = empty + kStages;
   uint64_t* tmem_empty = tmem_full + 2;
@@ -112,6 +132,10 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     prefetch_tensormap(&map_x);
     prefetch_tensormap(&map_w);
     prefetch_tensormap(&map_y);
+    if constexpr (BOTH) {
+      prefetch_tensormap(&map_xr);
+      prefetch_tensormap(&map_wr);
+    }
   }
   // A candidate half in front of which only the request half is still running streams X and W at once; its
   // epilogue waits.
@@ -125,6 +149,16 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     if (elect_one()) {
       uint32_t it = 0;
       bool ok = true;
+      if constexpr (BOTH) {  // the longer half first: its way to the rows overlaps the other's products
+        const int32_t r0 = rh.first[blockIdx.x / n_tiles], n0 = (int32_t)(blockIdx.x % n_tiles) * BN;
+        for (int32_t kb = 0; kb < rh.k_blocks; ++kb, ++it) {
+          const int s = it % kStages;
+          if (!mbar_wait(&empty[s], ((it / kStages) & 1) ^ 1, abort_flag, p.status, kStatusLinear | 1)) { ok = false; break; }
+          mbar_expect_tx(&full[s], rh.rows * (BK * 2) + Cfg::kBBytes);
+          tma_load_2d(smem + s * Cfg::kABytes, &map_xr, &full[s], kb * BK, r0);
+          tma_load_2d(smem + Cfg::kOffB + s * Cfg::kBBytes, &map_wr, &full[s], kb * BK, n0);
+        }
+      }
       for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
         const int32_t m0 = (int32_t)(t / n_tiles) * TM, n0 = (int32_t)(t % n_tiles) * BN;
         for (int32_t kb = 0; kb < k_blocks; ++kb, ++it) {
@@ -153,14 +187,10 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       constexpr uint32_t idesc = umma_idesc_bf16(BM, BN, false, false);
       uint32_t it = 0, lt = 0;
       bool ok = true;
-      for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++lt) {
-        const uint32_t acc = lt & 1;
-        if (!mbar_wait(&tmem_empty[acc], ((lt >> 1) & 1) ^ 1, abort_flag, p.status, kStatusLinear | 2)) { ok = false; break; }
-        tc_fence_after_sync();
-        const uint32_t d_tmem = tmem_base + acc * BN;
-        for (int32_t kb = 0; kb < k_blocks; ++kb, ++it) {
+      auto products = [&](uint32_t d_tmem, int32_t blocks) {
+        for (int32_t kb = 0; kb < blocks; ++kb, ++it) {
           const int s = it % kStages;
-          if (!mbar_wait(&full[s], (it / kStages) & 1, abort_flag, p.status, kStatusLinear | 3)) { ok = false; break; }
+          if (!mbar_wait(&full[s], (it / kStages) & 1, abort_flag, p.status, kStatusLinear | 3)) return false;
           tc_fence_after_sync();
           const uint64_t a_desc = smem_desc_sw128(smem_u32(smem + s * Cfg::kABytes), 1024, 16);
           const uint64_t b_desc = smem_desc_sw128(smem_u32(smem + Cfg::kOffB + s * Cfg::kBBytes), 1024, 16);
@@ -169,6 +199,17 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             umma_ss(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
           umma_commit(&empty[s]);  // frees the stage once these MMAs have read it
         }
+        return true;
+      };
+      if constexpr (BOTH) {
+        ok = products(tmem_base + BN, rh.k_blocks);
+        if (ok) umma_commit(&tmem_full[1]);
+      }
+      for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++lt) {
+        const uint32_t acc = lt & 1;
+        if (!mbar_wait(&tmem_empty[acc], ((lt >> 1) & 1) ^ 1, abort_flag, p.status, kStatusLinear | 2)) { ok = false; break; }
+        tc_fence_after_sync();
+        ok = products(tmem_base + acc * BN, k_blocks);
         if (ok) umma_commit(&tmem_full[acc]);
       }
       if (!ok) {
@@ -187,14 +228,44 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       griddep_wait();
       griddep_launch_dependents();
     }
+    if constexpr (BOTH) {
+      // the request half, bias included, to shared memory: row by row of X^R
+      const int32_t n0 = (int32_t)(blockIdx.x % n_tiles) * BN;
+      ok = mbar_wait(&tmem_full[1], 0, abort_flag, p.status, kStatusLinear | 4);
+      tc_fence_after_sync();
+      if (ok && q * 32 < rh.rows) {
+        float* z = z_rows + (q * 32 + lane) * Cfg::kZStride;
+#pragma unroll 1
+        for (int c = 0; c < BN; c += 32) {
+          uint32_t v[32];
+          tmem_ld_32x32b_x32(tmem_base + BN + c + ((uint32_t)(q * 32) << 16), v);
+          tmem_ld_wait();
+          if (q * 32 + lane < rh.rows) {
+#pragma unroll
+            for (int i = 0; i < 32; i += 4) {
+              float4 f = make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]), __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
+              if (p.bias != nullptr && n0 + c + i < p.d_out) {
+                const float4 b = __ldg(reinterpret_cast<const float4*>(p.bias + n0 + c + i));
+                f.x += b.x; f.y += b.y; f.z += b.z; f.w += b.w;
+              }
+              *reinterpret_cast<float4*>(z + c + i) = f;
+            }
+          }
+        }
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
+    }
     for (int64_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++lt) {
       const uint32_t acc = lt & 1;
       const int32_t m0 = (int32_t)(t / n_tiles) * TM, n0 = (int32_t)(t % n_tiles) * BN;
       const int64_t row = (int64_t)m0 + q * 32 + lane;
       const bool mine = TM == BM || q * 32 < TM;  // rows of the tile among this warp's
       const float* add_row = nullptr;
-      if (p.add != nullptr && mine && row < p.M)
-        add_row = p.add + (int64_t)p.map.of(row) * p.ld_add;
+      if constexpr (BOTH) {
+        if (mine && row < p.M) add_row = z_rows + (p.map.of(row) - rh.first[t / n_tiles]) * Cfg::kZStride - n0;
+      } else {
+        if (p.add != nullptr && mine && row < p.M) add_row = p.add + (int64_t)p.map.of(row) * p.ld_add;
+      }
       if (!mbar_wait(&tmem_full[acc], (lt >> 1) & 1, abort_flag, p.status, kStatusLinear | 4)) { ok = false; break; }
       tc_fence_after_sync();
       const uint32_t t_row = tmem_base + acc * BN + ((uint32_t)(q * 32) << 16);
@@ -225,12 +296,13 @@ linear_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 #pragma unroll
           for (int i = 0; i < CH; i += 4) {
             if (col0 + i < p.d_out) {
-              const float4 z = __ldg(reinterpret_cast<const float4*>(add_row + col0 + i));
+              const float4* from = reinterpret_cast<const float4*>(add_row + col0 + i);
+              const float4 z = BOTH ? *from : __ldg(from);
               f[i] += z.x; f[i + 1] += z.y; f[i + 2] += z.z; f[i + 3] += z.w;
             }
           }
         }
-        if (p.bias != nullptr) {
+        if (!BOTH && p.bias != nullptr) {
 #pragma unroll
           for (int i = 0; i < CH; i += 4) {
             if (col0 + i < p.d_out) {
@@ -299,10 +371,18 @@ int sm_count() {
   return n;
 }
 
-template <int TM, int BN, typename OutT>
+// What the request half of a split layer reads, and where its rows begin for each row tile.
+struct RequestArgs {
+  const void *XR, *W;
+  int64_t ld_xr, ld_w;
+  int32_t R, d_req;
+  RequestHalf half;
+};
+
+template <int TM, int BN, typename OutT, bool BOTH = false>
 rocs_status_t launch(int64_t M, int32_t d_in, int32_t d_out, const void* X, int64_t ld_x, const void* W,
                      int64_t ld_w, const float* bias, const float* add, int64_t ld_add, const RequestMap& map,
-                     int act, void* Y, int64_t ld_y, cudaStream_t stream, bool wait_late) {
+                     int act, void* Y, int64_t ld_y, cudaStream_t stream, bool wait_late, const RequestArgs* request = nullptr) {
   using Cfg = LinearCfg<TM, BN>;
   constexpr int CH = BN * (int)sizeof(OutT) < 128 ? BN : 128 / (int)sizeof(OutT);
   // A batch of fewer rows than a tile loads no more than it has: the loads of a small batch, 64 bytes per clock and
@@ -318,26 +398,55 @@ rocs_status_t launch(int64_t M, int32_t d_in, int32_t d_out, const void* X, int6
                           sizeof(OutT), (uint64_t)M, (uint64_t)d_out, (uint64_t)ld_y, 32, CH, CH * sizeof(OutT) == 128,
                           CH * sizeof(OutT) == 64))
     return ROCS_ERR_CUDA;
+  CUtensorMap map_xr = map_x, map_wr = map_w;
+  std::conditional_t<BOTH, RequestHalf, NoRequestHalf> rh{};
+  if constexpr (BOTH) {
+    rh = request->half;
+    if (!make_tensor_map_2d(&map_xr, request->XR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)request->R, (uint64_t)request->d_req,
+                            (uint64_t)request->ld_xr, (uint32_t)rh.rows, BK, true) ||
+        !make_tensor_map_2d(&map_wr, request->W, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)d_out, (uint64_t)request->d_req,
+                            (uint64_t)request->ld_w, BN, BK, true))
+      return ROCS_ERR_CUDA;
+  }
   uint32_t* status = device_status_word();
   if (!status) return ROCS_ERR_CUDA;
-  auto kernel = linear_umma_kernel<TM, BN, OutT>;
-  ROCS_ALLOW_SMEM(kernel, Cfg::kSmemBytes);
+  constexpr int kSmem = Cfg::kSmemBytes + (BOTH ? Cfg::kZBytes : 0);
+  auto kernel = linear_umma_kernel<TM, BN, OutT, BOTH>;
+  ROCS_ALLOW_SMEM(kernel, kSmem);
   const int64_t tiles = ((M + TM - 1) / TM) * ((d_out + BN - 1) / BN);
   const int grid = (int)std::min<int64_t>(tiles, sm_count());
   LinearParams p{M, d_in, d_out, bias, add, ld_add, map, act, x_rows, wait_late ? 1 : 0, status};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = Cfg::kSmemBytes;
+  cfg.dynamicSmemBytes = kSmem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, map_x, map_w, map_y, p));
+  ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, map_x, map_w, map_y, p, map_xr, map_wr, rh));
   ROCS_CUDA_TRY(cudaGetLastError());
   return ROCS_OK;
+}
+
+// Few tiles: the one that loads least (its rows of X and of W) among those that give every tile an SM of its own.
+// An SM loads 64 bytes per clock, which is the time of such a layer, down to about 240 cycles per K block (the
+// products of 128 rows, however few are used, and their hand-over).  In a chain of the same layer, with 128 x 64
+// tiles and with these: 500 x 1024 -> 1024 4.80 and 4.48 us (64 x 64), 500 x 1024 -> 256 4.63 and 4.09 (32 x 32),
+// 741 x 512 -> 512 3.69 and 3.40, 96 x 512 -> 1024 3.54 and 3.04, 128 x 256 -> 256 2.90 and 2.43.  Measured and not
+// taken: a tile's K blocks split over a cluster of 2 to 8 CTAs (5.64, 6.6, 4.86, 4.24, 4.26: clusters start later
+// and hold up the next launch), the two loads of a K block issued by two warps (4.53, 4.15, 3.43, 3.09, 2.49).
+bool small_tile(int64_t M, int32_t d_out, int* tm, int* bn) {
+  const int sms = sm_count();
+  int64_t least = INT64_MAX;
+  for (int t = 32; t <= 128; t *= 2)
+    for (int b = 32; b <= 64; b *= 2) {
+      const int64_t rows = std::min<int64_t>(t, (M + 7) / 8 * 8) + b;
+      if (((M + t - 1) / t) * ((d_out + b - 1) / b) <= sms && rows < least) { least = rows; *tm = t; *bn = b; }
+    }
+  return least != INT64_MAX;
 }
 
 }  // namespace
@@ -368,32 +477,52 @@ rocs_status_t umma_linear(int64_t M, int32_t d_in, int32_t d_out, const void* X,
                                      wait_late)                                                                      \
            : launch<TM_, BN_, __nv_bfloat16>(M, d_in, d_out, X, ld_x, W, ld_w, bias, add, ld_add, map, act, Y, ld_y, \
                                              stream, wait_late))
-  // Few tiles: the one that loads least (its rows of X and of W) among those that give every tile an SM of its own.
-  // An SM loads 64 bytes per clock, which is the time of such a layer, down to about 240 cycles per K block (the
-  // products of 128 rows, however few are used, and their hand-over).  In a chain of the same layer, with 128 x 64
-  // tiles and with these: 500 x 1024 -> 1024 4.80 and 4.48 us (64 x 64), 500 x 1024 -> 256 4.63 and 4.09 (32 x 32),
-  // 741 x 512 -> 512 3.69 and 3.40, 96 x 512 -> 1024 3.54 and 3.04, 128 x 256 -> 256 2.90 and 2.43.  Measured and not
-  // taken: a tile's K blocks split over a cluster of 2 to 8 CTAs (5.64, 6.6, 4.86, 4.24, 4.26: clusters start later
-  // and hold up the next launch), the two loads of a K block issued by two warps (4.53, 4.15, 3.43, 3.09, 2.49).
   const int sms = sm_count();
-  auto tiles = [&](int tm, int bn) { return ((M + tm - 1) / tm) * ((d_out + bn - 1) / bn); };
-  int tm = 128, bn = 64;
-  int64_t least = INT64_MAX;
-  for (int t = 32; t <= 128; t *= 2)
-    for (int b = 32; b <= 64; b *= 2) {
-      const int64_t rows = std::min<int64_t>(t, (M + 7) / 8 * 8) + b;
-      if (tiles(t, b) <= sms && rows < least) { least = rows; tm = t; bn = b; }
-    }
-  if (least != INT64_MAX) {
+  int tm, bn;
+  if (small_tile(M, d_out, &tm, &bn)) {
     if (bn == 32) return tm == 32 ? ROCS_LAUNCH(32, 32) : tm == 64 ? ROCS_LAUNCH(64, 32) : ROCS_LAUNCH(128, 32);
     return tm == 32 ? ROCS_LAUNCH(32, 64) : tm == 64 ? ROCS_LAUNCH(64, 64) : ROCS_LAUNCH(128, 64);
   }
   // Otherwise the widest tile that still gives every SM something to do.
   bn = d_out > 128 ? 256 : (d_out > 64 ? 128 : 64);
-  while (bn > 64 && tiles(128, bn) < sms) bn /= 2;
+  while (bn > 64 && ((M + 127) / 128) * ((d_out + bn - 1) / bn) < sms) bn /= 2;
   if (bn == 256) return ROCS_LAUNCH(128, 256);
   if (bn == 128) return ROCS_LAUNCH(128, 128);
   return ROCS_LAUNCH(128, 64);
+#undef ROCS_LAUNCH
+}
+
+// One launch for both halves where every tile has an SM of its own and its candidates' requests (their rows of X^R are
+// consecutive) are no more than its rows.
+rocs_status_t umma_linear_both(const rocs_plan* plan, int32_t d_req, int32_t d_cand, int32_t d_out, const void* XR, int64_t ld_xr,
+                               const void* XC, int64_t ld_xc, const void* W_CR, int64_t ld_wcr, const void* W_CC, int64_t ld_wcc,
+                               const float* bias, int act, void* Y, int64_t ld_y, cudaStream_t stream, bool* taken) {
+  *taken = false;
+  int tm, bn;
+  if (plan->N < 1 || plan->N > kSearchRows || d_req < 8 || d_cand < 8 || d_out < 8 || d_out % 4 != 0 || !small_tile(plan->N, d_out, &tm, &bn))
+    return ROCS_OK;
+  const int32_t m_tiles = (int32_t)((plan->N + tm - 1) / tm);
+  if (m_tiles > kMaxTilesBoth) return ROCS_OK;
+  RequestArgs request{XR, W_CR, ld_xr, ld_wcr, plan->R, d_req, {}};
+  const int32_t* off = plan->offsets_host.data();
+  int32_t r = 0, most = 1;  // r: the request that holds a row, the last one that does not begin behind it
+  for (int32_t t = 0; t < m_tiles; ++t) {
+    const int32_t row0 = t * tm, last = std::min(row0 + tm, (int32_t)plan->N) - 1;
+    while (off[r + 1] <= row0) ++r;
+    request.half.first[t] = r;
+    while (off[r + 1] <= last && r - request.half.first[t] < tm) ++r;
+    most = std::max(most, r - request.half.first[t] + 1);
+    if (most > tm) return ROCS_OK;  // requests without candidates in between
+  }
+  request.half.rows = (most + 7) / 8 * 8;
+  request.half.k_blocks = (d_req + BK - 1) / BK;
+  const RequestMap map{nullptr, plan->cand_offsets, plan->R};
+  *taken = true;
+#define ROCS_LAUNCH(TM_, BN_)                                                                                             \
+  launch<TM_, BN_, __nv_bfloat16, true>(plan->N, d_cand, d_out, XC, ld_xc, W_CC, ld_wcc, bias, nullptr, 0, map, act, Y, ld_y, \
+                                        stream, false, &request)
+  if (bn == 32) return tm == 32 ? ROCS_LAUNCH(32, 32) : tm == 64 ? ROCS_LAUNCH(64, 32) : ROCS_LAUNCH(128, 32);
+  return tm == 32 ? ROCS_LAUNCH(32, 64) : tm == 64 ? ROCS_LAUNCH(64, 64) : ROCS_LAUNCH(128, 64);
 #undef ROCS_LAUNCH
 }
 

@@ -172,6 +172,42 @@ def test_linear_halves_in_small_tiles(N):
     assert _run_linear(cfg, co, bias=True, relu=True) <= tol_for("bf16")
 
 
+def _counts_of(law, N, rng):
+    if law == "one":
+        return [N]
+    per = {"each": 1, "few": 6, "many": 300, "gaps": 40}[law]
+    counts = []
+    while sum(counts) < N:
+        counts.append(min(N - sum(counts), int(rng.integers(1, 2 * per)) if per > 1 else 1))
+        counts += [0] * int(rng.integers(0, 5)) if law == "gaps" else []
+    return [0, 0, *counts, 0] if law == "gaps" else counts
+
+
+@pytest.mark.parametrize("law", ["one", "each", "few", "many", "gaps"])
+@pytest.mark.parametrize("dtype,N,d_req,d_cand,d_out", [
+    ("bf16", 33, 200, 8, 72), ("bf16", 500, 520, 256, 512), ("bf16", 600, 8, 304, 256), ("bf16", 1100, 72, 264, 1000),   # tiles of their own
+    ("bf16", 1300, 520, 64, 1024), ("bf16", 4866, 200, 256, 1024), ("bf16", 20000, 64, 128, 328), ("bf16", 9500, 768, 8, 64),  # CTA pairs
+    ("f32", 1, 3, 5, 9), ("f32", 40, 65, 16, 300), ("f32", 300, 20, 40, 132)])
+def test_linear_halves_in_one_launch(dtype, N, d_req, d_cand, d_out, law):
+    # the request half in the candidates' launch: one request, as many as rows, so many or so spread out (empty ones
+    # in between) that some tiles or runs hold more than fit and the halves are two launches after all
+    co = wl.offsets_from_counts(_counts_of(law, N, np.random.default_rng(N)))
+    cfg = wl.CONFIGS[5].with_(R=len(co) - 1, dtype=dtype, d_req=d_req, d_cand=d_cand, d_out=d_out)
+    ends = np.concatenate([co[:-1], co[1:] - 1, np.arange(0, N, 97), np.arange(0, N, 256)])
+    sample = np.unique(np.clip(ends, 0, N - 1))[:1200]
+    if dtype == "f32" and (d_req * 4) % 16:
+        d = wl.linear_inputs(cfg, co, bias=True)
+        def rows(a):  # rows that start on 16-byte boundaries
+            t = torch.zeros(a.shape[0], (a.shape[1] + 3) // 4 * 4, device="cuda")
+            t[:, :a.shape[1]] = to_dev(a)
+            return t[:, :a.shape[1]]
+        Y = rocs.ikbo_linear(_plan(co), rows(d["XR"]), rows(d["XC"]), rows(d["W"][:, :d_req]), rows(d["W"][:, d_req:]), bias=to_dev(d["bias"]),
+                             out=rows(np.zeros((N, d_out), np.float32)))
+        assert rel_err(to_host_f64(Y), ref.ikbo_linear(co, d["XR"], d["XC"], d["W"], bias=d["bias"])) <= tol_for(dtype)
+        return
+    assert _run_linear(cfg, co, bias=True, relu=law == "few", sample=sample) <= tol_for(dtype)
+
+
 def test_linear_empty_batch():
     co = np.zeros(3, np.int32)
     cfg = wl.CONFIGS[2].with_(R=2, d_req=64, d_cand=64, d_out=64)
