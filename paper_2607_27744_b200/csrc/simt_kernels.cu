@@ -13,9 +13,10 @@ namespace {
 
 constexpr int kGlmThreads = 128;
 // Tiles (of about 64 rows) of a small batch, whose blocks have tiles of fewer candidates and share the lanes out over K, and
-// of one whose request side is not worth a launch of its own.  fp32, 25 candidates of one request, 32 + 2 embeddings x 128,
+// of one whose request side is not worth a launch of its own (2613 candidates of 24 requests, 24 + 8 x 128, compression to
+// 4 + 4, 337 tiles: 14.1 us with that launch, 17.0 without).  fp32, 25 candidates of one request, 32 + 2 embeddings x 128,
 // compression to 8 + 8: 15.7 us before both, 6.1 us; 288 candidates of 32 + 8: 15.2 and 8.6 us.
-constexpr int32_t kGlmSmallTiles = 296, kGlmFusedTiles = 592;
+constexpr int32_t kGlmSmallTiles = 296, kGlmFusedTiles = 148;
 
 __device__ __forceinline__ float ld_f(const float* p, int64_t i) { return p[i]; }
 __device__ __forceinline__ float ld_f(const __nv_bfloat16* p, int64_t i) { return __bfloat162float(p[i]); }
