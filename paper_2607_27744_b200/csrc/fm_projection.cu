@@ -15,6 +15,9 @@
 //   step 2   FC_i = X^C_i H             the accumulator layout of step 1 is the B-operand layout of
 //                                       step 2, so H never leaves registers; X^C_i is the M x K
 //                                       operand, read with ldmatrix
+// Candidates of up to 8 embeddings take their own term through the Gram matrix instead,
+//     FC[i] = X^C_i T[m_i] + (X^C_i X^C_i^T) P_C,
+// whose products are the same for the rows of all candidates that fit 16 rows.
 // A general kernel (any shape, fp32 or bf16 storage, fp32 FMA) covers everything else.
 #include <algorithm>
 #include <type_traits>
@@ -304,6 +307,22 @@ __device__ __forceinline__ void split_bf16(float a, float b, uint32_t (&part)[3]
   }
 }
 
+// T^T of a request, columns 16 kt .. and the 16 columns cp of d, in the accumulator layout of step 1.
+template <int D>
+__device__ __forceinline__ void load_t(const float* tt, int32_t k, int kt, int cp, int g, int tq, float (&f)[2][4]) {
+  const int c = kt * 16 + g;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int col = (2 * cp + h) * 8 + 2 * tq;
+    const float2 lo = c < k ? *reinterpret_cast<const float2*>(tt + c * D + col) : make_float2(0.f, 0.f);
+    const float2 hi = c + 8 < k ? *reinterpret_cast<const float2*>(tt + (c + 8) * D + col) : make_float2(0.f, 0.f);
+    f[h][0] = lo.x;
+    f[h][1] = lo.y;
+    f[h][2] = hi.x;
+    f[h][3] = hi.y;
+  }
+}
+
 // KT: blocks of 16 projection columns.  With one, the request's T stays in registers while consecutive
 // candidates share it; with two it would not fit beside H and comes from L1 for every candidate.
 template <int D, int KT, bool FULL>
@@ -390,19 +409,6 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
     const int trow = warp * n_c + (lane % 8) + ((lane / 8) % 2) * 8;
     const int lsel = lane / 16;
     float tfrag[KT == 1 ? kPairs : 1][2][4];  // T^T of the cached request in step-1 accumulator layout
-    auto load_t = [&](const float* tt, int kt, int cp, float (&f)[2][4]) {
-      const int c = kt * 16 + g;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int col = (2 * cp + h) * 8 + 2 * tq;
-        const float2 lo = c < p.k ? *reinterpret_cast<const float2*>(tt + c * D + col) : make_float2(0.f, 0.f);
-        const float2 hi = c + 8 < p.k ? *reinterpret_cast<const float2*>(tt + (c + 8) * D + col) : make_float2(0.f, 0.f);
-        f[h][0] = lo.x;
-        f[h][1] = lo.y;
-        f[h][2] = hi.x;
-        f[h][3] = hi.y;
-      }
-    };
     int32_t cached_req = -1;
     int s = 0;
     uint32_t phase = 0;
@@ -427,7 +433,7 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
           cached_req = r;
           if constexpr (KT == 1) {
 #pragma unroll
-            for (int cp = 0; cp < kPairs; ++cp) load_t(tt, 0, cp, tfrag[cp]);
+            for (int cp = 0; cp < kPairs; ++cp) load_t<D>(tt, p.k, 0, cp, g, tq, tfrag[cp]);
           }
         }
         const uint32_t tile = smem_u32(smem + s * stage_bytes) + trow * 128;
@@ -449,7 +455,7 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
 #pragma unroll
               for (int e = 0; e < 8; ++e) f[e / 4][e % 4] = tfrag[cp][e / 4][e % 4];
             } else {
-              load_t(tt, kt, cp, f);
+              load_t<D>(tt, p.k, kt, cp, g, tq, f);
             }
             mma_bf16(f[0], pa[kt], xb[0], xb[1]);
             mma_bf16(f[1], pa[kt], xb[2], xb[3]);
@@ -525,6 +531,276 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
   }
 }
 
+// Columns 16 kt .. of one candidate whose first row the lane's `tile` and `trow` point at, the way of the kernel above with H
+// in three bf16 parts, every bit of it: for values that the pairs cannot hold (an infinity, what rounds to one, a Gram matrix
+// past fp32), where the result has to be what fp32 arithmetic gives.
+template <int D>
+__device__ __forceinline__ void fm_candidate_by_parts(uint32_t tile, int trow, int32_t slab_bytes, const FmParams& p, const float* tt,
+                                                   int64_t cand, int kt) {
+  const int lane = threadIdx.x % 32, g = lane / 4, tq = lane % 4, lsel = lane / 16;
+  const __nv_bfloat16* pc = p.P + (int64_t)p.n_r * p.k;
+  auto at = [&](int row, int col) -> float {  // P_C[row][col], zero beyond n_c rows and k columns
+    return row < p.n_c && col < p.k ? __bfloat162float(pc[row * p.k + col]) : 0.f;
+  };
+  const int c = kt * 16 + g;
+  const uint32_t pa[4] = {pack_bf16(at(2 * tq, c), at(2 * tq + 1, c)), pack_bf16(at(2 * tq, c + 8), at(2 * tq + 1, c + 8)),
+                          pack_bf16(at(2 * tq + 8, c), at(2 * tq + 9, c)), pack_bf16(at(2 * tq + 8, c + 8), at(2 * tq + 9, c + 8))};
+  // rows of the K x N operand of step 1 that are this candidate's: 2 tq, 2 tq + 1 and the two 8 further on
+  auto row_mask = [&](int row) { return (row < p.n_c ? 0xffffu : 0u) | (row + 1 < p.n_c ? 0xffff0000u : 0u); };
+  const uint32_t keep_lo = row_mask(2 * tq), keep_hi = row_mask(2 * tq + 8);
+  float out[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll 1
+  for (int cp = 0; cp < D / 16; ++cp) {
+    const int chunk = 2 * cp + lsel;
+    const uint32_t from = tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4);
+    uint32_t xb[4], xa[4];
+    ldmatrix_x4_trans(from, xb);
+    ldmatrix_x4(from, xa);
+    float f[2][4];
+    load_t<D>(tt, p.k, kt, cp, g, tq, f);
+    mma_bf16(f[0], pa, xb[0] & keep_lo, xb[1] & keep_hi);
+    mma_bf16(f[1], pa, xb[2] & keep_lo, xb[3] & keep_hi);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      uint32_t b0[3], b1[3];
+      split_bf16(f[0][2 * h], f[0][2 * h + 1], b0);
+      split_bf16(f[1][2 * h], f[1][2 * h + 1], b1);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) mma_bf16(out[h], xa, b0[i], b1[i]);
+    }
+  }
+  __nv_bfloat16* fc = p.FC + cand * p.n_c * p.k;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int col = kt * 16 + 8 * h + 2 * tq;
+    if (col < p.k) {
+      if (g < p.n_c) *reinterpret_cast<uint32_t*>(fc + g * p.k + col) = pack_bf16(out[h][0], out[h][1]);
+      if (g + 8 < p.n_c) *reinterpret_cast<uint32_t*>(fc + (g + 8) * p.k + col) = pack_bf16(out[h][2], out[h][3]);
+    }
+  }
+}
+
+// n_c up to 8, even k up to 32: FC = X^C T + (X^C X^C^T) P_C on fragments of 16 rows, 16 / n_c candidates each.  Per
+// 16 columns of d six products (T as a pair 2 x 2, the Gram matrix 2) on one ldmatrix: the rows' fragment as the M x K operand
+// is also the K x N operand of the Gram matrix.  Entries of two different candidates are set to zero and the rest goes, as a
+// pair, by P_C repeated per candidate; no precision is lost against the kernel above.  Fragments that reach into another
+// request are computed once per request.  A candidate per warp there, several here: 20423 candidates of 4 embeddings x 128,
+// k = 16: 25.7 and 14.8 us; 50848 of 4 x 64, k = 8: 31.0 and 15.6 us.  With one candidate per fragment (12 embeddings) four
+// more products make it the slower way: 26.4 and 28.1 us.  KT: as above, T of two blocks comes from L1 for every fragment.
+template <int D, int KT>
+__global__ void __launch_bounds__((tile_cands<D, false>() + 1) * 32, 1)
+fm_candidate_gram_kernel(const __grid_constant__ CUtensorMap map_xc, const FmParams p) {
+  constexpr int kSlabs = D / 64;
+  constexpr int kSteps = D / 16;
+  constexpr int kWarps = tile_cands<D, false>();
+  extern __shared__ __align__(1024) uint8_t smem[];
+  const int32_t n_c = p.n_c, per_frag = kFragRows / n_c, frag_rows = per_frag * n_c;
+  const int32_t tile_rows = kWarps * frag_rows, tile_cands = kWarps * per_frag;
+  // 64 columns of the tile, 128-byte swizzled rows, to the 1024 bytes that the swizzle repeats in
+  const int32_t slab_bytes = (tile_rows * 128 + 1023) / 1024 * 1024;
+  const int32_t stage_bytes = kSlabs * slab_bytes;
+  // behind the stages: rows that the last warp's fragments read past the tile
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.stages * stage_bytes + kFragRows * 128);
+  uint64_t* empty = full + kMaxStages;
+  AbortFlag* abort_flag = reinterpret_cast<AbortFlag*>(empty + kMaxStages);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  if ((smem_u32(smem) & 1023u) != 0) {  // the swizzled tiles assume a 1024-byte aligned base
+    if (threadIdx.x == 0) atomicCAS(p.status, 0u, kStatusFm | 15);
+    return;
+  }
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], kWarps);
+    }
+    abort_flag->v = 0;
+    fence_mbar_init();
+  }
+  __syncthreads();
+  const int32_t tiles_per_cta = (p.num_tiles + (int32_t)gridDim.x - 1) / (int32_t)gridDim.x;
+  const int32_t tile_begin = min((int32_t)blockIdx.x * tiles_per_cta, p.num_tiles);
+  const int32_t tile_end = min(tile_begin + tiles_per_cta, p.num_tiles);
+
+  if (warp == kWarps) {
+    // ------------------------------ TMA producer ------------------------------------------
+    if (elect_one()) {
+      prefetch_tensormap(&map_xc);
+      int s = 0;
+      uint32_t phase = 0, it = 0;
+      for (int32_t t = tile_begin; t < tile_end; ++t, ++it) {
+        if (!mbar_wait(&empty[s], phase ^ 1, abort_flag, p.status, kStatusFm | 1)) break;
+        mbar_expect_tx(&full[s], kSlabs * tile_rows * 128);
+#pragma unroll
+        for (int sl = 0; sl < kSlabs; ++sl)
+          tma_load_2d(smem + s * stage_bytes + sl * slab_bytes, &map_xc, &full[s], sl * 64, t * tile_rows);
+        if (++s == p.stages) { s = 0; phase ^= 1; }
+      }
+      // loads in flight land in this CTA's shared memory: wait for them before the CTA may exit
+      for (int st = 0; st < p.stages; ++st) {
+        const uint32_t n_issued = it / p.stages + (((int)(it % p.stages) > st) ? 1 : 0);
+        if (n_issued == 0) continue;
+        const uint64_t t0 = globaltimer_ns();
+        while (!mbar_try_wait(&full[st], (n_issued - 1) & 1) && globaltimer_ns() - t0 < kWaitLimitNs) {}
+      }
+    }
+    return;
+  }
+  const int g = lane / 4, tq = lane % 4;  // fragment row group and column pair
+  const int own[2] = {g / n_c, (g + 8) / n_c};  // candidates of the fragment that the lane's rows g and g + 8 are of
+  uint32_t same = 0;  // entries of the Gram matrix whose two rows are of one candidate, in accumulator layout
+#pragma unroll
+  for (int t = 0; t < 2; ++t)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int col = t * 8 + 2 * tq + e % 2;
+      if (own[e / 2] == col / n_c && col < frag_rows) same |= 1u << (t * 4 + e);
+    }
+  uint32_t pb[KT][2][2];  // P_C, repeated per candidate, as the K x N operand
+  {
+    const __nv_bfloat16* pc = p.P + (int64_t)p.n_r * p.k;
+    auto at = [&](int row, int col) -> float { return row < frag_rows && col < p.k ? __bfloat162float(pc[row % n_c * p.k + col]) : 0.f; };
+#pragma unroll
+    for (int kt = 0; kt < KT; ++kt)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = kt * 16 + h * 8 + g;
+        pb[kt][h][0] = pack_bf16(at(2 * tq, c), at(2 * tq + 1, c));
+        pb[kt][h][1] = pack_bf16(at(2 * tq + 8, c), at(2 * tq + 9, c));
+      }
+  }
+  const int row0 = warp * frag_rows, in_frag = (lane % 8) + ((lane / 8) % 2) * 8, trow = row0 + in_frag, lsel = lane / 16;
+  // T as the K x N operand, as a pair: [part][b0, b1] of step s and columns 8 h of block kt
+  auto load_pair = [&](const float* tt, int kt, int h, int s, uint32_t (&b0)[2], uint32_t (&b1)[2]) {
+    const int c = kt * 16 + h * 8 + g;
+    float2 lo = make_float2(0.f, 0.f), hi = lo;
+    if (c < p.k) {
+      lo = *reinterpret_cast<const float2*>(tt + c * D + s * 16 + 2 * tq);
+      hi = *reinterpret_cast<const float2*>(tt + c * D + s * 16 + 8 + 2 * tq);
+    }
+    split_bf16(lo.x, lo.y, b0);
+    split_bf16(hi.x, hi.y, b1);
+  };
+  uint32_t tb[KT == 1 ? kSteps : 1][2][2][2];  // [step][h][b0 | b1][part]
+  int32_t cached_req = -1;
+  int s = 0;
+  uint32_t phase = 0;
+  // the request of this warp's first candidate, and its end, found one tile ahead of their use
+  int32_t r_next = 0, end_next = 0;
+  RequestWalk walk{p.offsets, p.R};
+  auto find = [&](int32_t t) {
+    const int64_t c = (int64_t)t * tile_cands + warp * per_frag;
+    if (t < tile_end && c < p.N) {
+      r_next = walk.of(c);
+      end_next = walk.end;
+    }
+  };
+  find(tile_begin);
+  for (int32_t t = tile_begin; t < tile_end; ++t) {
+    int32_t r = r_next, end = end_next;
+    find(t + 1);
+    if (!mbar_wait(&full[s], phase, abort_flag, p.status, kStatusFm | 2)) break;
+    const int64_t cand = (int64_t)t * tile_cands + warp * per_frag;
+    const int32_t valid = (int32_t)max((int64_t)0, min((int64_t)per_frag, p.N - cand));
+    const uint32_t stage = smem_u32(smem + s * stage_bytes), tile = stage + trow * 128;
+    for (int32_t lo = 0; lo < valid;) {
+      const int32_t hi = min(valid, (int32_t)(end - cand));  // candidates lo .. hi of the fragment are of request r
+      const float* tt = p.TT + (int64_t)r * p.k * D;
+      if (r != cached_req) {
+        if (cached_req < 0) griddep_wait();  // TT comes from the request kernel launched just before
+        cached_req = r;
+        if constexpr (KT == 1) {
+#pragma unroll
+          for (int st = 0; st < kSteps; ++st)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) load_pair(tt, 0, h, st, tb[st][h][0], tb[st][h][1]);
+        }
+      }
+      float out[KT][2][4], low[KT][2][4], gram[2][4];  // (two chains: of the rounded values and of the remainders)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          gram[h][e] = 0.f;
+#pragma unroll
+          for (int kt = 0; kt < KT; ++kt) out[kt][h][e] = low[kt][h][e] = 0.f;
+        }
+#pragma unroll
+      for (int st = 0; st < kSteps; ++st) {
+        const int chunk = 2 * st + lsel;  // 16-byte chunk along d
+        uint32_t xa[4];
+        ldmatrix_x4(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xa);
+        mma_bf16(gram[0], xa, xa[0], xa[2]);
+        mma_bf16(gram[1], xa, xa[1], xa[3]);
+#pragma unroll
+        for (int kt = 0; kt < KT; ++kt)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if constexpr (KT == 1) {
+              mma_bf16(out[kt][h], xa, tb[st][h][0][0], tb[st][h][1][0]);
+              mma_bf16(low[kt][h], xa, tb[st][h][0][1], tb[st][h][1][1]);
+            } else {
+              uint32_t b0[2], b1[2];
+              load_pair(tt, kt, h, st, b0, b1);
+              mma_bf16(out[kt][h], xa, b0[0], b1[0]);
+              mma_bf16(low[kt][h], xa, b0[1], b1[1]);
+            }
+          }
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if ((same >> e & 1u) == 0) gram[e / 4][e % 4] = 0.f;
+      // the accumulator layout of two 8-wide tiles is that of a 16 x 16 M x K operand
+      uint32_t part[4][2];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) split_bf16(gram[x / 2][x % 2 * 2], gram[x / 2][x % 2 * 2 + 1], part[x]);
+      const uint32_t ga[4] = {part[0][0], part[1][0], part[2][0], part[3][0]};
+      const uint32_t gb[4] = {part[0][1], part[1][1], part[2][1], part[3][1]};
+      uint32_t bad = 0;  // candidates with a NaN in a row of theirs
+#pragma unroll
+      for (int kt = 0; kt < KT; ++kt)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          mma_bf16(out[kt][h], ga, pb[kt][h][0], pb[kt][h][1]);
+          mma_bf16(low[kt][h], gb, pb[kt][h][0], pb[kt][h][1]);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            out[kt][h][e] += low[kt][h][e];
+            if (isnan(out[kt][h][e])) bad |= 1u << own[e / 2];
+          }
+        }
+      if (__any_sync(0xffffffffu, bad != 0)) {  // perhaps of an infinity, or of a value that rounds to one
+        bad = __reduce_or_sync(0xffffffffu, bad);
+        for (int32_t c = lo; c < hi; ++c)
+          if (bad >> c & 1u) {
+            const int row = row0 + c * n_c + in_frag;
+#pragma unroll 1
+            for (int kt = 0; kt < KT; ++kt) fm_candidate_by_parts<D>(stage + row * 128, row, slab_bytes, p, tt, cand + c, kt);
+          }
+      }
+      __nv_bfloat16* fc = p.FC + cand * n_c * p.k;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        if (own[j] < lo || own[j] >= hi || (bad >> own[j] & 1u)) continue;
+#pragma unroll
+        for (int kt = 0; kt < KT; ++kt)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int col = kt * 16 + 8 * h + 2 * tq;
+            if (col < p.k) *reinterpret_cast<uint32_t*>(fc + (g + 8 * j) * p.k + col) = pack_bf16(out[kt][h][2 * j], out[kt][h][2 * j + 1]);
+          }
+      }
+      lo = hi;
+      if (lo < valid) {  // on to the next request that has candidates
+        do { ++r; } while (p.offsets[r + 1] <= cand + lo);
+        end = p.offsets[r + 1];
+      }
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[s]);
+    if (++s == p.stages) { s = 0; phase ^= 1; }
+  }
+}
+
 int sm_count_fm() {
   static int n = 0;
   if (n == 0) {
@@ -535,15 +811,17 @@ int sm_count_fm() {
   return n;
 }
 
-template <int D, int KT, bool FULL>
+enum class FmKernel { kFull, kPair, kGram };
+template <int D, int KT, FmKernel WHICH>
 rocs_status_t launch_fm_mma_as(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t k,
                                const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
-  constexpr int kTileCands = tile_cands<D, FULL>();
-  const int stage_bytes = D / 64 * ((kTileCands * n_c * 128 + 1023) / 1024 * 1024);
+  constexpr int kWarps = tile_cands<D, WHICH == FmKernel::kFull>();
+  const int32_t tile_cands = WHICH == FmKernel::kGram ? kWarps * (kFragRows / n_c) : kWarps, tile_rows = tile_cands * n_c;
+  const int stage_bytes = D / 64 * ((tile_rows * 128 + 1023) / 1024 * 1024);
   constexpr int kFixed = kFragRows * 128 + 2 * kMaxStages * 8 + 16;
   CUtensorMap map_xc;
   if (!make_tensor_map_2d(&map_xc, XC, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)plan->N * n_c, D, D,
-                          (uint32_t)(kTileCands * n_c), 64, true))
+                          (uint32_t)tile_rows, 64, true))
     return ROCS_ERR_CUDA;
   uint32_t* status = device_status_word();
   if (!status) return ROCS_ERR_CUDA;
@@ -552,7 +830,7 @@ rocs_status_t launch_fm_mma_as(const rocs_plan* plan, int32_t n_r, int32_t n_c, 
   p.n_r = n_r;
   p.n_c = n_c;
   p.k = k;
-  p.num_tiles = (int32_t)((plan->N + kTileCands - 1) / kTileCands);
+  p.num_tiles = (int32_t)((plan->N + tile_cands - 1) / tile_cands);
   p.stages = std::min(kMaxStages, (227 * 1024 - kFixed) / stage_bytes);
   p.P = (const __nv_bfloat16*)P;
   p.offsets = plan->cand_offsets;
@@ -561,13 +839,15 @@ rocs_status_t launch_fm_mma_as(const rocs_plan* plan, int32_t n_r, int32_t n_c, 
   p.FC = (__nv_bfloat16*)FC;
   p.status = status;
   const int smem = p.stages * stage_bytes + kFixed;
-  auto kern = fm_candidate_mma_kernel<D, KT, FULL>;
+  void (*kern)(CUtensorMap, FmParams);
+  if constexpr (WHICH == FmKernel::kGram) kern = fm_candidate_gram_kernel<D, KT>;
+  else kern = fm_candidate_mma_kernel<D, KT, WHICH == FmKernel::kFull>;
   ROCS_ALLOW_SMEM(kern, kMaxDynamicSmem);
   // Launched so that it may overlap the request kernel in front of it on the stream (that kernel
   // releases its dependents at once); nothing else this kernel reads is written by that launch.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)std::min(p.num_tiles, sm_count_fm()));
-  cfg.blockDim = dim3((kTileCands + 1) * 32);
+  cfg.blockDim = dim3((kWarps + 1) * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -582,10 +862,11 @@ rocs_status_t launch_fm_mma_as(const rocs_plan* plan, int32_t n_r, int32_t n_c, 
 template <int D>
 rocs_status_t launch_fm_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t k,
                             const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
-  if (k > 16) return launch_fm_mma_as<D, 2, false>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
-  if (n_c == kFragRows && (k == 8 || k == 16))
-    return launch_fm_mma_as<D, 1, true>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
-  return launch_fm_mma_as<D, 1, false>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+#define ROCS_LAUNCH(KT_, WHICH_) launch_fm_mma_as<D, KT_, FmKernel::WHICH_>(plan, n_r, n_c, k, XC, P, TT, FC, stream)
+  if (n_c <= kFragRows / 2) return k > 16 ? ROCS_LAUNCH(2, kGram) : ROCS_LAUNCH(1, kGram);
+  if (k > 16) return ROCS_LAUNCH(2, kPair);
+  return n_c == kFragRows && (k == 8 || k == 16) ? ROCS_LAUNCH(1, kFull) : ROCS_LAUNCH(1, kPair);
+#undef ROCS_LAUNCH
 }
 
 template <typename T>
