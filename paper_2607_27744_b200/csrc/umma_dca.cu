@@ -217,13 +217,15 @@ __device__ __forceinline__ void row_by_hand(const __nv_bfloat16* q, const __nv_b
   }
 }
 
-// The item of index i in the order request, head, tile, found by one warp from the offsets.
-__device__ __forceinline__ DcaItem find_item(const int32_t* __restrict__ off, int32_t R, int32_t per, int32_t heads,
-                                             int32_t i, int lane) {
+// The item of index i in the order request, head, tile, found by one warp from the offsets, with its request's keys: their
+// offsets are loaded with the candidates' and not behind them, a second trip to memory in front of the item's first loads.
+__device__ __forceinline__ DcaItem find_item(const int32_t* __restrict__ off, const int32_t* __restrict__ seq, int32_t R, int32_t per,
+                                             int32_t heads, int32_t i, int lane, int32_t& s0, int32_t& L) {
   int32_t base = 0;
   for (int32_t r0 = 0; r0 < R; r0 += 32) {
     const int32_t r = r0 + lane;
     const int32_t c0 = r < R ? off[r] : 0, n = r < R ? off[r + 1] - c0 : 0;
+    const int32_t k0 = r < R ? seq[r] : 0, k1 = r < R ? seq[r + 1] : 0;
     const int32_t tiles = tiles_of(n, per), entries = tiles * heads;
     int32_t incl = entries;
 #pragma unroll
@@ -236,6 +238,8 @@ __device__ __forceinline__ DcaItem find_item(const int32_t* __restrict__ off, in
     if (hit != 0) {
       const int32_t local = i - first, h = tiles > 0 ? local / tiles : 0, c = (local - h * tiles) * per;
       const int src = __ffs(hit) - 1;
+      s0 = __shfl_sync(0xffffffffu, k0, src);
+      L = __shfl_sync(0xffffffffu, k1, src) - s0;
       return DcaItem{__shfl_sync(0xffffffffu, r, src), __shfl_sync(0xffffffffu, c0 + c, src),
                      __shfl_sync(0xffffffffu, min(per, n - c), src), __shfl_sync(0xffffffffu, h, src)};
     }
@@ -420,9 +424,13 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     int32_t next_s0 = 0, next_L = 0, total_L = 0;
     auto read_next = [&]() {
       if (i >= 0) {
-        next = p.items == nullptr ? find_item(p.cand_offsets, p.R, BQ / p.n_q, p.H, i, lane) : p.items[i];
-        next_s0 = p.seq_offsets[next.req];
-        next_L = p.seq_offsets[next.req + 1] - next_s0;
+        if (p.items == nullptr) {
+          next = find_item(p.cand_offsets, p.seq_offsets, p.R, BQ / p.n_q, p.H, i, lane, next_s0, next_L);
+        } else {
+          next = p.items[i];
+          next_s0 = p.seq_offsets[next.req];
+          next_L = p.seq_offsets[next.req + 1] - next_s0;
+        }
         if constexpr (SPLIT) {  // this side's run of the item's key blocks
           const int32_t nblk = (next_L + BKV - 1) / BKV, parts = 2 * (int32_t)cluster_size;
           const int32_t part = 2 * (int32_t)cluster_ctarank() + side;
@@ -880,7 +888,7 @@ static rocs_status_t launch_dca(const rocs_plan* plan, int32_t n_q, int32_t H, f
   if (num > 0x7fffffffLL) return ROCS_ERR_UNSUPPORTED;
   if (num == 0) return ROCS_OK;
   // Items that fit the SMs once are split along their keys (SPLIT): over the two sides of a CTA, and over the CTAs
-  // of the largest cluster of which every item still gets one at the same time, two key blocks per side at least.  Short
+  // of the largest cluster of which every item still gets one at the same time.  Short
   // sequences are not worth it.  How many clusters run at once differs from chip to chip (a cluster stays inside one of
   // its partitions, of which each chip has other SMs: 74 pairs, 33 of 4 and 15 of 8 on one), and an item more than that
   // takes a second round: 16 items of 4096 keys 26.1 us over clusters of 8 there, 14.6 us over 4.  The numbers below are a
@@ -889,8 +897,13 @@ static rocs_status_t launch_dca(const rocs_plan* plan, int32_t n_q, int32_t H, f
   const bool split = num <= sms && blocks >= 3;
   int32_t cluster = 1;
   const int32_t most[4] = {sms, 70, 32, 14};
+  // Blocks of 128 keys: one per CTA is enough (its sides then do not compete for the SM).  40 candidates of one request x 8
+  // heads of 64, in a chain, with two per side and this: 300 / 520 / 1000 keys 8.4 / 9.7 / 9.7 and 7.7 / 8.2 / 8.7 us; 2000 keys
+  // over 4 and 8 CTAs 10.6 and 11.2.  Blocks of 64 keys: 8 requests x 4 heads of 128, 300 / 520 keys, two per side and one per
+  // CTA 9.2 / 10.3 and 10.3 / 11.6.
+  auto worth = [&](int i) { return (4 << i) <= blocks || (BKV == 128 && (1 << i) <= blocks && (i < 3 || blocks < 12)); };
   for (int i = 1; i < 4 && split; ++i)
-    if (num <= most[i] && (4 << i) <= blocks) cluster = 1 << i;
+    if (num <= most[i] && worth(i)) cluster = 1 << i;
   // Requests that a producer warp looks through itself, at every item; the list is a launch in front.  What looking
   // costs grows with the requests times the items.  Plan and attention, 8 heads of 64, 200 to 400 keys, without and with
   // the list: 27 candidates of each of 64 / 256 / 288 / 512 requests 15.9 / 44.4 / 54.1 / 105 us and 18.4 / 46.2 / 52.2 /
