@@ -13,9 +13,12 @@
 // candidate's own n_c x n_c block on the diagonal (the off-diagonal products are discarded: the
 // kernel is bound by reading X^C from HBM, the tensor pipe has slack).
 //
-// Persistent CTA, 10 warps: warp 0 TMA producer, warp 1 MMA issuer, two epilogue groups of four
-// warps that alternate tiles (each owns one TMEM accumulator), so one group drains a tile while the
-// tensor pipe fills the other accumulator.  An epilogue warp owns 32 rows = 32 / n_c whole
+// Persistent CTA, 14 or 10 warps: warp 0 TMA producer, warp 1 MMA issuer, three epilogue groups of four
+// warps that take tiles in turn (each owns one TMEM accumulator), so groups drain tiles while the
+// tensor pipe fills the next accumulator.  Three where that many accumulators fit the 512 columns (up to 32 embeddings of a
+// request) and the third row buffer does not take a stage of the ring: the way of a tile through its group is the longer one
+// (128 requests x 1024 candidates, 32 + 16 embeddings x 128 to 8 + 8: 125.7 us with two groups, 117.9 us with three, 5.4 TB/s).
+// An epilogue warp owns 32 rows = 32 / n_c whole
 // candidates: it rounds their YC rows to bf16 into a private shared-memory buffer, copies them out
 // if the raw block is wanted, and forms OC = ZR + W_CC YC per candidate with warp-level
 // mma.sync m16n8k16 (W_CC fragments live in registers, YC fragments come through ldmatrix), so the
@@ -30,9 +33,10 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kThreads = 320;
+constexpr int threads_of(int groups) { return 64 + 128 * groups; }
 constexpr uint32_t kStatusGlm = 0x200;
-constexpr int kAccStride = 256;  // TMEM columns per accumulator
+constexpr uint32_t kTmemCols = 512;
+constexpr int acc_stride(int groups) { return groups == 3 ? 160 : 256; }  // TMEM columns per accumulator
 
 struct GlmParams {
   const Tile* tiles;       // the list, or null
@@ -48,18 +52,19 @@ struct GlmParams {
 };
 
 // WALK: the tiles are found in the offsets, otherwise read from the list.
-template <int NC, bool WALK>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int NC, bool WALK, int G>
+__global__ void __launch_bounds__(threads_of(G), 1)
 glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constant__ CUtensorMap map_xc,
                 const GlmParams p) {
+  constexpr int kAccStride = acc_stride(G);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* staging = smem + p.stages * p.stage_bytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(staging + 2 * p.group_staging_bytes);
+  uint64_t* full = reinterpret_cast<uint64_t*>(staging + G * p.group_staging_bytes);
   uint64_t* empty = full + 8;
   uint64_t* tmem_full = empty + 8;
-  uint64_t* tmem_empty = tmem_full + 2;
-  uint64_t* drain = tmem_empty + 2;
+  uint64_t* tmem_empty = tmem_full + G;
+  uint64_t* drain = tmem_empty + G;
   uint32_t* tmem_ptr = reinterpret_cast<uint32_t*>(drain + 1);
   AbortFlag* abort_flag = reinterpret_cast<AbortFlag*>(tmem_ptr + 1);
 
@@ -78,7 +83,7 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    for (int a = 0; a < 2; ++a) {
+    for (int a = 0; a < G; ++a) {
       mbar_init(&tmem_full[a], 1);
       mbar_init(&tmem_empty[a], 4);
     }
@@ -87,7 +92,7 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
     fence_mbar_init();
   }
   if (warp == 1) {
-    tmem_alloc(tmem_ptr, 2 * kAccStride);
+    tmem_alloc(tmem_ptr, kTmemCols);
     tmem_relinquish();
   }
   tc_fence_before_sync();
@@ -131,9 +136,9 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
       uint32_t it = 0;
       bool ok = true;
       for (int32_t t = t_begin; t < t_end; ++t, ++it) {
-        const uint32_t acc = it & 1;
+        const uint32_t acc = it % G;
         const int s = it % p.stages;
-        if (!mbar_wait(&tmem_empty[acc], ((it >> 1) & 1) ^ 1, abort_flag, p.status, kStatusGlm | 2)) { ok = false; break; }
+        if (!mbar_wait(&tmem_empty[acc], ((it / G) & 1) ^ 1, abort_flag, p.status, kStatusGlm | 2)) { ok = false; break; }
         if (!mbar_wait(&full[s], (it / p.stages) & 1, abort_flag, p.status, kStatusGlm | 3)) { ok = false; break; }
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + acc * kAccStride;
@@ -156,7 +161,7 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
   } else {
     // ------------------------------ epilogue groups ----------------------------------------
     // Everything below is local to one warp: a warp owns 32 tile rows = 32 / NC whole candidates.
-    const int g = (warp - 2) / 4;  // group 0: warps 2-5, group 1: warps 6-9
+    const int g = (warp - 2) / 4;  // group 0: warps 2-5, group 1: warps 6-9, ...
     const int q = warp % 4;        // TMEM lane quadrant = rows 32q .. 32q+31 of the tile
     const int n8 = n / 8;
     // bf16 copy of this warp's 32 rows of YC, row stride yc_stride bytes (16 mod 32: no conflicts)
@@ -189,9 +194,9 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
     for (int32_t t = t_begin; t < t_end; ++t, ++it) {
       Tile tile;
       if (WALK) tile = walk.take(t + 1 < t_end);
-      if ((int)(it & 1) != g) continue;
+      if ((int)(it % G) != g) continue;
       if (!WALK) tile = p.tiles[t];
-      if (!mbar_wait(&tmem_full[g], (it >> 1) & 1, abort_flag, p.status, kStatusGlm | 4)) break;
+      if (!mbar_wait(&tmem_full[g], (it / G) & 1, abort_flag, p.status, kStatusGlm | 4)) break;
       tc_fence_after_sync();
       const uint32_t t_row = tmem_base + g * kAccStride + ((uint32_t)(q * 32) << 16);
       // All TMEM reads of the tile are issued before the first wait: the first 32 columns of the
@@ -318,7 +323,7 @@ glm_umma_kernel(const __grid_constant__ CUtensorMap map_xr, const __grid_constan
   __syncthreads();
   if (warp == 1) {
     tc_fence_after_sync();
-    tmem_dealloc(tmem_base, 2 * kAccStride);
+    tmem_dealloc(tmem_base, kTmemCols);
   }
 }
 
@@ -335,7 +340,7 @@ int sm_count_glm() {
 constexpr int kMaxSmem = 227 * 1024;
 
 struct GlmLayout {
-  int32_t n_r_pad, stage_bytes, group_staging_bytes, yc_stride, stages, smem_bytes;
+  int32_t n_r_pad, stage_bytes, group_staging_bytes, yc_stride, groups, stages, smem_bytes;
   bool ok;
 };
 
@@ -348,11 +353,20 @@ GlmLayout glm_layout(int32_t n_r, int32_t n_c, int32_t d, int32_t n_co) {
   L.yc_stride = (n * 2) % 32 == 0 ? n * 2 + 16 : n * 2;
   (void)n_co;
   L.group_staging_bytes = (128 * L.yc_stride + 127) & ~127;
-  const int32_t fixed = 2 * L.group_staging_bytes + 512 + 1024;
-  L.stages = std::min(6, (kMaxSmem - fixed) / L.stage_bytes);
-  L.smem_bytes = L.stages * L.stage_bytes + fixed;
+  auto fixed = [&](int groups) { return groups * L.group_staging_bytes + 512 + 1024; };
+  auto stages = [&](int groups) { return std::min(6, (kMaxSmem - fixed(groups)) / L.stage_bytes); };
+  L.groups = L.n_r_pad + 128 <= acc_stride(3) && stages(3) == stages(2) ? 3 : 2;
+  L.stages = stages(L.groups);
+  L.smem_bytes = L.stages * L.stage_bytes + fixed(L.groups);
   L.ok = L.stages >= 2;
   return L;
+}
+
+template <int NC, bool WALK, int G>
+rocs_status_t launch(const cudaLaunchConfig_t& cfg, const CUtensorMap& map_xr, const CUtensorMap& map_xc, const GlmParams& p) {
+  ROCS_ALLOW_SMEM((glm_umma_kernel<NC, WALK, G>), kMaxSmem);
+  ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, glm_umma_kernel<NC, WALK, G>, map_xr, map_xc, p));
+  return ROCS_OK;
 }
 
 }  // namespace
@@ -399,7 +413,7 @@ rocs_status_t umma_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t 
   // this kernel sets itself up and streams X^C beside it and waits for it only before it reads ZR, if it does.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3((unsigned)threads_of(L.groups));
   cfg.dynamicSmemBytes = L.smem_bytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -407,22 +421,14 @@ rocs_status_t umma_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-#define ROCS_GLM_LAUNCH(NC_)                                                                                  \
-  do {                                                                                                        \
-    if (tl.dev == nullptr) {                                                                                  \
-      ROCS_ALLOW_SMEM((glm_umma_kernel<NC_, true>), kMaxSmem);                                                \
-      ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, glm_umma_kernel<NC_, true>, map_xr, map_xc, p));                 \
-    } else {                                                                                                  \
-      ROCS_ALLOW_SMEM((glm_umma_kernel<NC_, false>), kMaxSmem);                                               \
-      ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, glm_umma_kernel<NC_, false>, map_xr, map_xc, p));                \
-    }                                                                                                         \
-  } while (0)
-  if (n_c == 8) ROCS_GLM_LAUNCH(8);
-  else if (n_c == 16) ROCS_GLM_LAUNCH(16);
-  else ROCS_GLM_LAUNCH(32);
-#undef ROCS_GLM_LAUNCH
-  ROCS_CUDA_TRY(cudaGetLastError());
-  return ROCS_OK;
+#define ROCS_LAUNCH(NC_)                                                                                                        \
+  st = tl.dev == nullptr ? (L.groups == 3 ? launch<NC_, true, 3>(cfg, map_xr, map_xc, p) : launch<NC_, true, 2>(cfg, map_xr, map_xc, p)) \
+                         : (L.groups == 3 ? launch<NC_, false, 3>(cfg, map_xr, map_xc, p) : launch<NC_, false, 2>(cfg, map_xr, map_xc, p))
+  if (n_c == 8) ROCS_LAUNCH(8);
+  else if (n_c == 16) ROCS_LAUNCH(16);
+  else ROCS_LAUNCH(32);
+#undef ROCS_LAUNCH
+  return st;
 }
 
 }  // namespace rocs

@@ -758,6 +758,18 @@ def test_glm_tiles_walked_in_the_offsets(R, n_c):
     assert _run_glm(wl.CONFIGS[5].with_(R=R, n_r=8, n_c=n_c, d_emb=64, n_ro=2, n_co=4), co) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("R,most", [(150, 16), (60, 400)])
+@pytest.mark.parametrize("n_r,n_c,d,n_co", [(32, 16, 128, 8), (16, 8, 64, 0), (24, 32, 128, 16), (40, 16, 128, 4), (32, 8, 256, 5)])
+def test_glm_epilogue_groups(R, most, n_r, n_c, d, n_co):
+    # three groups of epilogue warps (two behind 40 embeddings of a request, or where a third takes a stage): runs of fewer
+    # tiles than groups and runs that take each of them several times, with tiles that leave warps without rows
+    co = wl.offsets_from_counts(np.random.default_rng(most).integers(0, most, R).tolist())
+    cfg = wl.CONFIGS[5].with_(R=R, n_r=n_r, n_c=n_c, d_emb=d, n_ro=min(2, n_co), n_co=n_co)
+    N = int(co[-1])
+    sample = np.unique(np.concatenate([np.clip(np.stack([co[:-1], co[1:] - 1]).ravel(), 0, N - 1), np.arange(0, N, 61)]))
+    assert _run_glm(cfg, co, sample=sample) <= tol_for("bf16")
+
+
 def test_glm_config4_full_size_sampled():
     cfg = wl.CONFIGS[4]
     co = wl.cand_offsets(cfg)
