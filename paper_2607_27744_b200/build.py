@@ -13,7 +13,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "librocs.so")
 EXT = os.path.join(HERE, "_native.so")
-SOURCES = ["api.cu", "simt_kernels.cu", "linear_simt.cu", "tensor_map.cu", "umma_linear.cu", "umma_linear_ws2.cu", "umma_linear_pair.cu", "umma_dca.cu", "dca_simt.cu", "umma_glm.cu", "glm_mma.cu", "fm_projection.cu", "group_norm.cu", "no_alloc.cu", "selftest.cu", "row_stats.cu", "glm_request_mma.cu"]
+SOURCES = ["api.cu", "simt_kernels.cu", "linear_simt.cu", "tensor_map.cu", "umma_linear.cu", "umma_linear_ws2.cu", "umma_linear_pair.cu", "umma_dca.cu", "dca_simt.cu", "umma_glm.cu", "glm_mma.cu", "fm_projection.cu", "fm_umma.cu", "group_norm.cu", "no_alloc.cu", "selftest.cu", "row_stats.cu", "glm_request_mma.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",

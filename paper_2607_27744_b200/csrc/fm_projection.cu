@@ -7,17 +7,14 @@
 // so a candidate reads its own 2 n_c d bytes and nothing of the request but the d x k block T,
 // which stays in registers while consecutive candidates belong to the same request.
 //
-// The candidate side is bound by HBM (about 30 flop per byte): the bf16 kernel streams candidate
-// tiles through a TMA ring and gives every warp one candidate at a time, whose two small products
-// (16 x d x 16 each) run on mma.sync m16n8k16 straight out of the swizzled tile:
+// The candidate side is bound by HBM (about 30 flop per byte).  Two bf16 kernels: fm_umma.cu, and here, for candidates of 16
+// embeddings, a kernel that streams candidate tiles through a TMA ring and gives every warp one candidate at a time, whose
+// two small products (16 x d x 16 each) run on mma.sync m16n8k16 straight out of the swizzled tile:
 //   step 1   H^T = T^T + P_C^T X^C_i    accumulators start at T^T (fp32); X^C_i is the K x N
 //                                       operand, read with ldmatrix.trans
 //   step 2   FC_i = X^C_i H             the accumulator layout of step 1 is the B-operand layout of
 //                                       step 2, so H never leaves registers; X^C_i is the M x K
 //                                       operand, read with ldmatrix
-// Candidates of up to 8 embeddings take their own term through the Gram matrix instead,
-//     FC[i] = X^C_i T[m_i] + (X^C_i X^C_i^T) P_C,
-// whose products are the same for the rows of all candidates that fit 16 rows.
 // A general kernel (any shape, fp32 or bf16 storage, fp32 FMA) covers everything else.
 #include <algorithm>
 #include <type_traits>
@@ -36,13 +33,25 @@ __device__ __forceinline__ float ld_f(const __nv_bfloat16* p, int64_t i) { retur
 __device__ __forceinline__ void st_f(float* p, int64_t i, float v) { p[i] = v; }
 __device__ __forceinline__ void st_f(__nv_bfloat16* p, int64_t i, float v) { p[i] = __float2bfloat16_rn(v); }
 
+// TT as the candidate kernels read it: fp32 [R, k, d], or (PAIR) bf16 [R, 2, k, d], value and remainder.
+template <bool PAIR>
+using TermOf = std::conditional_t<PAIR, __nv_bfloat16, float>;
+// What is left of an infinity or a NaN is 0; a finite value does not round to infinity.
+__device__ __forceinline__ __nv_bfloat16 pair_value(float x) {
+  const __nv_bfloat16 v = __float2bfloat16_rn(x);
+  return __hisinf(v) ? __ushort_as_bfloat16((unsigned short)(__float_as_uint(x) >> 16)) : v;
+}
+__device__ __forceinline__ __nv_bfloat16 pair_remainder(float x, __nv_bfloat16 value) {
+  return __float2bfloat16_rn(isfinite(x) ? x - __bfloat162float(value) : 0.f);
+}
+
 // ---------------------------------------------------------------------------------------------
 // Request side, one block per request:  TT[r] = P_R^T X^R_r  ([k, d] fp32, the transpose of T)
 // and FR[r] = X^R_r T[r].
 // ---------------------------------------------------------------------------------------------
-template <typename T>
+template <typename T, bool PAIR>
 __global__ void __launch_bounds__(256) fm_request_kernel(int32_t n_r, int32_t d, int32_t k, const T* __restrict__ XR,
-                                                         const T* __restrict__ P, float* __restrict__ TT,
+                                                         const T* __restrict__ P, TermOf<PAIR>* __restrict__ TT,
                                                          T* __restrict__ FR) {
   extern __shared__ float sm[];
   const int32_t ds = d + 1;           // padded row stride: rows land in different banks
@@ -75,7 +84,14 @@ __global__ void __launch_bounds__(256) fm_request_kernel(int32_t n_r, int32_t d,
     for (int u = 0; u < kCg; ++u)
       if (c0 + u < k) {
         tt[(c0 + u) * ds + e] = acc[u];
-        TT[((int64_t)r * k + c0 + u) * d + e] = acc[u];
+        if constexpr (PAIR) {
+          __nv_bfloat16* at = TT + ((int64_t)r * 2 * k + c0 + u) * d + e;
+          const __nv_bfloat16 value = pair_value(acc[u]);
+          at[0] = value;
+          at[(int64_t)k * d] = pair_remainder(acc[u], value);
+        } else {
+          TT[((int64_t)r * k + c0 + u) * d + e] = acc[u];
+        }
       }
   }
   if (!FR) return;
@@ -130,24 +146,12 @@ __global__ void __launch_bounds__(128) fm_candidate_simt_kernel(int32_t n_r, int
 }
 
 // ---------------------------------------------------------------------------------------------
-// Candidate side, bf16 streaming kernel: n_c up to 16, even k up to 32, d a multiple of 64 up to 256.
-// The fragments hold 16 candidate rows: of a candidate with fewer the rest are the next candidate's, which
-// step 1 masks to zero (0 x NaN of a neighbour must not arise) and step 2 computes and drops.
-// 16 embeddings and 8 or 16 columns (FULL) round H to bf16 and are bound by HBM.  Every other shape takes H as a bf16 pair
-// (value and remainder) through two products in step 2, and is bound by the products: error of FC against 64 bits on 128
-// requests x 1024 candidates, 32 + 12 embeddings x 128, k = 16, 1.6568e-3 as with fp32 FMA throughout (all of it the
-// rounding of FC) at 120.3 us; 1.8657e-3 at 81.8 us with H rounded; three parts, every bit of H, about 30 us more.
-// 18 400 candidates of 12 embeddings x 128, k = 16: 26.9 us; the general kernel, a block per candidate, 284 us.
+// Candidate side, bf16 streaming kernel: 16 embeddings, 8 or 16 columns, d a multiple of 64 up to 256.  H is rounded to bf16.
+// Bound by HBM; against fm_umma.cu: 29 / 300 / 1000 / 8000 / 131072 candidates x 128, k = 16, 5.6 / 6.1 / 7.4 / 21.5 / 103 us
+// and 6.3 / 6.6 / 8.9 / 22.6 / 106, 10000 x 64, k = 8, 14.9 and 18.6: one candidate per warp is done sooner behind its loads.
 // ---------------------------------------------------------------------------------------------
-constexpr int kFragRows = 16;      // rows of a candidate's fragments
-// Candidates per tile = compute warps per CTA.  Two per scheduler are enough for a stream that HBM bounds; the chains of the
-// pair's products want more of them: as many as leave them their registers (11 and the producer are three per scheduler, at
-// 168 registers, 15 four at 128).  With 8: 128.4 us for the batch above, 223 for 183 us on 128 x 512 candidates of 12
-// embeddings x 256, 54.2 for 49.9 on 64 x 512 of 16 x 64 to 24 columns.
-template <int D, bool FULL>
-constexpr int tile_cands() {
-  return FULL ? 8 : D == 64 ? 15 : 11;
-}
+constexpr int kFragRows = 16;      // embeddings of a candidate = rows of its fragments
+constexpr int kTileCands = 8;      // candidates per tile = compute warps per CTA
 constexpr int kMaxStages = 12;
 constexpr uint32_t kStatusFm = 0x600;
 
@@ -185,9 +189,10 @@ __device__ __forceinline__ void ldmatrix_x2(uint32_t addr, uint32_t (&r)[2]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
 }
 
+template <bool PAIR>
 __global__ void __launch_bounds__(256) fm_request_mma_kernel(int32_t n_r, int32_t d, int32_t k,
                                                              const __nv_bfloat16* __restrict__ XR,
-                                                             const __nv_bfloat16* __restrict__ P, float* __restrict__ TT,
+                                                             const __nv_bfloat16* __restrict__ P, TermOf<PAIR>* __restrict__ TT,
                                                              __nv_bfloat16* __restrict__ FR) {
   extern __shared__ __align__(16) uint8_t smem_fmr[];
   const int32_t n_rp = (n_r + 15) / 16 * 16, kp = (k + 15) / 16 * 16;
@@ -245,7 +250,16 @@ __global__ void __launch_bounds__(256) fm_request_mma_kernel(int32_t n_r, int32_
       for (int j = 0; j < 2; ++j) {
         const int32_t c = c0 + g8 + j * 8, e = e0 + h * 8 + 2 * t4;
         const float v0 = acc[h][2 * j], v1 = acc[h][2 * j + 1];
-        if (c < k) *reinterpret_cast<float2*>(TT + ((int64_t)r * k + c) * d + e) = make_float2(v0, v1);
+        if constexpr (PAIR) {
+          if (c < k) {
+            __nv_bfloat16* at = TT + ((int64_t)r * 2 * k + c) * d + e;
+            const __nv_bfloat162 value(pair_value(v0), pair_value(v1));
+            *reinterpret_cast<__nv_bfloat162*>(at) = value;
+            *reinterpret_cast<__nv_bfloat162*>(at + (int64_t)k * d) = __nv_bfloat162(pair_remainder(v0, value.x), pair_remainder(v1, value.y));
+          }
+        } else {
+          if (c < k) *reinterpret_cast<float2*>(TT + ((int64_t)r * k + c) * d + e) = make_float2(v0, v1);
+        }
         const __nv_bfloat162 hi = __floats2bfloat162_rn(v0, v1);
         const __nv_bfloat162 lo = __floats2bfloat162_rn(v0 - __low2float(hi), v1 - __high2float(hi));
         *reinterpret_cast<__nv_bfloat162*>(th + c * x_row + e * 2) = hi;
@@ -282,7 +296,7 @@ __global__ void __launch_bounds__(256) fm_request_mma_kernel(int32_t n_r, int32_
 
 struct FmParams {
   int64_t N;
-  int32_t n_r, n_c, k, num_tiles, stages;
+  int32_t n_r, k, num_tiles, stages;
   const __nv_bfloat16* P;        // [n_r + n_c, k]
   const int32_t* offsets;        // [R + 1]
   int32_t R;
@@ -291,26 +305,10 @@ struct FmParams {
   uint32_t* status;
 };
 
-// Two fp32 values as bf16 pairs that add up to them.  Rounded value and rounded remainder: 17 bits.
-__device__ __forceinline__ void split_bf16(float a, float b, uint32_t (&part)[2]) {
-  part[0] = pack_bf16(a, b);
-  part[1] = pack_bf16(a - __uint_as_float(part[0] << 16), b - __uint_as_float(part[0] & 0xffff0000u));
-}
-// Upper halves of the values, of what is left and of what is left then: every bit.  An infinity is infinite in every part.
-__device__ __forceinline__ void split_bf16(float a, float b, uint32_t (&part)[3]) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
-    part[i] = __byte_perm(ua, ub, 0x7632);
-    a = fabsf(a) == INFINITY ? a : a - __uint_as_float(ua & 0xffff0000u);
-    b = fabsf(b) == INFINITY ? b : b - __uint_as_float(ub & 0xffff0000u);
-  }
-}
-
-// T^T of a request, columns 16 kt .. and the 16 columns cp of d, in the accumulator layout of step 1.
+// T^T of a request, the 16 columns cp of d, in the accumulator layout of step 1.
 template <int D>
-__device__ __forceinline__ void load_t(const float* tt, int32_t k, int kt, int cp, int g, int tq, float (&f)[2][4]) {
-  const int c = kt * 16 + g;
+__device__ __forceinline__ void load_t(const float* tt, int32_t k, int cp, int g, int tq, float (&f)[2][4]) {
+  const int c = g;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int col = (2 * cp + h) * 8 + 2 * tq;
@@ -323,21 +321,16 @@ __device__ __forceinline__ void load_t(const float* tt, int32_t k, int kt, int c
   }
 }
 
-// KT: blocks of 16 projection columns.  With one, the request's T stays in registers while consecutive
-// candidates share it; with two it would not fit beside H and comes from L1 for every candidate.
-template <int D, int KT, bool FULL>
-__global__ void __launch_bounds__((tile_cands<D, FULL>() + 1) * 32, 1)
+template <int D>
+__global__ void __launch_bounds__((kTileCands + 1) * 32, 1)
 fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmParams p) {
   constexpr int kSlabs = D / 64;
   constexpr int kPairs = D / 16;  // pairs of 8-column groups = k-steps of step 2
   extern __shared__ __align__(1024) uint8_t smem[];
-  const int32_t n_c = FULL ? kFragRows : p.n_c;
-  constexpr int kTileCands = tile_cands<D, FULL>();
-  // 64 columns of the tile, 128-byte swizzled rows, to the 1024 bytes that the swizzle repeats in
-  const int32_t slab_bytes = (kTileCands * n_c * 128 + 1023) / 1024 * 1024;
-  const int32_t stage_bytes = kSlabs * slab_bytes;
-  // behind the stages: rows that the last candidate's fragments read past the tile
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.stages * stage_bytes + (FULL ? 0 : kFragRows * 128));
+  constexpr int32_t n_c = kFragRows;
+  constexpr int32_t slab_bytes = kTileCands * n_c * 128;  // 64 columns of the tile, 128-byte swizzled rows
+  constexpr int32_t stage_bytes = kSlabs * slab_bytes;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.stages * stage_bytes);
   uint64_t* empty = full + kMaxStages;
   AbortFlag* abort_flag = reinterpret_cast<AbortFlag*>(empty + kMaxStages);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -386,29 +379,22 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
     // ------------------------------ one candidate per warp ---------------------------------
     const int g = lane / 4, tq = lane % 4;  // fragment row group and column pair
     // P_C^T as the M x K operand of step 1: A[m = projection column][kk = candidate row]
-    uint32_t pa[KT][4];
+    uint32_t pa[4];
     {
       const __nv_bfloat16* pc = p.P + (int64_t)p.n_r * p.k;
-      auto at = [&](int row, int col) -> float {  // P_C[row][col], zero beyond n_c rows and k columns
-        return row < n_c && col < p.k ? __bfloat162float(pc[row * p.k + col]) : 0.f;
+      auto at = [&](int row, int col) -> float {  // P_C[row][col], zero beyond k columns
+        return col < p.k ? __bfloat162float(pc[row * p.k + col]) : 0.f;
       };
-#pragma unroll
-      for (int kt = 0; kt < KT; ++kt) {
-        const int c = kt * 16 + g;
-        pa[kt][0] = pack_bf16(at(2 * tq, c), at(2 * tq + 1, c));
-        pa[kt][1] = pack_bf16(at(2 * tq, c + 8), at(2 * tq + 1, c + 8));
-        pa[kt][2] = pack_bf16(at(2 * tq + 8, c), at(2 * tq + 9, c));
-        pa[kt][3] = pack_bf16(at(2 * tq + 8, c + 8), at(2 * tq + 9, c + 8));
-      }
+      pa[0] = pack_bf16(at(2 * tq, g), at(2 * tq + 1, g));
+      pa[1] = pack_bf16(at(2 * tq, g + 8), at(2 * tq + 1, g + 8));
+      pa[2] = pack_bf16(at(2 * tq + 8, g), at(2 * tq + 9, g));
+      pa[3] = pack_bf16(at(2 * tq + 8, g + 8), at(2 * tq + 9, g + 8));
     }
-    // rows of the K x N operand of step 1 that are this candidate's: 2 tq, 2 tq + 1 and the two 8 further on
-    auto row_mask = [&](int row) { return (row < n_c ? 0xffffu : 0u) | (row + 1 < n_c ? 0xffff0000u : 0u); };
-    const uint32_t keep_lo = row_mask(2 * tq), keep_hi = row_mask(2 * tq + 8);
     // this lane's address pattern inside a candidate's 16 rows: row, and which of the two
     // 8-column groups of a pair
     const int trow = warp * n_c + (lane % 8) + ((lane / 8) % 2) * 8;
     const int lsel = lane / 16;
-    float tfrag[KT == 1 ? kPairs : 1][2][4];  // T^T of the cached request in step-1 accumulator layout
+    float tfrag[kPairs][2][4];  // T^T of the cached request in step-1 accumulator layout
     int32_t cached_req = -1;
     int s = 0;
     uint32_t phase = 0;
@@ -431,96 +417,44 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
         if (r != cached_req) {
           if (cached_req < 0) griddep_wait();  // TT comes from the request kernel launched just before
           cached_req = r;
-          if constexpr (KT == 1) {
 #pragma unroll
-            for (int cp = 0; cp < kPairs; ++cp) load_t<D>(tt, p.k, 0, cp, g, tq, tfrag[cp]);
-          }
+          for (int cp = 0; cp < kPairs; ++cp) load_t<D>(tt, p.k, cp, g, tq, tfrag[cp]);
         }
         const uint32_t tile = smem_u32(smem + s * stage_bytes) + trow * 128;
         __nv_bfloat16* fc = p.FC + cand * n_c * p.k;
+        // step 1: H^T (16 x D) = T^T + P_C^T X^C, whose accumulator is the K x N operand of step 2 as it stands
+        uint32_t hb[kPairs][2][2];  // [k-step][projection columns 0-7 | 8-15][b0, b1]
 #pragma unroll
-        for (int kt = 0; kt < KT; ++kt) {
-          // step 1: H^T (16 x D) = T^T + P_C^T X^C, whose accumulator is the K x N operand of step 2 as it stands
-          auto step1 = [&](int cp, float (&f)[2][4]) {
-            const int chunk = 2 * cp + lsel;  // 16-byte chunk along d
-            uint32_t xb[4];
-            ldmatrix_x4_trans(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xb);
-            if constexpr (!FULL) {
-              xb[0] &= keep_lo;
-              xb[1] &= keep_hi;
-              xb[2] &= keep_lo;
-              xb[3] &= keep_hi;
-            }
-            if constexpr (KT == 1) {
+        for (int cp = 0; cp < kPairs; ++cp) {
+          const int chunk = 2 * cp + lsel;  // 16-byte chunk along d
+          uint32_t xb[4];
+          ldmatrix_x4_trans(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xb);
+          float f[2][4];
 #pragma unroll
-              for (int e = 0; e < 8; ++e) f[e / 4][e % 4] = tfrag[cp][e / 4][e % 4];
-            } else {
-              load_t<D>(tt, p.k, kt, cp, g, tq, f);
-            }
-            mma_bf16(f[0], pa[kt], xb[0], xb[1]);
-            mma_bf16(f[1], pa[kt], xb[2], xb[3]);
-          };
-          // step 2: FC (16 x 16) = X^C H
-          float out[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-          auto rows_of = [&](int cp, uint32_t (&xa)[4]) {
-            const int chunk = 2 * cp + lsel;
-            ldmatrix_x4(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xa);
-          };
-          if constexpr (FULL) {
-            uint32_t hb[kPairs][2][2];  // [k-step][projection columns 0-7 | 8-15][b0, b1]
+          for (int e = 0; e < 8; ++e) f[e / 4][e % 4] = tfrag[cp][e / 4][e % 4];
+          mma_bf16(f[0], pa, xb[0], xb[1]);
+          mma_bf16(f[1], pa, xb[2], xb[3]);
+          hb[cp][0][0] = pack_bf16(f[0][0], f[0][1]);
+          hb[cp][0][1] = pack_bf16(f[1][0], f[1][1]);
+          hb[cp][1][0] = pack_bf16(f[0][2], f[0][3]);
+          hb[cp][1][1] = pack_bf16(f[1][2], f[1][3]);
+        }
+        // step 2: FC (16 x 16) = X^C H
+        float out[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
-            for (int cp = 0; cp < kPairs; ++cp) {
-              float f[2][4];
-              step1(cp, f);
-              hb[cp][0][0] = pack_bf16(f[0][0], f[0][1]);
-              hb[cp][0][1] = pack_bf16(f[1][0], f[1][1]);
-              hb[cp][1][0] = pack_bf16(f[0][2], f[0][3]);
-              hb[cp][1][1] = pack_bf16(f[1][2], f[1][3]);
-            }
+        for (int cp = 0; cp < kPairs; ++cp) {
+          const int chunk = 2 * cp + lsel;
+          uint32_t xa[4];
+          ldmatrix_x4(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xa);
+          mma_bf16(out[0], xa, hb[cp][0][0], hb[cp][0][1]);
+          mma_bf16(out[1], xa, hb[cp][1][0], hb[cp][1][1]);
+        }
 #pragma unroll
-            for (int cp = 0; cp < kPairs; ++cp) {
-              uint32_t xa[4];
-              rows_of(cp, xa);
-              mma_bf16(out[0], xa, hb[cp][0][0], hb[cp][0][1]);
-              mma_bf16(out[1], xa, hb[cp][1][0], hb[cp][1][1]);
-            }
-          } else {
-            auto product = [&](auto parts) {
-              constexpr int kParts = decltype(parts)::value;
-#pragma unroll
-              for (int cp = 0; cp < kPairs; ++cp) {
-                float f[2][4];
-                uint32_t xa[4];
-                step1(cp, f);
-                rows_of(cp, xa);
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                  uint32_t b0[kParts], b1[kParts];
-                  split_bf16(f[0][2 * h], f[0][2 * h + 1], b0);
-                  split_bf16(f[1][2 * h], f[1][2 * h + 1], b1);
-#pragma unroll
-                  for (int i = 0; i < kParts; ++i) mma_bf16(out[h], xa, b0[i], b1[i]);
-                }
-              }
-            };
-            product(std::integral_constant<int, 2>());
-            bool nan = false;  // in this candidate's rows: what the next one's hold must not decide
-#pragma unroll
-            for (int e = 0; e < 8; ++e) nan = nan || (g + 8 * (e / 2 % 2) < n_c && isnan(out[e / 4][e % 4]));
-            if (__any_sync(0xffffffffu, nan)) {  // perhaps of an infinity, or of a value that rounds to one
-#pragma unroll
-              for (int e = 0; e < 8; ++e) out[e / 4][e % 4] = 0.f;
-              product(std::integral_constant<int, 3>());
-            }
-          }
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int col = kt * 16 + 8 * h + 2 * tq;
-            if (col < p.k) {
-              if (FULL || g < n_c) *reinterpret_cast<uint32_t*>(fc + g * p.k + col) = pack_bf16(out[h][0], out[h][1]);
-              if (FULL || g + 8 < n_c)
-                *reinterpret_cast<uint32_t*>(fc + (g + 8) * p.k + col) = pack_bf16(out[h][2], out[h][3]);
-            }
+        for (int h = 0; h < 2; ++h) {
+          const int col = 8 * h + 2 * tq;
+          if (col < p.k) {
+            *reinterpret_cast<uint32_t*>(fc + g * p.k + col) = pack_bf16(out[h][0], out[h][1]);
+            *reinterpret_cast<uint32_t*>(fc + (g + 8) * p.k + col) = pack_bf16(out[h][2], out[h][3]);
           }
         }
       }
@@ -528,276 +462,6 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
       if (lane == 0) mbar_arrive(&empty[s]);
       if (++s == p.stages) { s = 0; phase ^= 1; }
     }
-  }
-}
-
-// Columns 16 kt .. of one candidate whose first row the lane's `tile` and `trow` point at, the way of the kernel above with H
-// in three bf16 parts, every bit of it: for values that the pairs cannot hold (an infinity, what rounds to one, a Gram matrix
-// past fp32), where the result has to be what fp32 arithmetic gives.
-template <int D>
-__device__ __forceinline__ void fm_candidate_by_parts(uint32_t tile, int trow, int32_t slab_bytes, const FmParams& p, const float* tt,
-                                                   int64_t cand, int kt) {
-  const int lane = threadIdx.x % 32, g = lane / 4, tq = lane % 4, lsel = lane / 16;
-  const __nv_bfloat16* pc = p.P + (int64_t)p.n_r * p.k;
-  auto at = [&](int row, int col) -> float {  // P_C[row][col], zero beyond n_c rows and k columns
-    return row < p.n_c && col < p.k ? __bfloat162float(pc[row * p.k + col]) : 0.f;
-  };
-  const int c = kt * 16 + g;
-  const uint32_t pa[4] = {pack_bf16(at(2 * tq, c), at(2 * tq + 1, c)), pack_bf16(at(2 * tq, c + 8), at(2 * tq + 1, c + 8)),
-                          pack_bf16(at(2 * tq + 8, c), at(2 * tq + 9, c)), pack_bf16(at(2 * tq + 8, c + 8), at(2 * tq + 9, c + 8))};
-  // rows of the K x N operand of step 1 that are this candidate's: 2 tq, 2 tq + 1 and the two 8 further on
-  auto row_mask = [&](int row) { return (row < p.n_c ? 0xffffu : 0u) | (row + 1 < p.n_c ? 0xffff0000u : 0u); };
-  const uint32_t keep_lo = row_mask(2 * tq), keep_hi = row_mask(2 * tq + 8);
-  float out[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll 1
-  for (int cp = 0; cp < D / 16; ++cp) {
-    const int chunk = 2 * cp + lsel;
-    const uint32_t from = tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4);
-    uint32_t xb[4], xa[4];
-    ldmatrix_x4_trans(from, xb);
-    ldmatrix_x4(from, xa);
-    float f[2][4];
-    load_t<D>(tt, p.k, kt, cp, g, tq, f);
-    mma_bf16(f[0], pa, xb[0] & keep_lo, xb[1] & keep_hi);
-    mma_bf16(f[1], pa, xb[2] & keep_lo, xb[3] & keep_hi);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      uint32_t b0[3], b1[3];
-      split_bf16(f[0][2 * h], f[0][2 * h + 1], b0);
-      split_bf16(f[1][2 * h], f[1][2 * h + 1], b1);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) mma_bf16(out[h], xa, b0[i], b1[i]);
-    }
-  }
-  __nv_bfloat16* fc = p.FC + cand * p.n_c * p.k;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int col = kt * 16 + 8 * h + 2 * tq;
-    if (col < p.k) {
-      if (g < p.n_c) *reinterpret_cast<uint32_t*>(fc + g * p.k + col) = pack_bf16(out[h][0], out[h][1]);
-      if (g + 8 < p.n_c) *reinterpret_cast<uint32_t*>(fc + (g + 8) * p.k + col) = pack_bf16(out[h][2], out[h][3]);
-    }
-  }
-}
-
-// n_c up to 8, even k up to 32: FC = X^C T + (X^C X^C^T) P_C on fragments of 16 rows, 16 / n_c candidates each.  Per
-// 16 columns of d six products (T as a pair 2 x 2, the Gram matrix 2) on one ldmatrix: the rows' fragment as the M x K operand
-// is also the K x N operand of the Gram matrix.  Entries of two different candidates are set to zero and the rest goes, as a
-// pair, by P_C repeated per candidate; no precision is lost against the kernel above.  Fragments that reach into another
-// request are computed once per request.  A candidate per warp there, several here: 20423 candidates of 4 embeddings x 128,
-// k = 16: 25.7 and 14.8 us; 50848 of 4 x 64, k = 8: 31.0 and 15.6 us.  With one candidate per fragment (12 embeddings) four
-// more products make it the slower way: 26.4 and 28.1 us.  KT: as above, T of two blocks comes from L1 for every fragment.
-template <int D, int KT>
-__global__ void __launch_bounds__((tile_cands<D, false>() + 1) * 32, 1)
-fm_candidate_gram_kernel(const __grid_constant__ CUtensorMap map_xc, const FmParams p) {
-  constexpr int kSlabs = D / 64;
-  constexpr int kSteps = D / 16;
-  constexpr int kWarps = tile_cands<D, false>();
-  extern __shared__ __align__(1024) uint8_t smem[];
-  const int32_t n_c = p.n_c, per_frag = kFragRows / n_c, frag_rows = per_frag * n_c;
-  const int32_t tile_rows = kWarps * frag_rows, tile_cands = kWarps * per_frag;
-  // 64 columns of the tile, 128-byte swizzled rows, to the 1024 bytes that the swizzle repeats in
-  const int32_t slab_bytes = (tile_rows * 128 + 1023) / 1024 * 1024;
-  const int32_t stage_bytes = kSlabs * slab_bytes;
-  // behind the stages: rows that the last warp's fragments read past the tile
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.stages * stage_bytes + kFragRows * 128);
-  uint64_t* empty = full + kMaxStages;
-  AbortFlag* abort_flag = reinterpret_cast<AbortFlag*>(empty + kMaxStages);
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  if ((smem_u32(smem) & 1023u) != 0) {  // the swizzled tiles assume a 1024-byte aligned base
-    if (threadIdx.x == 0) atomicCAS(p.status, 0u, kStatusFm | 15);
-    return;
-  }
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < p.stages; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], kWarps);
-    }
-    abort_flag->v = 0;
-    fence_mbar_init();
-  }
-  __syncthreads();
-  const int32_t tiles_per_cta = (p.num_tiles + (int32_t)gridDim.x - 1) / (int32_t)gridDim.x;
-  const int32_t tile_begin = min((int32_t)blockIdx.x * tiles_per_cta, p.num_tiles);
-  const int32_t tile_end = min(tile_begin + tiles_per_cta, p.num_tiles);
-
-  if (warp == kWarps) {
-    // ------------------------------ TMA producer ------------------------------------------
-    if (elect_one()) {
-      prefetch_tensormap(&map_xc);
-      int s = 0;
-      uint32_t phase = 0, it = 0;
-      for (int32_t t = tile_begin; t < tile_end; ++t, ++it) {
-        if (!mbar_wait(&empty[s], phase ^ 1, abort_flag, p.status, kStatusFm | 1)) break;
-        mbar_expect_tx(&full[s], kSlabs * tile_rows * 128);
-#pragma unroll
-        for (int sl = 0; sl < kSlabs; ++sl)
-          tma_load_2d(smem + s * stage_bytes + sl * slab_bytes, &map_xc, &full[s], sl * 64, t * tile_rows);
-        if (++s == p.stages) { s = 0; phase ^= 1; }
-      }
-      // loads in flight land in this CTA's shared memory: wait for them before the CTA may exit
-      for (int st = 0; st < p.stages; ++st) {
-        const uint32_t n_issued = it / p.stages + (((int)(it % p.stages) > st) ? 1 : 0);
-        if (n_issued == 0) continue;
-        const uint64_t t0 = globaltimer_ns();
-        while (!mbar_try_wait(&full[st], (n_issued - 1) & 1) && globaltimer_ns() - t0 < kWaitLimitNs) {}
-      }
-    }
-    return;
-  }
-  const int g = lane / 4, tq = lane % 4;  // fragment row group and column pair
-  const int own[2] = {g / n_c, (g + 8) / n_c};  // candidates of the fragment that the lane's rows g and g + 8 are of
-  uint32_t same = 0;  // entries of the Gram matrix whose two rows are of one candidate, in accumulator layout
-#pragma unroll
-  for (int t = 0; t < 2; ++t)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int col = t * 8 + 2 * tq + e % 2;
-      if (own[e / 2] == col / n_c && col < frag_rows) same |= 1u << (t * 4 + e);
-    }
-  uint32_t pb[KT][2][2];  // P_C, repeated per candidate, as the K x N operand
-  {
-    const __nv_bfloat16* pc = p.P + (int64_t)p.n_r * p.k;
-    auto at = [&](int row, int col) -> float { return row < frag_rows && col < p.k ? __bfloat162float(pc[row % n_c * p.k + col]) : 0.f; };
-#pragma unroll
-    for (int kt = 0; kt < KT; ++kt)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int c = kt * 16 + h * 8 + g;
-        pb[kt][h][0] = pack_bf16(at(2 * tq, c), at(2 * tq + 1, c));
-        pb[kt][h][1] = pack_bf16(at(2 * tq + 8, c), at(2 * tq + 9, c));
-      }
-  }
-  const int row0 = warp * frag_rows, in_frag = (lane % 8) + ((lane / 8) % 2) * 8, trow = row0 + in_frag, lsel = lane / 16;
-  // T as the K x N operand, as a pair: [part][b0, b1] of step s and columns 8 h of block kt
-  auto load_pair = [&](const float* tt, int kt, int h, int s, uint32_t (&b0)[2], uint32_t (&b1)[2]) {
-    const int c = kt * 16 + h * 8 + g;
-    float2 lo = make_float2(0.f, 0.f), hi = lo;
-    if (c < p.k) {
-      lo = *reinterpret_cast<const float2*>(tt + c * D + s * 16 + 2 * tq);
-      hi = *reinterpret_cast<const float2*>(tt + c * D + s * 16 + 8 + 2 * tq);
-    }
-    split_bf16(lo.x, lo.y, b0);
-    split_bf16(hi.x, hi.y, b1);
-  };
-  uint32_t tb[KT == 1 ? kSteps : 1][2][2][2];  // [step][h][b0 | b1][part]
-  int32_t cached_req = -1;
-  int s = 0;
-  uint32_t phase = 0;
-  // the request of this warp's first candidate, and its end, found one tile ahead of their use
-  int32_t r_next = 0, end_next = 0;
-  RequestWalk walk{p.offsets, p.R};
-  auto find = [&](int32_t t) {
-    const int64_t c = (int64_t)t * tile_cands + warp * per_frag;
-    if (t < tile_end && c < p.N) {
-      r_next = walk.of(c);
-      end_next = walk.end;
-    }
-  };
-  find(tile_begin);
-  for (int32_t t = tile_begin; t < tile_end; ++t) {
-    int32_t r = r_next, end = end_next;
-    find(t + 1);
-    if (!mbar_wait(&full[s], phase, abort_flag, p.status, kStatusFm | 2)) break;
-    const int64_t cand = (int64_t)t * tile_cands + warp * per_frag;
-    const int32_t valid = (int32_t)max((int64_t)0, min((int64_t)per_frag, p.N - cand));
-    const uint32_t stage = smem_u32(smem + s * stage_bytes), tile = stage + trow * 128;
-    for (int32_t lo = 0; lo < valid;) {
-      const int32_t hi = min(valid, (int32_t)(end - cand));  // candidates lo .. hi of the fragment are of request r
-      const float* tt = p.TT + (int64_t)r * p.k * D;
-      if (r != cached_req) {
-        if (cached_req < 0) griddep_wait();  // TT comes from the request kernel launched just before
-        cached_req = r;
-        if constexpr (KT == 1) {
-#pragma unroll
-          for (int st = 0; st < kSteps; ++st)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) load_pair(tt, 0, h, st, tb[st][h][0], tb[st][h][1]);
-        }
-      }
-      float out[KT][2][4], low[KT][2][4], gram[2][4];  // (two chains: of the rounded values and of the remainders)
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          gram[h][e] = 0.f;
-#pragma unroll
-          for (int kt = 0; kt < KT; ++kt) out[kt][h][e] = low[kt][h][e] = 0.f;
-        }
-#pragma unroll
-      for (int st = 0; st < kSteps; ++st) {
-        const int chunk = 2 * st + lsel;  // 16-byte chunk along d
-        uint32_t xa[4];
-        ldmatrix_x4(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xa);
-        mma_bf16(gram[0], xa, xa[0], xa[2]);
-        mma_bf16(gram[1], xa, xa[1], xa[3]);
-#pragma unroll
-        for (int kt = 0; kt < KT; ++kt)
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            if constexpr (KT == 1) {
-              mma_bf16(out[kt][h], xa, tb[st][h][0][0], tb[st][h][1][0]);
-              mma_bf16(low[kt][h], xa, tb[st][h][0][1], tb[st][h][1][1]);
-            } else {
-              uint32_t b0[2], b1[2];
-              load_pair(tt, kt, h, st, b0, b1);
-              mma_bf16(out[kt][h], xa, b0[0], b1[0]);
-              mma_bf16(low[kt][h], xa, b0[1], b1[1]);
-            }
-          }
-      }
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        if ((same >> e & 1u) == 0) gram[e / 4][e % 4] = 0.f;
-      // the accumulator layout of two 8-wide tiles is that of a 16 x 16 M x K operand
-      uint32_t part[4][2];
-#pragma unroll
-      for (int x = 0; x < 4; ++x) split_bf16(gram[x / 2][x % 2 * 2], gram[x / 2][x % 2 * 2 + 1], part[x]);
-      const uint32_t ga[4] = {part[0][0], part[1][0], part[2][0], part[3][0]};
-      const uint32_t gb[4] = {part[0][1], part[1][1], part[2][1], part[3][1]};
-      uint32_t bad = 0;  // candidates with a NaN in a row of theirs
-#pragma unroll
-      for (int kt = 0; kt < KT; ++kt)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          mma_bf16(out[kt][h], ga, pb[kt][h][0], pb[kt][h][1]);
-          mma_bf16(low[kt][h], gb, pb[kt][h][0], pb[kt][h][1]);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            out[kt][h][e] += low[kt][h][e];
-            if (isnan(out[kt][h][e])) bad |= 1u << own[e / 2];
-          }
-        }
-      if (__any_sync(0xffffffffu, bad != 0)) {  // perhaps of an infinity, or of a value that rounds to one
-        bad = __reduce_or_sync(0xffffffffu, bad);
-        for (int32_t c = lo; c < hi; ++c)
-          if (bad >> c & 1u) {
-            const int row = row0 + c * n_c + in_frag;
-#pragma unroll 1
-            for (int kt = 0; kt < KT; ++kt) fm_candidate_by_parts<D>(stage + row * 128, row, slab_bytes, p, tt, cand + c, kt);
-          }
-      }
-      __nv_bfloat16* fc = p.FC + cand * n_c * p.k;
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        if (own[j] < lo || own[j] >= hi || (bad >> own[j] & 1u)) continue;
-#pragma unroll
-        for (int kt = 0; kt < KT; ++kt)
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int col = kt * 16 + 8 * h + 2 * tq;
-            if (col < p.k) *reinterpret_cast<uint32_t*>(fc + (g + 8 * j) * p.k + col) = pack_bf16(out[kt][h][2 * j], out[kt][h][2 * j + 1]);
-          }
-      }
-      lo = hi;
-      if (lo < valid) {  // on to the next request that has candidates
-        do { ++r; } while (p.offsets[r + 1] <= cand + lo);
-        end = p.offsets[r + 1];
-      }
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&empty[s]);
-    if (++s == p.stages) { s = 0; phase ^= 1; }
   }
 }
 
@@ -811,43 +475,36 @@ int sm_count_fm() {
   return n;
 }
 
-enum class FmKernel { kFull, kPair, kGram };
-template <int D, int KT, FmKernel WHICH>
-rocs_status_t launch_fm_mma_as(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t k,
-                               const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
-  constexpr int kWarps = tile_cands<D, WHICH == FmKernel::kFull>();
-  const int32_t tile_cands = WHICH == FmKernel::kGram ? kWarps * (kFragRows / n_c) : kWarps, tile_rows = tile_cands * n_c;
-  const int stage_bytes = D / 64 * ((tile_rows * 128 + 1023) / 1024 * 1024);
-  constexpr int kFixed = kFragRows * 128 + 2 * kMaxStages * 8 + 16;
+template <int D>
+rocs_status_t launch_fm_mma(const rocs_plan* plan, int32_t n_r, int32_t k, const void* XC, const void* P, const float* TT,
+                            void* FC, cudaStream_t stream) {
+  constexpr int kStageBytes = kTileCands * kFragRows * D * 2, kFixed = 2 * kMaxStages * 8 + 16;
   CUtensorMap map_xc;
-  if (!make_tensor_map_2d(&map_xc, XC, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)plan->N * n_c, D, D,
-                          (uint32_t)tile_rows, 64, true))
+  if (!make_tensor_map_2d(&map_xc, XC, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)plan->N * kFragRows, D, D,
+                          kTileCands * kFragRows, 64, true))
     return ROCS_ERR_CUDA;
   uint32_t* status = device_status_word();
   if (!status) return ROCS_ERR_CUDA;
   FmParams p{};
   p.N = plan->N;
   p.n_r = n_r;
-  p.n_c = n_c;
   p.k = k;
-  p.num_tiles = (int32_t)((plan->N + tile_cands - 1) / tile_cands);
-  p.stages = std::min(kMaxStages, (227 * 1024 - kFixed) / stage_bytes);
+  p.num_tiles = (int32_t)((plan->N + kTileCands - 1) / kTileCands);
+  p.stages = std::min(kMaxStages, (227 * 1024 - kFixed) / kStageBytes);
   p.P = (const __nv_bfloat16*)P;
   p.offsets = plan->cand_offsets;
   p.R = plan->R;
   p.TT = TT;
   p.FC = (__nv_bfloat16*)FC;
   p.status = status;
-  const int smem = p.stages * stage_bytes + kFixed;
-  void (*kern)(CUtensorMap, FmParams);
-  if constexpr (WHICH == FmKernel::kGram) kern = fm_candidate_gram_kernel<D, KT>;
-  else kern = fm_candidate_mma_kernel<D, KT, WHICH == FmKernel::kFull>;
+  const int smem = p.stages * kStageBytes + kFixed;
+  auto kern = fm_candidate_mma_kernel<D>;
   ROCS_ALLOW_SMEM(kern, kMaxDynamicSmem);
   // Launched so that it may overlap the request kernel in front of it on the stream (that kernel
   // releases its dependents at once); nothing else this kernel reads is written by that launch.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)std::min(p.num_tiles, sm_count_fm()));
-  cfg.blockDim = dim3((kWarps + 1) * 32);
+  cfg.blockDim = dim3((kTileCands + 1) * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -857,16 +514,6 @@ rocs_status_t launch_fm_mma_as(const rocs_plan* plan, int32_t n_r, int32_t n_c, 
   cfg.numAttrs = 1;
   ROCS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, map_xc, p));
   return ROCS_OK;
-}
-
-template <int D>
-rocs_status_t launch_fm_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t k,
-                            const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
-#define ROCS_LAUNCH(KT_, WHICH_) launch_fm_mma_as<D, KT_, FmKernel::WHICH_>(plan, n_r, n_c, k, XC, P, TT, FC, stream)
-  if (n_c <= kFragRows / 2) return k > 16 ? ROCS_LAUNCH(2, kGram) : ROCS_LAUNCH(1, kGram);
-  if (k > 16) return ROCS_LAUNCH(2, kPair);
-  return n_c == kFragRows && (k == 8 || k == 16) ? ROCS_LAUNCH(1, kFull) : ROCS_LAUNCH(1, kPair);
-#undef ROCS_LAUNCH
 }
 
 template <typename T>
@@ -879,24 +526,31 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
   if (smem_r > kMaxSmem || smem_c > kMaxSmem) return ROCS_ERR_UNSUPPORTED;
   const size_t n_rp = (size_t)(n_r + 15) / 16 * 16, kp = (size_t)(k + 15) / 16 * 16;
   const size_t smem_mma = n_rp * ((size_t)(d + 8) * 2 + (kp + 8) * 2) + 2 * kp * (size_t)(d + 8) * 2;
-  if (plan->R > 0 && tensor_core_request && sizeof(T) == 2 && d % 16 == 0 && k % 8 == 0 && smem_mma <= kMaxSmem) {
-    ROCS_ALLOW_SMEM(fm_request_mma_kernel, kMaxSmem);
-    const rocs_status_t st = launch_dependent(fm_request_mma_kernel, dim3((unsigned)plan->R), 256, smem_mma, stream, n_r, d, k,
-                                              (const __nv_bfloat16*)XR, (const __nv_bfloat16*)P, TT, (__nv_bfloat16*)FR);
-    if (st != ROCS_OK) return st;
-  } else if (plan->R > 0) {
-    ROCS_ALLOW_SMEM(fm_request_kernel<T>, kMaxSmem);
-    const rocs_status_t st = launch_dependent(fm_request_kernel<T>, dim3((unsigned)plan->R), 256, smem_r, stream, n_r, d, k,
-                                              (const T*)XR, (const T*)P, TT, (T*)FR);
+  const bool pair = fast_candidates && FC != nullptr && !(n_c == kFragRows && (k == 8 || k == 16));  // fm_umma.cu reads TT
+  if (plan->R > 0) {
+    const bool mma = tensor_core_request && sizeof(T) == 2 && d % 16 == 0 && k % 8 == 0 && smem_mma <= kMaxSmem;
+    auto run = [&](auto with_pair) {
+      constexpr bool kPair = decltype(with_pair)::value;
+      if (mma) {
+        ROCS_ALLOW_SMEM(fm_request_mma_kernel<kPair>, kMaxSmem);
+        return launch_dependent(fm_request_mma_kernel<kPair>, dim3((unsigned)plan->R), 256, smem_mma, stream, n_r, d, k,
+                                (const __nv_bfloat16*)XR, (const __nv_bfloat16*)P, (TermOf<kPair>*)TT, (__nv_bfloat16*)FR);
+      }
+      ROCS_ALLOW_SMEM((fm_request_kernel<T, kPair>), kMaxSmem);
+      return launch_dependent(fm_request_kernel<T, kPair>, dim3((unsigned)plan->R), 256, smem_r, stream, n_r, d, k,
+                              (const T*)XR, (const T*)P, (TermOf<kPair>*)TT, (T*)FR);
+    };
+    const rocs_status_t st = pair ? run(std::true_type()) : run(std::false_type());
     if (st != ROCS_OK) return st;
   }
   if (plan->N == 0 || !FC) return ROCS_OK;
+  if (pair) return fm_umma(plan, n_r, n_c, d, k, XC, P, TT, FC, stream);
   if (fast_candidates) {
     switch (d) {
-      case 64: return launch_fm_mma<64>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
-      case 128: return launch_fm_mma<128>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
-      case 192: return launch_fm_mma<192>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
-      case 256: return launch_fm_mma<256>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 64: return launch_fm_mma<64>(plan, n_r, k, XC, P, TT, FC, stream);
+      case 128: return launch_fm_mma<128>(plan, n_r, k, XC, P, TT, FC, stream);
+      case 192: return launch_fm_mma<192>(plan, n_r, k, XC, P, TT, FC, stream);
+      case 256: return launch_fm_mma<256>(plan, n_r, k, XC, P, TT, FC, stream);
       default: break;
     }
   }

@@ -219,6 +219,40 @@ struct TileWalk {
     const int32_t c = first + local * per;
     next = Tile{r, c, min(per, end - c), 0};
   }
+  // The same by all THREADS threads of a block, each with its share of the requests; scratch: THREADS / 32 + 2 words.
+  template <int THREADS>
+  __device__ __forceinline__ void start_in_block(int32_t t, int32_t* scratch) {
+    int32_t *found = scratch, *warp_sum = scratch + 2;
+    const int32_t chunk = (R + THREADS - 1) / THREADS, r0 = min((int32_t)threadIdx.x * chunk, R), r1 = min(r0 + chunk, R);
+    const int32_t lane = threadIdx.x % 32, w = threadIdx.x / 32;
+    int32_t sum = 0;
+#pragma unroll 4
+    for (int32_t r = r0; r < r1; ++r) sum += tiles_of(offsets[r + 1] - offsets[r], per);
+    int32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += up;
+    }
+    if (lane == 31) warp_sum[w] = incl;
+    __syncthreads();
+    int32_t local = t - (incl - sum);
+    for (int x = 0; x < w; ++x) local -= warp_sum[x];
+    if (0 <= local && local < sum) {
+      int32_t r = r0, n;
+      while (local >= (n = tiles_of(offsets[r + 1] - offsets[r], per))) {
+        local -= n;
+        ++r;
+      }
+      found[0] = r;
+      found[1] = offsets[r] + local * per;
+    }
+    __syncthreads();
+    next = Tile{found[0], found[1], 0, 0};
+    end = offsets[next.req + 1];
+    next_end = offsets[min(next.req + 2, R)];
+    next.count = min(per, end - next.cand0);
+  }
   // The tile at hand; moves on to the next one if there is `more`.
   __device__ __forceinline__ Tile take(bool more) {
     const Tile t = next;
@@ -288,6 +322,9 @@ rocs_status_t group_norm(rocs_dtype_t dt, int kind, int64_t M, int32_t d, const 
 // F = G P on the request-once form; tt_workspace [R, k, d] fp32 receives P_R^T X^R per request.
 // allow_fast: use the bf16 streaming kernel for the candidate side where the shape allows it.
 bool fm_projection_fast_supported(int32_t n_c, int32_t d, int32_t k);
+// Candidate rows on tcgen05 (fm_umma.cu), for the shapes above; TT as bf16 pairs [R, 2, k, d].
+rocs_status_t fm_umma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, int32_t k, const void* XC, const void* P,
+                      const void* TT, void* FC, cudaStream_t stream);
 rocs_status_t fm_projection(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, int32_t k,
                             const void* XR, const void* XC, const void* P, void* FR, void* FC, float* tt_workspace,
                             bool allow_fast, cudaStream_t stream);

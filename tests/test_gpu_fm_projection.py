@@ -102,6 +102,21 @@ def test_bf16_partial_fragments_are_as_exact_as_fp32_arithmetic(n_c, k, d_emb):
     assert np.array_equal(kinds[0], kinds[1]) and np.any(kinds[1][60] != 0)
 
 
+@pytest.mark.parametrize("law", ["few", "many", "sparse"])
+@pytest.mark.parametrize("n_r,n_c,d_emb,k", [(20, 12, 128, 16), (5, 3, 64, 2), (24, 4, 192, 24), (16, 5, 64, 14), (48, 8, 256, 32), (7, 9, 128, 22),
+                                             (20, 16, 64, 24), (33, 15, 192, 8), (16, 1, 128, 16)])
+def test_bf16_tiles_of_one_request(n_r, n_c, d_emb, k, law):
+    # tiles of 8 to 32 candidates of one request, rows behind a candidate's embeddings and columns behind k; fewer tiles than a
+    # ring has stages and runs that take ring and accumulators several times; more requests than threads, most of them empty
+    g = np.random.default_rng(k)
+    counts = {"few": [3, 0, 33, 1], "many": g.integers(0, 130, 300), "sparse": np.where(g.random(3000) < 0.2, g.integers(1, 40, 3000), 0)}[law]
+    co = wl.offsets_from_counts(np.asarray(counts).tolist())
+    cfg = wl.CONFIGS[4].with_(R=len(co) - 1, n_r=n_r, n_c=n_c, d_emb=d_emb)
+    N = int(co[-1])
+    sample = np.unique(np.concatenate([g.integers(0, N, 400), [0, N - 1]]))
+    assert _run(cfg, co, k, sample=sample) <= tol_for("bf16")
+
+
 @pytest.mark.parametrize("path", PATHS)
 def test_bf16_shapes_outside_the_streaming_kernel(path):
     co = wl.offsets_from_counts([20, 3, 41])
