@@ -132,6 +132,7 @@ struct DcaParams {
   int32_t R;
   int32_t n_q, H;
   float scale_log2e;  // scale * log2(e)
+  float per_key;      // 1 / average keys of a request where items go by length, otherwise 0
   const int32_t* seq_offsets;
   const __nv_bfloat16 *Q, *K, *V;  // plain pointers for rows that are computed by hand
   __nv_bfloat16* O;
@@ -204,16 +205,59 @@ __device__ __forceinline__ void row_by_hand(const __nv_bfloat16* q, const __nv_b
   }
 }
 
-// The item of index i in the order request, head, tile, found by one warp from the offsets, with its request's keys: their
+// Classes of requests by their number of keys, most keys first, an eighth of the average apart: the order of the items where
+// they are a few rounds of the chip, so that the last to be claimed are short ones.  Lane c of a warp has the index of class
+// c's first item and the number of its items.
+constexpr int kLengthClasses = 8;
+__device__ __forceinline__ int length_class(int32_t L, float per_key) {
+  return min(max((int)((1.5f - (float)L * per_key) * 8.f), 0), kLengthClasses - 1);
+}
+struct ClassItems {
+  int32_t first, count;
+};
+__device__ __forceinline__ ClassItems count_classes(const int32_t* __restrict__ off, const int32_t* __restrict__ seq, int32_t R,
+                                                    int32_t per, int32_t heads, float per_key, int lane) {
+  int32_t count = 0;
+  for (int32_t r0 = 0; r0 < R; r0 += 32) {
+    const int32_t r = r0 + lane;
+    const int32_t entries = r < R ? tiles_of(off[r + 1] - off[r], per) * heads : 0;
+    const int c = r < R ? length_class(seq[r + 1] - seq[r], per_key) : 0;
+#pragma unroll
+    for (int x = 0; x < kLengthClasses; ++x) {
+      const int32_t sum = __reduce_add_sync(0xffffffffu, c == x ? entries : 0);
+      if (lane == x) count += sum;
+    }
+  }
+  int32_t incl = count;
+#pragma unroll
+  for (int o = 1; o < kLengthClasses; o <<= 1) {
+    const int32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += up;
+  }
+  return ClassItems{incl - count, lane < kLengthClasses ? count : 0};
+}
+
+// The item of index i in the order class, request, head, tile, found by one warp from the offsets, with its request's keys: their
 // offsets are loaded with the candidates' and not behind them, a second trip to memory in front of the item's first loads.
+template <bool BY_LENGTH>
 __device__ __forceinline__ DcaItem find_item(const int32_t* __restrict__ off, const int32_t* __restrict__ seq, int32_t R, int32_t per,
-                                             int32_t heads, int32_t i, int lane, int32_t& s0, int32_t& L) {
+                                             int32_t heads, float per_key, const ClassItems& classes, int32_t i, int lane,
+                                             int32_t& s0, int32_t& L) {
   int32_t base = 0;
+  int cls = 0;
+  const bool by_length = BY_LENGTH && per_key != 0.f;
+  if (by_length) {
+    const uint32_t in_class = __ballot_sync(0xffffffffu, classes.first <= i && i - classes.first < classes.count);
+    if (in_class == 0) return DcaItem{-1, 0, 0, 0};
+    cls = __ffs(in_class) - 1;
+    base = __shfl_sync(0xffffffffu, classes.first, cls);
+  }
   for (int32_t r0 = 0; r0 < R; r0 += 32) {
     const int32_t r = r0 + lane;
     const int32_t c0 = r < R ? off[r] : 0, n = r < R ? off[r + 1] - c0 : 0;
     const int32_t k0 = r < R ? seq[r] : 0, k1 = r < R ? seq[r + 1] : 0;
-    const int32_t tiles = tiles_of(n, per), entries = tiles * heads;
+    const int32_t tiles = tiles_of(n, per);
+    const int32_t entries = !by_length || length_class(k1 - k0, per_key) == cls ? tiles * heads : 0;
     int32_t incl = entries;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -407,12 +451,15 @@ dca_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     };
     Claims* claims = reinterpret_cast<Claims*>(smem + C::kOffClaim);
     int32_t i = SPLIT ? (int32_t)(blockIdx.x / cluster_size) : (int32_t)blockIdx.x;  // -1: no more
+    ClassItems classes{0, 0};
+    constexpr bool kByLength = DH == 128 && !SPLIT;
+    if (kByLength && p.per_key != 0.f) classes = count_classes(p.cand_offsets, p.seq_offsets, p.R, BQ / p.n_q, p.H, p.per_key, lane);
     DcaItem next{-1, 0, 0, 0};
     int32_t next_s0 = 0, next_L = 0, total_L = 0;
     auto read_next = [&]() {
       if (i >= 0) {
         if (p.items == nullptr) {
-          next = find_item(p.cand_offsets, p.seq_offsets, p.R, BQ / p.n_q, p.H, i, lane, next_s0, next_L);
+          next = find_item<kByLength>(p.cand_offsets, p.seq_offsets, p.R, BQ / p.n_q, p.H, p.per_key, classes, i, lane, next_s0, next_L);
         } else {
           next = p.items[i];
           next_s0 = p.seq_offsets[next.req];
@@ -927,6 +974,13 @@ static rocs_status_t launch_dca(const rocs_plan* plan, int32_t n_q, int32_t H, f
   p.n_q = n_q;
   p.H = H;
   p.scale_log2e = scale * 1.4426950408889634f;
+  // Items of the longest requests first where a side takes one to three and a half of them and they are long: 40 requests x
+  // about 20 candidates of 32 query tokens x 4 heads of 128 over 500..1500 keys 68.4 -> 63.2 us, 40 x 500 candidates over 1000..2000 73.1 ->
+  // 68.5, 20 x 600 over 750..1500 42.6 -> 40.2.  Not with many requests or short ones, which pay for the counting (60 x 200 over
+  // 200..400 23.9 -> 24.4, 120 x 100 over 60..120 19.4 -> 21.5), nor with heads of 64, where sides of an SM in step with one
+  // another cost more than the end gains (80 x 200 over 500..1000 54.8 -> 57.3, 64 x 300 over 150..300 30.8 -> 32.7).
+  const bool by_length = BKV == 64 && plan->R <= 64 && blocks >= 10 && num > 2 * sms && num <= 7 * sms;
+  p.per_key = by_length ? (float)plan->R / (float)T : 0.f;
   p.seq_offsets = seq_offsets;
   p.Q = (const __nv_bfloat16*)Q;
   p.K = (const __nv_bfloat16*)K;

@@ -497,6 +497,22 @@ def test_dca_general_kernel_groups_of_keys(L, dh):
     assert rel_err(to_host_f64(O), want) <= tol_for("f32")
 
 
+@pytest.mark.parametrize("R", [12, 33, 64, 65])
+def test_dca_bf16_items_by_length(R):
+    # up to 64 requests with long sequences: items in the order of their number of keys, from none to several times the
+    # average, requests without candidates in between; one more request and the order is that of the requests
+    g = np.random.default_rng(R)
+    lengths = g.choice([0, 1, 130, 640, 700, 1400, 2500], R)
+    lengths[0] = 3000
+    counts = g.integers(0, 36000 // R, R) * (g.random(R) < 0.8)
+    counts[-1] = 500
+    co, so = wl.offsets_from_counts(counts.tolist()), np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    cfg = wl.CONFIGS[3].with_(R=R, H=4, dh=128)
+    N = int(co[-1])
+    sample = np.unique(np.concatenate([np.clip(np.stack([co[:-1], co[1:] - 1]).ravel(), 0, N - 1), g.integers(0, N, 150)]))
+    assert _run_dca(cfg, co, so, sample=sample) <= tol_for("bf16")
+
+
 def test_dca_bf16_64_query_tokens_per_candidate():
     # two candidates fill a 128-row tile (Section 4.3.2 names query tiles of 32 and 64 tokens)
     co = wl.offsets_from_counts([5, 1, 12, 2])
