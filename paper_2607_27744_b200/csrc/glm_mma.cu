@@ -9,7 +9,7 @@
 // kernel 286 us.  The compression takes the fp32 block as a bf16 pair (value and remainder) through two products, as
 // exact as that kernel: error of OC against 64 bits 1.6573e-3 on 128 requests x 1024 candidates, 32 + 12 embeddings x
 // 128 to 8, at 187 us; 1.9116e-3 and 140 us with the block rounded first.  The tcgen05 kernel rounds it: where both
-// apply it is the faster also without the pair (128 x 1024 candidates, 32 + 16 embeddings with compression: 127 us,
+// apply it is the faster also without the pair (128 x 1024 candidates, 32 + 16 embeddings with compression: 118 us,
 // this one 145 us with 15 compute warps, 161 us with 8 that take two fragments each).
 //
 // A persistent CTA takes a contiguous run of tiles (tiles never cross a request); a producer warp streams the

@@ -179,7 +179,7 @@ struct RequestWalk {
 // Making the list is a launch in front of the request kernel, which a small batch feels and a large one does not: a
 // block of 8 requests x 697 candidates (attention's list made in its kernel too) 40.0 us with lists and 35.4 without,
 // one of 2 x 17 36.4 and 26.0; 128 x 1024 candidates (16384 tiles) 127.0 us with the list and 130.7 walked, the walk
-// being on every warp's path from tile to tile.  (One kernel for both ran the list in 136.4 us for 132.0: two instantiations.)
+// being on every warp's path from tile to tile (with a third group of epilogue warps 120.7 and 120.5: it is no longer the longest).  (One kernel for both ran the list in 136.4 us for 132.0: two instantiations.)
 // Plan and interaction with compression, 32 + 16 embeddings x 128, walked and with the list: 64 requests with 627 / 1230 /
 // 2432 / 4826 / 9628 tiles 14.0 / 18.6 / 27.5 / 43.9 / 85.9 us and 17.0 / 20.6 / 28.6 / 44.3 / 82.0 us.  About 2200 tiles of
 // 256 / 512 / 768 / 1024 requests 28.3 / 30.9 / 34.0 / 42.1 and 28.8 / 30.8 / 34.5 / 39.0; with 12 embeddings 39.1 / 44.0 /
