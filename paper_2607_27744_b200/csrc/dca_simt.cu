@@ -273,8 +273,11 @@ rocs_status_t dispatch(const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh
   // Two groups share the blocks of a request that has more than one.  One group and two, 1 x 25 candidates x 2 heads of 64
   // over 72..144 keys 9.9 and 8.5 us, 1 x 288 x 16 heads of 32 over 58..116 8.4 and 6.9 us, 24 x 109 x 8 heads of 64 over
   // 64..384 the same; four groups with blocks of 32 keys 9.3, 7.8 and 83 us for 69: an SM's FMAs are then the limit.
+  // 64 wide they also pay in long grids (100 x 27 candidates x 8 heads over 200..400 keys 101 and 93 us, 20 x 60 over 70..140
+  // 28.7 and 26.1); 32 wide, where twice the blocks of one group fit an SM, not (76 x 9 x 16 heads over 51..103 29.7 and 38.1).
   const int64_t keys = T_rows / plan->R;  // of an average request
-  const bool two = keys > KEYS;
+  constexpr int32_t kOneRound = 296;  // blocks of two groups
+  const bool two = keys > KEYS && (dh > 32 || items.num <= kOneRound);
   // smallest compiled width that holds the head: columns beyond dh are zeros in shared memory
   if (dh <= 32) {
     if (two) ROCS_LAUNCH(32, 2);
