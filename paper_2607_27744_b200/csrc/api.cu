@@ -577,7 +577,7 @@ static rocs_status_t ikbo_linear_impl(const rocs_plan_t* plan, rocs_dtype_t dtyp
                                      stream);
       if (taken) return st;
     }
-    if (row_stats == nullptr && dtype == ROCS_F32 && d_cand > 0 && simt_linear_both_supported(plan->N, d_req, d_out))
+    if (row_stats == nullptr && dtype == ROCS_F32 && d_cand > 0 && simt_linear_both_supported(plan->N, plan->R, d_req, d_out))
       return simt_linear_both(plan, d_req, d_cand, d_out, XR, ld_xr, XC, ld_xc, W_CR, ld_wcr, W_CC, ld_wcc, bias, act, Y, ld_y, stream);
     // Request half, once per request (Section 4.1): Z = X^R W_CR^T + bias, fp32.  The map, where a table of it has to be
     // made, beside it on the SMs that it leaves idle; the candidate kernel waits for both before it reads either.

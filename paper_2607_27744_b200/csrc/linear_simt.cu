@@ -281,10 +281,11 @@ rocs_status_t simt_linear(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_ou
 
 // The request half is computed for every candidate: worth it while that is less than a launch.  In a chain, two launches and
 // one: 25 x 80 | 64 -> 64 3.6 and 2.5 us (5.7 and 2.8 with the host in front), 48 x 128 | 64 -> 512 4.2 and 5.1 (5.7 and 5.3),
-// 27 x 64 | 256 -> 512 4.5 and 4.9 (5.6 and 4.9), 341 x 112 | 256 -> 512 9.4 and 11.7.
-bool simt_linear_both_supported(int64_t N, int32_t d_req, int32_t d_out) {
+// 27 x 64 | 256 -> 512 4.5 and 4.9 (5.6 and 4.9), 341 x 112 | 256 -> 512 9.4 and 11.7.  Nor with many candidates of a request,
+// whose row all of them fetch from the same place at the same time: 64 | 32 -> 64, 800 of 20 requests 6.2 and 5.3, 700 of one 5.1 and 8.3.
+bool simt_linear_both_supported(int64_t N, int32_t R, int32_t d_req, int32_t d_out) {
   constexpr int64_t kMost = 1 << 22;
-  return N > 0 && N <= kSearchRows && N * d_req * d_out <= kMost && ((N + 31) / 32) * ((d_out + 31) / 32) < 148;
+  return N > 0 && N <= kSearchRows && N <= 64 * (int64_t)R && N * d_req * d_out <= kMost && ((N + 31) / 32) * ((d_out + 31) / 32) < 148;
 }
 rocs_status_t simt_linear_both(const rocs_plan* plan, int32_t d_req, int32_t d_cand, int32_t d_out, const void* XR, int64_t ld_xr,
                                const void* XC, int64_t ld_xc, const void* W_CR, int64_t ld_wcr, const void* W_CC, int64_t ld_wcc,

@@ -302,7 +302,7 @@ rocs_status_t simt_linear(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_ou
                           const float* add, int64_t ld_add, const RequestMap& map, int act,
                           void* Y, int64_t ld_y, bool out_f32, cudaStream_t stream);
 // Both halves of an fp32 split layer in one launch, for few candidates.
-bool simt_linear_both_supported(int64_t N, int32_t d_req, int32_t d_out);
+bool simt_linear_both_supported(int64_t N, int32_t R, int32_t d_req, int32_t d_out);
 rocs_status_t simt_linear_both(const rocs_plan* plan, int32_t d_req, int32_t d_cand, int32_t d_out, const void* XR, int64_t ld_xr,
                                const void* XC, int64_t ld_xc, const void* W_CR, int64_t ld_wcr, const void* W_CC, int64_t ld_wcc,
                                const float* bias, int act, void* Y, int64_t ld_y, cudaStream_t stream);
