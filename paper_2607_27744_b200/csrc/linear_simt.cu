@@ -170,6 +170,27 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
       if constexpr (BOTH) part[(KS * BM + ty + 8 * i) * PS + tx + 8 * j] = acc_r[i][j];
     }
   __syncthreads();
+  if constexpr (BM * BN <= kGroup * KS) {
+    // a value per thread: a chain of four-wide sums on few threads was longer (1850 candidates, 64|32 -> 64, fp32:
+    // 9.1 us, 8.8 so)
+    const int32_t r = threadIdx.x / BN, c = threadIdx.x % BN, n = n0 + c;
+    if (r >= BM || m0 + r >= M || n >= d_out) return;
+    const float z = add ? add[(int64_t)req[r] * ld_add + n] : 0.f, b = bias ? bias[n] : 0.f;
+    float v = sm[r * PS + c], zr = 0.f;
+#pragma unroll
+    for (int g = 1; g < KS; ++g) v += sm[(g * BM + r) * PS + c];
+    if constexpr (BOTH) {
+#pragma unroll
+      for (int g = 0; g < KS; ++g) zr += sm[((KS + g) * BM + r) * PS + c];
+      v += zr + b;
+    } else {
+      v += b;
+      v += z;
+    }
+    if (act == ROCS_ACT_RELU) v = fmaxf(v, 0.f);
+    st_f(Y + (m0 + r) * ld_y + n, v);
+    return;
+  }
   // Four neighbouring columns of kRowsEach rows per thread.  The request rows are all asked for before the first is
   // used: one at a time, every row of a tile waited for the L2 cache.
   constexpr int kPerRow = BN / 4, kThreads = kGroup * KS, kRowStep = kThreads / kPerRow, kRowsEach = BM / kRowStep;
@@ -280,12 +301,13 @@ rocs_status_t simt_linear(rocs_dtype_t dt, int64_t M, int32_t d_in, int32_t d_ou
 }
 
 // The request half is computed for every candidate: worth it while that is less than a launch.  In a chain, two launches and
-// one: 25 x 80 | 64 -> 64 3.6 and 2.5 us (5.7 and 2.8 with the host in front), 48 x 128 | 64 -> 512 4.2 and 5.1 (5.7 and 5.3),
-// 27 x 64 | 256 -> 512 4.5 and 4.9 (5.6 and 4.9), 341 x 112 | 256 -> 512 9.4 and 11.7.  Nor with many candidates of a request,
-// whose row all of them fetch from the same place at the same time: 64 | 32 -> 64, 800 of 20 requests 6.2 and 5.3, 700 of one 5.1 and 8.3.
+// one: 25 x 80 | 64 -> 64 3.6 and 2.5 us (5.7 and 2.8 with the host in front), 341 x 112 | 256 -> 512 9.4 and 11.7.  Nor where a
+// request's row is fetched by too many at the same time, its candidates in every block of columns: 64 | 32 -> 64, 800 of 20
+// requests 6.2 and 5.3, 64 of one 4.0 and 2.8, 700 of one 5.1 and 8.3; 128 | 64 -> 512, 48 of two 4.6 and 6.7.
 bool simt_linear_both_supported(int64_t N, int32_t R, int32_t d_req, int32_t d_out) {
   constexpr int64_t kMost = 1 << 22;
-  return N > 0 && N <= kSearchRows && N <= 64 * (int64_t)R && N * d_req * d_out <= kMost && ((N + 31) / 32) * ((d_out + 31) / 32) < 148;
+  return N > 0 && N <= kSearchRows && N * d_out <= 4096 * (int64_t)R && N * d_req * d_out <= kMost &&
+         ((N + 31) / 32) * ((d_out + 31) / 32) < 148;
 }
 rocs_status_t simt_linear_both(const rocs_plan* plan, int32_t d_req, int32_t d_cand, int32_t d_out, const void* XR, int64_t ld_xr,
                                const void* XC, int64_t ld_xc, const void* W_CR, int64_t ld_wcr, const void* W_CC, int64_t ld_wcc,
