@@ -14,7 +14,9 @@
 // on mma.sync, whose products were what took the time (some 25 cycles of a scheduler each): 18400 candidates of 12
 // embeddings x 128, k = 16, 28.7 -> 20.2 us with their request kernel; 56721 of 12 x 192, k = 24, 205 -> 66; 32768 of 16 x 64,
 // k = 24, 50 -> 32.5; 19236 of 4 x 128, k = 16, 24.9 -> 11.1; 15 of 8 x 64 5.7 -> 5.4.  12000 requests of two candidates, a tile each
-// of which they fill a sixteenth, 81 -> 92.  The tiles are walked and not listed, in any number: the walk is short against a tile
+// of which they fill a sixteenth, 81 -> 92, and a few thousand of 12 embeddings in two or three rounds of tiles: 2959 of one
+// request x 128 8.4 -> 8.9, 5000 x 64, k = 8, 7.4 -> 9.1.  T kept in a ring of its own, loaded once per request and multiplied apart
+// from the Gram matrix, was slower (23.1 us for 18400 to 21000 candidates of 12 x 128 as above, 26.9 us so).  The tiles are walked and not listed, in any number: the walk is short against a tile
 // (2700 tiles 25.3 us with the list, 23.0 walked).
 #include <algorithm>
 
