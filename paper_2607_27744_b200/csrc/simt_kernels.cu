@@ -178,8 +178,8 @@ __global__ void __launch_bounds__(kGlmThreads) glm_candidate_simt_kernel(
   float* wr = wc + (w_shared ? (size_t)n_c * n_co : 0);        // [n_co, n_r]: W_CR (extra)
   const int tid = threadIdx.x;
   int32_t block = blockIdx.x;
-  if constexpr (FUSED) {
-    ptx::griddep_wait();
+  if constexpr (FUSED) {  // the call's first launch: the one in front may be what writes its inputs
+    ptx::griddep_wait_for(XR, XC, W, cand_offsets, tiles);
     ptx::griddep_launch_dependents();
     if (block < R) {
       glm_request_side<T, kGlmThreads>(block, n_r, n_c, d, XR, W, n_ro, n_co, YR, OR_, nullptr, sm);
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kGlmThreads) glm_candidate_simt_kernel(
     for (int32_t e = tid; e < rows * n; e += kGlmThreads) st_f(out, e, yc[e]);
   }
   // Launched beside the request kernel: its ZR is read from here on, and whoever waits for this grid counts on both.
-  if constexpr (!FUSED) ptx::griddep_wait();
+  if constexpr (!FUSED) ptx::griddep_wait_for(ZR);
   if (!compress) return;
   const float* zr = FUSED ? yc + (size_t)rows * n : ZR + (int64_t)tile.req * n_co * n;  // FUSED: columns of requests only
   const int32_t zr_cols = FUSED ? n_r : n;

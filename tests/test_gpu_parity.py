@@ -691,6 +691,31 @@ def test_glm_general_kernel_batch_sizes(dtype, n_r, n_c, d, n_co, per, R):
     assert _run_glm(cfg, co) <= tol_for(dtype)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_glm_small_batch_behind_the_kernel_that_writes_its_rows(dtype):
+    # the interaction's only launch may start while the kernel in front of it still writes X^R and X^C
+    co = wl.offsets_from_counts([7, 1, 12])
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    plan, d, n_r, n_c = _plan(co), 64, 20, 4
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    W = torch.randn(8, n_r + n_c, device="cuda", generator=gen).to(dt)
+    ER, EC = torch.empty(3, n_r, d, dtype=dt, device="cuda"), torch.empty(20, n_c, d, dtype=dt, device="cuda")
+    ws = torch.empty(rocs.glm_interaction_workspace(plan, n_r, n_c, 4), dtype=torch.uint8, device="cuda")
+    raw = [(torch.randn(3 * n_r, d, device="cuda", generator=gen).to(dt), torch.randn(20 * n_c, d, device="cuda", generator=gen).to(dt)) for _ in range(20)]
+    got = []
+    for r, c in raw:
+        rocs.group_norm(r, out=ER.view(-1, d))
+        rocs.group_norm(c, out=EC.view(-1, d))
+        got.append({k: v.clone() for k, v in rocs.glm_interaction(plan, ER, EC, W, 4, 4, want_raw=True, workspace=ws).items()})
+    for (r, c), out in zip(raw, got):
+        rocs.group_norm(r, out=ER.view(-1, d))
+        rocs.group_norm(c, out=EC.view(-1, d))
+        torch.cuda.synchronize()
+        want = rocs.glm_interaction(plan, ER, EC, W, 4, 4, want_raw=True, workspace=ws)
+        for k in want:
+            assert torch.equal(out[k], want[k]), k
+
+
 @pytest.mark.parametrize("n_r,n_c,d,n_co,raw", [(32, 16, 128, 8, False), (20, 12, 64, 4, True), (4, 4, 192, 16, True), (44, 8, 256, 3, False),
                                                   (20, 8, 128, 0, True), (16, 4, 64, 8, False), (100, 16, 64, 16, True),
                                                   (128, 12, 256, 1, False), (44, 16, 128, 0, True), (24, 12, 128, 8, False)])
