@@ -7,8 +7,8 @@
 // so a candidate reads its own 2 n_c d bytes and nothing of the request but the d x k block T,
 // which stays in registers while consecutive candidates belong to the same request.
 //
-// The candidate side is bound by HBM (about 30 flop per byte).  Two bf16 kernels: fm_umma.cu, and here, for candidates of 16
-// embeddings, a kernel that streams candidate tiles through a TMA ring and gives every warp one candidate at a time, whose
+// The candidate side is bound by HBM (about 30 flop per byte).  Two bf16 kernels: fm_umma.cu, and here
+// a kernel that streams candidate tiles through a TMA ring and gives every warp one candidate at a time, whose
 // two small products (16 x d x 16 each) run on mma.sync m16n8k16 straight out of the swizzled tile:
 //   step 1   H^T = T^T + P_C^T X^C_i    accumulators start at T^T (fp32); X^C_i is the K x N
 //                                       operand, read with ldmatrix.trans
@@ -146,12 +146,24 @@ __global__ void __launch_bounds__(128) fm_candidate_simt_kernel(int32_t n_r, int
 }
 
 // ---------------------------------------------------------------------------------------------
-// Candidate side, bf16 streaming kernel: 16 embeddings, 8 or 16 columns, d a multiple of 64 up to 256.  H is rounded to bf16.
-// Bound by HBM; against fm_umma.cu: 29 / 300 / 1000 / 8000 / 131072 candidates x 128, k = 16, 5.6 / 6.1 / 7.4 / 21.5 / 103 us
-// and 6.3 / 6.6 / 8.9 / 22.6 / 106, 10000 x 64, k = 8, 14.9 and 18.6: one candidate per warp is done sooner behind its loads.
+// Candidate side, bf16 streaming kernel: n_c up to 16, even k up to 32, d a multiple of 64 up to 256.
+// The fragments hold 16 candidate rows: of a candidate with fewer the rest are the next candidate's, which
+// step 1 masks to zero (0 x NaN of a neighbour must not arise) and step 2 computes and drops.
+// 16 embeddings and 8 or 16 columns (FULL) round H to bf16 and are bound by HBM.  Every other shape takes H as a bf16 pair
+// (value and remainder) through two products in step 2, and is bound by the products: error of FC against 64 bits on 128
+// requests x 1024 candidates, 32 + 12 embeddings x 128, k = 16, 1.6568e-3 as with fp32 FMA throughout (all of it the
+// rounding of FC) at 120.3 us; 1.8657e-3 at 81.8 us with H rounded; three parts, every bit of H, about 30 us more.
+// 18 400 candidates of 12 embeddings x 128, k = 16: 26.9 us; the general kernel, a block per candidate, 284 us.
 // ---------------------------------------------------------------------------------------------
-constexpr int kFragRows = 16;      // embeddings of a candidate = rows of its fragments
-constexpr int kTileCands = 8;      // candidates per tile = compute warps per CTA
+constexpr int kFragRows = 16;      // rows of a candidate's fragments
+// Candidates per tile = compute warps per CTA.  Two per scheduler are enough for a stream that HBM bounds; the chains of the
+// pair's products want more of them: as many as leave them their registers (11 and the producer are three per scheduler, at
+// 168 registers, 15 four at 128).  With 8: 128.4 us for the batch above, 223 for 183 us on 128 x 512 candidates of 12
+// embeddings x 256, 54.2 for 49.9 on 64 x 512 of 16 x 64 to 24 columns.
+template <int D, bool FULL>
+constexpr int tile_cands() {
+  return FULL ? 8 : D == 64 ? 15 : 11;
+}
 constexpr int kMaxStages = 12;
 constexpr uint32_t kStatusFm = 0x600;
 
@@ -296,7 +308,7 @@ __global__ void __launch_bounds__(256) fm_request_mma_kernel(int32_t n_r, int32_
 
 struct FmParams {
   int64_t N;
-  int32_t n_r, k, num_tiles, stages;
+  int32_t n_r, n_c, k, num_tiles, stages;
   const __nv_bfloat16* P;        // [n_r + n_c, k]
   const int32_t* offsets;        // [R + 1]
   int32_t R;
@@ -305,32 +317,37 @@ struct FmParams {
   uint32_t* status;
 };
 
-// T^T of a request, the 16 columns cp of d, in the accumulator layout of step 1.
-template <int D>
-__device__ __forceinline__ void load_t(const float* tt, int32_t k, int cp, int g, int tq, float (&f)[2][4]) {
-  const int c = g;
+// Two fp32 values as bf16 pairs that add up to them.  Rounded value and rounded remainder: 17 bits.
+__device__ __forceinline__ void split_bf16(float a, float b, uint32_t (&part)[2]) {
+  part[0] = pack_bf16(a, b);
+  part[1] = pack_bf16(a - __uint_as_float(part[0] << 16), b - __uint_as_float(part[0] & 0xffff0000u));
+}
+// Upper halves of the values, of what is left and of what is left then: every bit.  An infinity is infinite in every part.
+__device__ __forceinline__ void split_bf16(float a, float b, uint32_t (&part)[3]) {
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int col = (2 * cp + h) * 8 + 2 * tq;
-    const float2 lo = c < k ? *reinterpret_cast<const float2*>(tt + c * D + col) : make_float2(0.f, 0.f);
-    const float2 hi = c + 8 < k ? *reinterpret_cast<const float2*>(tt + (c + 8) * D + col) : make_float2(0.f, 0.f);
-    f[h][0] = lo.x;
-    f[h][1] = lo.y;
-    f[h][2] = hi.x;
-    f[h][3] = hi.y;
+  for (int i = 0; i < 3; ++i) {
+    const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
+    part[i] = __byte_perm(ua, ub, 0x7632);
+    a = fabsf(a) == INFINITY ? a : a - __uint_as_float(ua & 0xffff0000u);
+    b = fabsf(b) == INFINITY ? b : b - __uint_as_float(ub & 0xffff0000u);
   }
 }
 
-template <int D>
-__global__ void __launch_bounds__((kTileCands + 1) * 32, 1)
+// KT: blocks of 16 projection columns.  With one, the request's T stays in registers while consecutive
+// candidates share it; with two it would not fit beside H and comes from L1 for every candidate.
+template <int D, int KT, bool FULL>
+__global__ void __launch_bounds__((tile_cands<D, FULL>() + 1) * 32, 1)
 fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmParams p) {
   constexpr int kSlabs = D / 64;
   constexpr int kPairs = D / 16;  // pairs of 8-column groups = k-steps of step 2
   extern __shared__ __align__(1024) uint8_t smem[];
-  constexpr int32_t n_c = kFragRows;
-  constexpr int32_t slab_bytes = kTileCands * n_c * 128;  // 64 columns of the tile, 128-byte swizzled rows
-  constexpr int32_t stage_bytes = kSlabs * slab_bytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.stages * stage_bytes);
+  const int32_t n_c = FULL ? kFragRows : p.n_c;
+  constexpr int kTileCands = tile_cands<D, FULL>();
+  // 64 columns of the tile, 128-byte swizzled rows, to the 1024 bytes that the swizzle repeats in
+  const int32_t slab_bytes = (kTileCands * n_c * 128 + 1023) / 1024 * 1024;
+  const int32_t stage_bytes = kSlabs * slab_bytes;
+  // behind the stages: rows that the last candidate's fragments read past the tile
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + p.stages * stage_bytes + (FULL ? 0 : kFragRows * 128));
   uint64_t* empty = full + kMaxStages;
   AbortFlag* abort_flag = reinterpret_cast<AbortFlag*>(empty + kMaxStages);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -379,22 +396,42 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
     // ------------------------------ one candidate per warp ---------------------------------
     const int g = lane / 4, tq = lane % 4;  // fragment row group and column pair
     // P_C^T as the M x K operand of step 1: A[m = projection column][kk = candidate row]
-    uint32_t pa[4];
+    uint32_t pa[KT][4];
     {
       const __nv_bfloat16* pc = p.P + (int64_t)p.n_r * p.k;
-      auto at = [&](int row, int col) -> float {  // P_C[row][col], zero beyond k columns
-        return col < p.k ? __bfloat162float(pc[row * p.k + col]) : 0.f;
+      auto at = [&](int row, int col) -> float {  // P_C[row][col], zero beyond n_c rows and k columns
+        return row < n_c && col < p.k ? __bfloat162float(pc[row * p.k + col]) : 0.f;
       };
-      pa[0] = pack_bf16(at(2 * tq, g), at(2 * tq + 1, g));
-      pa[1] = pack_bf16(at(2 * tq, g + 8), at(2 * tq + 1, g + 8));
-      pa[2] = pack_bf16(at(2 * tq + 8, g), at(2 * tq + 9, g));
-      pa[3] = pack_bf16(at(2 * tq + 8, g + 8), at(2 * tq + 9, g + 8));
+#pragma unroll
+      for (int kt = 0; kt < KT; ++kt) {
+        const int c = kt * 16 + g;
+        pa[kt][0] = pack_bf16(at(2 * tq, c), at(2 * tq + 1, c));
+        pa[kt][1] = pack_bf16(at(2 * tq, c + 8), at(2 * tq + 1, c + 8));
+        pa[kt][2] = pack_bf16(at(2 * tq + 8, c), at(2 * tq + 9, c));
+        pa[kt][3] = pack_bf16(at(2 * tq + 8, c + 8), at(2 * tq + 9, c + 8));
+      }
     }
+    // rows of the K x N operand of step 1 that are this candidate's: 2 tq, 2 tq + 1 and the two 8 further on
+    auto row_mask = [&](int row) { return (row < n_c ? 0xffffu : 0u) | (row + 1 < n_c ? 0xffff0000u : 0u); };
+    const uint32_t keep_lo = row_mask(2 * tq), keep_hi = row_mask(2 * tq + 8);
     // this lane's address pattern inside a candidate's 16 rows: row, and which of the two
     // 8-column groups of a pair
     const int trow = warp * n_c + (lane % 8) + ((lane / 8) % 2) * 8;
     const int lsel = lane / 16;
-    float tfrag[kPairs][2][4];  // T^T of the cached request in step-1 accumulator layout
+    float tfrag[KT == 1 ? kPairs : 1][2][4];  // T^T of the cached request in step-1 accumulator layout
+    auto load_t = [&](const float* tt, int kt, int cp, float (&f)[2][4]) {
+      const int c = kt * 16 + g;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int col = (2 * cp + h) * 8 + 2 * tq;
+        const float2 lo = c < p.k ? *reinterpret_cast<const float2*>(tt + c * D + col) : make_float2(0.f, 0.f);
+        const float2 hi = c + 8 < p.k ? *reinterpret_cast<const float2*>(tt + (c + 8) * D + col) : make_float2(0.f, 0.f);
+        f[h][0] = lo.x;
+        f[h][1] = lo.y;
+        f[h][2] = hi.x;
+        f[h][3] = hi.y;
+      }
+    };
     int32_t cached_req = -1;
     int s = 0;
     uint32_t phase = 0;
@@ -417,44 +454,96 @@ fm_candidate_mma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmPara
         if (r != cached_req) {
           if (cached_req < 0) griddep_wait();  // TT comes from the request kernel launched just before
           cached_req = r;
+          if constexpr (KT == 1) {
 #pragma unroll
-          for (int cp = 0; cp < kPairs; ++cp) load_t<D>(tt, p.k, cp, g, tq, tfrag[cp]);
+            for (int cp = 0; cp < kPairs; ++cp) load_t(tt, 0, cp, tfrag[cp]);
+          }
         }
         const uint32_t tile = smem_u32(smem + s * stage_bytes) + trow * 128;
         __nv_bfloat16* fc = p.FC + cand * n_c * p.k;
-        // step 1: H^T (16 x D) = T^T + P_C^T X^C, whose accumulator is the K x N operand of step 2 as it stands
-        uint32_t hb[kPairs][2][2];  // [k-step][projection columns 0-7 | 8-15][b0, b1]
 #pragma unroll
-        for (int cp = 0; cp < kPairs; ++cp) {
-          const int chunk = 2 * cp + lsel;  // 16-byte chunk along d
-          uint32_t xb[4];
-          ldmatrix_x4_trans(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xb);
-          float f[2][4];
+        for (int kt = 0; kt < KT; ++kt) {
+          // step 1: H^T (16 x D) = T^T + P_C^T X^C, whose accumulator is the K x N operand of step 2 as it stands
+          auto step1 = [&](int cp, float (&f)[2][4]) {
+            const int chunk = 2 * cp + lsel;  // 16-byte chunk along d
+            uint32_t xb[4];
+            ldmatrix_x4_trans(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xb);
+            if constexpr (!FULL) {
+              xb[0] &= keep_lo;
+              xb[1] &= keep_hi;
+              xb[2] &= keep_lo;
+              xb[3] &= keep_hi;
+            }
+            if constexpr (KT == 1) {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) f[e / 4][e % 4] = tfrag[cp][e / 4][e % 4];
-          mma_bf16(f[0], pa, xb[0], xb[1]);
-          mma_bf16(f[1], pa, xb[2], xb[3]);
-          hb[cp][0][0] = pack_bf16(f[0][0], f[0][1]);
-          hb[cp][0][1] = pack_bf16(f[1][0], f[1][1]);
-          hb[cp][1][0] = pack_bf16(f[0][2], f[0][3]);
-          hb[cp][1][1] = pack_bf16(f[1][2], f[1][3]);
-        }
-        // step 2: FC (16 x 16) = X^C H
-        float out[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+              for (int e = 0; e < 8; ++e) f[e / 4][e % 4] = tfrag[cp][e / 4][e % 4];
+            } else {
+              load_t(tt, kt, cp, f);
+            }
+            mma_bf16(f[0], pa[kt], xb[0], xb[1]);
+            mma_bf16(f[1], pa[kt], xb[2], xb[3]);
+          };
+          // step 2: FC (16 x 16) = X^C H
+          float out[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+          auto rows_of = [&](int cp, uint32_t (&xa)[4]) {
+            const int chunk = 2 * cp + lsel;
+            ldmatrix_x4(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xa);
+          };
+          if constexpr (FULL) {
+            uint32_t hb[kPairs][2][2];  // [k-step][projection columns 0-7 | 8-15][b0, b1]
 #pragma unroll
-        for (int cp = 0; cp < kPairs; ++cp) {
-          const int chunk = 2 * cp + lsel;
-          uint32_t xa[4];
-          ldmatrix_x4(tile + (chunk / 8) * slab_bytes + (((chunk % 8) ^ (trow & 7)) << 4), xa);
-          mma_bf16(out[0], xa, hb[cp][0][0], hb[cp][0][1]);
-          mma_bf16(out[1], xa, hb[cp][1][0], hb[cp][1][1]);
-        }
+            for (int cp = 0; cp < kPairs; ++cp) {
+              float f[2][4];
+              step1(cp, f);
+              hb[cp][0][0] = pack_bf16(f[0][0], f[0][1]);
+              hb[cp][0][1] = pack_bf16(f[1][0], f[1][1]);
+              hb[cp][1][0] = pack_bf16(f[0][2], f[0][3]);
+              hb[cp][1][1] = pack_bf16(f[1][2], f[1][3]);
+            }
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int col = 8 * h + 2 * tq;
-          if (col < p.k) {
-            *reinterpret_cast<uint32_t*>(fc + g * p.k + col) = pack_bf16(out[h][0], out[h][1]);
-            *reinterpret_cast<uint32_t*>(fc + (g + 8) * p.k + col) = pack_bf16(out[h][2], out[h][3]);
+            for (int cp = 0; cp < kPairs; ++cp) {
+              uint32_t xa[4];
+              rows_of(cp, xa);
+              mma_bf16(out[0], xa, hb[cp][0][0], hb[cp][0][1]);
+              mma_bf16(out[1], xa, hb[cp][1][0], hb[cp][1][1]);
+            }
+          } else {
+            auto product = [&](auto parts) {
+              constexpr int kParts = decltype(parts)::value;
+#pragma unroll
+              for (int cp = 0; cp < kPairs; ++cp) {
+                float f[2][4];
+                uint32_t xa[4];
+                step1(cp, f);
+                rows_of(cp, xa);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                  uint32_t b0[kParts], b1[kParts];
+                  split_bf16(f[0][2 * h], f[0][2 * h + 1], b0);
+                  split_bf16(f[1][2 * h], f[1][2 * h + 1], b1);
+#pragma unroll
+                  for (int i = 0; i < kParts; ++i) mma_bf16(out[h], xa, b0[i], b1[i]);
+                }
+              }
+            };
+            product(std::integral_constant<int, 2>());
+            bool nan = false;  // in this candidate's rows: what the next one's hold must not decide
+#pragma unroll
+            for (int e = 0; e < 8; ++e) nan = nan || (g + 8 * (e / 2 % 2) < n_c && isnan(out[e / 4][e % 4]));
+            if (__any_sync(0xffffffffu, nan)) {  // perhaps of an infinity, or of a value that rounds to one
+#pragma unroll
+              for (int e = 0; e < 8; ++e) out[e / 4][e % 4] = 0.f;
+              product(std::integral_constant<int, 3>());
+            }
+          }
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int col = kt * 16 + 8 * h + 2 * tq;
+            if (col < p.k) {
+              if (FULL || g < n_c) *reinterpret_cast<uint32_t*>(fc + g * p.k + col) = pack_bf16(out[h][0], out[h][1]);
+              if (FULL || g + 8 < n_c)
+                *reinterpret_cast<uint32_t*>(fc + (g + 8) * p.k + col) = pack_bf16(out[h][2], out[h][3]);
+            }
           }
         }
       }
@@ -475,30 +564,33 @@ int sm_count_fm() {
   return n;
 }
 
-template <int D>
-rocs_status_t launch_fm_mma(const rocs_plan* plan, int32_t n_r, int32_t k, const void* XC, const void* P, const float* TT,
-                            void* FC, cudaStream_t stream) {
-  constexpr int kStageBytes = kTileCands * kFragRows * D * 2, kFixed = 2 * kMaxStages * 8 + 16;
+template <int D, int KT, bool FULL>
+rocs_status_t launch_fm_mma_as(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t k,
+                               const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
+  constexpr int kTileCands = tile_cands<D, FULL>();
+  const int stage_bytes = D / 64 * ((kTileCands * n_c * 128 + 1023) / 1024 * 1024);
+  constexpr int kFixed = kFragRows * 128 + 2 * kMaxStages * 8 + 16;
   CUtensorMap map_xc;
-  if (!make_tensor_map_2d(&map_xc, XC, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)plan->N * kFragRows, D, D,
-                          kTileCands * kFragRows, 64, true))
+  if (!make_tensor_map_2d(&map_xc, XC, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)plan->N * n_c, D, D,
+                          (uint32_t)(kTileCands * n_c), 64, true))
     return ROCS_ERR_CUDA;
   uint32_t* status = device_status_word();
   if (!status) return ROCS_ERR_CUDA;
   FmParams p{};
   p.N = plan->N;
   p.n_r = n_r;
+  p.n_c = n_c;
   p.k = k;
   p.num_tiles = (int32_t)((plan->N + kTileCands - 1) / kTileCands);
-  p.stages = std::min(kMaxStages, (227 * 1024 - kFixed) / kStageBytes);
+  p.stages = std::min(kMaxStages, (227 * 1024 - kFixed) / stage_bytes);
   p.P = (const __nv_bfloat16*)P;
   p.offsets = plan->cand_offsets;
   p.R = plan->R;
   p.TT = TT;
   p.FC = (__nv_bfloat16*)FC;
   p.status = status;
-  const int smem = p.stages * kStageBytes + kFixed;
-  auto kern = fm_candidate_mma_kernel<D>;
+  const int smem = p.stages * stage_bytes + kFixed;
+  auto kern = fm_candidate_mma_kernel<D, KT, FULL>;
   ROCS_ALLOW_SMEM(kern, kMaxDynamicSmem);
   // Launched so that it may overlap the request kernel in front of it on the stream (that kernel
   // releases its dependents at once); nothing else this kernel reads is written by that launch.
@@ -516,6 +608,15 @@ rocs_status_t launch_fm_mma(const rocs_plan* plan, int32_t n_r, int32_t k, const
   return ROCS_OK;
 }
 
+template <int D>
+rocs_status_t launch_fm_mma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t k,
+                            const void* XC, const void* P, const float* TT, void* FC, cudaStream_t stream) {
+  if (k > 16) return launch_fm_mma_as<D, 2, false>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+  if (n_c == kFragRows && (k == 8 || k == 16))
+    return launch_fm_mma_as<D, 1, true>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+  return launch_fm_mma_as<D, 1, false>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+}
+
 template <typename T>
 rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, int32_t k, const void* XR,
                         const void* XC, const void* P, void* FR, void* FC, float* TT, bool fast_candidates,
@@ -526,7 +627,7 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
   if (smem_r > kMaxSmem || smem_c > kMaxSmem) return ROCS_ERR_UNSUPPORTED;
   const size_t n_rp = (size_t)(n_r + 15) / 16 * 16, kp = (size_t)(k + 15) / 16 * 16;
   const size_t smem_mma = n_rp * ((size_t)(d + 8) * 2 + (kp + 8) * 2) + 2 * kp * (size_t)(d + 8) * 2;
-  const bool pair = fast_candidates && FC != nullptr && !(n_c == kFragRows && (k == 8 || k == 16));  // fm_umma.cu reads TT
+  const bool pair = fast_candidates && FC != nullptr && fm_umma_pays(plan, n_c, d, k);  // fm_umma.cu reads TT
   if (plan->R > 0) {
     const bool mma = tensor_core_request && sizeof(T) == 2 && d % 16 == 0 && k % 8 == 0 && smem_mma <= kMaxSmem;
     auto run = [&](auto with_pair) {
@@ -547,10 +648,10 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
   if (pair) return fm_umma(plan, n_r, n_c, d, k, XC, P, TT, FC, stream);
   if (fast_candidates) {
     switch (d) {
-      case 64: return launch_fm_mma<64>(plan, n_r, k, XC, P, TT, FC, stream);
-      case 128: return launch_fm_mma<128>(plan, n_r, k, XC, P, TT, FC, stream);
-      case 192: return launch_fm_mma<192>(plan, n_r, k, XC, P, TT, FC, stream);
-      case 256: return launch_fm_mma<256>(plan, n_r, k, XC, P, TT, FC, stream);
+      case 64: return launch_fm_mma<64>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 128: return launch_fm_mma<128>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 192: return launch_fm_mma<192>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
+      case 256: return launch_fm_mma<256>(plan, n_r, n_c, k, XC, P, TT, FC, stream);
       default: break;
     }
   }

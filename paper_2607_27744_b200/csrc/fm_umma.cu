@@ -13,11 +13,9 @@
 // Bound by HBM, and in small batches by what a short run of tiles takes to start and end.  In place of a candidate per warp
 // on mma.sync, whose products were what took the time (some 25 cycles of a scheduler each): 18400 candidates of 12
 // embeddings x 128, k = 16, 28.7 -> 20.2 us with their request kernel; 56721 of 12 x 192, k = 24, 205 -> 66; 32768 of 16 x 64,
-// k = 24, 50 -> 32.5; 19236 of 4 x 128, k = 16, 24.9 -> 11.1; 15 of 8 x 64 5.7 -> 5.4.  12000 requests of two candidates, a tile each
-// of which they fill a sixteenth, 81 -> 92, and a few thousand of 12 embeddings in two or three rounds of tiles: 2959 of one
-// request x 128 8.4 -> 8.9, 5000 x 64, k = 8, 7.4 -> 9.1.  T kept in a ring of its own, loaded once per request and multiplied apart
-// from the Gram matrix, was slower (23.1 us for 18400 to 21000 candidates of 12 x 128 as above, 26.9 us so).  The tiles are walked and not listed, in any number: the walk is short against a tile
-// (2700 tiles 25.3 us with the list, 23.0 walked).
+// k = 24, 50 -> 32.5; 19236 of 4 x 128, k = 16, 24.9 -> 11.1.  T kept in a ring of its own, loaded once per request and multiplied
+// apart from the Gram matrix, was slower (23.1 us for 18400 to 21000 candidates of 12 x 128 as above, 26.9 us so).  The tiles are
+// walked and not listed, in any number: the walk is short against a tile (2700 tiles 25.3 us with the list, 23.0 walked).
 #include <algorithm>
 
 #include "rocs_internal.h"
@@ -296,6 +294,26 @@ rocs_status_t launch(int smem, const CUtensorMap& map_tt, const CUtensorMap& map
 int rows_of(int32_t n_c) { return n_c <= 4 ? 4 : n_c <= 8 ? 8 : 16; }
 
 }  // namespace
+
+// Where this kernel is the faster one of the two on bf16 rows.  fm_projection.cu's has as many candidates at work on an SM as
+// warps and takes a candidate's bytes alone; this one takes a tile's 128 rows however few of them a request fills, and its run of
+// tiles starts and ends slower.  Request kernel included, on a plan that is kept, that one and this one, in us:
+//   few candidates per tile, of 1000 requests 4 x 128, k = 16: one / two / eight each 13.4 / 16.4 / 24.5 and 17.4 / 17.4 / 17.6;
+//   12000 x 2 of 8 x 64, k = 8, 77 and 96; 100 x 3 of 12 x 128, k = 16, 7.0 and 7.9; of 12 x 192, k = 24, 1000 x 1 / 2 24.2 / 28.9 and
+//   27.4 / 27.6
+//   d = 64, few requests, their products being short: 12 embeddings, k = 8, 1 x 3000 / 5000 / 10000 6.6 / 7.6 / 9.8 and 8.4 / 9.6 / 11.9,
+//   100 x 10 / 30 / 100 7.1 / 8.2 / 12.0 and 8.0 / 8.8 / 12.3, 1000 x 8 / 30 17.0 / 27.8 and 14.8 / 25.6; 8 embeddings, 1 x 300 /
+//   3000 / 5000 / 10000 5.3 / 6.6 / 7.6 / 9.8 and 5.5 / 7.6 / 8.2 / 9.5, 100 x 30 8.2 and 7.8
+//   d = 128, k = 16, 12 embeddings in two or three rounds of tiles of a request or a few: 3000 8.4 and 9.2, 5000 11.1 and 10.9
+// 16 embeddings to 8 or 16 columns take H rounded once there (103 and 106 us on 131072 x 128, k = 16; 5.6 and 6.3 on 29).
+bool fm_umma_pays(const rocs_plan* plan, int32_t n_c, int32_t d, int32_t k) {
+  if (n_c == 16 && (k == 8 || k == 16)) return false;
+  const int64_t N = plan->N, R = plan->R, tiles = plan_entries(plan, 128 / rows_of(n_c));
+  if (R > 64 && (d <= 128 ? N <= 3 * tiles : N < 2 * tiles)) return false;
+  if (d == 64 && k <= 16 && n_c > 4 && (n_c > 8 ? R <= 128 && N <= 16384 : R <= 32 && N <= 6144)) return false;
+  if (d == 128 && k <= 16 && n_c > 8 && R <= 4 && tiles > 148 && tiles <= 3 * 148) return false;
+  return true;
+}
 
 rocs_status_t fm_umma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, int32_t k, const void* XC, const void* P,
                       const void* TT, void* FC, cudaStream_t stream) {
