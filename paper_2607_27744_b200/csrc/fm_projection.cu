@@ -33,25 +33,13 @@ __device__ __forceinline__ float ld_f(const __nv_bfloat16* p, int64_t i) { retur
 __device__ __forceinline__ void st_f(float* p, int64_t i, float v) { p[i] = v; }
 __device__ __forceinline__ void st_f(__nv_bfloat16* p, int64_t i, float v) { p[i] = __float2bfloat16_rn(v); }
 
-// TT as the candidate kernels read it: fp32 [R, k, d], or (PAIR) bf16 [R, 2, k, d], value and remainder.
-template <bool PAIR>
-using TermOf = std::conditional_t<PAIR, __nv_bfloat16, float>;
-// What is left of an infinity or a NaN is 0; a finite value does not round to infinity.
-__device__ __forceinline__ __nv_bfloat16 pair_value(float x) {
-  const __nv_bfloat16 v = __float2bfloat16_rn(x);
-  return __hisinf(v) ? __ushort_as_bfloat16((unsigned short)(__float_as_uint(x) >> 16)) : v;
-}
-__device__ __forceinline__ __nv_bfloat16 pair_remainder(float x, __nv_bfloat16 value) {
-  return __float2bfloat16_rn(isfinite(x) ? x - __bfloat162float(value) : 0.f);
-}
-
 // ---------------------------------------------------------------------------------------------
 // Request side, one block per request:  TT[r] = P_R^T X^R_r  ([k, d] fp32, the transpose of T)
 // and FR[r] = X^R_r T[r].
 // ---------------------------------------------------------------------------------------------
-template <typename T, bool PAIR>
+template <typename T>
 __global__ void __launch_bounds__(256) fm_request_kernel(int32_t n_r, int32_t d, int32_t k, const T* __restrict__ XR,
-                                                         const T* __restrict__ P, TermOf<PAIR>* __restrict__ TT,
+                                                         const T* __restrict__ P, float* __restrict__ TT,
                                                          T* __restrict__ FR) {
   extern __shared__ float sm[];
   const int32_t ds = d + 1;           // padded row stride: rows land in different banks
@@ -84,14 +72,7 @@ __global__ void __launch_bounds__(256) fm_request_kernel(int32_t n_r, int32_t d,
     for (int u = 0; u < kCg; ++u)
       if (c0 + u < k) {
         tt[(c0 + u) * ds + e] = acc[u];
-        if constexpr (PAIR) {
-          __nv_bfloat16* at = TT + ((int64_t)r * 2 * k + c0 + u) * d + e;
-          const __nv_bfloat16 value = pair_value(acc[u]);
-          at[0] = value;
-          at[(int64_t)k * d] = pair_remainder(acc[u], value);
-        } else {
-          TT[((int64_t)r * k + c0 + u) * d + e] = acc[u];
-        }
+        TT[((int64_t)r * k + c0 + u) * d + e] = acc[u];
       }
   }
   if (!FR) return;
@@ -201,10 +182,9 @@ __device__ __forceinline__ void ldmatrix_x2(uint32_t addr, uint32_t (&r)[2]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
 }
 
-template <bool PAIR>
 __global__ void __launch_bounds__(256) fm_request_mma_kernel(int32_t n_r, int32_t d, int32_t k,
                                                              const __nv_bfloat16* __restrict__ XR,
-                                                             const __nv_bfloat16* __restrict__ P, TermOf<PAIR>* __restrict__ TT,
+                                                             const __nv_bfloat16* __restrict__ P, float* __restrict__ TT,
                                                              __nv_bfloat16* __restrict__ FR) {
   extern __shared__ __align__(16) uint8_t smem_fmr[];
   const int32_t n_rp = (n_r + 15) / 16 * 16, kp = (k + 15) / 16 * 16;
@@ -262,16 +242,7 @@ __global__ void __launch_bounds__(256) fm_request_mma_kernel(int32_t n_r, int32_
       for (int j = 0; j < 2; ++j) {
         const int32_t c = c0 + g8 + j * 8, e = e0 + h * 8 + 2 * t4;
         const float v0 = acc[h][2 * j], v1 = acc[h][2 * j + 1];
-        if constexpr (PAIR) {
-          if (c < k) {
-            __nv_bfloat16* at = TT + ((int64_t)r * 2 * k + c) * d + e;
-            const __nv_bfloat162 value(pair_value(v0), pair_value(v1));
-            *reinterpret_cast<__nv_bfloat162*>(at) = value;
-            *reinterpret_cast<__nv_bfloat162*>(at + (int64_t)k * d) = __nv_bfloat162(pair_remainder(v0, value.x), pair_remainder(v1, value.y));
-          }
-        } else {
-          if (c < k) *reinterpret_cast<float2*>(TT + ((int64_t)r * k + c) * d + e) = make_float2(v0, v1);
-        }
+        if (c < k) *reinterpret_cast<float2*>(TT + ((int64_t)r * k + c) * d + e) = make_float2(v0, v1);
         const __nv_bfloat162 hi = __floats2bfloat162_rn(v0, v1);
         const __nv_bfloat162 lo = __floats2bfloat162_rn(v0 - __low2float(hi), v1 - __high2float(hi));
         *reinterpret_cast<__nv_bfloat162*>(th + c * x_row + e * 2) = hi;
@@ -627,25 +598,19 @@ rocs_status_t launch_fm(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t
   if (smem_r > kMaxSmem || smem_c > kMaxSmem) return ROCS_ERR_UNSUPPORTED;
   const size_t n_rp = (size_t)(n_r + 15) / 16 * 16, kp = (size_t)(k + 15) / 16 * 16;
   const size_t smem_mma = n_rp * ((size_t)(d + 8) * 2 + (kp + 8) * 2) + 2 * kp * (size_t)(d + 8) * 2;
-  const bool pair = fast_candidates && FC != nullptr && fm_umma_pays(plan, n_c, d, k);  // fm_umma.cu reads TT
-  if (plan->R > 0) {
-    const bool mma = tensor_core_request && sizeof(T) == 2 && d % 16 == 0 && k % 8 == 0 && smem_mma <= kMaxSmem;
-    auto run = [&](auto with_pair) {
-      constexpr bool kPair = decltype(with_pair)::value;
-      if (mma) {
-        ROCS_ALLOW_SMEM(fm_request_mma_kernel<kPair>, kMaxSmem);
-        return launch_dependent(fm_request_mma_kernel<kPair>, dim3((unsigned)plan->R), 256, smem_mma, stream, n_r, d, k,
-                                (const __nv_bfloat16*)XR, (const __nv_bfloat16*)P, (TermOf<kPair>*)TT, (__nv_bfloat16*)FR);
-      }
-      ROCS_ALLOW_SMEM((fm_request_kernel<T, kPair>), kMaxSmem);
-      return launch_dependent(fm_request_kernel<T, kPair>, dim3((unsigned)plan->R), 256, smem_r, stream, n_r, d, k,
-                              (const T*)XR, (const T*)P, (TermOf<kPair>*)TT, (T*)FR);
-    };
-    const rocs_status_t st = pair ? run(std::true_type()) : run(std::false_type());
+  if (plan->R > 0 && tensor_core_request && sizeof(T) == 2 && d % 16 == 0 && k % 8 == 0 && smem_mma <= kMaxSmem) {
+    ROCS_ALLOW_SMEM(fm_request_mma_kernel, kMaxSmem);
+    const rocs_status_t st = launch_dependent(fm_request_mma_kernel, dim3((unsigned)plan->R), 256, smem_mma, stream, n_r, d, k,
+                                              (const __nv_bfloat16*)XR, (const __nv_bfloat16*)P, TT, (__nv_bfloat16*)FR);
+    if (st != ROCS_OK) return st;
+  } else if (plan->R > 0) {
+    ROCS_ALLOW_SMEM(fm_request_kernel<T>, kMaxSmem);
+    const rocs_status_t st = launch_dependent(fm_request_kernel<T>, dim3((unsigned)plan->R), 256, smem_r, stream, n_r, d, k,
+                                              (const T*)XR, (const T*)P, TT, (T*)FR);
     if (st != ROCS_OK) return st;
   }
   if (plan->N == 0 || !FC) return ROCS_OK;
-  if (pair) return fm_umma(plan, n_r, n_c, d, k, XC, P, TT, FC, stream);
+  if (fast_candidates && fm_umma_pays(plan, n_c, d, k)) return fm_umma(plan, n_r, n_c, d, k, XC, P, TT, FC, stream);
   if (fast_candidates) {
     switch (d) {
       case 64: return launch_fm_mma<64>(plan, n_r, n_c, k, XC, P, TT, FC, stream);

@@ -322,10 +322,10 @@ rocs_status_t group_norm(rocs_dtype_t dt, int kind, int64_t M, int32_t d, const 
 // F = G P on the request-once form; tt_workspace [R, k, d] fp32 receives P_R^T X^R per request.
 // allow_fast: use the bf16 streaming kernel for the candidate side where the shape allows it.
 bool fm_projection_fast_supported(int32_t n_c, int32_t d, int32_t k);
-// Candidate rows on tcgen05 (fm_umma.cu), for the shapes above; TT as bf16 pairs [R, 2, k, d].
+// Candidate rows on tcgen05 (fm_umma.cu), for the shapes above.
 bool fm_umma_pays(const rocs_plan* plan, int32_t n_c, int32_t d, int32_t k);
 rocs_status_t fm_umma(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, int32_t k, const void* XC, const void* P,
-                      const void* TT, void* FC, cudaStream_t stream);
+                      const float* TT, void* FC, cudaStream_t stream);
 rocs_status_t fm_projection(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, int32_t k,
                             const void* XR, const void* XC, const void* P, void* FR, void* FC, float* tt_workspace,
                             bool allow_fast, cudaStream_t stream);

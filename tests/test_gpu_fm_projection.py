@@ -81,7 +81,7 @@ def test_bf16_streaming_kernel_with_partial_fragments(n_c, k, d_emb):
 
 @pytest.mark.parametrize("n_c,k,d_emb", [(12, 16, 128), (4, 24, 192), (15, 32, 256), (16, 18, 128), (16, 12, 64), (8, 8, 64)])
 def test_bf16_partial_fragments_are_as_exact_as_fp32_arithmetic(n_c, k, d_emb):
-    # Both kernels hold H to fp32 and round the result to bf16 once.  Sums of fp32 in another order differ by some 2^-20,
+    # Both kernels hold T and the candidate's own term to fp32 and round the result to bf16 once.  Sums of fp32 in another order differ by some 2^-20,
     # against the 2^-9 of that rounding: the errors against fp64 are the same up to which way close values are rounded
     # (well below 1 % of the norm over these thousands of values; H in bf16 would add about 40 %).
     co = wl.offsets_from_counts([1, 0, 9, 8, 33, 7, 0, 133])
@@ -115,6 +115,58 @@ def test_bf16_tiles_of_one_request(n_r, n_c, d_emb, k, law):
     N = int(co[-1])
     sample = np.unique(np.concatenate([g.integers(0, N, 400), [0, N - 1]]))
     assert _run(cfg, co, k, sample=sample) <= tol_for("bf16")
+def _bf16(a):
+    return torch.from_numpy(np.asarray(a, np.float32)).bfloat16()
+
+
+def _error_by_path(co, XR, XC, P):
+    """Relative error (2-norm) of FC against 64 bits on either path, and the 64-bit values."""
+    want = ref.glm_fm_projection(co, *[t.view(torch.uint16).numpy() for t in (XR, XC, P)])[:, XR.shape[1]:]
+    plan = rocs.plan_create(to_dev(co), co)
+    err = []
+    for path in PATHS:
+        rocs.set_path(path)
+        got = to_host_f64(rocs.glm_fm_projection(plan, XR.cuda(), XC.cuda(), P.cuda())["FC"])
+        err.append(np.linalg.norm(got - want) / np.linalg.norm(want))
+    return err, want
+
+
+@pytest.mark.parametrize("n_c,k,d_emb", [(12, 16, 128), (4, 24, 192), (15, 32, 256), (8, 8, 128), (5, 2, 192)])
+def test_bf16_request_term_keeps_its_24_bits(n_c, k, d_emb):
+    # T is M + M / 256 + delta, delta some 2^-14, and neighbouring values of the candidates cancel what the first two give: FC is
+    # X^C delta.  fp32 holds T to 2^-24 (2^-23 where a product's sum is cut off and not rounded), 2^-9 of delta at most; 17 bits
+    # to 2^-18, 4 % of FC.
+    g = np.random.default_rng(k)
+    co = wl.offsets_from_counts([4000, 0, 3, 2500])  # as many tiles as the tcgen05 kernel is taken for
+    R, N = len(co) - 1, int(co[-1])
+    M = np.repeat(1.0 + g.random((R, 2, d_emb // 2)), 2, axis=2) * np.array([[1.0], [2.0 ** -8]])
+    XR = _bf16(np.concatenate([M, 2.0 ** -14 * g.standard_normal((R, 1, d_emb))], axis=1))
+    half = g.standard_normal((N, n_c, d_emb // 2, 1))
+    XC = _bf16(np.concatenate([half, -half], axis=3).reshape(N, n_c, d_emb))
+    P = _bf16(np.concatenate([np.ones((3, k)), 2.0 ** -30 * g.standard_normal((n_c, k))]))
+    err, _ = _error_by_path(co, XR, XC, P)
+    assert err[1] <= 3e-3 and err[0] <= (1.01 * err[1] ** 2 + 2.0 ** -18) ** 0.5, err
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -70])
+@pytest.mark.parametrize("n_c,k,d_emb", [(12, 16, 128), (4, 24, 192), (15, 32, 256), (8, 8, 128), (5, 2, 192)])
+def test_bf16_terms_that_cancel(n_c, k, d_emb, scale):
+    # The candidates are small changes of their request's rows, and P_R = -P_C: X^C T and (X^C X^C^T) P_C are thousands of times
+    # their sum.  Both are fp32 sums, off by a few 2^-24 of what they add up (numpy: up to 2, 4 allowed), beside FC's rounding.
+    # Scaled, the squares lie below fp32's range, and their products with P_C do not.
+    g = np.random.default_rng(n_c)
+    co = wl.offsets_from_counts([7000, 0, 3, 90])
+    base = _bf16(g.standard_normal((4, n_c, d_emb))).double().numpy()
+    PC = _bf16(g.standard_normal((n_c, k)) / n_c ** 0.5).double().numpy()
+    X = np.repeat(base, np.diff(co), axis=0)
+    at = g.integers(0, n_c * d_emb, (len(X), 4))
+    np.put_along_axis(X.reshape(len(X), -1), at, np.take_along_axis(X.reshape(len(X), -1), at, 1) * (1 + 2.0 ** -6), 1)
+    X = _bf16(X).double().numpy()
+    err, want = _error_by_path(co, _bf16(base * scale), _bf16(X * scale), _bf16(np.concatenate([-PC, PC]) / scale))
+    T = -np.repeat(base.transpose(0, 2, 1) @ PC, np.diff(co), axis=0)
+    terms = np.abs(X) @ np.abs(T) + np.abs(X @ X.transpose(0, 2, 1)) @ np.abs(PC)
+    lost = 4 * 2.0 ** -24 * np.linalg.norm(terms * scale) / np.linalg.norm(want)
+    assert err[1] <= 2e-3 and err[0] <= (1.01 * err[1] ** 2 + lost ** 2) ** 0.5, (err, lost)
 
 
 @pytest.mark.parametrize("path", PATHS)
