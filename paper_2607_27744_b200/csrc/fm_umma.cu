@@ -74,21 +74,54 @@ __device__ __forceinline__ uint32_t take_upper(float& a, float& b) {
   return __byte_perm(ua, ub, 0x7632);
 }
 
-// One row in plain fp32, the request's and the candidate's own term added up before the row's product: for values that the
-// parts or the Gram matrix cannot hold (an infinity, a square out of fp32's range), where the result has to be what fp32 arithmetic gives.
-__device__ __noinline__ void row_by_hand(const __nv_bfloat16* xc, const __nv_bfloat16* row, const float* tt,
-                                         const __nv_bfloat16* pc, int32_t n_c, int32_t d, int32_t k, __nv_bfloat16* out) {
+// Rows of a warp's candidates in plain fp32, by the whole warp, the request's and the candidate's own term added up before a row's
+// product: for values that the parts or the Gram matrix cannot hold (an infinity, a square out of fp32's range), where the result
+// has to be what fp32 arithmetic gives.  A NaN in the request's term or among a candidate's values is one either way and is not
+// computed again: with a thread per row, which was done for those too, 18400 candidates with a NaN in two of their 100 requests took 20.7 ms.
+template <int NC>
+__device__ __noinline__ void rows_by_hand(uint32_t rows, const __nv_bfloat16* x, const float* tt, const __nv_bfloat16* pc,
+                                          int32_t n_c, int32_t d, int32_t k, __nv_bfloat16* out, int lane) {
+  constexpr int kMost = 8;  // d / 32
 #pragma unroll 1
-  for (int32_t c = 0; c < k; ++c) {
-    float acc = 0.f;
+  for (; rows != 0; rows >>= NC, x += n_c * d, out += n_c * k) {
+    const uint32_t mine = rows & ((1u << NC) - 1u);
+    if (mine == 0) continue;
+    bool looked = false;
 #pragma unroll 1
-    for (int32_t e = 0; e < d; ++e) {
-      float h = tt[c * d + e];
+    for (int32_t c = 0; c < k; ++c) {
+      float h[kMost];
+      bool nan = false;
+#pragma unroll
+      for (int i = 0; i < kMost; ++i) {
+        h[i] = 32 * i < d ? tt[c * d + 32 * i + lane] : 0.f;
+        nan = nan || isnan(h[i]);
+      }
+      if (__any_sync(0xffffffffu, nan)) continue;
+      if (!looked) {
+#pragma unroll 4
+        for (int32_t e = lane; e < n_c * d; e += 32) nan = nan || __hisnan(x[e]);
+        if (__any_sync(0xffffffffu, nan)) break;
+        looked = true;
+      }
+#pragma unroll 2
+      for (int32_t a = 0; a < n_c; ++a) {
+        const float w = __bfloat162float(pc[a * k + c]);
+#pragma unroll
+        for (int i = 0; i < kMost; ++i)
+          if (32 * i < d) h[i] = fmaf(w, __bfloat162float(x[a * d + 32 * i + lane]), h[i]);
+      }
 #pragma unroll 1
-      for (int32_t a = 0; a < n_c; ++a) h = fmaf(__bfloat162float(pc[a * k + c]), __bfloat162float(xc[a * d + e]), h);
-      acc = fmaf(__bfloat162float(row[e]), h, acc);
+      for (uint32_t left = mine; left != 0; left &= left - 1) {
+        const int32_t a = __ffs(left) - 1;
+        float sum = 0.f;
+#pragma unroll
+        for (int i = 0; i < kMost; ++i)
+          if (32 * i < d) sum = fmaf(__bfloat162float(x[a * d + 32 * i + lane]), h[i], sum);
+#pragma unroll
+        for (int o = 16; o > 0; o /= 2) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) out[a * k + c] = __float2bfloat16_rn(sum);
+      }
     }
-    out[c] = __float2bfloat16_rn(acc);
   }
 }
 
@@ -281,13 +314,13 @@ fm_umma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmUmmaParams p)
       tc_fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tmem_empty[acc]);
+      bool by_hand = false;
       if (a_row < p.n_c && cand_l < tile.count) {
         uint64_t out[KP / 2];
 #pragma unroll
         for (int c = 0; c < KP; c += 2)
           out[c / 2] = pack2(__uint_as_float(val[c]) + __uint_as_float(rem[c]), __uint_as_float(val[c + 1]) + __uint_as_float(rem[c + 1]));
-        float probe = 0.f;  // not 0 behind an infinity or a NaN among this row's values
-        float most = 0.f;   // the largest of the row's products with its candidate's rows
+        float most = 0.f;  // the largest of the row's products with its candidate's rows
 #pragma unroll
         for (int j = 0; j < NC; ++j) {
           if (j >= p.n_c) break;
@@ -296,7 +329,6 @@ fm_umma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmUmmaParams p)
 #pragma unroll
           for (int s = 1; s < 32 / NC; ++s) x = sub == s ? vcc[s * NC + j] : x;
           const float gram = __uint_as_float(x);
-          probe = fmaf(gram, 0.f, probe);
           most = fmaxf(most, fabsf(gram));
           const uint64_t gram2 = pack2(gram, gram);
 #pragma unroll
@@ -307,23 +339,15 @@ fm_umma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmUmmaParams p)
           }
         }
         float f[KP];
+        float probe = 0.f;  // not 0 behind an infinity or a NaN among this row's values, which one of its products also gives
 #pragma unroll
         for (int c = 0; c < KP; c += 2) {
           unpack2(out[c / 2], f[c], f[c + 1]);
           if (c < p.k) probe = fmaf(f[c], 0.f, fmaf(f[c + 1], 0.f, probe));  // (k is even)
         }
-        if (most < kSmallProduct) {
-          bool zeros = most == 0.f;
-#pragma unroll
-          for (int c = 0; c < KP; ++c) zeros = zeros && (c >= p.k || f[c] == 0.f);
-          if (!zeros) probe = 1.f;
-        }
         const int64_t cand = (int64_t)tile.cand0 + cand_l;
         __nv_bfloat16* dst = p.FC + (cand * p.n_c + a_row) * p.k;
-        if (probe != 0.f) {
-          const __nv_bfloat16* xc = p.XC + cand * p.n_c * p.d;
-          row_by_hand(xc, xc + a_row * p.d, p.TT + (int64_t)tile.req * p.k * p.d, p.P + (int64_t)p.n_r * p.k, p.n_c, p.d, p.k, dst);
-        } else if (p.k % 8 == 0) {
+        if (p.k % 8 == 0) {
 #pragma unroll
           for (int c = 0; c < KP; c += 8)
             if (c < p.k)
@@ -334,6 +358,20 @@ fm_umma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmUmmaParams p)
           for (int c = 0; c < KP; c += 2)
             if (c < p.k) *reinterpret_cast<uint32_t*>(dst + c) = pack_bf16(f[c], f[c + 1]);
         }
+        by_hand = probe != 0.f;
+        if (most < kSmallProduct) {
+          bool zeros = most == 0.f;  // a row of zeros
+#pragma unroll
+          for (int c = 0; c < KP; ++c) zeros = zeros && (c >= p.k || f[c] == 0.f);
+          by_hand = !zeros;
+        }
+      }
+      const uint32_t rows = __ballot_sync(0xffffffffu, by_hand);
+      if (rows != 0) {
+        __syncwarp();  // their values are written again
+        const int64_t first = (int64_t)tile.cand0 + q * 32 / NC;  // the warp's candidates
+        rows_by_hand<NC>(rows, p.XC + first * p.n_c * p.d, p.TT + (int64_t)tile.req * p.k * p.d, p.P + (int64_t)p.n_r * p.k, p.n_c, p.d, p.k,
+                         p.FC + first * p.n_c * p.k, lane);
       }
       __syncwarp();
     }

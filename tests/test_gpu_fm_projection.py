@@ -169,6 +169,42 @@ def test_bf16_terms_that_cancel(n_c, k, d_emb, scale):
     assert err[1] <= 2e-3 and err[0] <= (1.01 * err[1] ** 2 + lost ** 2) ** 0.5, (err, lost)
 
 
+@pytest.mark.parametrize("where", ["XR nan", "XR inf", "XC nan", "XC inf", "P request nan", "P candidate inf", "XC huge"])
+@pytest.mark.parametrize("n_c,k,d_emb", [(12, 16, 128), (4, 24, 192), (16, 20, 128), (8, 10, 128), (15, 32, 256)])
+def test_bf16_values_out_of_range_show_as_in_fp32(n_c, k, d_emb, where):
+    # NaN, infinity and squares past fp32 in some rows of a batch of many tiles: the same values are NaN or infinite as on the
+    # general path, and the others' bits do not change
+    g = np.random.default_rng(n_c)
+    co = wl.offsets_from_counts(g.integers(0, 100, 130).tolist())
+    cfg = wl.CONFIGS[4].with_(R=len(co) - 1, n_r=20, n_c=n_c, d_emb=d_emb)
+    d = wl.glm_inputs(cfg, co)
+    d["P"] = wl.fm_projection_weight(cfg, k)
+    plan = rocs.plan_create(to_dev(co), co)
+    run = lambda: rocs.glm_fm_projection(plan, *[to_dev(d[n]) for n in ("XR", "XC", "P")])["FC"]
+    before = _bits(run())
+    bits = {"nan": 0x7fc0, "inf": 0x7f80, "huge": 0x6500}[where.split()[-1]]
+    if where.startswith("P"):
+        d["P"][3 if "request" in where else 20 + n_c - 1, k // 2] = bits
+        touched = np.ones(len(before), bool)
+    elif where.startswith("XR"):
+        d["XR"][[5, 77], [2, 19], [7, 63]] = bits
+        touched = np.isin(np.repeat(np.arange(cfg.R), np.diff(co)), [5, 77])
+    else:
+        rows = [0, 33, 34, len(before) - 1]
+        d["XC"][rows, [0, n_c - 1, 1, 2], [1, 0, d_emb - 1, 5]] = bits
+        touched = np.isin(np.arange(len(before)), rows)
+    kinds, got = [], None
+    for path in PATHS:
+        rocs.set_path(path)
+        out = run()
+        got = _bits(out) if got is None else got
+        out = to_host_f64(out)
+        kinds.append(np.where(np.isnan(out), 2, np.where(np.isinf(out), np.sign(out), 0)))
+    assert np.array_equal(kinds[0], kinds[1])
+    assert np.any(kinds[1][touched] != 0) or where == "XC huge"
+    assert np.array_equal(got[~touched], before[~touched])
+
+
 @pytest.mark.parametrize("path", PATHS)
 def test_bf16_shapes_outside_the_streaming_kernel(path):
     co = wl.offsets_from_counts([20, 3, 41])
