@@ -735,13 +735,9 @@ rocs_status_t rocs_glm_interaction(const rocs_plan_t* plan, rocs_dtype_t dtype, 
       return ROCS_ERR_WORKSPACE;
     zr = (float*)workspace;
   }
-  // Few products: the general kernels, whose request side is in the candidates' launch.  bf16, plan kept, tensor cores and
-  // general kernels: 20 / 320 / 640 candidates of 24 + 8 embeddings x 128, raw (0.6 / 10 / 20 M products), 6.9 / 7.0 / 6.8 and
-  // 4.6 / 5.7 / 7.9 us; 40 / 160 / 320 of 20 + 12 x 64 to 4 + 4 (0.9 / 3.8 / 7.5 M) 6.8 / 6.8 / 6.8 and 5.7 / 6.1 / 7.3;
-  // 640 of 8 + 4 x 64, raw (1.9 M), 6.8 and 4.1; but 8 of 32 + 16 x 128 to 8 + 8 (0.8 M) 7.1 and 7.7: W_CR X^R is then long.
-  constexpr int64_t kFewProducts = 1 << 22;
-  if (dtype == ROCS_BF16 && g_path.load() == ROCS_PATH_AUTO && plan->R <= 128 && (YC || OC) &&
-      plan->N * n_c * (n_r + n_c) * d <= kFewProducts && (!OC || n_co == 0 || n_r * d <= 2048)) {
+  // Few products: the general kernels, whose request side is in the candidates' launch.
+  if (dtype == ROCS_BF16 && g_path.load() == ROCS_PATH_AUTO && (YC || OC) &&
+      simt_glm_pays(plan, n_r, n_c, d, n_co, OC != nullptr && n_co > 0)) {
     const rocs_status_t st = simt_glm(dtype, plan, n_r, n_c, d, XR, XC, W, n_ro, n_co, YR, YC, OR_, OC, zr, stream);
     if (st != ROCS_ERR_UNSUPPORTED) return st;
   }

@@ -309,6 +309,7 @@ rocs_status_t simt_linear_both(const rocs_plan* plan, int32_t d_req, int32_t d_c
 rocs_status_t simt_dca(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_q, int32_t H, int32_t dh,
                        float scale, const void* Q, const void* K, const void* V,
                        const int32_t* seq_offsets, int64_t T, void* O, cudaStream_t stream);
+bool simt_glm_pays(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, int32_t n_co, bool compress);
 rocs_status_t simt_glm(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d,
                        const void* XR, const void* XC, const void* W, int32_t n_ro, int32_t n_co,
                        void* YR, void* YC, void* OR_, void* OC, float* zr_workspace,

@@ -353,6 +353,25 @@ static rocs_status_t launch_glm(const rocs_plan* plan, int32_t n_r, int32_t n_c,
 #undef ROCS_LAUNCH
 }
 
+// Where a small bf16 batch is faster here than on the tensor-core kernels, which are two launches: few products, and none of the
+// chains long that a block's lanes make of a request's own products or of a candidate's (with compression W_CR X^R and its products
+// too).  Plan kept, tensor cores and general kernels, us: 20 / 320 / 640 candidates of 24 + 8 embeddings x 128, raw (0.6 / 10 / 20 M
+// products), 6.9 / 7.0 / 6.8 and 4.6 / 5.7 / 7.9; 40 / 160 / 320 of 20 + 12 x 64 to 4 + 4 (0.9 / 3.8 / 7.5 M) 6.8 / 6.8 / 6.8 and 5.7 / 6.1 /
+// 7.3; 640 of 8 + 4 x 64, raw (1.9 M), 6.8 and 4.1.  Chains, a candidate each of one / of 100 requests, raw: 32 embeddings x 64 / 128 / 192 (32 /
+// 64 / 96 steps) 4.9 / 5.1 / 4.5 and 3.9 / 4.7 / 5.7, 6.2 / 6.8 / 6.8 and 4.6 / 6.0 / 7.0; 40 x 64 (64) 5.1 and 5.1, 7.2 and 6.0; 48 x 64 (128) 4.5
+// and 7.2, 7.4 and 8.3; 48 x 192 (384) 5.6 and 13.4, 9.2 and 16.2.  To 8 + 8, 8 of one request: 16 + 8 x 128 (32) 6.2 and 6.0, 16 + 16 x
+// 128 (64) 5.6 and 7.1, 32 + 16 x 128 7.1 and 7.7.
+bool simt_glm_pays(const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d, int32_t n_co, bool compress) {
+  constexpr int64_t kFewProducts = 1 << 22;
+  if (plan->R > kGlmThreads || plan->N * n_c * (n_r + n_c) * d > kFewProducts) return false;
+  auto steps = [&](int32_t items) {
+    const int32_t ks = lanes_per_item(items, kGlmThreads);
+    return (int64_t)((items + kGlmThreads / ks - 1) / (kGlmThreads / ks)) * (d / ks);
+  };
+  const int32_t q = (n_r + 3) / 4, own = (n_c + 3) / 4, rows = (n_c + (compress ? n_co : 0) + 3) / 4;
+  return steps(q * q) <= 64 && steps(rows * q + own * own) <= (compress ? 32 : 64) && (!compress || (int64_t)n_r * d <= 2048);
+}
+
 // YC == OC == nullptr runs only the request side (used in front of the tensor-core candidate
 // kernel); XC == nullptr is then allowed.
 rocs_status_t simt_glm(rocs_dtype_t dt, const rocs_plan* plan, int32_t n_r, int32_t n_c, int32_t d,
