@@ -50,16 +50,18 @@ def test_bf16_ragged_segments_and_tail_tile(path, k, d_emb):
     assert _run(cfg, co, k, path=path) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("n_c,k", [(16, 8), (16, 16), (12, 8), (4, 8)])
 @pytest.mark.parametrize("law", ["short", "gaps", "long"])
-def test_bf16_streaming_kernel_walks_the_requests(law):
-    # a warp's candidates ascend by 8: the next request, the one behind a run of empty ones, the same one
+def test_bf16_streaming_kernel_walks_the_requests(law, n_c, k):
+    # a warp's candidates ascend by 8 or 15, in several tiles per CTA: the next request, the one behind a run of empty ones, the same
+    # one (4 embeddings: by more than two candidates per tile the walk over tiles of the tcgen05 kernel)
     g = np.random.default_rng(5)
     counts = {"short": g.integers(0, 4, 9000), "gaps": np.where(g.random(9000) < 0.02, g.integers(1, 150, 9000), 0),
               "long": g.integers(500, 3000, 9)}[law]
     co = wl.offsets_from_counts(counts.tolist())
-    cfg = wl.CONFIGS[4].with_(R=len(co) - 1, n_r=4, n_c=4, d_emb=64)
+    cfg = wl.CONFIGS[4].with_(R=len(co) - 1, n_r=4, n_c=n_c, d_emb=64)
     sample = np.unique(np.concatenate([g.integers(0, co[-1], 600), [0, co[-1] - 1]]))
-    assert _run(cfg, co, 8, sample=sample) <= tol_for("bf16")
+    assert _run(cfg, co, k, sample=sample) <= tol_for("bf16")
 
 
 @pytest.mark.parametrize("n_c,k,d_emb", [(12, 16, 128), (4, 24, 192), (1, 2, 64), (15, 32, 256), (16, 18, 128), (8, 10, 64)])

@@ -62,12 +62,13 @@ def test_linear_bf16_ragged_segments_several_tiles(path, relu, bias):
     assert _run_linear(cfg, co, bias=bias, relu=relu, path=path) <= tol_for("bf16")
 
 
+@pytest.mark.parametrize("requests,most", [(70, 41), (800, 21)])
 @pytest.mark.parametrize("relu,bias", [(False, False), (True, True)])
-def test_linear_bf16_narrow_input_many_short_segments(relu, bias):
-    # N >= 512 with d_cand <= 256 takes the weight-stationary kernel; segments of 0..40 rows put
-    # several requests into every 32-row slab, so both the shared-memory and the global request
-    # rows are exercised; d_out = 328 leaves a ragged last column slice
-    counts = [(i * 7) % 41 for i in range(70)]
+def test_linear_bf16_narrow_input_many_short_segments(relu, bias, requests, most):
+    # 8000 rows with d_cand <= 256 take the weight-stationary kernel, and segments of 0..20 rows put more requests into a run of
+    # 256 rows than one launch holds: several in every 32-row slab, so both the shared-memory and the global request rows are
+    # exercised; d_out = 328 leaves a ragged last column slice.  1393 rows are one launch of small tiles
+    counts = [(i * 7) % most for i in range(requests)]
     co = wl.offsets_from_counts(counts)
     cfg = wl.CONFIGS[5].with_(R=len(counts), d_req=64, d_cand=200, d_out=328)
     assert _run_linear(cfg, co, bias=bias, relu=relu) <= tol_for("bf16")
@@ -139,8 +140,8 @@ def test_plain_linear_tile_widths(M, d_out):
 
 @pytest.mark.parametrize("N", [1, 7, 9, 127, 129, 500, 511, 16384, 16385])
 def test_linear_few_rows_and_both_request_maps(N):
-    # X tiles of fewer than 128 rows, the candidate half that waits for the request half in its epilogue only
-    # (below 512 rows), the request searched in the offsets (up to 16384 rows) or read from the table
+    # X tiles of fewer than 128 rows, both halves in one launch (few requests per tile or run of rows), on small tiles
+    # below 512 rows and on CTA pairs
     counts = [0, N // 3, 1, 0, N - N // 3 - 1, 0] if N > 1 else [0, 1]
     co = wl.offsets_from_counts(counts)
     cfg = wl.CONFIGS[2].with_(R=len(counts), d_req=136, d_cand=320 if N < 512 else 72, d_out=192)
@@ -165,10 +166,21 @@ def test_plain_linear_small_tiles(M, d_in, d_out):
 
 @pytest.mark.parametrize("N", [1, 40, 129, 300])
 def test_linear_halves_in_small_tiles(N):
-    # the request half in fp32 tiles of 32 columns, the candidate half waiting for it in its epilogue only
+    # a request half longer than the candidate half, in one launch
     counts = [0, N // 3, 1, 0, N - N // 3 - 1, 0] if N > 1 else [0, 1]
     co = wl.offsets_from_counts(counts)
     cfg = wl.CONFIGS[2].with_(R=len(counts), d_req=1032, d_cand=520, d_out=200)
+    assert _run_linear(cfg, co, bias=True, relu=True) <= tol_for("bf16")
+
+
+@pytest.mark.parametrize("N", [2, 33, 127, 500])
+@pytest.mark.parametrize("d_req,d_cand", [(136, 72), (136, 320), (1032, 520)])
+def test_linear_halves_apart_in_small_tiles(N, d_req, d_cand):
+    # a run of 150 requests without candidates inside a tile, more than its rows: the halves are two launches, the candidate
+    # half waits for the request half in its epilogue only and searches the request in the offsets
+    counts = [0, N // 2, *[0] * 150, N - N // 2, 0]
+    co = wl.offsets_from_counts(counts)
+    cfg = wl.CONFIGS[2].with_(R=len(counts), d_req=d_req, d_cand=d_cand, d_out=192)
     assert _run_linear(cfg, co, bias=True, relu=True) <= tol_for("bf16")
 
 
@@ -664,8 +676,10 @@ def test_glm_bf16_ragged(path, which):
 
 
 @pytest.mark.parametrize("path", PATHS)
-def test_glm_bf16_other_split(path):
-    co = wl.offsets_from_counts([20, 3])
+@pytest.mark.parametrize("per", [20, 200])
+def test_glm_bf16_other_split(path, per):
+    # 203 candidates are more products than the general kernels take of themselves
+    co = wl.offsets_from_counts([per, 3])
     cfg = wl.CONFIGS[4].with_(R=2, n_r=16, n_c=16, d_emb=64, n_ro=4, n_co=12)
     assert _run_glm(cfg, co, path=path) <= tol_for("bf16")
 
@@ -725,7 +739,8 @@ def test_glm_fragments(n_r, n_c, d, n_co, raw, many):
     # columns that end inside a group of 16 and take several passes, fewer fragments than warps; a candidate
     # and a request full of NaN must show in their own rows only
     counts = [1, 0, 9, 8, 33, 7, 0, 133] * (30 if many else 1)
-    co = wl.offsets_from_counts(counts + ([3000] if many and n_c < 8 else []))
+    counts += [3000] if many and n_c < 8 else [0] * 125  # (few products of up to 128 requests are the general kernels')
+    co = wl.offsets_from_counts(counts)
     cfg = wl.CONFIGS[4].with_(R=len(co) - 1, n_r=n_r, n_c=n_c, d_emb=d, n_ro=min(2, n_co), n_co=n_co)
     g = wl.glm_inputs(cfg, co)
     plan, W = _plan(co), to_dev(g["W"]) if n_co else None
@@ -756,7 +771,7 @@ def test_glm_fragments_are_as_exact_as_fp32_arithmetic(n_r, n_c, d, n_co, raw):
     # Both kernels compress the fp32 products and round the result to bf16 once.  Sums of fp32 in another order differ by
     # some 2^-20, against the 2^-9 of that rounding: the errors against fp64 are the same up to which way close values are
     # rounded (well below 1 % of the norm over these thousands of values; products rounded first would add about 20 %).
-    co = wl.offsets_from_counts([1, 0, 9, 8, 33, 7, 0, 133])
+    co = wl.offsets_from_counts([1, 0, 9, 8, 33, 7, 0, 133] + [0] * 125)  # (few products of up to 128 requests are one kernel on both paths)
     cfg = wl.CONFIGS[4].with_(R=len(co) - 1, n_r=n_r, n_c=n_c, d_emb=d, n_ro=2, n_co=n_co)
     g = wl.glm_inputs(cfg, co)
     want = ref.glm_interaction(co, g["XR"], g["XC"], g["W"], cfg.n_ro, n_co)[1][:, cfg.n_ro:]
@@ -768,12 +783,14 @@ def test_glm_fragments_are_as_exact_as_fp32_arithmetic(n_r, n_c, d, n_co, raw):
     XC, W = g["XC"].copy(), g["W"].copy()
     XC[60, 1, 5] = 0x7f80                          # infinities show in the same values either way
     W[cfg.n_ro + n_co - 1, n_r + n_c - 1] = 0xff80
-    err, kinds = [], []
+    err, kinds, values = [], [], []
     for path in PATHS:
         rocs.set_path(path)
         got = run(g["XC"], g["W"])
+        values.append(got)
         err.append(np.linalg.norm(got - want) / np.linalg.norm(want))
         kinds.append([np.where(np.isnan(o), 2, np.where(np.isinf(o), np.sign(o), 0)) for o in (run(XC, g["W"]), run(g["XC"], W))])
+    assert not np.array_equal(*values), "the same kernel on both paths"
     assert err[0] <= 1.01 * err[1]
     for auto, general in zip(*kinds):
         assert np.array_equal(auto, general) and np.any(auto[60] != 0)
@@ -784,7 +801,8 @@ def test_work_lists_of_many_requests(R):
     # the lists are scanned by 256 threads per block up to 12000 requests and on the host beyond: counts of
     # 0..3 candidates put empty requests at both ends of every thread's share
     co = wl.offsets_from_counts([(i * 5 + 3) % 4 for i in range(R)])
-    assert _run_glm(wl.CONFIGS[5].with_(R=R, n_r=8, d_emb=64, n_ro=0, n_co=0), co) <= tol_for("bf16")
+    # (48 embeddings of up to 128 requests: with 8 so few products are the general kernels')
+    assert _run_glm(wl.CONFIGS[5].with_(R=R, n_r=48 if R <= 128 else 8, d_emb=64, n_ro=0, n_co=0), co) <= tol_for("bf16")
     so = wl.offsets_from_counts([(i * 3) % 5 for i in range(R)])
     assert _run_dca(wl.CONFIGS[3].with_(R=R, H=2, dh=8), co, so) <= tol_for("bf16")
     assert _run_dca(wl.CONFIGS[3].with_(R=R, H=2, dh=32), co, so) <= tol_for("bf16")
@@ -795,7 +813,7 @@ def test_work_lists_of_many_requests(R):
 def test_glm_tiles_walked_in_the_offsets(R, n_c):
     # runs of tiles that begin and end inside requests, behind partial last tiles and runs of empty requests
     g = np.random.default_rng(R)
-    co = wl.offsets_from_counts([int(c) for c in g.choice([0, 0, 1, 7, 16, 17, 40], R - 1)] + [23])
+    co = wl.offsets_from_counts([int(c) for c in g.choice([0, 0, 1, 7, 16, 17, 40], R - 1)] + [23 if R > 128 else 623])  # (more products than the general kernels take)
     assert _run_glm(wl.CONFIGS[5].with_(R=R, n_r=8, n_c=n_c, d_emb=64, n_ro=2, n_co=4), co) <= tol_for("bf16")
 
 
