@@ -82,11 +82,12 @@ def test_bf16_streaming_kernel_with_partial_fragments(n_c, k, d_emb):
 
 
 @pytest.mark.parametrize("n_c,k,d_emb", [(12, 16, 128), (4, 24, 192), (15, 32, 256), (16, 18, 128), (16, 12, 64), (8, 8, 64)])
-def test_bf16_partial_fragments_are_as_exact_as_fp32_arithmetic(n_c, k, d_emb):
+@pytest.mark.parametrize("counts", [[1, 0, 9, 8, 33, 7, 0, 133], [1, 0, 2] * 70])
+def test_bf16_partial_fragments_are_as_exact_as_fp32_arithmetic(n_c, k, d_emb, counts):
     # Both kernels hold T and the candidate's own term to fp32 and round the result to bf16 once.  Sums of fp32 in another order differ by some 2^-20,
     # against the 2^-9 of that rounding: the errors against fp64 are the same up to which way close values are rounded
     # (well below 1 % of the norm over these thousands of values; H in bf16 would add about 40 %).
-    co = wl.offsets_from_counts([1, 0, 9, 8, 33, 7, 0, 133])
+    co = wl.offsets_from_counts(counts)  # (short requests are the streaming kernel's)
     cfg = wl.CONFIGS[4].with_(R=len(co) - 1, n_r=20, n_c=n_c, d_emb=d_emb)
     d, P = wl.glm_inputs(cfg, co), wl.fm_projection_weight(cfg, k)
     want = ref.glm_fm_projection(co, d["XR"], d["XC"], P)[:, cfg.n_r:]
@@ -104,14 +105,16 @@ def test_bf16_partial_fragments_are_as_exact_as_fp32_arithmetic(n_c, k, d_emb):
     assert np.array_equal(kinds[0], kinds[1]) and np.any(kinds[1][60] != 0)
 
 
-@pytest.mark.parametrize("law", ["few", "many", "sparse"])
+@pytest.mark.parametrize("law", ["few", "many", "sparse", "short"])
 @pytest.mark.parametrize("n_r,n_c,d_emb,k", [(20, 12, 128, 16), (5, 3, 64, 2), (24, 4, 192, 24), (16, 5, 64, 14), (48, 8, 256, 32), (7, 9, 128, 22),
                                              (20, 16, 64, 24), (33, 15, 192, 8), (16, 1, 128, 16)])
 def test_bf16_tiles_of_one_request(n_r, n_c, d_emb, k, law):
     # tiles of 8 to 32 candidates of one request, rows behind a candidate's embeddings and columns behind k; fewer tiles than a
-    # ring has stages and runs that take ring and accumulators several times; more requests than threads, most of them empty
+    # ring has stages and runs that take ring and accumulators several times; more requests than threads, most of them empty;
+    # a candidate or two per request, which the streaming kernel takes
     g = np.random.default_rng(k)
-    counts = {"few": [3, 0, 33, 1], "many": g.integers(0, 130, 300), "sparse": np.where(g.random(3000) < 0.2, g.integers(1, 40, 3000), 0)}[law]
+    counts = {"few": [3, 0, 33, 1], "many": g.integers(0, 130, 300), "sparse": np.where(g.random(3000) < 0.2, g.integers(1, 40, 3000), 0),
+              "short": g.integers(0, 3, 600)}[law]
     co = wl.offsets_from_counts(np.asarray(counts).tolist())
     cfg = wl.CONFIGS[4].with_(R=len(co) - 1, n_r=n_r, n_c=n_c, d_emb=d_emb)
     N = int(co[-1])
