@@ -170,6 +170,7 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
       if constexpr (BOTH) part[(KS * BM + ty + 8 * i) * PS + tx + 8 * j] = acc_r[i][j];
     }
   __syncthreads();
+  static_assert(!BOTH || BM * BN <= kGroup * KS, "the request half's sums are added up below only");
   if constexpr (BM * BN <= kGroup * KS) {
     // a value per thread: a chain of four-wide sums on few threads was longer (1850 candidates, 64|32 -> 64, fp32:
     // 9.1 us, 8.8 so)
@@ -189,72 +190,62 @@ __global__ void __launch_bounds__(kGroup* KS, TM == 8 ? 3 : 1) linear_simt_kerne
     }
     if (act == ROCS_ACT_RELU) v = fmaxf(v, 0.f);
     st_f(Y + (m0 + r) * ld_y + n, v);
-    return;
-  }
-  // Four neighbouring columns of kRowsEach rows per thread.  The request rows are all asked for before the first is
-  // used: one at a time, every row of a tile waited for the L2 cache.
-  constexpr int kPerRow = BN / 4, kThreads = kGroup * KS, kRowStep = kThreads / kPerRow, kRowsEach = BM / kRowStep;
-  static_assert(kThreads % kPerRow == 0 && (BM % kRowStep == 0 || kRowStep > BM), "rows of a tile over the threads");
-  const int32_t c4 = threadIdx.x % kPerRow * 4, r0 = threadIdx.x / kPerRow, n = n0 + c4;
-  const int32_t cols = min(d_out - n, 4);
-  if (r0 >= BM || cols <= 0) return;
-  constexpr int kEach = kRowsEach > 0 ? kRowsEach : 1;
-  float4 z[kEach];
+  } else {
+    // Four neighbouring columns of kRowsEach rows per thread.  The request rows are all asked for before the first is
+    // used: one at a time, every row of a tile waited for the L2 cache.
+    constexpr int kPerRow = BN / 4, kThreads = kGroup * KS, kRowStep = kThreads / kPerRow, kRowsEach = BM / kRowStep;
+    static_assert(kThreads % kPerRow == 0 && BM % kRowStep == 0, "rows of a tile over the threads");
+    const int32_t c4 = threadIdx.x % kPerRow * 4, r0 = threadIdx.x / kPerRow, n = n0 + c4;
+    const int32_t cols = min(d_out - n, 4);
+    if (cols <= 0) return;
+    float4 z[kRowsEach];
 #pragma unroll
-  for (int u = 0; u < kEach; ++u) {
-    const int32_t r = r0 + u * kRowStep;
-    z[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (add && m0 + r < M) {
-      const float* from = add + (int64_t)req[r] * ld_add + n;
-      if (cols == 4 && ld_add % 4 == 0) {
-        z[u] = *reinterpret_cast<const float4*>(from);
-      } else {
-        z[u].x = from[0];
-        if (cols > 1) z[u].y = from[1];
-        if (cols > 2) z[u].z = from[2];
-        if (cols > 3) z[u].w = from[3];
+    for (int u = 0; u < kRowsEach; ++u) {
+      const int32_t r = r0 + u * kRowStep;
+      z[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (add && m0 + r < M) {
+        const float* from = add + (int64_t)req[r] * ld_add + n;
+        if (cols == 4 && ld_add % 4 == 0) {
+          z[u] = *reinterpret_cast<const float4*>(from);
+        } else {
+          z[u].x = from[0];
+          if (cols > 1) z[u].y = from[1];
+          if (cols > 2) z[u].z = from[2];
+          if (cols > 3) z[u].w = from[3];
+        }
       }
     }
-  }
-  float b4[4] = {0.f, 0.f, 0.f, 0.f};
-  if (bias)
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-      if (c < cols) b4[c] = bias[n + c];
-#pragma unroll
-  for (int u = 0; u < kEach; ++u) {
-    const int32_t r = r0 + u * kRowStep;
-    if (m0 + r >= M) break;
-    float4 v4 = *reinterpret_cast<const float4*>(sm + r * PS + c4);
-#pragma unroll
-    for (int g = 1; g < KS; ++g) {
-      const float4 o = *reinterpret_cast<const float4*>(sm + (g * BM + r) * PS + c4);
-      v4.x += o.x; v4.y += o.y; v4.z += o.z; v4.w += o.w;
-    }
-    float v[4] = {v4.x, v4.y, v4.z, v4.w};
-    if constexpr (BOTH) {
-#pragma unroll
-      for (int g = 0; g < KS; ++g) {
-        const float4 o = *reinterpret_cast<const float4*>(sm + ((KS + g) * BM + r) * PS + c4);
-        z[u].x += o.x; z[u].y += o.y; z[u].z += o.z; z[u].w += o.w;
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) v[c] += lane_of(z[u], c) + b4[c];
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      if (!BOTH && bias) v[c] += b4[c];
-      if (add) v[c] += lane_of(z[u], c);
-      if (act == ROCS_ACT_RELU) v[c] = fmaxf(v[c], 0.f);
-    }
-    TOut* out = Y + (m0 + r) * ld_y + n;  // rows start on 16-byte boundaries and n is a multiple of 4
-    if (cols == 4) {
-      store_pair(out, v[0], v[1]);
-      store_pair(out + 2, v[2], v[3]);
-    } else {
+    float b4[4] = {0.f, 0.f, 0.f, 0.f};
+    if (bias)
 #pragma unroll
       for (int c = 0; c < 4; ++c)
-        if (c < cols) st_f(out + c, v[c]);
+        if (c < cols) b4[c] = bias[n + c];
+#pragma unroll
+    for (int u = 0; u < kRowsEach; ++u) {
+      const int32_t r = r0 + u * kRowStep;
+      if (m0 + r >= M) break;
+      float4 v4 = *reinterpret_cast<const float4*>(sm + r * PS + c4);
+#pragma unroll
+      for (int g = 1; g < KS; ++g) {
+        const float4 o = *reinterpret_cast<const float4*>(sm + (g * BM + r) * PS + c4);
+        v4.x += o.x; v4.y += o.y; v4.z += o.z; v4.w += o.w;
+      }
+      float v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (bias) v[c] += b4[c];
+        if (add) v[c] += lane_of(z[u], c);
+        if (act == ROCS_ACT_RELU) v[c] = fmaxf(v[c], 0.f);
+      }
+      TOut* out = Y + (m0 + r) * ld_y + n;  // rows start on 16-byte boundaries and n is a multiple of 4
+      if (cols == 4) {
+        store_pair(out, v[0], v[1]);
+        store_pair(out + 2, v[2], v[3]);
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (c < cols) st_f(out + c, v[c]);
+      }
     }
   }
 }
