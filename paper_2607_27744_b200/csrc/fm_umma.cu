@@ -7,7 +7,7 @@
 // T, of what is left and of what is left then, which add up to its 24 bits: four warps split it into the tile's stage, where it
 // stays as long as the stage's tiles are of that request.  (Two parts, 17 bits, are as exact on independent inputs; where X^C T is
 // what little its values do not cancel of each other they are not.)  Both terms are fp32 sums and meet behind their
-// products: where they cancel, FC is exact to fp32 of the terms, not of their sum.
+// products; rows in which they cancel to less than a 64th are computed by hand, both terms added up in front of the product.
 // Per 64-wide slice of d shared memory holds [T_3 ; T_2 ; T_1 ; X^C tile] back to back, each part k rows (to a multiple of 8),
 // so that a single tcgen05.mma per 16-deep K step computes
 //     D[128, 3 kp + 128] = X^C_tile * [T_3 ; T_2 ; T_1 ; X^C_tile]^T
@@ -65,6 +65,9 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // Rows whose products with their candidate's rows are all below this are computed by hand: what fp32's range cuts off of them
 // may count where P_C is large.
 constexpr float kSmallProduct = 0x1p-90f;
+// And rows in which the two terms cancel to less than this part of the request's: what fp32 sums lose of the terms (some 2^-21 of them)
+// stays below 2^-15 of the row then, a hundredth of its rounding to bf16.
+constexpr float kCancelled = 64.f;
 
 // The upper halves of two values as a bf16 pair, and what is left of them.
 __device__ __forceinline__ uint32_t take_upper(float& a, float& b) {
@@ -341,9 +344,12 @@ fm_umma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmUmmaParams p)
       bool by_hand = false;
       if (a_row < p.n_c && cand_l < tile.count) {
         uint64_t out[KP / 2];
+        uint64_t square_t = 0, square_f = 0;  // of the request's term and of the sum, two chains each
 #pragma unroll
-        for (int c = 0; c < KP; c += 2)
+        for (int c = 0; c < KP; c += 2) {
           out[c / 2] = pack2(__uint_as_float(val[c]) + __uint_as_float(rem[c]), __uint_as_float(val[c + 1]) + __uint_as_float(rem[c + 1]));
+          if (c < p.k) square_t = ffma2(out[c / 2], out[c / 2], square_t);  // (k is even)
+        }
         float most = 0.f;  // the largest of the row's products with its candidate's rows
 #pragma unroll
         for (int j = 0; j < NC; ++j) {
@@ -363,11 +369,10 @@ fm_umma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmUmmaParams p)
           }
         }
         float f[KP];
-        float probe = 0.f;  // not 0 behind an infinity or a NaN among this row's values, which one of its products also gives
 #pragma unroll
         for (int c = 0; c < KP; c += 2) {
           unpack2(out[c / 2], f[c], f[c + 1]);
-          if (c < p.k) probe = fmaf(f[c], 0.f, fmaf(f[c + 1], 0.f, probe));  // (k is even)
+          if (c < p.k) square_f = ffma2(out[c / 2], out[c / 2], square_f);
         }
         const int64_t cand = (int64_t)tile.cand0 + cand_l;
         __nv_bfloat16* dst = p.FC + (cand * p.n_c + a_row) * p.k;
@@ -382,7 +387,11 @@ fm_umma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmUmmaParams p)
           for (int c = 0; c < KP; c += 2)
             if (c < p.k) *reinterpret_cast<uint32_t*>(dst + c) = pack_bf16(f[c], f[c + 1]);
         }
-        by_hand = probe != 0.f;
+        float t0, t1, f0, f1;
+        unpack2(square_t, t0, t1);
+        unpack2(square_f, f0, f1);
+        // not finite behind an infinity or a NaN among this row's values, which one of its products also gives
+        by_hand = !(f0 + f1 < INFINITY) || (f0 + f1) * (kCancelled * kCancelled) < t0 + t1;
         if (most < kSmallProduct) {
           bool zeros = most == 0.f;  // a row of zeros
 #pragma unroll
