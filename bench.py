@@ -536,7 +536,7 @@ def run_rocs(args):
         "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": "bf16", "data": "synthetic",
         "config": {"workload": WORKLOAD, "l2": f"{N_SETS} rotating input/activation sets, larger than L2",
-                   "step": "plan + request half + candidate half (in-kernel broadcast) + 2 plain layers",
+                   "step": "plan + split layer (both halves in one launch, in-kernel broadcast) + 2 plain layers",
                    "sharding": f"global batch = {world} x the workload's requests, split by request "
                                f"(sharding.shard_batch), {shard.requests.size} requests / {N} candidates per rank"},
         "clocks": clock_summary,

@@ -14,8 +14,9 @@
 // requests x 8 heads of 64 over 64..384 keys, fp32: 69 us; one warp per query row, which re-read the keys
 // for every row, 1450 us.  32 rows and not 64: ragged requests leave less of a tile empty (74 us with 64);
 // 8 x 4 scores per thread 71-90 us, packed fma.rn.f32x2 68 us: the reads, not the issue slots, are the limit.
-// Every row is computed by a fixed sequence over its own request's keys, so results are deterministic
-// and independent of neighbouring candidates (Eq. 1).
+// A row is computed from its own request's keys alone, in a sequence that the batch's shape fixes (whether its blocks of keys go to
+// one group or two follows from the average length and the number of tiles): for a batch of given shape results are deterministic
+// and independent of the other candidates' values (Eq. 1), in batches of different shape the last bits can differ.
 #include <algorithm>
 
 #include "rocs_internal.h"

@@ -401,6 +401,7 @@ fm_umma_kernel(const __grid_constant__ CUtensorMap map_xc, const FmUmmaParams p)
       }
       const uint32_t rows = __ballot_sync(0xffffffffu, by_hand);
       if (rows != 0) {
+        griddep_wait();  // T is read here by threads that have not waited for it themselves
         __syncwarp();  // their values are written again
         const int64_t first = (int64_t)tile.cand0 + q * 32 / NC;  // the warp's candidates
         rows_by_hand<NC>(rows, p.XC + first * p.n_c * p.d, p.TT + (int64_t)tile.req * p.k * p.d, p.P + (int64_t)p.n_r * p.k, p.n_c, p.d, p.k,

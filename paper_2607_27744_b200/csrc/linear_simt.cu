@@ -15,7 +15,7 @@
 // 256 -> 1024 behind it, 46 us for both (56 us with the request rows of the epilogue read one at a time and a part's rows
 // on the same banks; one 64 x 64 tile of 16-wide synchronous slices for every shape:
 // 160 us, half of it the 16 blocks of the request half).
-// Every output is produced by a sequence that depends on the shape only, so results are deterministic and
+// Every output is produced by a sequence that depends on the batch's shape only, so results are deterministic and
 // independent of the other rows' values (Eq. 1).
 #include "rocs_internal.h"
 #include "simt_util.cuh"

@@ -1,7 +1,8 @@
 // General CUDA-core kernels: fp32 FMA arithmetic on fp32 or bf16 storage.  They accept every
 // legal shape, carry the fp32 path, and serve bf16 shapes the tensor-core kernels do not take.
-// Every output row is produced by a fixed instruction sequence over that row's own inputs, so
-// results are bitwise deterministic and independent of neighbouring candidates (Eq. 1).
+// An output row is produced from its own inputs alone, in a sequence that the batch's shape fixes (how many lanes share a product,
+// and whether the request term is W (X X^T) or (W X) X^T, follow from the number of candidates): for a batch of given shape
+// results are bitwise deterministic and independent of the other candidates' values (Eq. 1).
 #include <algorithm>
 
 #include "rocs_internal.h"
