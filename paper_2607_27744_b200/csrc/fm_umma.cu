@@ -7,7 +7,7 @@
 // T, of what is left and of what is left then, which add up to its 24 bits: four warps split it into the tile's stage, where it
 // stays as long as the stage's tiles are of that request.  (Two parts, 17 bits, are as exact on independent inputs; where X^C T is
 // what little its values do not cancel of each other they are not.)  Both terms are fp32 sums and meet behind their
-// products; rows in which they cancel to less than a 64th are computed by hand, both terms added up in front of the product.
+// products; rows in which they cancel to less than a 256th are computed by hand, both terms added up in front of the product.
 // Per 64-wide slice of d shared memory holds [T_3 ; T_2 ; T_1 ; X^C tile] back to back, each part k rows (to a multiple of 8),
 // so that a single tcgen05.mma per 16-deep K step computes
 //     D[128, 3 kp + 128] = X^C_tile * [T_3 ; T_2 ; T_1 ; X^C_tile]^T
@@ -42,7 +42,7 @@ struct FmUmmaParams {
   int32_t stages, stage_bytes;
   const __nv_bfloat16 *P, *XC;  // [n_r + n_c, k], [N, n_c, d]
   const float* TT;              // [R, k, d]
-  __nv_bfloat16* FC;                 // [N, n_c, k]
+  __nv_bfloat16* FC;            // [N, n_c, k]
   uint32_t* status;
 };
 
@@ -66,8 +66,9 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // may count where P_C is large.
 constexpr float kSmallProduct = 0x1p-90f;
 // And rows in which the two terms cancel to less than this part of the request's: what fp32 sums lose of the terms (some 2^-21 of them)
-// stays below 2^-15 of the row then, a hundredth of its rounding to bf16.
-constexpr float kCancelled = 64.f;
+// stays below 2^-13 of the row then, a sixteenth of its rounding to bf16.  (With 64 in place of 256 independent values meet it often
+// enough with two columns, one row in some thousands, to cost a batch of one round of tiles 2.8 us.)
+constexpr float kCancelled = 256.f;
 
 // The upper halves of two values as a bf16 pair, and what is left of them.
 __device__ __forceinline__ uint32_t take_upper(float& a, float& b) {

@@ -157,8 +157,8 @@ def test_bf16_request_term_keeps_its_24_bits(n_c, k, d_emb):
 @pytest.mark.parametrize("n_c,k,d_emb", [(12, 16, 128), (4, 24, 192), (15, 32, 256), (8, 8, 128), (5, 2, 192)])
 def test_bf16_terms_that_cancel(n_c, k, d_emb, scale):
     # The candidates are small changes of their request's rows, and P_R = -P_C: X^C T and (X^C X^C^T) P_C are thousands of times
-    # their sum, and would be off by up to a few 1e-3 of it as sums of their own.  Rows whose sum is below a 64th of a term are added
-    # up before the product; what the others lose (64 times some 2^-21) is a hundredth of FC's rounding.
+    # their sum, and would be off by up to a few 1e-3 of it as sums of their own.  Rows whose sum is below a 256th of a term are added
+    # up before the product; what the others lose (256 times some 2^-21) is a sixteenth of FC's rounding, 2^-8 of it in the norm.
     # Scaled, the squares lie below fp32's range, and their products with P_C do not.
     g = np.random.default_rng(n_c)
     co = wl.offsets_from_counts([7000, 0, 3, 90])
